@@ -94,15 +94,17 @@ gt_status gt_check(void* workspace, void* stream);
  * The traversal runs to exhaustion, so pairs farther than max_dist (bucket max_dist) stay
  * distinct from unreachable pairs (bucket max_dist+1).  Bit-exact and deterministic.
  * Out-of-range col_idx entries are undefined behaviour.
- * Workspace: about 4(G+1) + 4 n_total + 4 G + 1 KB for a packed batch whose graphs have at most 17 066 nodes each and
- * for a single graph below 14 500 nodes (per-graph offsets, and the connected-component label of every node: the search
- * of an undirected graph without a vertex of more than 64 out-edges stops at level max_dist); a single larger graph (it takes a bit-matrix traversal, which is the faster one from there)
- * needs about 7 KB per node for each of min(4, ceil(n/8192)) groups of thread blocks (seven bit
- * matrices of 1 KB rows per group: visited, and one frontier per level up to 5; later levels reuse two of
- * them) plus 1 KB per 33 edges per group (rows for vertices with more than 32 out-edges) and 16 bytes per
- * 32 edges -- 2.0 GB at 65 536 nodes with 786 000 edges -- and a device that supports cooperative
- * launches; a batch that contains a larger graph needs 12 bytes per node of the largest graph for each
- * of up to 2 x (number of SMs) thread blocks.
+ * Workspace (gt_spd_build_workspace says how much): 256 bytes for graphs of up to about 5 000 nodes, whose whole traversal
+ * state fits shared memory; a single graph of up to 22 000 nodes: its edge list once more (2 bytes per edge) and bit planes of
+ * 4 bytes per node, bit of max_dist + 1 and thread block in flight (up to two per SM; 24 MB at 8 192 nodes); a single graph
+ * from 14 500 nodes on at least what its bit-matrix traversal needs (the one used beyond 22 000 nodes): about 7 KB per node
+ * for each of min(4, ceil(n/8192)) groups of thread blocks (seven bit matrices of 1 KB rows per group: visited, and one
+ * frontier per level up to 5; later levels reuse two of them) plus 1 KB per 33 edges per group (rows for vertices with more
+ * than 32 out-edges) and 16 bytes per 32 edges -- 2.0 GB at 65 536 nodes with 786 000 edges -- and a device that supports
+ * cooperative launches; other batches with a larger graph: 4(G+1) + 4 n_total + 4 G bytes (per-graph offsets, and the
+ * connected-component label of every node: the search of an undirected graph without a vertex of more than 64 out-edges
+ * stops at level max_dist), and beyond 17 066 nodes 12 bytes per node of the largest graph for each of up to
+ * 2 x (number of SMs) thread blocks.
  * ------------------------------------------------------------------------------------- */
 size_t gt_spd_build_workspace(const gt_batch* batch, int64_t nnz, int32_t max_dist);
 gt_status gt_spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
@@ -122,10 +124,11 @@ gt_status gt_spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t n
  * holds until the process exits.  The call itself allocates and frees nothing.
  *
  * Same arguments, results and error codes as gt_spd_build, minus the workspace, with these rules:
- *  - Size limit: the batch must satisfy gt_spd_build_workspace(batch, nnz, max_dist) <=
- *    gt_spd_build_static_limit(); in practice a packed batch whose graphs have at most 17 066 nodes each, or a
- *    single graph below 14 500 nodes (larger ones keep their traversal state in the workspace and need far more).  Otherwise
- *    GT_ERR_WORKSPACE is returned and nothing is launched.
+ *  - Size limit: a packed batch whose graphs have at most 17 066 nodes each, or a single graph below 14 500 nodes
+ *    (larger ones keep their traversal state in the workspace and need far more), as far as the offsets and component labels
+ *    of the batch fit the array; every batch with gt_spd_build_workspace(batch, nnz, max_dist) <= gt_spd_build_static_limit()
+ *    does.  (gt_spd_build may use more workspace than that on a graph that this call still builds, more slowly, without it.)
+ *    Otherwise GT_ERR_WORKSPACE is returned and nothing is launched.
  *  - First call per device: the first call made with a given device current looks up the
  *    device address of the built-in array (a one-off set-up step).  Make that first call outside
  *    any stream capture.

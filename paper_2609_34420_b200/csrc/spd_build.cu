@@ -1,21 +1,25 @@
-// gt_spd_build: shortest-path-distance index matrix from CSR by bit-parallel multi-source BFS.
+// gt_spd_build: shortest-path-distance index matrix from CSR.
 //
 // The paper builds the structural-encoding bias from batch topology on the CPU while
 // loading data (Sec. "Preliminaries"; the data-loading stall of the latency model).  Here
-// the index form of that bias is built on the GPU.
+// the index form of that bias is built on the GPU, by one of four kernels (make_plan below):
+//   graphs of up to about 5 000 nodes       pull in shared memory (spd_pull.cu)
+//   one graph of up to 22 000 nodes         the same with edge list and code planes in the workspace (spd_pull_large.cu)
+//   one larger graph                        bit matrices in the workspace (further down)
+//   batches with a larger graph             multi-source frontier push (here)
 //
 // One CTA advances 32 sources at once: bit b of a vertex's 32-bit word belongs to source
 // s0+b.  Per BFS level every vertex with a non-empty frontier word pushes that word to its
-// out-neighbours with a shared-memory OR (high-degree vertices are expanded by the whole
+// out-neighbours with an atomic OR (high-degree vertices are expanded by the whole
 // warp, the rest by their own lane); the newly reached (source, vertex) pairs are then
 // written to the output, lanes holding consecutive vertices so that one warp store fills a
 // contiguous run of one SPD row.  Distances below max_dist are written when they are discovered; at level
 // max_dist everything not reached yet is written as "max_dist or farther" in one pass of full runs, the later
 // levels only push, and "unreachable" (overwriting those bytes) and row padding follow at the end: every byte is
-// written once, unreachable pairs of graphs deeper than max_dist twice, so the HBM traffic is the matrix plus the CSR.  The frontier / next / visited words live in shared memory
-// when 12 bytes per vertex fit, otherwise in an L2-resident slice of the workspace (batches with a
-// graph beyond that size); a single graph beyond that size takes the bit-matrix build further down.
-#include "gt_common.cuh"
+// written once, unreachable pairs of graphs deeper than max_dist twice, so the HBM traffic is the matrix plus the CSR.
+// The frontier / next / visited words live in shared memory when 12 bytes per vertex fit, otherwise in an L2-resident slice
+// of the workspace.
+#include "spd_pull.cuh"
 
 namespace gt {
 namespace {
@@ -887,6 +891,8 @@ constexpr size_t kSmemStateLimit = 200 * 1024;
 constexpr int32_t kDenseMinNodes = 14500;
 
 struct SpdPlan {
+    PullPlan pull;             // used where it fits
+    PullLargePlan large;       // used where it fits
     bool smem_state;
     bool dense;                // single large graph: bit-matrix BFS (persistent cooperative kernel)
     int dense_groups;
@@ -899,9 +905,17 @@ struct SpdPlan {
     size_t batch_start_off, scratch_off, scratch_words_per_cta, comp_off, sym_off, total_bytes;
 };
 
-SpdPlan make_plan(const gt_batch* b, int64_t nnz)
+// `in_place`: the caller has no workspace to speak of (gt_spd_build_static).
+SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_place = false)
 {
     SpdPlan pl{};
+    if (nnz < 0) nnz = 0;
+    // The pull wherever rows and edge list fit shared memory (graphs of about 5 000 nodes); one larger graph without the list,
+    // up to the size from which the bit matrices are faster; the push for batches that contain a larger graph.
+    pl.pull = spd_pull_plan(b, nnz, max_dist);
+    if (pl.pull.fits) { pl.total_bytes = kHeaderBytes; return pl; }
+    if (!in_place) pl.large = spd_pull_large_plan(b, nnz, max_dist);
+    if (pl.large.fits && b->n_total < kDenseMinNodes) { pl.total_bytes = pl.large.total_bytes; return pl; }
     size_t state = spd_state_bytes(b->max_seqlen);
     pl.smem_state = state <= kSmemStateLimit;
     pl.threads = b->max_seqlen <= 1024 ? 256 : (b->max_seqlen <= 4096 ? 512 : 1024);
@@ -930,7 +944,7 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz)
     pl.sym_off = align_up(pl.comp_off + sizeof(int32_t) * (size_t)b->n_total, 256);
     pl.total_bytes = pl.sym_off + sizeof(int32_t) * (size_t)b->n_graphs;
     pl.dense = false;
-    // A single graph takes the bit-matrix build from kDenseMinNodes up: measured on power-law graphs of average degree 12 it
+    // A single graph takes the bit-matrix build from kDenseMinNodes up (where the pull does not serve it): measured on power-law graphs of average degree 12 it
     // overtakes the multi-source BFS between 14 000 and 15 000 nodes (16 384 nodes: 0.98 against 1.65 ms), before the BFS
     // state stops fitting shared memory at 17 066.
     if ((!pl.smem_state || b->n_total >= kDenseMinNodes) && b->n_graphs == 1) {
@@ -965,6 +979,7 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz)
             cudaGetLastError();
         }
     }
+    if (pl.large.total_bytes > pl.total_bytes) pl.total_bytes = pl.large.total_bytes;      // room for both: the test hook asks for the bit matrices
     return pl;
 }
 
@@ -973,27 +988,31 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz)
 
 extern "C" size_t gt_spd_build_workspace(const gt_batch* batch, int64_t nnz, int32_t max_dist)
 {
-    (void)max_dist;
     if (gt::validate_batch(batch) != GT_OK) return 0;
-    return gt::make_plan(batch, nnz).total_bytes;
+    return gt::make_plan(batch, nnz, max_dist < 1 ? 1 : (max_dist > 254 ? 254 : max_dist)).total_bytes;
 }
 
-extern "C" gt_status gt_spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
-                                  const gt_batch* batch, int32_t max_dist,
-                                  const int64_t* spd_offsets, uint8_t* spd_out,
-                                  void* workspace, size_t workspace_bytes, void* stream)
+namespace gt {
+namespace {
+
+gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz, const gt_batch* batch, int32_t max_dist,
+                    const int64_t* spd_offsets, uint8_t* spd_out, void* workspace, size_t workspace_bytes, void* stream, bool in_place)
 {
-    using namespace gt;
     gt_status st = validate_batch(batch);
     if (st != GT_OK) return st;
     if (row_ptr == nullptr || spd_out == nullptr || nnz < 0 || (nnz > 0 && col_idx == nullptr)) return GT_ERR_INVALID_ARG;
     if (max_dist < 1 || max_dist > 254) return GT_ERR_INVALID_ARG;
     if (batch->n_graphs > 1 && spd_offsets == nullptr) return GT_ERR_INVALID_ARG;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
-    SpdPlan pl = make_plan(batch, nnz);
+    SpdPlan pl = make_plan(batch, nnz, max_dist, in_place);
     if (workspace == nullptr || workspace_bytes < pl.total_bytes || misaligned16(workspace)) return GT_ERR_WORKSPACE;
 
     cudaStream_t s = (cudaStream_t)stream;
+    if (pl.pull.fits)
+        return spd_pull_launch(pl.pull, row_ptr, col_idx, batch->n_graphs > 1 ? batch->cu_seqlens : nullptr,
+                               batch->n_graphs > 1 ? spd_offsets : nullptr, batch, max_dist, spd_out, s);
+    if (pl.large.fits && !(pl.dense && g_barrier_overcount))
+        return spd_pull_large_launch(pl.large, row_ptr, col_idx, nnz, batch, max_dist, spd_out, workspace, s);
     uint8_t* ws = (uint8_t*)workspace;
     SpdParams p{};
     p.row_ptr = row_ptr;
@@ -1072,6 +1091,17 @@ extern "C" gt_status gt_spd_build(const int32_t* row_ptr, const int32_t* col_idx
     return GT_OK;
 }
 
+}  // namespace
+}  // namespace gt
+
+extern "C" gt_status gt_spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
+                                  const gt_batch* batch, int32_t max_dist,
+                                  const int64_t* spd_offsets, uint8_t* spd_out,
+                                  void* workspace, size_t workspace_bytes, void* stream)
+{
+    return gt::spd_build(row_ptr, col_idx, nnz, batch, max_dist, spd_offsets, spd_out, workspace, workspace_bytes, stream, false);
+}
+
 extern "C" void gt_test_hook_barrier_overcount(int32_t extra)
 {
     gt::g_barrier_overcount = extra > 0 ? (uint32_t)extra : 0u;
@@ -1124,8 +1154,8 @@ extern "C" gt_status gt_spd_build_static(const int32_t* row_ptr, const int32_t* 
     gt_status st = validate_batch(batch);
     if (st != GT_OK) return st;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
-    const size_t need = gt_spd_build_workspace(batch, nnz, max_dist);
-    if (need == 0) return GT_ERR_INVALID_ARG;
+    if (max_dist < 1 || max_dist > 254) return GT_ERR_INVALID_ARG;
+    const size_t need = make_plan(batch, nnz, max_dist, true).total_bytes;
     if (need > kStaticScratchBytes) {
         if (getenv("GT_DEBUG"))
             fprintf(stderr, "[gt_attn] gt_spd_build_static: this batch needs %zu bytes of scratch, the built-in "
@@ -1136,5 +1166,5 @@ extern "C" gt_status gt_spd_build_static(const int32_t* row_ptr, const int32_t* 
     if ((st = static_scratch_ptr(&scratch)) != GT_OK) return st;
     // the array keeps whatever the previous call left: status words and work counters start at zero
     GT_CUDA_TRY(cudaMemsetAsync(scratch, 0, kHeaderBytes, (cudaStream_t)stream));
-    return gt_spd_build(row_ptr, col_idx, nnz, batch, max_dist, spd_offsets, spd_out, scratch, kStaticScratchBytes, stream);
+    return spd_build(row_ptr, col_idx, nnz, batch, max_dist, spd_offsets, spd_out, scratch, kStaticScratchBytes, stream, true);
 }
