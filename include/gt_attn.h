@@ -355,8 +355,8 @@ gt_status gt_biased_attn_fwd_chunked(const void* q, const void* k, const void* v
  * a contraction instead of the bucket form's scatter.  The backward takes the forward's lse but not its output:
  * the per-query term dout_i . out_i is recomputed in fp32 as sum_j P_ij (dout_i . v_j), because the features have
  * a large common part and a term taken from the rounded bf16 output would leak it into dweights.  Single graph only (n_graphs == 1, else
- * GT_ERR_UNSUPPORTED); head_dim in {32, 64}.  This variant is a correctness-first fp32 path on the CUDA
- * cores (no tensor cores): it is meant for the model sizes the paper trains (1 024 - 8 192 nodes per
+ * GT_ERR_UNSUPPORTED); head_dim in {32, 64}.  This variant keeps fp32 probabilities and score gradients (they enter the
+ * tensor-core products as three bf16 terms each): it is meant for the model sizes the paper trains (1 024 - 8 192 nodes per
  * batch), not for the 65 536-node benchmark.  The forward needs no workspace and has no device status.
  * ------------------------------------------------------------------------------------- */
 gt_status gt_feature_attn_fwd(const void* q, const void* k, const void* v, const uint8_t* features, const float* weights,

@@ -4,12 +4,24 @@
 // only, the linear form is the reading taken here).  The bias gradient is a plain contraction,
 // dW[h][c] = sum_ij dS_ij f[i][j][c], instead of the scatter of the bucket form.
 //
-// This path is written for correctness first (plain fp32 CUDA cores, no tensor cores): one warp owns a few
-// query rows (forward; backward pass for dQ and dW) or a few key rows (backward pass for dK and dV) and walks
-// over 32-row tiles of the other side that the thread block stages in shared memory, transposed with a padded pitch
-// ([channel][row], 33 floats per channel), so that a lane reads either its row's column or its channels' entries
-// without bank conflicts; the rest are broadcasts.
-// Every output element has one owning warp: no atomics except the fp64 adds of the 4 x H weight gradients.
+// The contractions run on the tensor cores without giving up fp32: the bf16 inputs are exact operands, and a probability or
+// a score gradient, an fp32 number, goes in as three bf16 terms (8 + 8 + 8 bits of mantissa: the sum is the number), so the
+// products are those of the fp32 form; sums are fp32 and the elementwise part is unchanged fp32.  Three kernels of one shape:
+//   forward      a warp owns 16 query rows and walks over keys:   S = Q K^T, online softmax, O += P V
+//   query side   the same rows and keys:  S, dP = dO V^T, then in ONE walk the sums of P dP K and P K (and of P dP f, P f and
+//                P dP); with Delta_i = sum_j P_ij dP_ij known at the end,  dQ_i = sum P dP K - Delta_i sum P K,  and dW alike
+//   key side     a warp owns 16 key rows and walks over queries:  S^T, dP^T, dV += P^T dO, dK += dS^T Q
+// The score fragments of one product are the operand fragments of the next (mma.sync keeps both in registers), a pair's four
+// features are read straight into the lane that holds its score, and Delta is formed from the same P as the gradients: the
+// features have a large common part, which a Delta from a rounded output would turn into an error of dW.  A thread block is
+// two row groups times two halves of each 64-row tile of the other side (small graphs have few rows: the halves keep twice as
+// many warps busy), whose partial results are added at the end.
+//
+// mma.sync and not tcgen05: at the 500 - 8 192 nodes this form is meant for, a 128-row tile per thread block would leave
+// most SMs empty, and the three-term operands would have to travel through tensor memory.
+// What bounds it: latency at ten warps per SM (1 500 nodes have no more rows), with the warp-level MMAs at 36-46 % of their
+// pipe (14 of the 20 contractions are the terms of P and dS) and the issue slots at 41-50 %.  1 500 nodes, H = 8, d = 64:
+// forward 55 us, query side 92 us, key side 85 us; the same sums on the fp32 pipes took 3 000 us.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -19,314 +31,629 @@ namespace gt {
 namespace {
 
 constexpr int kFeat = 4;              // bias features per node pair
-constexpr int kWarps = 8;
-constexpr int kOwn = 4;               // rows owned by a warp
-constexpr int kBlockRows = kWarps * kOwn;
-constexpr int kOther = 32;            // rows of the other side per shared-memory tile (one per lane)
+constexpr int kRows = 32;             // rows of a thread block: two groups of 16
+constexpr int kTile = 64;             // rows of the other side per stage: two halves of 32
+constexpr int kThreads = 128;
 
-__device__ __forceinline__ float warp_max(float x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
-}
-__device__ __forceinline__ float warp_sum(float x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-__device__ __forceinline__ float bf16_at(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Stage rows [r0, r0+32) of head h of a bf16 [n, H, D] tensor: row-major into `rm` [32][D] and, if `tr` is
-// given, transposed into `tr` [D][33].  Rows past n are zero.
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldm4_trans(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool valid)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16u : 0u) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kLeft>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kLeft) : "memory"); }
+
+// Two fp32 numbers as three pairs of bf16 whose sum they are.
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo)
+{
+    auto pack = [](float a, float b) {
+        uint32_t r;
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+        return r;
+    };
+    hi = pack(x0, x1);
+    x0 -= __uint_as_float(hi << 16);
+    x1 -= __uint_as_float(hi & 0xffff0000u);
+    mid = pack(x0, x1);
+    x0 -= __uint_as_float(mid << 16);
+    x1 -= __uint_as_float(mid & 0xffff0000u);
+    lo = pack(x0, x1);
+}
+
+// A tile of rows of D bf16 in shared memory: 16-byte chunks, XOR-swizzled so that eight rows of one chunk column lie in
+// different banks (ldmatrix reads them together).
 template <int D>
-__device__ __forceinline__ void stage_tile(const __nv_bfloat16* __restrict__ x, int32_t n, int32_t n_heads, int32_t h, int32_t r0,
-                                           float* rm, float* tr)
+struct Tile {
+    static constexpr int kRowBytes = 2 * D;
+    static __device__ __forceinline__ uint32_t at(uint32_t base, int row, int chunk)
+    {
+        const int x = D == 64 ? (row & 7) : ((row >> 1) & 3);
+        return base + (uint32_t)(row * kRowBytes + ((chunk ^ x) * 16));
+    }
+    // rows [r0, r0 + kCount) of head h of a [n, H, D] tensor; rows past n are zero
+    template <int kCount>
+    static __device__ __forceinline__ void fetch(uint32_t base, const __nv_bfloat16* __restrict__ x, int32_t n, int32_t n_heads, int32_t h, int32_t r0)
+    {
+        constexpr int kChunks = D / 8;
+#pragma unroll
+        for (int e = 0; e < kCount * kChunks / kThreads; ++e) {
+            const int i = e * kThreads + (int)threadIdx.x, r = i / kChunks, c = i % kChunks;
+            const bool ok = r0 + r < n;
+            cp16(at(base, r, c), x + ((size_t)(ok ? r0 + r : 0) * n_heads + h) * D + c * 8, ok);
+        }
+    }
+    // A fragments (16 rows from `row`, all of D)
+    static __device__ __forceinline__ void load_a(uint32_t (&a)[D / 16][4], uint32_t base, int row, int lane)
+    {
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k) ldm4(a[k], at(base, row + (lane & 15), 2 * k + (lane >> 4)));
+    }
+    // B fragments of 16 rows (two column tiles of the product) for channels 16 k .. : b[0..1] first tile, b[2..3] second
+    static __device__ __forceinline__ void load_b(uint32_t (&b)[4], uint32_t base, int row, int k, int lane)
+    {
+        ldm4(b, at(base, row + (lane & 7) + ((lane >> 4) << 3), 2 * k + ((lane >> 3) & 1)));
+    }
+    // B fragments of 16 rows as the contracted index, channels 16 c .. (two column tiles)
+    static __device__ __forceinline__ void load_bt(uint32_t (&b)[4], uint32_t base, int row, int c, int lane)
+    {
+        ldm4_trans(b, at(base, row + (lane & 15), 2 * c + (lane >> 4)));
+    }
+};
+
+// S (16 x 32, two blocks of 16 columns) = A (16 x D) B^T, B = 32 rows of a tile
+template <int D>
+__device__ __forceinline__ void scores(float (&s)[2][2][4], const uint32_t (&a)[D / 16][4], uint32_t base, int row, int lane)
 {
-    for (int e = threadIdx.x; e < kOther * D; e += blockDim.x) {
-        const int r = e / D, c = e % D;
-        const float v = (r0 + r < n) ? bf16_at(x + ((size_t)(r0 + r) * n_heads + h) * D + c) : 0.f;
-        if (rm) rm[r * D + c] = v;
-        if (tr) tr[c * (kOther + 1) + r] = v;
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) s[b][t][x] = 0.f;
+#pragma unroll
+    for (int k = 0; k < D / 16; ++k) {
+        uint32_t b[4], c[4];
+        Tile<D>::load_b(b, base, row, k, lane);
+        Tile<D>::load_b(c, base, row + 16, k, lane);
+        mma16816(s[0][0], a[k], b[0], b[1]);
+        mma16816(s[0][1], a[k], b[2], b[3]);
+        mma16816(s[1][0], a[k], c[0], c[1]);
+        mma16816(s[1][1], a[k], c[2], c[3]);
     }
 }
 
-__device__ __forceinline__ float feature_bias(const uint8_t* __restrict__ feat, int32_t n, int32_t i, int32_t j, const float (&w)[kFeat],
-                                              uint32_t* raw = nullptr)
+// Two such products with A read from 16 rows of a tile as it goes.  Their steps alternate: an MMA that adds to the result of
+// the one before it would wait for it.
+template <int D>
+__device__ __forceinline__ void two_scores(float (&s)[2][4], uint32_t own_s, float (&u)[2][4], uint32_t own_u, int own_row,
+                                           uint32_t base_s, uint32_t base_u, int row, int lane)
 {
-    const uint32_t f4 = *(const uint32_t*)(feat + ((size_t)i * n + j) * kFeat);
-    if (raw) *raw = f4;
-    return w[0] * (float)(f4 & 0xffu) + w[1] * (float)((f4 >> 8) & 0xffu) + w[2] * (float)((f4 >> 16) & 0xffu) + w[3] * (float)(f4 >> 24);
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) s[t][x] = u[t][x] = 0.f;
+#pragma unroll
+    for (int k = 0; k < D / 16; ++k) {
+        uint32_t a[4], b[4], c[4], d[4];
+        ldm4(a, Tile<D>::at(own_s, own_row + (lane & 15), 2 * k + (lane >> 4)));
+        Tile<D>::load_b(b, base_s, row, k, lane);
+        ldm4(c, Tile<D>::at(own_u, own_row + (lane & 15), 2 * k + (lane >> 4)));
+        Tile<D>::load_b(d, base_u, row, k, lane);
+        mma16816(s[0], a, b[0], b[1]);
+        mma16816(u[0], c, d[0], d[1]);
+        mma16816(s[1], a, b[2], b[3]);
+        mma16816(u[1], c, d[2], d[3]);
+    }
+}
+
+// a 16 x 16 block of fp32 in score fragments -> its three bf16 operand fragments
+__device__ __forceinline__ void split_block(const float (&p)[2][4], uint32_t (&t)[3][4])
+{
+    split3(p[0][0], p[0][1], t[0][0], t[1][0], t[2][0]);
+    split3(p[0][2], p[0][3], t[0][1], t[1][1], t[2][1]);
+    split3(p[1][0], p[1][1], t[0][2], t[1][2], t[2][2]);
+    split3(p[1][2], p[1][3], t[0][3], t[1][3], t[2][3]);
+}
+
+// Two sums (16 x 16 of 16 x D): acc += P (16 x 16, three terms; smallest first) times 16 rows of a tile, steps alternating.
+__device__ __forceinline__ void two_sums(float (&u0)[4], float (&u1)[4], const uint32_t (&t)[3][4], const uint32_t (&b)[4],
+                                         float (&v0)[4], float (&v1)[4], const uint32_t (&r)[3][4], const uint32_t (&d)[4])
+{
+#pragma unroll
+    for (int x = 2; x >= 0; --x) {
+        mma16816(u0, t[x], b[0], b[1]);
+        mma16816(v0, r[x], d[0], d[1]);
+        mma16816(u1, t[x], b[2], b[3]);
+        mma16816(v1, r[x], d[2], d[3]);
+    }
+}
+
+__device__ __forceinline__ void unpack_features(uint32_t f4, float (&f)[kFeat])
+{
+    // byte -> fp32 without the conversion pipe: 2^15 + b has b in its mantissa's second byte, and 2^15 comes off exactly
+#pragma unroll
+    for (int c = 0; c < kFeat; ++c) f[c] = __uint_as_float(__byte_perm(f4, 0x47000000u, 0x7404u | ((uint32_t)c << 4))) - 32768.f;
+}
+
+struct FeatureArgs {
+    const __nv_bfloat16 *q, *k, *v, *dout;
+    const uint32_t* feat;         // the four features of a pair as one word, [n][n]
+    const float* weights;
+    const float* lse_in;
+    float* lse;
+    float* delta;                 // [H][n]
+    double* dw_part;              // [H][row blocks][4]
+    __nv_bfloat16 *out, *dq, *dk, *dv;
+    float* dweights;
+    int32_t n, n_heads;
+    float scale;                  // 1 / sqrt(d)
+};
+
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+
+// 2^x to 2 ulp (0 for -inf)
+__device__ __forceinline__ float exp2_of(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// words of pairs (i, j) and (i, j + 1), j even; out of range: 0
+__device__ __forceinline__ uint2 feature_pair(const uint32_t* __restrict__ feat, int32_t n, bool pairs, int32_t i, int32_t j)
+{
+    uint2 r = make_uint2(0u, 0u);
+    if (i < n && j < n) {
+        const uint32_t* at = feat + (size_t)i * n + j;
+        if (pairs) r = __ldg((const uint2*)at);            // n even: j + 1 < n too
+        else {
+            r.x = __ldg(at);
+            if (j + 1 < n) r.y = __ldg(at + 1);
+        }
+    }
+    return r;
+}
+__device__ __forceinline__ float bias_of(uint32_t f4, const float (&w)[kFeat])
+{
+    float f[kFeat];
+    unpack_features(f4, f);
+    return w[0] * f[0] + w[1] * f[1] + w[2] * f[2] + w[3] * f[3];
+}
+// sum over the four lanes that share a fragment row
+__device__ __forceinline__ float quad_sum(float x)
+{
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    return x + __shfl_xor_sync(0xffffffffu, x, 2);
+}
+__device__ __forceinline__ float quad_max(float x)
+{
+    x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
+    return fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Forward: a warp owns kOwn query rows; lane l takes key j0 + l of the current key tile.
+// Forward: a warp owns 16 query rows and one half of the keys.
 // ---------------------------------------------------------------------------------------------------
 template <int D>
-__global__ void __launch_bounds__(kWarps * 32) feature_fwd_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                                                                   const __nv_bfloat16* __restrict__ v, const uint8_t* __restrict__ feat,
-                                                                   const float* __restrict__ weights, __nv_bfloat16* __restrict__ out,
-                                                                   float* __restrict__ lse, int32_t n, int32_t n_heads)
+__global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 {
-    __shared__ float s_q[kBlockRows * D];
-    __shared__ float s_kt[D * (kOther + 1)];
-    __shared__ float s_v[kOther * D];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kTileBytes = kTile * 2 * D;
+    __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];                    // two stages of K and V
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
     const int h = blockIdx.y;
-    const int32_t i0 = blockIdx.x * kBlockRows;
-    const float scale = 1.0f / sqrtf((float)D);
+    const int32_t n = p.n, i0 = (int32_t)blockIdx.x * kRows + 16 * group;
+    const int g = lane >> 2, t4 = lane & 3;
+    const uint32_t base = smem_addr(s_tiles);
+    const bool pairs = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.feat) & 7u) == 0;
     float w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = weights[h * kFeat + c];
-    for (int e = threadIdx.x; e < kBlockRows * D; e += blockDim.x) {
-        const int r = e / D, c = e % D;
-        s_q[e] = (i0 + r < n) ? bf16_at(q + ((size_t)(i0 + r) * n_heads + h) * D + c) * scale : 0.f;
-    }
-    constexpr int kC = D / 32;                 // output channels per lane: c = lane + 32 * t
-    float m[kOwn], l[kOwn], o[kOwn][kC];
+    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c] * kLog2e;      // scores in units of log 2
+    const float scale = p.scale * kLog2e;
+
+    uint32_t qa[D / 16][4];
+    Tile<D>::template fetch<kRows>(base, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    cp_commit();
+    cp_wait<0>();
+    __syncthreads();
+    Tile<D>::load_a(qa, base, 16 * group, lane);
+    __syncthreads();
+
+    float o[D / 8][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
 #pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-        m[r] = -INFINITY; l[r] = 0.f;
+    for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-        for (int t = 0; t < kC; ++t) o[r][t] = 0.f;
-    }
-    for (int32_t j0 = 0; j0 < n; j0 += kOther) {
+        for (int x = 0; x < 4; ++x) o[c][x] = 0.f;
+    const int32_t n_tiles = (n + kTile - 1) / kTile;
+    auto stage = [&](int32_t tile) {
+        const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
+        Tile<D>::template fetch<kTile>(at, p.k, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
+        cp_commit();
+    };
+    stage(0);
+    for (int32_t tile = 0; tile < n_tiles; ++tile) {
+        const int32_t j0 = tile * kTile + 32 * half;
+        uint2 f[2][2][2];                                                        // [16 keys][column tile][row g, g + 8]
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) f[b][t][r] = feature_pair(p.feat, n, pairs, i0 + g + 8 * r, j0 + 16 * b + 8 * t + 2 * t4);
+        if (tile + 1 < n_tiles) { stage(tile + 1); cp_wait<1>(); } else cp_wait<0>();
         __syncthreads();
-        stage_tile<D>(k, n, n_heads, h, j0, nullptr, s_kt);
-        stage_tile<D>(v, n, n_heads, h, j0, s_v, nullptr);
-        __syncthreads();
-        const int32_t j = j0 + lane;
+        const uint32_t kt = base + (uint32_t)(tile & 1) * 2 * kTileBytes, vt = kt + kTileBytes;
+        const bool ragged = j0 + 32 > n;
+        float s[2][2][4], top[2] = {m[0], m[1]};
+        scores<D>(s, qa, kt, 32 * half, lane);
 #pragma unroll
-        for (int r = 0; r < kOwn; ++r) {
-            const int32_t i = i0 + warp * kOwn + r;
-            if (i >= n) continue;                                   // warp-uniform
-            float s = -INFINITY;
-            if (j < n) {
-                float acc = 0.f;
-                const float* qr = s_q + (warp * kOwn + r) * D;
-#pragma unroll 8
-                for (int c = 0; c < D; ++c) acc += qr[c] * s_kt[c * (kOther + 1) + lane];
-                s = acc + feature_bias(feat, n, i, j, w);           // bias added before the softmax statistics
+        for (int b = 0; b < 2; ++b) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
+                    const float bias = bias_of(x & 1 ? f[b][t][x >> 1].y : f[b][t][x >> 1].x, w);
+                    s[b][t][x] = s[b][t][x] * scale + bias;                      // bias added before the softmax statistics
+                    if (ragged && j >= n) s[b][t][x] = -INFINITY;
+                    top[x >> 1] = fmaxf(top[x >> 1], s[b][t][x]);
+                }
+        }
+        top[0] = quad_max(top[0]);
+        top[1] = quad_max(top[1]);
+        if (__any_sync(0xffffffffu, top[0] > m[0] || top[1] > m[1])) {
+            const float a0 = m[0] == top[0] ? 1.f : exp2_of(m[0] - top[0]), a1 = m[1] == top[1] ? 1.f : exp2_of(m[1] - top[1]);
+            l[0] *= a0; l[1] *= a1;
+#pragma unroll
+            for (int c = 0; c < D / 8; ++c) { o[c][0] *= a0; o[c][1] *= a0; o[c][2] *= a1; o[c][3] *= a1; }
+            m[0] = top[0]; m[1] = top[1];
+        }
+        const float ref0 = m[0] == -INFINITY ? 0.f : m[0], ref1 = m[1] == -INFINITY ? 0.f : m[1];     // a half without keys so far
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    s[b][t][x] = exp2_of(s[b][t][x] - (x < 2 ? ref0 : ref1));            // 0 for keys past the end
+                    l[x >> 1] += s[b][t][x];
+                }
+            uint32_t pt[3][4];
+            split_block(s[b], pt);
+#pragma unroll
+            for (int c = 0; c < D / 16; c += 2) {
+                uint32_t v0[4], v1[4];
+                Tile<D>::load_bt(v0, vt, 32 * half + 16 * b, c, lane);
+                Tile<D>::load_bt(v1, vt, 32 * half + 16 * b, c + 1, lane);
+                two_sums(o[2 * c], o[2 * c + 1], pt, v0, o[2 * c + 2], o[2 * c + 3], pt, v1);
             }
-            const float m_new = fmaxf(m[r], warp_max(s));
-            const float alpha = expf(m[r] - m_new);                 // first tile: exp(-inf) = 0
-            const float p = expf(s - m_new);                        // 0 for keys past the end
-            l[r] = l[r] * alpha + warp_sum(p);
-            m[r] = m_new;
+        }
+        __syncthreads();
+    }
+    l[0] = quad_sum(l[0]);
+    l[1] = quad_sum(l[1]);
+    // the second half's share, merged by the first
+    float* part = (float*)s_tiles + group * (16 * (D + 2));
+    if (half == 1) {
 #pragma unroll
-            for (int t = 0; t < kC; ++t) o[r][t] *= alpha;
-            for (int jj = 0; jj < kOther; ++jj) {
-                const float pj = __shfl_sync(0xffffffffu, p, jj);
+        for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-                for (int t = 0; t < kC; ++t) o[r][t] += pj * s_v[jj * D + lane + 32 * t];
+            for (int x = 0; x < 4; ++x) part[(g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1)] = o[c][x];
+        if (t4 == 0) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) { part[16 * D + g + 8 * r] = m[r]; part[16 * D + 16 + g + 8 * r] = l[r]; }
+        }
+    }
+    __syncthreads();
+    if (half == 0) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int32_t i = i0 + g + 8 * r;
+            const float m2 = part[16 * D + g + 8 * r], l2 = part[16 * D + 16 + g + 8 * r];
+            const float mm = fmaxf(m[r], m2), a = exp2_of(m[r] - mm), b = m2 == -INFINITY ? 0.f : exp2_of(m2 - mm);
+            const float ll = l[r] * a + l2 * b, inv = 1.0f / ll;
+            if (i < n) {
+#pragma unroll
+                for (int c = 0; c < D / 8; ++c) {
+                    const float* o2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
+                    const float x = (o[c][2 * r] * a + o2[0] * b) * inv, y = (o[c][2 * r + 1] * a + o2[1] * b) * inv;
+                    *(__nv_bfloat162*)(p.out + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) = __floats2bfloat162_rn(x, y);
+                }
+                if (t4 == 0) p.lse[(size_t)h * n + i] = mm * kLn2 + logf(ll);
             }
         }
     }
-#pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-        const int32_t i = i0 + warp * kOwn + r;
-        if (i >= n) continue;
-        const float inv = 1.0f / l[r];
-#pragma unroll
-        for (int t = 0; t < kC; ++t) out[((size_t)i * n_heads + h) * D + lane + 32 * t] = __float2bfloat16_rn(o[r][t] * inv);
-        if (lane == 0) lse[(size_t)h * n + i] = m[r] + logf(l[r]);
-    }
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Backward, query side: a warp owns kOwn query rows and produces their dQ and their share of dW.  It walks over
-// the keys twice: first for Delta_i = sum_j P_ij (dO_i . v_j) (formed from the same fp32 P that the gradients use, so
-// that every row of dS sums to zero to rounding -- the features have a large common part, which a Delta taken from the
-// rounded bf16 output would turn into an error of dW), then for dS.  Delta is also written out for the key-side pass.
+// Backward, query side: dQ, Delta and the row block's share of dW.
 // ---------------------------------------------------------------------------------------------------
 template <int D>
-__global__ void __launch_bounds__(kWarps * 32) feature_bwd_q_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                                                                     const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ dout,
-                                                                     const float* __restrict__ lse, float* __restrict__ delta,
-                                                                     const uint8_t* __restrict__ feat, const float* __restrict__ weights,
-                                                                     __nv_bfloat16* __restrict__ dq, double* __restrict__ dw_acc,
-                                                                     int32_t n, int32_t n_heads)
+__global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs p)
 {
-    __shared__ float s_q[kBlockRows * D];
-    __shared__ float s_do[kBlockRows * D];
-    __shared__ float s_kt[D * (kOther + 1)];     // [channel][key]: a lane reads its key's column, or its channels' row entry
-    __shared__ float s_vt[D * (kOther + 1)];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kTileBytes = kTile * 2 * D;
+    __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];
+    __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' Q and dO (in registers they would cost a block per SM)
+    __shared__ float s_sums[2][16][kFeat + 1];                                    // the second half's P dP and P f per row
+    __shared__ double s_dw[4][kFeat];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
     const int h = blockIdx.y;
-    const int32_t i0 = blockIdx.x * kBlockRows;
-    const float scale = 1.0f / sqrtf((float)D);
+    const int32_t n = p.n, i0 = (int32_t)blockIdx.x * kRows + 16 * group;
+    const int g = lane >> 2, t4 = lane & 3;
+    const uint32_t base = smem_addr(s_tiles);
+    const bool pairs = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.feat) & 7u) == 0;
     float w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = weights[h * kFeat + c];
-    for (int e = threadIdx.x; e < kBlockRows * D; e += blockDim.x) {
-        const int r = e / D, c = e % D;
-        const bool ok = i0 + r < n;
-        s_q[e] = ok ? bf16_at(q + ((size_t)(i0 + r) * n_heads + h) * D + c) * scale : 0.f;
-        s_do[e] = ok ? bf16_at(dout + ((size_t)(i0 + r) * n_heads + h) * D + c) : 0.f;
+    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c] * kLog2e;
+    const float scale = p.scale * kLog2e;
+
+    const uint32_t own_q = smem_addr(s_own), own_d = own_q + kRows * 2 * D;
+    Tile<D>::template fetch<kRows>(own_q, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows>(own_d, p.dout, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    cp_commit();
+
+    float lse[2], xk[D / 8][4], pk[D / 8][4];                                     // sums of P dP K and of P K
+    float xs[2] = {0.f, 0.f}, pf[2][kFeat], xf[kFeat];                            // sums of P dP, P f (per row) and P dP f
+#pragma unroll
+    for (int r = 0; r < 2; ++r) lse[r] = i0 + g + 8 * r < n ? p.lse_in[(size_t)h * n + i0 + g + 8 * r] * kLog2e : INFINITY;     // P = 0
+#pragma unroll
+    for (int c = 0; c < D / 8; ++c)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) xk[c][x] = pk[c][x] = 0.f;
+#pragma unroll
+    for (int c = 0; c < kFeat; ++c) xf[c] = pf[0][c] = pf[1][c] = 0.f;
+    const int32_t n_tiles = (n + kTile - 1) / kTile;
+    auto stage = [&](int32_t tile) {
+        const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
+        Tile<D>::template fetch<kTile>(at, p.k, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
+        cp_commit();
+    };
+    stage(0);
+    for (int32_t tile = 0; tile < n_tiles; ++tile) {
+        const int32_t j0 = tile * kTile + 32 * half;
+        uint2 f[2][2];                                                            // of the next 16 keys
+        auto fetch_features = [&](int b) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) f[t][r] = feature_pair(p.feat, n, pairs, i0 + g + 8 * r, j0 + 16 * b + 8 * t + 2 * t4);
+        };
+        fetch_features(0);
+        if (tile + 1 < n_tiles) { stage(tile + 1); cp_wait<1>(); } else cp_wait<0>();
+        __syncthreads();
+        const uint32_t kt = base + (uint32_t)(tile & 1) * 2 * kTileBytes, vt = kt + kTileBytes;
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b) {
+            float s[2][4], dp[2][4];
+            two_scores<D>(s, own_q, dp, own_d, 16 * group, kt, vt, 32 * half + 16 * b, lane);
+            const bool ragged = j0 + 16 * b + 16 > n;
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int r = x >> 1;
+                    const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
+                    float fv[kFeat];
+                    unpack_features(x & 1 ? f[t][r].y : f[t][r].x, fv);
+                    const float bias = w[0] * fv[0] + w[1] * fv[1] + w[2] * fv[2] + w[3] * fv[3];
+                    float pr = exp2_of(s[t][x] * scale + (bias - lse[r]));
+                    if (ragged && j >= n) pr = 0.f;
+                    const float px = pr * dp[t][x];
+                    s[t][x] = pr;
+                    dp[t][x] = px;
+                    xs[r] += px;
+#pragma unroll
+                    for (int c = 0; c < kFeat; ++c) { pf[r][c] += pr * fv[c]; xf[c] += px * fv[c]; }
+                }
+            if (b == 0) fetch_features(1);
+            uint32_t pt[3][4], xt[3][4];
+            split_block(s, pt);
+            split_block(dp, xt);
+#pragma unroll
+            for (int c = 0; c < D / 16; ++c) {
+                uint32_t kb[4];
+                Tile<D>::load_bt(kb, kt, 32 * half + 16 * b, c, lane);
+                two_sums(pk[2 * c], pk[2 * c + 1], pt, kb, xk[2 * c], xk[2 * c + 1], xt, kb);
+            }
+        }
+        __syncthreads();
     }
-    constexpr int kC = D / 32;
-    float acc_dq[kOwn][kC], acc_dw[kFeat];
 #pragma unroll
-    for (int r = 0; r < kOwn; ++r)
+    for (int r = 0; r < 2; ++r) {
+        xs[r] = quad_sum(xs[r]);
 #pragma unroll
-        for (int t = 0; t < kC; ++t) acc_dq[r][t] = 0.f;
-#pragma unroll
-    for (int c = 0; c < kFeat; ++c) acc_dw[c] = 0.f;
-    float lse_r[kOwn], delta_r[kOwn];
-#pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-        const int32_t i = i0 + warp * kOwn + r;
-        lse_r[r] = i < n ? lse[(size_t)h * n + i] : 0.f;
-        delta_r[r] = 0.f;
+        for (int c = 0; c < kFeat; ++c) pf[r][c] = quad_sum(pf[r][c]);
     }
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int32_t j0 = 0; j0 < n; j0 += kOther) {
-            __syncthreads();
-            stage_tile<D>(k, n, n_heads, h, j0, nullptr, s_kt);
-            stage_tile<D>(v, n, n_heads, h, j0, nullptr, s_vt);
-            __syncthreads();
-            const int32_t j = j0 + lane;
+    float* part = (float*)s_tiles + group * (2 * 16 * D);
+    if (half == 1) {
 #pragma unroll
-            for (int r = 0; r < kOwn; ++r) {
-                const int32_t i = i0 + warp * kOwn + r;
-                if (i >= n) continue;
-                float p = 0.f, dp = 0.f;
-                uint32_t f4 = 0u;
-                if (j < n) {
-                    float s = 0.f;
-                    const float* qr = s_q + (warp * kOwn + r) * D;
-                    const float* dr = s_do + (warp * kOwn + r) * D;
-#pragma unroll 8
-                    for (int c = 0; c < D; ++c) {
-                        s += qr[c] * s_kt[c * (kOther + 1) + lane];
-                        dp += dr[c] * s_vt[c * (kOther + 1) + lane];
-                    }
-                    s += feature_bias(feat, n, i, j, w, &f4);
-                    p = expf(s - lse_r[r]);
-                }
-                if (pass == 0) {
-                    delta_r[r] += warp_sum(p * dp);
-                    continue;
-                }
-                const float ds = p * (dp - delta_r[r]);
-                acc_dw[0] += ds * (float)(f4 & 0xffu);
-                acc_dw[1] += ds * (float)((f4 >> 8) & 0xffu);
-                acc_dw[2] += ds * (float)((f4 >> 16) & 0xffu);
-                acc_dw[3] += ds * (float)(f4 >> 24);
-                for (int jj = 0; jj < kOther; ++jj) {
-                    const float dsj = __shfl_sync(0xffffffffu, ds, jj);
+        for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-                    for (int t = 0; t < kC; ++t) acc_dq[r][t] += dsj * s_kt[(lane + 32 * t) * (kOther + 1) + jj];
-                }
+            for (int x = 0; x < 4; ++x) {
+                const int at = (g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1);
+                part[at] = xk[c][x];
+                part[16 * D + at] = pk[c][x];
+            }
+        if (t4 == 0) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                s_sums[group][g + 8 * r][kFeat] = xs[r];
+#pragma unroll
+                for (int c = 0; c < kFeat; ++c) s_sums[group][g + 8 * r][c] = pf[r][c];
             }
         }
     }
+    __syncthreads();
+    double dw[kFeat];
 #pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-        const int32_t i = i0 + warp * kOwn + r;
-        if (i < n && lane == 0) delta[(size_t)h * n + i] = delta_r[r];
-    }
+    for (int c = 0; c < kFeat; ++c) dw[c] = (double)xf[c];
+    if (half == 0) {
 #pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-        const int32_t i = i0 + warp * kOwn + r;
-        if (i >= n) continue;
+        for (int r = 0; r < 2; ++r) {
+            const int32_t i = i0 + g + 8 * r;
+            const float delta = xs[r] + s_sums[group][g + 8 * r][kFeat];
+            if (i < n) {
 #pragma unroll
-        for (int t = 0; t < kC; ++t) dq[((size_t)i * n_heads + h) * D + lane + 32 * t] = __float2bfloat16_rn(acc_dq[r][t] * scale);
+                for (int c = 0; c < D / 8; ++c) {
+                    const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
+                    const float a = (xk[c][2 * r] + x2[0]) - delta * (pk[c][2 * r] + x2[16 * D]);
+                    const float b = (xk[c][2 * r + 1] + x2[1]) - delta * (pk[c][2 * r + 1] + x2[16 * D + 1]);
+                    *(__nv_bfloat162*)(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) = __floats2bfloat162_rn(a * p.scale, b * p.scale);
+                }
+                if (t4 == 0) p.delta[(size_t)h * n + i] = delta;
+            }
+            if (t4 == 0) {
+#pragma unroll
+                for (int c = 0; c < kFeat; ++c) dw[c] -= (double)delta * ((double)pf[r][c] + (double)s_sums[group][g + 8 * r][c]);
+            }
+        }
     }
 #pragma unroll
     for (int c = 0; c < kFeat; ++c) {
-        const float tot = warp_sum(acc_dw[c]);
-        if (lane == 0) atomicAdd(&dw_acc[h * kFeat + c], (double)tot);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) dw[c] += __shfl_xor_sync(0xffffffffu, dw[c], off);
+        if (lane == 0) s_dw[warp][c] = dw[c];
     }
+    __syncthreads();
+    if (threadIdx.x < kFeat)
+        p.dw_part[((size_t)h * gridDim.x + blockIdx.x) * kFeat + threadIdx.x] =
+            s_dw[0][threadIdx.x] + s_dw[1][threadIdx.x] + s_dw[2][threadIdx.x] + s_dw[3][threadIdx.x];
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Backward, key side: a warp owns kOwn key rows and produces their dK and dV; lane l takes query i0 + l.
+// Backward, key side: dK and dV (and, by the first block of a head, the sum of the row blocks' shares of dW).
 // ---------------------------------------------------------------------------------------------------
 template <int D>
-__global__ void __launch_bounds__(kWarps * 32) feature_bwd_kv_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                                                                      const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ dout,
-                                                                      const float* __restrict__ lse, const float* __restrict__ delta,
-                                                                      const uint8_t* __restrict__ feat, const float* __restrict__ weights,
-                                                                      __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-                                                                      int32_t n, int32_t n_heads)
+__global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs p)
 {
-    __shared__ float s_k[kBlockRows * D];
-    __shared__ float s_v[kBlockRows * D];
-    __shared__ float s_qt[D * (kOther + 1)];     // [channel][query]
-    __shared__ float s_dot[D * (kOther + 1)];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kTileBytes = kTile * 2 * D;
+    __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];                    // two stages of Q and dO
+    __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' K and V
+    __shared__ float2 s_row[2][kTile];                                            // {lse / ln 2, Delta} of the queries
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
     const int h = blockIdx.y;
-    const int32_t j0 = blockIdx.x * kBlockRows;
-    const float scale = 1.0f / sqrtf((float)D);
+    const int32_t n = p.n, j0 = (int32_t)blockIdx.x * kRows + 16 * group;
+    const int g = lane >> 2, t4 = lane & 3;
+    const uint32_t base = smem_addr(s_tiles);
+    if (blockIdx.x == 0 && warp == 0) {
+        double dw = 0.0;                                                          // lane: feature lane & 3, every eighth block
+        for (unsigned b = lane >> 2; b < gridDim.x; b += 8) dw += p.dw_part[((size_t)h * gridDim.x + b) * kFeat + (lane & 3)];
+#pragma unroll
+        for (int off = 16; off >= 4; off >>= 1) dw += __shfl_xor_sync(0xffffffffu, dw, off);
+        if (lane < kFeat) p.dweights[h * kFeat + lane] = (float)dw;
+    }
     float w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = weights[h * kFeat + c];
-    for (int e = threadIdx.x; e < kBlockRows * D; e += blockDim.x) {
-        const int r = e / D, c = e % D;
-        const bool ok = j0 + r < n;
-        s_k[e] = ok ? bf16_at(k + ((size_t)(j0 + r) * n_heads + h) * D + c) * scale : 0.f;
-        s_v[e] = ok ? bf16_at(v + ((size_t)(j0 + r) * n_heads + h) * D + c) : 0.f;
-    }
-    constexpr int kC = D / 32;
-    float acc_dk[kOwn][kC], acc_dv[kOwn][kC];
-#pragma unroll
-    for (int r = 0; r < kOwn; ++r)
-#pragma unroll
-        for (int t = 0; t < kC; ++t) { acc_dk[r][t] = 0.f; acc_dv[r][t] = 0.f; }
-    for (int32_t i0 = 0; i0 < n; i0 += kOther) {
-        __syncthreads();
-        stage_tile<D>(q, n, n_heads, h, i0, nullptr, s_qt);
-        stage_tile<D>(dout, n, n_heads, h, i0, nullptr, s_dot);
-        __syncthreads();
-        const int32_t i = i0 + lane;
-        const float lse_i = i < n ? lse[(size_t)h * n + i] : 0.f;
-        const float delta_i = i < n ? delta[(size_t)h * n + i] : 0.f;
-#pragma unroll
-        for (int r = 0; r < kOwn; ++r) {
-            const int32_t j = j0 + warp * kOwn + r;
-            if (j >= n) continue;
-            float p = 0.f, ds = 0.f;
-            if (i < n) {
-                float s = 0.f, dp = 0.f;
-                const float* kr = s_k + (warp * kOwn + r) * D;
-                const float* vr = s_v + (warp * kOwn + r) * D;
-#pragma unroll 8
-                for (int c = 0; c < D; ++c) {
-                    s += kr[c] * s_qt[c * (kOther + 1) + lane];
-                    dp += vr[c] * s_dot[c * (kOther + 1) + lane];
-                }
-                s += feature_bias(feat, n, i, j, w);                // the pair is (query i -> key j)
-                p = expf(s - lse_i);
-                ds = p * (dp - delta_i);
-            }
-            for (int ii = 0; ii < kOther; ++ii) {
-                const float pi = __shfl_sync(0xffffffffu, p, ii), dsi = __shfl_sync(0xffffffffu, ds, ii);
-#pragma unroll
-                for (int t = 0; t < kC; ++t) {
-                    acc_dv[r][t] += pi * s_dot[(lane + 32 * t) * (kOther + 1) + ii];
-                    acc_dk[r][t] += dsi * s_qt[(lane + 32 * t) * (kOther + 1) + ii];
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-        const int32_t j = j0 + warp * kOwn + r;
-        if (j >= n) continue;
-#pragma unroll
-        for (int t = 0; t < kC; ++t) {
-            dv[((size_t)j * n_heads + h) * D + lane + 32 * t] = __float2bfloat16_rn(acc_dv[r][t]);
-            dk[((size_t)j * n_heads + h) * D + lane + 32 * t] = __float2bfloat16_rn(acc_dk[r][t] * scale);
-        }
-    }
-}
+    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c] * kLog2e;
+    const float scale = p.scale * kLog2e;
 
-__global__ void feature_dw_finalize_kernel(const double* __restrict__ dw_acc, float* __restrict__ dweights, int32_t n_w)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_w) dweights[i] = (float)dw_acc[i];
+    const uint32_t own_k = smem_addr(s_own), own_v = own_k + kRows * 2 * D;
+    Tile<D>::template fetch<kRows>(own_k, p.k, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows>(own_v, p.v, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    cp_commit();
+
+    float dk[D / 8][4], dv[D / 8][4];
+#pragma unroll
+    for (int c = 0; c < D / 8; ++c)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) dk[c][x] = dv[c][x] = 0.f;
+    const int32_t n_tiles = (n + kTile - 1) / kTile;
+    auto stage = [&](int32_t tile) {
+        const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
+        Tile<D>::template fetch<kTile>(at, p.q, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile>(at + kTileBytes, p.dout, n, p.n_heads, h, tile * kTile);
+        cp_commit();
+        if (threadIdx.x < kTile) {
+            const int32_t i = tile * kTile + (int32_t)threadIdx.x;
+            s_row[tile & 1][threadIdx.x] = i < n ? make_float2(p.lse_in[(size_t)h * n + i] * kLog2e, p.delta[(size_t)h * n + i]) : make_float2(INFINITY, 0.f);
+        }
+    };
+    stage(0);
+    for (int32_t tile = 0; tile < n_tiles; ++tile) {
+        const int32_t i0 = tile * kTile + 32 * half;
+        uint32_t f[2][4];                                                         // fragment order: (key g, query 2t4), (g, 2t4+1), (g+8, ..)
+        auto fetch_features = [&](int b) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int32_t i = i0 + 16 * b + 8 * t + 2 * t4 + (x & 1), j = j0 + g + 8 * (x >> 1);
+                    f[t][x] = i < n && j < n ? __ldg(p.feat + (size_t)i * n + j) : 0u;         // the pair is (query i -> key j)
+                }
+        };
+        fetch_features(0);
+        if (tile + 1 < n_tiles) { stage(tile + 1); cp_wait<1>(); } else cp_wait<0>();
+        __syncthreads();
+        const uint32_t qt = base + (uint32_t)(tile & 1) * 2 * kTileBytes, dt = qt + kTileBytes;
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b) {
+            float s[2][4], dp[2][4];
+            two_scores<D>(s, own_k, dp, own_v, 16 * group, qt, dt, 32 * half + 16 * b, lane);
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const float2 row = s_row[tile & 1][32 * half + 16 * b + 8 * t + 2 * t4 + (x & 1)];
+                    s[t][x] = exp2_of(s[t][x] * scale + (bias_of(f[t][x], w) - row.x));        // 0 for queries past the end
+                    dp[t][x] = s[t][x] * (dp[t][x] - row.y);
+                }
+            if (b == 0) fetch_features(1);
+            uint32_t pt[3][4], st[3][4];
+            split_block(s, pt);
+            split_block(dp, st);
+#pragma unroll
+            for (int c = 0; c < D / 16; ++c) {
+                uint32_t ob[4], qb[4];
+                Tile<D>::load_bt(ob, dt, 32 * half + 16 * b, c, lane);
+                Tile<D>::load_bt(qb, qt, 32 * half + 16 * b, c, lane);
+                two_sums(dv[2 * c], dv[2 * c + 1], pt, ob, dk[2 * c], dk[2 * c + 1], st, qb);
+            }
+        }
+        __syncthreads();
+    }
+    float* part = (float*)s_tiles + group * (2 * 16 * D);
+    if (half == 1) {
+#pragma unroll
+        for (int c = 0; c < D / 8; ++c)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int at = (g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1);
+                part[at] = dk[c][x];
+                part[16 * D + at] = dv[c][x];
+            }
+    }
+    __syncthreads();
+    if (half == 0) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int32_t j = j0 + g + 8 * r;
+            if (j >= n) continue;
+#pragma unroll
+            for (int c = 0; c < D / 8; ++c) {
+                const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
+                const size_t at = ((size_t)j * p.n_heads + h) * D + 8 * c + 2 * t4;
+                *(__nv_bfloat162*)(p.dk + at) = __floats2bfloat162_rn((dk[c][2 * r] + x2[0]) * p.scale, (dk[c][2 * r + 1] + x2[1]) * p.scale);
+                *(__nv_bfloat162*)(p.dv + at) = __floats2bfloat162_rn(dv[c][2 * r] + x2[16 * D], dv[c][2 * r + 1] + x2[16 * D + 1]);
+            }
+        }
+    }
 }
 
 gt_status check_feature_common(const gt_batch* batch, int32_t n_heads, int32_t head_dim)
@@ -337,6 +664,11 @@ gt_status check_feature_common(const gt_batch* batch, int32_t n_heads, int32_t h
     if (head_dim != 32 && head_dim != 64) return GT_ERR_UNSUPPORTED;
     if (batch->n_graphs != 1 || n_heads > 65535) return GT_ERR_UNSUPPORTED;
     return GT_OK;
+}
+
+size_t dw_part_bytes(int32_t n, int32_t n_heads)
+{
+    return align_up((size_t)n_heads * (size_t)((n + kRows - 1) / kRows) * kFeat * sizeof(double), 256);
 }
 
 }  // namespace
@@ -352,15 +684,18 @@ extern "C" gt_status gt_feature_attn_fwd(const void* q, const void* k, const voi
     if (!q || !k || !v || !features || !weights || !out || !lse) return GT_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(features) & 3u) != 0) return GT_ERR_INVALID_ARG;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
-    const int32_t n = batch->n_total;
-    dim3 grid((unsigned)((n + kBlockRows - 1) / kBlockRows), (unsigned)n_heads);
-    cudaStream_t s = (cudaStream_t)stream;
-    if (head_dim == 64)
-        feature_fwd_kernel<64><<<grid, kWarps * 32, 0, s>>>((const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
-                                                            features, weights, (__nv_bfloat16*)out, lse, n, n_heads);
-    else
-        feature_fwd_kernel<32><<<grid, kWarps * 32, 0, s>>>((const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
-                                                            features, weights, (__nv_bfloat16*)out, lse, n, n_heads);
+    FeatureArgs p{};
+    p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v;
+    p.feat = (const uint32_t*)features;
+    p.weights = weights;
+    p.lse = lse;
+    p.out = (__nv_bfloat16*)out;
+    p.n = batch->n_total;
+    p.n_heads = n_heads;
+    p.scale = 1.0f / sqrtf((float)head_dim);
+    const dim3 grid((unsigned)((p.n + kRows - 1) / kRows), (unsigned)n_heads);
+    if (head_dim == 64) feature_fwd_kernel<64><<<grid, kThreads, 0, (cudaStream_t)stream>>>(p);
+    else feature_fwd_kernel<32><<<grid, kThreads, 0, (cudaStream_t)stream>>>(p);
     GT_CUDA_TRY(cudaGetLastError());
     return GT_OK;
 }
@@ -368,7 +703,7 @@ extern "C" gt_status gt_feature_attn_fwd(const void* q, const void* k, const voi
 extern "C" size_t gt_feature_attn_bwd_workspace(const gt_batch* batch, int32_t n_heads)
 {
     if (gt::validate_batch(batch) != GT_OK || n_heads < 1) return 0;
-    return gt::kHeaderBytes + gt::align_up((size_t)n_heads * gt::kFeat * sizeof(double), 256) + (size_t)batch->n_total * n_heads * sizeof(float);
+    return gt::kHeaderBytes + gt::dw_part_bytes(batch->n_total, n_heads) + (size_t)batch->n_total * n_heads * sizeof(float);
 }
 
 extern "C" gt_status gt_feature_attn_bwd(const void* q, const void* k, const void* v, const void* dout, const float* lse,
@@ -384,24 +719,30 @@ extern "C" gt_status gt_feature_attn_bwd(const void* q, const void* k, const voi
     if ((reinterpret_cast<uintptr_t>(features) & 3u) != 0) return GT_ERR_INVALID_ARG;
     if (workspace == nullptr || workspace_bytes < gt_feature_attn_bwd_workspace(batch, n_heads) || misaligned16(workspace)) return GT_ERR_WORKSPACE;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
-    const int32_t n = batch->n_total;
-    cudaStream_t s = (cudaStream_t)stream;
     uint8_t* ws = (uint8_t*)workspace;
-    double* dw_acc = (double*)(ws + kHeaderBytes);
-    float* delta = (float*)(ws + kHeaderBytes + align_up((size_t)n_heads * kFeat * sizeof(double), 256));
-    GT_CUDA_TRY(cudaMemsetAsync(dw_acc, 0, (size_t)n_heads * kFeat * sizeof(double), s));
-    dim3 grid((unsigned)((n + kBlockRows - 1) / kBlockRows), (unsigned)n_heads);
-    const __nv_bfloat16 *qb = (const __nv_bfloat16*)q, *kb = (const __nv_bfloat16*)k, *vb = (const __nv_bfloat16*)v;
-    const __nv_bfloat16* dob = (const __nv_bfloat16*)dout;
+    FeatureArgs p{};
+    p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v; p.dout = (const __nv_bfloat16*)dout;
+    p.feat = (const uint32_t*)features;
+    p.weights = weights;
+    p.lse_in = lse;
+    p.dw_part = (double*)(ws + kHeaderBytes);
+    p.delta = (float*)(ws + kHeaderBytes + dw_part_bytes(batch->n_total, n_heads));
+    p.dq = (__nv_bfloat16*)dq; p.dk = (__nv_bfloat16*)dk; p.dv = (__nv_bfloat16*)dv;
+    p.dweights = dweights;
+    p.n = batch->n_total;
+    p.n_heads = n_heads;
+    p.scale = 1.0f / sqrtf((float)head_dim);
+    const dim3 grid((unsigned)((p.n + kRows - 1) / kRows), (unsigned)n_heads);
+    cudaStream_t s = (cudaStream_t)stream;
     if (head_dim == 64) {
-        feature_bwd_q_kernel<64><<<grid, kWarps * 32, 0, s>>>(qb, kb, vb, dob, lse, delta, features, weights, (__nv_bfloat16*)dq, dw_acc, n, n_heads);
-        feature_bwd_kv_kernel<64><<<grid, kWarps * 32, 0, s>>>(qb, kb, vb, dob, lse, delta, features, weights, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n, n_heads);
+        feature_bwd_q_kernel<64><<<grid, kThreads, 0, s>>>(p);
+        GT_CUDA_TRY(cudaGetLastError());
+        feature_bwd_kv_kernel<64><<<grid, kThreads, 0, s>>>(p);
     } else {
-        feature_bwd_q_kernel<32><<<grid, kWarps * 32, 0, s>>>(qb, kb, vb, dob, lse, delta, features, weights, (__nv_bfloat16*)dq, dw_acc, n, n_heads);
-        feature_bwd_kv_kernel<32><<<grid, kWarps * 32, 0, s>>>(qb, kb, vb, dob, lse, delta, features, weights, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n, n_heads);
+        feature_bwd_q_kernel<32><<<grid, kThreads, 0, s>>>(p);
+        GT_CUDA_TRY(cudaGetLastError());
+        feature_bwd_kv_kernel<32><<<grid, kThreads, 0, s>>>(p);
     }
-    GT_CUDA_TRY(cudaGetLastError());
-    feature_dw_finalize_kernel<<<1, 256, 0, s>>>(dw_acc, dweights, n_heads * kFeat);
     GT_CUDA_TRY(cudaGetLastError());
     return GT_OK;
 }
