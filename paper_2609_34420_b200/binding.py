@@ -146,9 +146,24 @@ class Batch:
     cu_seqlens: Optional[torch.Tensor] = None
     spd_offsets: Optional[torch.Tensor] = None
 
+    def __setattr__(self, name, value):
+        self.__dict__.pop("_c", None)
+        self.__dict__[name] = value
+
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k != "_c"}      # (pointers do not travel)
+
     def c_struct(self) -> _GtBatch:
-        return _GtBatch(self.n_total, self.n_graphs, _ptr(self.cu_seqlens),
-                        self.n_total if self.max_seqlen is None else self.max_seqlen)
+        return self._c_pair()[0]
+
+    def _c_pair(self):
+        """The C struct and its ctypes reference, made once: a call on a batch passes the same ones every time."""
+        cu = _ptr(self.cu_seqlens)
+        pair = self.__dict__.get("_c")
+        if pair is None or pair[2] != cu:
+            c = _GtBatch(self.n_total, self.n_graphs, cu, self.n_total if self.max_seqlen is None else self.max_seqlen)
+            pair = self.__dict__["_c"] = (c, ctypes.byref(c), cu)
+        return pair
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -160,7 +175,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """Handle of torch's current stream on the current device (without making a Stream object for it)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _raise(status: int, where: str) -> None:
@@ -181,8 +197,8 @@ def gt_check(workspace: torch.Tensor) -> None:
 
 # ------------------------------------------------------------------------------------------
 def gt_spd_build_workspace(batch: Batch, nnz: int, max_dist: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_spd_build_workspace(ctypes.byref(b), int(nnz), int(max_dist)))
+    b = batch._c_pair()[1]
+    return int(lib().gt_spd_build_workspace(b, int(nnz), int(max_dist)))
 
 
 def gt_spd_build(row_ptr: torch.Tensor, col_idx: torch.Tensor, batch: Batch, max_dist: int,
@@ -191,8 +207,8 @@ def gt_spd_build(row_ptr: torch.Tensor, col_idx: torch.Tensor, batch: Batch, max
     nnz = int(col_idx.numel())
     if workspace is None:
         workspace = _workspace(gt_spd_build_workspace(batch, nnz, max_dist), row_ptr.device)
-    b = batch.c_struct()
-    st = lib().gt_spd_build(_ptr(row_ptr), _ptr(col_idx) if nnz else None, nnz, ctypes.byref(b), int(max_dist),
+    b = batch._c_pair()[1]
+    st = lib().gt_spd_build(_ptr(row_ptr), _ptr(col_idx) if nnz else None, nnz, b, int(max_dist),
                             _ptr(batch.spd_offsets), _ptr(spd_out), _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_spd_build")
     return workspace
@@ -208,15 +224,15 @@ def gt_spd_build_static(row_ptr: torch.Tensor, col_idx: torch.Tensor, batch: Bat
     library (one per device, shared by every call, so calls that overlap on the GPU race).
     Raises GtError(GT_ERR_WORKSPACE) when the batch needs more than gt_spd_build_static_limit()."""
     nnz = int(col_idx.numel())
-    b = batch.c_struct()
-    st = lib().gt_spd_build_static(_ptr(row_ptr), _ptr(col_idx) if nnz else None, nnz, ctypes.byref(b), int(max_dist),
+    b = batch._c_pair()[1]
+    st = lib().gt_spd_build_static(_ptr(row_ptr), _ptr(col_idx) if nnz else None, nnz, b, int(max_dist),
                                    _ptr(batch.spd_offsets), _ptr(spd_out), _stream())
     _raise(st, "gt_spd_build_static")
 
 
 def gt_biased_attn_fwd_workspace(batch: Batch, n_heads: int, head_dim: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_biased_attn_fwd_workspace(ctypes.byref(b), n_heads, head_dim))
+    b = batch._c_pair()[1]
+    return int(lib().gt_biased_attn_fwd_workspace(b, n_heads, head_dim))
 
 
 def gt_biased_attn_fwd(q, k, v, spd, bias, batch: Batch, max_dist: int, out, lse,
@@ -224,9 +240,9 @@ def gt_biased_attn_fwd(q, k, v, spd, bias, batch: Batch, max_dist: int, out, lse
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_fwd_workspace(batch, H, d), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_biased_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(spd), _ptr(batch.spd_offsets), _ptr(bias),
-                                  ctypes.byref(b), H, d, int(max_dist), _ptr(out), _ptr(lse),
+                                  b, H, d, int(max_dist), _ptr(out), _ptr(lse),
                                   _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_biased_attn_fwd")
     return workspace
@@ -238,17 +254,17 @@ def gt_biased_attn_fwd_ex(q, k, v, spd, bias, batch: Batch, max_dist: int, out, 
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_fwd_workspace(batch, H, d), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_biased_attn_fwd_ex(_ptr(q), _ptr(k), _ptr(v), _ptr(spd), _ptr(batch.spd_offsets), _ptr(bias),
-                                     ctypes.byref(b), H, d, int(max_dist), _ptr(out), _ptr(lse), _ptr(out_f32),
+                                     b, H, d, int(max_dist), _ptr(out), _ptr(lse), _ptr(out_f32),
                                      _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_biased_attn_fwd_ex")
     return workspace
 
 
 def gt_biased_attn_bwd_workspace(batch: Batch, n_heads: int, head_dim: int, max_dist: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_biased_attn_bwd_workspace(ctypes.byref(b), n_heads, head_dim, max_dist))
+    b = batch._c_pair()[1]
+    return int(lib().gt_biased_attn_bwd_workspace(b, n_heads, head_dim, max_dist))
 
 
 def gt_biased_attn_bwd(q, k, v, out, dout, lse, spd, bias, batch: Batch, max_dist: int, dq, dk, dv, dbias,
@@ -256,9 +272,9 @@ def gt_biased_attn_bwd(q, k, v, out, dout, lse, spd, bias, batch: Batch, max_dis
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_bwd_workspace(batch, H, d, max_dist), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_biased_attn_bwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(dout), _ptr(lse), _ptr(spd),
-                                  _ptr(batch.spd_offsets), _ptr(bias), ctypes.byref(b), H, d, int(max_dist),
+                                  _ptr(batch.spd_offsets), _ptr(bias), b, H, d, int(max_dist),
                                   _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbias),
                                   _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_biased_attn_bwd")
@@ -271,9 +287,9 @@ def gt_biased_attn_bwd_ex(q, k, v, out, dout, lse, spd, bias, batch: Batch, max_
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_bwd_workspace(batch, H, d, max_dist), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_biased_attn_bwd_ex(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(dout), _ptr(lse), _ptr(spd),
-                                     _ptr(batch.spd_offsets), _ptr(bias), ctypes.byref(b), H, d, int(max_dist),
+                                     _ptr(batch.spd_offsets), _ptr(bias), b, H, d, int(max_dist),
                                      _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbias), _ptr(out_f32),
                                      _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_biased_attn_bwd_ex")
@@ -285,8 +301,8 @@ def gt_spd_validate(spd, batch: Batch, max_dist: int, workspace: Optional[torch.
     workspace raises GtError(GT_ERR_BAD_SPD) if there are any, ``gt_spd_validate_count`` gives their number."""
     if workspace is None:
         workspace = _workspace(int(lib().gt_spd_validate_workspace()), spd.device)
-    b = batch.c_struct()
-    st = lib().gt_spd_validate(_ptr(spd), _ptr(batch.spd_offsets), ctypes.byref(b), int(max_dist),
+    b = batch._c_pair()[1]
+    st = lib().gt_spd_validate(_ptr(spd), _ptr(batch.spd_offsets), b, int(max_dist),
                                _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_spd_validate")
     return workspace
@@ -304,8 +320,8 @@ def gt_test_hook_barrier_overcount(extra: int) -> None:
 
 
 def gt_biased_attn_fwd_chunked_workspace(batch: Batch, n_heads: int, head_dim: int, n_kv_chunks: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_biased_attn_fwd_chunked_workspace(ctypes.byref(b), n_heads, head_dim, n_kv_chunks))
+    b = batch._c_pair()[1]
+    return int(lib().gt_biased_attn_fwd_chunked_workspace(b, n_heads, head_dim, n_kv_chunks))
 
 
 def gt_biased_attn_fwd_chunked(q, k, v, spd, bias, batch: Batch, max_dist: int, out, lse, n_kv_chunks: int,
@@ -314,9 +330,9 @@ def gt_biased_attn_fwd_chunked(q, k, v, spd, bias, batch: Batch, max_dist: int, 
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_fwd_chunked_workspace(batch, H, d, n_kv_chunks), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_biased_attn_fwd_chunked(_ptr(q), _ptr(k), _ptr(v), _ptr(spd), _ptr(batch.spd_offsets), _ptr(bias),
-                                          ctypes.byref(b), H, d, int(max_dist), _ptr(out), _ptr(lse),
+                                          b, H, d, int(max_dist), _ptr(out), _ptr(lse),
                                           int(n_kv_chunks), _ptr(lse_chunks),
                                           _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_biased_attn_fwd_chunked")
@@ -324,8 +340,8 @@ def gt_biased_attn_fwd_chunked(q, k, v, spd, bias, batch: Batch, max_dist: int, 
 
 
 def gt_biased_attn_bwd_chunked_workspace(batch: Batch, n_heads: int, head_dim: int, max_dist: int, n_kv_chunks: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_biased_attn_bwd_chunked_workspace(ctypes.byref(b), n_heads, head_dim, max_dist, n_kv_chunks))
+    b = batch._c_pair()[1]
+    return int(lib().gt_biased_attn_bwd_chunked_workspace(b, n_heads, head_dim, max_dist, n_kv_chunks))
 
 
 def gt_biased_attn_bwd_chunked(q, k, v, out, dout, lse, spd, bias, batch: Batch, max_dist: int, n_kv_chunks: int,
@@ -334,9 +350,9 @@ def gt_biased_attn_bwd_chunked(q, k, v, out, dout, lse, spd, bias, batch: Batch,
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_bwd_chunked_workspace(batch, H, d, max_dist, n_kv_chunks), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_biased_attn_bwd_chunked(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(dout), _ptr(lse), _ptr(spd),
-                                          _ptr(bias), ctypes.byref(b), H, d, int(max_dist), int(n_kv_chunks),
+                                          _ptr(bias), b, H, d, int(max_dist), int(n_kv_chunks),
                                           _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbias), _ptr(dbias_chunks),
                                           _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_biased_attn_bwd_chunked")
@@ -344,8 +360,8 @@ def gt_biased_attn_bwd_chunked(q, k, v, out, dout, lse, spd, bias, batch: Batch,
 
 
 def gt_biased_attn_fwd_step_workspace(batch: Batch, n_heads: int, head_dim: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_biased_attn_fwd_step_workspace(ctypes.byref(b), n_heads, head_dim))
+    b = batch._c_pair()[1]
+    return int(lib().gt_biased_attn_fwd_step_workspace(b, n_heads, head_dim))
 
 
 def gt_biased_attn_fwd_step(q, k, v, spd, bias, batch: Batch, max_dist: int, q_range, kv_range0, kv_range1,
@@ -354,8 +370,8 @@ def gt_biased_attn_fwd_step(q, k, v, spd, bias, batch: Batch, max_dist: int, q_r
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_biased_attn_fwd_step_workspace(batch, H, d), q.device)
-    b = batch.c_struct()
-    st = lib().gt_biased_attn_fwd_step(_ptr(q), _ptr(k), _ptr(v), _ptr(spd), _ptr(bias), ctypes.byref(b), H, d,
+    b = batch._c_pair()[1]
+    st = lib().gt_biased_attn_fwd_step(_ptr(q), _ptr(k), _ptr(v), _ptr(spd), _ptr(bias), b, H, d,
                                        int(max_dist), int(q_range[0]), int(q_range[1]),
                                        int(kv_range0[0]), int(kv_range0[1]), int(kv_range1[0]), int(kv_range1[1]),
                                        _ptr(o_acc), _ptr(lse_acc), _ptr(out),
@@ -365,8 +381,8 @@ def gt_biased_attn_fwd_step(q, k, v, spd, bias, batch: Batch, max_dist: int, q_r
 
 
 def gt_biased_attn_bwd_step_context_bytes(batch: Batch, n_heads: int, head_dim: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_biased_attn_bwd_step_context_bytes(ctypes.byref(b), n_heads, head_dim))
+    b = batch._c_pair()[1]
+    return int(lib().gt_biased_attn_bwd_step_context_bytes(b, n_heads, head_dim))
 
 
 def gt_biased_attn_bwd_step_prepare(out, dout, lse, spd, batch: Batch, max_dist: int,
@@ -376,13 +392,13 @@ def gt_biased_attn_bwd_step_prepare(out, dout, lse, spd, batch: Batch, max_dist:
     _, H, d = dout.shape
     if context is None:
         context = _workspace(gt_biased_attn_bwd_step_context_bytes(batch, H, d), dout.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     if out_f32 is None:
-        st = lib().gt_biased_attn_bwd_step_prepare(_ptr(out), _ptr(dout), _ptr(lse), _ptr(spd), ctypes.byref(b), H, d,
+        st = lib().gt_biased_attn_bwd_step_prepare(_ptr(out), _ptr(dout), _ptr(lse), _ptr(spd), b, H, d,
                                                    int(max_dist), _ptr(context), context.numel(), _stream())
     else:
         st = lib().gt_biased_attn_bwd_step_prepare_ex(_ptr(out), _ptr(out_f32), _ptr(dout), _ptr(lse), _ptr(spd),
-                                                      ctypes.byref(b), H, d, int(max_dist),
+                                                      b, H, d, int(max_dist),
                                                       _ptr(context), context.numel(), _stream())
     _raise(st, "gt_biased_attn_bwd_step_prepare")
     return context
@@ -391,8 +407,8 @@ def gt_biased_attn_bwd_step_prepare(out, dout, lse, spd, batch: Batch, max_dist:
 def gt_biased_attn_bwd_step(q, k, v, dout, bias, batch: Batch, max_dist: int, q_range, kv_range0, kv_range1,
                             dq_acc, dk_acc, dv_acc, dbias_acc, context: torch.Tensor) -> None:
     _, H, d = q.shape
-    b = batch.c_struct()
-    st = lib().gt_biased_attn_bwd_step(_ptr(q), _ptr(k), _ptr(v), _ptr(dout), _ptr(bias), ctypes.byref(b), H, d, int(max_dist),
+    b = batch._c_pair()[1]
+    st = lib().gt_biased_attn_bwd_step(_ptr(q), _ptr(k), _ptr(v), _ptr(dout), _ptr(bias), b, H, d, int(max_dist),
                                        int(q_range[0]), int(q_range[1]), int(kv_range0[0]), int(kv_range0[1]),
                                        int(kv_range1[0]), int(kv_range1[1]),
                                        _ptr(dq_acc), _ptr(dk_acc), _ptr(dv_acc), _ptr(dbias_acc),
@@ -402,8 +418,8 @@ def gt_biased_attn_bwd_step(q, k, v, dout, bias, batch: Batch, max_dist: int, q_
 
 def gt_biased_attn_bwd_step_finish(dq_acc, dk_acc, dv_acc, dbias_acc, batch: Batch, max_dist: int, dq, dk, dv, dbias) -> None:
     _, H, d = dq_acc.shape
-    b = batch.c_struct()
-    st = lib().gt_biased_attn_bwd_step_finish(_ptr(dq_acc), _ptr(dk_acc), _ptr(dv_acc), _ptr(dbias_acc), ctypes.byref(b), H, d,
+    b = batch._c_pair()[1]
+    st = lib().gt_biased_attn_bwd_step_finish(_ptr(dq_acc), _ptr(dk_acc), _ptr(dv_acc), _ptr(dbias_acc), b, H, d,
                                               int(max_dist), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dbias), _stream())
     _raise(st, "gt_biased_attn_bwd_step_finish")
 
@@ -411,15 +427,15 @@ def gt_biased_attn_bwd_step_finish(dq_acc, dk_acc, dv_acc, dbias_acc, batch: Bat
 def gt_feature_attn_fwd(q, k, v, features, weights, batch: Batch, out, lse) -> None:
     """Forward with the feature bias: features uint8 [N, N, 4], weights fp32 [H, 4]."""
     _, H, d = q.shape
-    b = batch.c_struct()
-    st = lib().gt_feature_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(features), _ptr(weights), ctypes.byref(b), H, d,
+    b = batch._c_pair()[1]
+    st = lib().gt_feature_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(features), _ptr(weights), b, H, d,
                                    _ptr(out), _ptr(lse), _stream())
     _raise(st, "gt_feature_attn_fwd")
 
 
 def gt_feature_attn_bwd_workspace(batch: Batch, n_heads: int) -> int:
-    b = batch.c_struct()
-    return int(lib().gt_feature_attn_bwd_workspace(ctypes.byref(b), n_heads))
+    b = batch._c_pair()[1]
+    return int(lib().gt_feature_attn_bwd_workspace(b, n_heads))
 
 
 def gt_feature_attn_bwd(q, k, v, dout, lse, features, weights, batch: Batch, dq, dk, dv, dweights,
@@ -427,9 +443,9 @@ def gt_feature_attn_bwd(q, k, v, dout, lse, features, weights, batch: Batch, dq,
     _, H, d = q.shape
     if workspace is None:
         workspace = _workspace(gt_feature_attn_bwd_workspace(batch, H), q.device)
-    b = batch.c_struct()
+    b = batch._c_pair()[1]
     st = lib().gt_feature_attn_bwd(_ptr(q), _ptr(k), _ptr(v), _ptr(dout), _ptr(lse), _ptr(features), _ptr(weights),
-                                   ctypes.byref(b), H, d, _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dweights),
+                                   b, H, d, _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dweights),
                                    _ptr(workspace), workspace.numel(), _stream())
     _raise(st, "gt_feature_attn_bwd")
     return workspace
@@ -459,8 +475,8 @@ def gt_feature_encode(features, batch: Batch, codes, vectors, workspace: Optiona
     """Categorical features uint8 [N, N, 4] -> codes (uint8, N rows of pitch N rounded up to 16) and vectors (int32/uint32 [256])."""
     if workspace is None:
         workspace = _workspace(int(lib().gt_feature_encode_workspace()), features.device)
-    b = batch.c_struct()
-    st = lib().gt_feature_encode(_ptr(features), ctypes.byref(b), _ptr(codes), _ptr(vectors), _ptr(workspace),
+    b = batch._c_pair()[1]
+    st = lib().gt_feature_encode(_ptr(features), b, _ptr(codes), _ptr(vectors), _ptr(workspace),
                                  workspace.numel(), _stream())
     _raise(st, "gt_feature_encode")
     return workspace

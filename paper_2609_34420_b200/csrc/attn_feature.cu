@@ -205,8 +205,6 @@ struct FeatureArgs {
     float scale;                  // 1 / sqrt(d)
 };
 
-constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
-
 // 2^x to 2 ulp (0 for -inf)
 __device__ __forceinline__ float exp2_of(float x)
 {
@@ -253,6 +251,8 @@ __device__ __forceinline__ float quad_max(float x)
 template <int D>
 __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 {
+    grid_wait();
+    grid_release();
     constexpr int kTileBytes = kTile * 2 * D;
     __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];                    // two stages of K and V
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
@@ -387,6 +387,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 template <int D>
 __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs p)
 {
+    grid_wait();
+    grid_release();
     constexpr int kTileBytes = kTile * 2 * D;
     __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];
     __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' Q and dO (in registers they would cost a block per SM)
@@ -543,6 +545,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs p)
 {
+    grid_wait();
+    grid_release();
     constexpr int kTileBytes = kTile * 2 * D;
     __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];                    // two stages of Q and dO
     __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' K and V
@@ -694,10 +698,7 @@ extern "C" gt_status gt_feature_attn_fwd(const void* q, const void* k, const voi
     p.n_heads = n_heads;
     p.scale = 1.0f / sqrtf((float)head_dim);
     const dim3 grid((unsigned)((p.n + kRows - 1) / kRows), (unsigned)n_heads);
-    if (head_dim == 64) feature_fwd_kernel<64><<<grid, kThreads, 0, (cudaStream_t)stream>>>(p);
-    else feature_fwd_kernel<32><<<grid, kThreads, 0, (cudaStream_t)stream>>>(p);
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    return launch_overlapped(head_dim == 64 ? feature_fwd_kernel<64> : feature_fwd_kernel<32>, grid, kThreads, 0, (cudaStream_t)stream, p);
 }
 
 extern "C" size_t gt_feature_attn_bwd_workspace(const gt_batch* batch, int32_t n_heads)
@@ -734,15 +735,7 @@ extern "C" gt_status gt_feature_attn_bwd(const void* q, const void* k, const voi
     p.scale = 1.0f / sqrtf((float)head_dim);
     const dim3 grid((unsigned)((p.n + kRows - 1) / kRows), (unsigned)n_heads);
     cudaStream_t s = (cudaStream_t)stream;
-    if (head_dim == 64) {
-        feature_bwd_q_kernel<64><<<grid, kThreads, 0, s>>>(p);
-        GT_CUDA_TRY(cudaGetLastError());
-        feature_bwd_kv_kernel<64><<<grid, kThreads, 0, s>>>(p);
-    } else {
-        feature_bwd_q_kernel<32><<<grid, kThreads, 0, s>>>(p);
-        GT_CUDA_TRY(cudaGetLastError());
-        feature_bwd_kv_kernel<32><<<grid, kThreads, 0, s>>>(p);
-    }
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    st = launch_overlapped(head_dim == 64 ? feature_bwd_q_kernel<64> : feature_bwd_q_kernel<32>, grid, kThreads, 0, s, p);
+    if (st != GT_OK) return st;
+    return launch_overlapped(head_dim == 64 ? feature_bwd_kv_kernel<64> : feature_bwd_kv_kernel<32>, grid, kThreads, 0, s, p);
 }

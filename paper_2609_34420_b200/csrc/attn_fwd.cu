@@ -157,6 +157,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int g = kPartial ? 0 : (int)blockIdx.z;
     const int chunk = kPartial ? (int)blockIdx.z : 0;
 
+    if (p.cu_seqlens) grid_wait();          // a single graph's blocks set up their barriers and tensor memory before they wait
     const int32_t node0 = p.cu_seqlens ? p.cu_seqlens[g] : 0;
     const int32_t n_g = p.cu_seqlens ? p.cu_seqlens[g + 1] - node0 : p.n_total;
     const int32_t q0 = ((int32_t)blockIdx.y + p.q_block0) * kRowsPerCta;
@@ -168,6 +169,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int32_t n_kv = kv_end > kv_begin ? (kv_end - kv_begin + kKvTile - 1) / kKvTile : 0;
 
     if (kPartial && n_kv == 0) {            // empty chunk: weight zero in the merge
+        grid_wait();
         for (int i = tid; i < kRowsPerCta; i += kFwdThreads) {
             int q = q0 + i;
             if (q < n_g) {
@@ -201,6 +203,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         if (p.spd_tma) prefetch_tensormap(&tmap_spd);
     }
     if (warp == 1) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
+    grid_wait();
+    grid_release();
     for (int i = tid; i < 256; i += kFwdThreads)
         s_bias[i] = p.bias[(size_t)h * p.n_buckets + min(i, p.n_buckets - 1)] * kLog2e;
     tc_fence_before();
@@ -636,6 +640,8 @@ __global__ void chunk_merge_kernel(const float* __restrict__ part_o, const float
                                    __nv_bfloat16* __restrict__ out, float* __restrict__ lse, float* __restrict__ lse_chunks,
                                    int32_t n_total, int32_t n_heads, int32_t n_chunks)
 {
+    grid_wait();
+    grid_release();
     constexpr int kVec = D / 4;
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t n_rows = (size_t)n_total * n_heads;
@@ -673,6 +679,8 @@ __global__ void step_merge_kernel(const float* __restrict__ part_o, const float*
                                   float* __restrict__ o_acc, float* __restrict__ lse_acc, __nv_bfloat16* __restrict__ out,
                                   int32_t q_begin, int32_t q_end, int32_t n_total, int32_t n_heads)
 {
+    grid_wait();
+    grid_release();
     constexpr int kVec = D / 4;
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t n_rows = (size_t)(q_end - q_begin) * n_heads;
@@ -730,11 +738,11 @@ gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
         if (p.out_f32 != nullptr)
             kern = p.n_buckets <= 32 ? attn_fwd_kernel<D, false, true, true> : attn_fwd_kernel<D, false, false, true>;
     }
-    GT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::kDynamic));
+    static std::atomic<uint64_t> granted[4] = {};
+    const gt_status st = grant_smem(kern, granted[(p.n_buckets <= 32 ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0)], FwdSmem<D>::kDynamic);
+    if (st != GT_OK) return st;
     dim3 grid((unsigned)p.n_heads, (unsigned)(grid_y > 0 ? grid_y : (batch->max_seqlen + kRowsPerCta - 1) / kRowsPerCta), (unsigned)grid_z);
-    kern<<<grid, kFwdThreads, FwdSmem<D>::kDynamic, s>>>(tq, tk, tv, tspd, p);
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    return launch_overlapped(kern, grid, kFwdThreads, FwdSmem<D>::kDynamic, s, tq, tk, tv, tspd, p);
 }
 
 gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint8_t* spd, const int64_t* spd_offsets,
@@ -855,13 +863,12 @@ extern "C" gt_status gt_biased_attn_fwd_chunked(const void* q, const void* k, co
     const size_t n_thr = rows * (head_dim / 4);
     const unsigned blocks = (unsigned)((n_thr + 255) / 256);
     if (head_dim == 64)
-        chunk_merge_kernel<64><<<blocks, 256, 0, s>>>(p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
+        st = launch_overlapped(chunk_merge_kernel<64>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
                                                       batch->n_total, n_heads, n_kv_chunks);
     else
-        chunk_merge_kernel<32><<<blocks, 256, 0, s>>>(p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
+        st = launch_overlapped(chunk_merge_kernel<32>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
                                                       batch->n_total, n_heads, n_kv_chunks);
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    return st;
 }
 
 extern "C" size_t gt_biased_attn_fwd_step_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim)
@@ -930,11 +937,10 @@ extern "C" gt_status gt_biased_attn_fwd_step(const void* q, const void* k, const
     const size_t n_thr = (size_t)(q_end - q_begin) * n_heads * (head_dim / 4);
     const unsigned blocks = (unsigned)((n_thr + 255) / 256);
     if (head_dim == 64)
-        step_merge_kernel<64><<<blocks, 256, 0, s>>>(p.part_o, p.part_lse, n_parts, o_acc, lse_acc, (__nv_bfloat16*)out,
+        st = launch_overlapped(step_merge_kernel<64>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, n_parts, o_acc, lse_acc, (__nv_bfloat16*)out,
                                                      q_begin, q_end, n, n_heads);
     else
-        step_merge_kernel<32><<<blocks, 256, 0, s>>>(p.part_o, p.part_lse, n_parts, o_acc, lse_acc, (__nv_bfloat16*)out,
+        st = launch_overlapped(step_merge_kernel<32>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, n_parts, o_acc, lse_acc, (__nv_bfloat16*)out,
                                                      q_begin, q_end, n, n_heads);
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    return st;
 }

@@ -4,6 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdio.h>
+#include <stdlib.h>
+
+#include <atomic>
 
 #include "../../include/gt_attn.h"
 
@@ -38,6 +41,44 @@ inline gt_status validate_batch(const gt_batch* b)
             return GT_ERR_CUDA;                                                        \
         }                                                                              \
     } while (0)
+
+// Kernels of this library are launched so that a kernel may start while the one before it in the stream is still running
+// (programmatic dependent launch): its set-up -- barriers, tensor memory, tables in registers -- and the launch itself then
+// overlap with the other's end.  Every such kernel calls grid_wait() before its first access to global memory, which returns
+// when everything before it in the stream is complete and visible, and grid_release() as soon as the next kernel may start
+// its own set-up.  (A kernel that is not of this library releases at its end; one that does not wait starts when all is done.)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+inline gt_status launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem_bytes, cudaStream_t stream, Args&&... args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    GT_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...));
+    return GT_OK;
+}
+
+// Lets a kernel use up to `bytes` of dynamic shared memory, once per device: `granted` is that kernel's own (a bit per device),
+// `bytes` always the same, so it does not matter how many threads ask at once.
+template <class Kernel>
+inline gt_status grant_smem(Kernel kernel, std::atomic<uint64_t>& granted, size_t bytes)
+{
+    int dev = 0;
+    GT_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 64 && ((granted.load(std::memory_order_relaxed) >> dev) & 1u)) return GT_OK;
+    GT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (dev < 64) granted.fetch_or(1ull << dev, std::memory_order_relaxed);
+    return GT_OK;
+}
 
 // Number of SMs of the current device (cached per device).
 int sm_count();

@@ -18,8 +18,6 @@
 // What bounds it: the shared-memory pipe in the level passes (a gathered row costs the bank conflicts of 32 random rows:
 // 3.5 wavefronts for 32 lanes of 4 bytes, 6.2 of 8, 10.6 of 16: wider rows cost less per target), and the stores of the
 // output at the end.
-#include <atomic>
-
 #include "spd_pull.cuh"
 
 namespace gt {
@@ -55,6 +53,8 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
     __shared__ uint16_t s_tpos[kT];          // position of target t
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    grid_wait();
+    grid_release();
     // Which targets of which graph?  In a batch of up to kSorted graphs the larger graphs come first (their blocks take
     // longer, and the last wave is short then): a graph's first block is the number of blocks of all graphs before it in
     // that order.  In a batch of more, graph g owns the blocks from cu[g]/kT + g up to the next graph's first, at least
@@ -480,16 +480,10 @@ size_t pull_state_bytes(int targets, int32_t n, int planes)
 template <int kT>
 gt_status launch(const PullParams& p, const PullPlan& pl, cudaStream_t s)
 {
-    static std::atomic<uint64_t> opted_in{0};          // devices on which the kernel may use the large shared memory
-    int dev = 0;
-    GT_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev >= 64 || !((opted_in.load(std::memory_order_relaxed) >> dev) & 1u)) {
-        GT_CUDA_TRY(cudaFuncSetAttribute(spd_pull_kernel<kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPullSmemLimit));
-        if (dev < 64) opted_in.fetch_or(1ull << dev, std::memory_order_relaxed);
-    }
-    spd_pull_kernel<kT><<<pl.blocks, pl.threads, pl.smem_bytes, s>>>(p);
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    static std::atomic<uint64_t> granted{0};
+    const gt_status st = grant_smem(spd_pull_kernel<kT>, granted, kPullSmemLimit);
+    if (st != GT_OK) return st;
+    return launch_overlapped(spd_pull_kernel<kT>, dim3(pl.blocks), (unsigned)pl.threads, pl.smem_bytes, s, p);
 }
 
 }  // namespace

@@ -12,7 +12,6 @@
 // those of its edges), then the bank conflicts of the row gathers, 3.5 wavefronts for 32 edges (spd_pull.cu).  Power-law
 // graphs of degree 12 against the frontier push that served them before: 12 000 nodes 915 -> 417 us, 14 400 nodes 1 395 ->
 // 632 us; against the bit-matrix build 16 384 nodes 920 -> 738 us; a graph of degree 10 and 8 192 nodes 374 -> 163 us.
-#include <atomic>
 #include <type_traits>
 
 #include "spd_pull.cuh"
@@ -55,6 +54,8 @@ __global__ void __launch_bounds__(1024, 1) spd_large_order_kernel(LargeParams p)
     uint16_t* degree = (uint16_t*)(key + n);           // of a vertex
     uint16_t* sorted = degree + n;                     // by position
     if (threadIdx.x < kLargeBins) s_bin[threadIdx.x] = 0;
+    grid_wait();
+    grid_release();
     for (int v0 = threadIdx.x; v0 < n; v0 += 8 * blockDim.x) {
         int32_t e0[8], e1[8];
 #pragma unroll
@@ -118,6 +119,8 @@ __global__ void __launch_bounds__(1024, 1) spd_large_order_kernel(LargeParams p)
 // The lists; a thread block per hub or group, so that no warp walks along many edges.  A vertex' own number fills up.
 __global__ void __launch_bounds__(256) spd_large_lists_kernel(LargeParams p)
 {
+    grid_wait();
+    grid_release();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n_hubs = (int)p.counts[0];
     int task = (int)blockIdx.x;
@@ -152,6 +155,8 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
     extern __shared__ __align__(16) uint8_t large_smem[];
     __shared__ uint32_t s_live[3], s_hub_at[kCachedHubs + 1];
     __shared__ uint16_t s_tpos[kTargets], s_hub[kCachedHubs];
+    grid_wait();
+    grid_release();
     const int n = p.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const uint32_t row_words = (uint32_t)pull_align(4 * (size_t)n) / 4;
     uint32_t* const rows0 = (uint32_t*)large_smem;
@@ -338,17 +343,6 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
     }
 }
 
-gt_status opt_in(const void* kernel, std::atomic<uint64_t>& done)
-{
-    int dev = 0;
-    GT_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev >= 64 || !((done.load(std::memory_order_relaxed) >> dev) & 1u)) {
-        GT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLargeSmemLimit));
-        if (dev < 64) done.fetch_or(1ull << dev, std::memory_order_relaxed);
-    }
-    return GT_OK;
-}
-
 }  // namespace
 
 PullLargePlan spd_pull_large_plan(const gt_batch* b, int64_t nnz, int32_t max_dist)
@@ -393,18 +387,14 @@ gt_status spd_pull_large_launch(const PullLargePlan& pl, const int32_t* row_ptr,
     p.n_pad = pl.n_pad;
     p.max_dist = max_dist;
     p.n_planes = pull_planes(max_dist);
-    static std::atomic<uint64_t> order_done{0}, pull_done{0};
+    static std::atomic<uint64_t> order_granted{0}, pull_granted{0};
     gt_status st;
-    if ((st = opt_in((const void*)spd_large_order_kernel, order_done)) != GT_OK) return st;
-    if ((st = opt_in((const void*)spd_large_pull_kernel, pull_done)) != GT_OK) return st;
-    spd_large_order_kernel<<<1, 1024, 8 * (size_t)p.n, s>>>(p);
-    GT_CUDA_TRY(cudaGetLastError());
+    if ((st = grant_smem(spd_large_order_kernel, order_granted, kLargeSmemLimit)) != GT_OK) return st;
+    if ((st = grant_smem(spd_large_pull_kernel, pull_granted, kLargeSmemLimit)) != GT_OK) return st;
+    if ((st = launch_overlapped(spd_large_order_kernel, dim3(1), 1024, 8 * (size_t)p.n, s, p)) != GT_OK) return st;
     const size_t tasks = (size_t)p.n / 32 + 2 + (size_t)nnz / (kLargeHubDegree + 1);
-    spd_large_lists_kernel<<<(unsigned)tasks, 256, 0, s>>>(p);
-    GT_CUDA_TRY(cudaGetLastError());
-    spd_large_pull_kernel<<<pl.blocks, pl.threads, pl.smem_bytes, s>>>(p);
-    GT_CUDA_TRY(cudaGetLastError());
-    return GT_OK;
+    if ((st = launch_overlapped(spd_large_lists_kernel, dim3((unsigned)tasks), 256, 0, s, p)) != GT_OK) return st;
+    return launch_overlapped(spd_large_pull_kernel, dim3(pl.blocks), (unsigned)pl.threads, pl.smem_bytes, s, p);
 }
 
 }  // namespace gt

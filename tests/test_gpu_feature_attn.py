@@ -164,3 +164,27 @@ def test_more_than_256_distinct_vectors_are_reported_and_the_fallback_is_the_cal
     assert e.value.status == 2
     assert gt.gt_feature_encode_count(ws) > 256
     gt.gt_check(ws)                                                  # the status was cleared by the first check
+
+
+@pytest.mark.parametrize("n", [3, 64, 65, 515])
+@pytest.mark.parametrize("n_vec", [1, 60, 256])
+def test_encoding_of_features_that_start_between_vectors(n, n_vec):
+    """Features that begin 4 bytes past a 16-byte boundary (the aligned middle is read as vectors, the ends one by one), rows
+    whose pitch is not a multiple of 16 bytes, the vector 0 among the words, more columns than a warp takes at a time."""
+    rng = np.random.Generator(np.random.PCG64(1000 * n + n_vec))
+    vec = np.unique(rng.integers(0, 256, size=(n_vec, 4), dtype=np.uint8), axis=0)
+    vec[0] = 0
+    f = vec[rng.integers(0, len(vec), size=(n, n))]
+    store = torch.zeros(n * n * 4 + 4, dtype=torch.uint8, device="cuda")
+    feat = store[4:].view(n, n, 4)
+    feat.copy_(torch.from_numpy(f))
+    ld = (n + 15) // 16 * 16
+    codes = torch.full((n * ld,), 77, dtype=torch.uint8, device="cuda")
+    vectors = torch.full((256,), -1, dtype=torch.int32, device="cuda")
+    ws = gt.gt_feature_encode(feat, gt.Batch(n), codes, vectors)
+    gt.gt_check(ws)
+    ref_code, ref_vec = ofeat.encode_features(f)
+    assert gt.gt_feature_encode_count(ws) == len(ref_vec)
+    got = codes.cpu().numpy().reshape(n, ld)
+    np.testing.assert_array_equal(got[:, :n], ref_code)
+    assert (got[:, n:] == 255).all()
