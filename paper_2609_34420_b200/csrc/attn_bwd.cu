@@ -29,8 +29,7 @@
 // reads each thread's 32 bucket bytes as two 16-byte words instead of 32 byte loads.
 //
 //   warp 0        TMA producer: K, V, the constant tiles once; Q_i, dO_i, the per-query rows and
-//                 (single graph) the SPD^T tile through a 2-stage ring
-//                 (packed batches: the SPD^T tile by cp.async, per-graph pitch)
+//                 the SPD^T tile through a 2-stage ring
 //   warps 1, 3, 2 MMA issuers: dV and the next S^T; dK and the next dP^T; dQ
 //   warps 4-19    softmax: warps 4-11 own queries [0,64) of every tile, warps 12-19 queries [64,128);
 //                 within a half, four warps per 32 query columns (32 score elements per thread)
@@ -59,8 +58,6 @@ constexpr int kExtCols = 16;                // bf16 per (query, head) row of fol
 constexpr int kExtTileBytes = kTile * kExtCols * 2;
 
 struct BwdParams {
-    const uint8_t* spd_t;    // transposed, clamped copy of the SPD blocks (workspace)
-    const int64_t* spd_offsets;
     const int32_t* cu_seqlens;
     const float* bias;
     float* dq_acc;           // [T,H,D] fp32             (workspace, zeroed)
@@ -71,7 +68,7 @@ struct BwdParams {
     int32_t n_total;
     int32_t n_heads;
     int32_t n_buckets;
-    int32_t spd_tma;         // 1: single graph, SPD tiles come by TMA
+    const uint8_t* maps;     // packed batch: tensor maps of the graphs' SPD^T blocks (workspace); nullptr: single graph
     int32_t kv_row0;         // key rows [kv_row0, kv_row_end) of a graph are this launch's (chunked / step entry points)
     int32_t kv_row_end;
     int32_t q_row0;          // query rows [q_row0, q_row_end) take part (step entry point; else the whole graph)
@@ -169,8 +166,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (kv0 >= kv_lim) return;
     const int32_t q_lo = p.q_row0, q_hi = min(n_g, p.q_row_end);
     if (q_hi <= q_lo) return;
-    const int64_t ld = (int64_t)((n_g + 15) & ~15);
-    const uint8_t* spd_g = p.spd_t + (p.spd_offsets ? p.spd_offsets[g] : 0);
     const int32_t n_q = (q_hi - q_lo + kTile - 1) / kTile;
 
     uint64_t* bars = (uint64_t*)(smem + L::kBars);
@@ -197,7 +192,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         mbar_init(bar(kBarDqFull), 1);
         mbar_init(bar(kBarDqFree), 4);
         mbar_init(bar(kBarKvTmem), 8);
-        mbar_init(bar(kBarSpdFull), p.spd_tma ? 1 : 32);
+        mbar_init(bar(kBarSpdFull), 1);
         mbar_init(bar(kBarSpdEmpty), 16);
         mbar_init(bar(kBarFinal), 3);
         fence_mbar_init();
@@ -207,7 +202,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         prefetch_tensormap(&tmap_do);
         prefetch_tensormap(&tmap_ext);
         prefetch_tensormap(&tmap_dq);
-        if (p.spd_tma) prefetch_tensormap(&tmap_spd);
+        if (!p.maps) prefetch_tensormap(&tmap_spd);
     }
     if (warp == 2) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
     for (int i = tid; i < n_bin_floats; i += kBwdThreads) s_bins[i] = 0.f;
@@ -235,7 +230,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         setmaxnreg_dec_40();
         if (warp == 0) {
             // ------------------------------ TMA producer ------------------------------
+            const void* spd_map = p.maps ? (const void*)(p.maps + (size_t)g * kMapBytes) : &tmap_spd;
             if (lane == 0) {
+                if (p.maps) acquire_tensor_map(spd_map);
                 mbar_arrive_expect_tx(bar(kBarKvFull), 2 * L::kTileBytes);
                 tma_load_3d(smem_u32(smem + L::kK), &tmap_k, bar(kBarKvFull), 0, h, node0 + kv0);
                 tma_load_3d(smem_u32(smem + L::kV), &tmap_v, bar(kBarKvFull), 0, h, node0 + kv0);
@@ -252,37 +249,11 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 }
                 __syncwarp();
                 if (i > 0) mbar_wait(bar(kBarSpdEmpty), (i - 1) & 1, abort_flag, p.status, 111);
-                if (p.spd_tma) {
-                    if (lane == 0) {
-                        mbar_arrive_expect_tx(bar(kBarSpdFull), L::kSpdBytes);
-                        tma_load_2d(smem_u32(smem + L::kSpd), &tmap_spd, bar(kBarSpdFull), q_lo + i * kTile, kv0);
-                    }
-                    __syncwarp();
-                } else {
-                    // packed batch (per-graph pitch): cp.async in the layout of the TMA 128-byte swizzle,
-                    // 16-byte chunk c of row r at chunk c ^ (r & 7)
-                    // (a lane copies chunk cc of rows lr, lr + 4, ...: the swizzle depends on the parity of the round only)
-                    const int32_t q0 = q_lo + i * kTile;
-                    const uint32_t dst0 = smem_u32(smem + L::kSpd);
-                    const int cc = lane & 7, lr = lane >> 3;
-                    const uint32_t dst_even = dst0 + (uint32_t)(lr * 128 + ((cc ^ lr) << 4)), dst_odd = dst0 + (uint32_t)(lr * 128 + ((cc ^ (4 + lr)) << 4));
-                    const uint32_t step = 4u * (uint32_t)ld;
-                    const uint8_t* src = spd_g + (int64_t)(kv0 + lr) * ld + q0 + cc * 16;
-                    const int32_t lim = ((int64_t)q0 + cc * 16 < ld) ? n_g - kv0 - lr : 0;       // rounds 4 it < lim are in range
-                    if (kv0 + kTile <= n_g && (int64_t)q0 + kTile <= ld) {
-#pragma unroll 8
-                        for (int it = 0; it < kTile / 4; ++it) {
-                            cp_async_16(((it & 1) ? dst_odd : dst_even) + it * 512, src + (uint64_t)step * (uint32_t)it, 16u);
-                        }
-                    } else {
-#pragma unroll 8
-                        for (int it = 0; it < kTile / 4; ++it) {
-                            const bool valid = 4 * it < lim;
-                            cp_async_16(((it & 1) ? dst_odd : dst_even) + it * 512, valid ? src + (uint64_t)step * (uint32_t)it : spd_g, valid ? 16u : 0u);
-                        }
-                    }
-                    cp_async_mbar_arrive_noinc(bar(kBarSpdFull));
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(bar(kBarSpdFull), L::kSpdBytes);
+                    tma_load_2d(smem_u32(smem + L::kSpd), spd_map, bar(kBarSpdFull), q_lo + i * kTile, kv0);
                 }
+                __syncwarp();
             }
         } else if (warp == 1 || warp == 3) {
             // ------------------------------- MMA issuers -------------------------------
@@ -684,6 +655,7 @@ __device__ __forceinline__ void split3_bf16(float v, uint32_t& w01, uint32_t& w2
 struct PrepareParams {
     const uint8_t* spd;
     uint8_t* spd_t;
+    uint8_t* maps;             // packed batch: tensor maps of the spd_t blocks, made from `model`
     const int64_t* spd_offsets;
     const int32_t* cu_seqlens;
     const __nv_bfloat16* out;
@@ -698,6 +670,7 @@ struct PrepareParams {
     uint32_t row_blocks;       // thread blocks that work on rows; the others transpose
     uint32_t last_bucket;
     float sqrt_d;
+    CUtensorMap model;
 };
 
 // Everything the main kernel wants done before it, in one launch (two fills and two kernels in a row spend more time starting
@@ -710,7 +683,7 @@ struct PrepareParams {
 // 64 graphs of 512-2 048 nodes, H = 16, d = 64: 197 us in two fills and two kernels before.
 constexpr int kPrepareRows = 128;
 template <int D>
-__global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const PrepareParams p)
+__global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const __grid_constant__ PrepareParams p)
 {
     __shared__ __align__(16) uint8_t s_rows[kPrepareRows * 6 * D];      // dO, then O (bf16 or fp32); or a tile to transpose
     static_assert(sizeof(s_rows) >= 128 * 128);
@@ -722,6 +695,8 @@ __global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const Prep
         const int32_t n_g = p.cu_seqlens ? p.cu_seqlens[g + 1] - p.cu_seqlens[g] : p.n_total;
         const int32_t i0 = (r / p.tiles) * 128, j0 = (r % p.tiles) * 128;
         if (i0 >= n_g || j0 >= n_g) return;
+        if (r == 0 && threadIdx.x == 0 && p.maps != nullptr)
+            make_spd_map(p.maps + (size_t)g * kMapBytes, p.model, p.spd_t + p.spd_offsets[g], n_g);
         transpose_tile(p.spd, p.spd_t, n_g, p.spd_offsets ? p.spd_offsets[g] : 0, i0, j0, p.last_bucket, (uint32_t*)s_rows);
         return;
     }
@@ -833,7 +808,7 @@ __global__ void bwd_finalize_kernel(const float* __restrict__ dq_acc, __nv_bfloa
 }
 
 struct BwdWorkspace {
-    size_t db_off, ext_off, dq_off, spdt_off, total;
+    size_t db_off, ext_off, dq_off, maps_off, spdt_off, total;
 };
 
 BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim, int32_t max_dist, int32_t n_chunks = 1)
@@ -843,7 +818,8 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
     w.db_off = kHeaderBytes;
     w.ext_off = w.db_off + align_up((size_t)n_chunks * n_heads * (max_dist + 2) * sizeof(double), 256);
     w.dq_off = w.ext_off + align_up(rows * kExtCols * 2, 256);
-    w.spdt_off = w.dq_off + align_up(rows * head_dim * sizeof(float), 256);
+    w.maps_off = w.dq_off + align_up(rows * head_dim * sizeof(float), 256);
+    w.spdt_off = w.maps_off + maps_bytes(b->n_graphs);
     // transposed SPD copy: at most sum n_g * round_up(n_g,16) <= n_total * round_up(max_seqlen,16) bytes
     w.total = w.spdt_off + align_up((size_t)b->n_total * (size_t)((b->max_seqlen + 15) & ~15), 256);
     return w;
@@ -930,13 +906,11 @@ static gt_status gt_bwd_run(const void* q, const void* k, const void* v, const v
     uint8_t* ws = (uint8_t*)workspace;
     const size_t rows = (size_t)batch->n_total * n_heads;
     const int32_t n_db = n_heads * (max_dist + 2);
-    CUtensorMap tspd = tq;                       // placeholder when the cp.async loader is used
+    CUtensorMap tspd;
     BwdParams p{};
-    p.spd_tma = batch->n_graphs == 1 ? 1 : 0;
     uint8_t* spd_t = ws + wsp.spdt_off;
-    if (p.spd_tma && (st = encode_spd_map(&tspd, spd_t, batch->n_total, 128)) != GT_OK) return st;
-    p.spd_t = spd_t;
-    p.spd_offsets = batch->n_graphs > 1 ? spd_offsets : nullptr;
+    if ((st = encode_spd_map(&tspd, spd_t, batch->max_seqlen, 128)) != GT_OK) return st;
+    if (batch->n_graphs > 1) p.maps = maps_at(ws + wsp.maps_off);
     p.cu_seqlens = batch->n_graphs > 1 ? batch->cu_seqlens : nullptr;
     p.bias = bias;
     p.dq_acc = (float*)(ws + wsp.dq_off);
@@ -952,7 +926,9 @@ static gt_status gt_bwd_run(const void* q, const void* k, const void* v, const v
 
     uint4* ext = (uint4*)(ws + wsp.ext_off);
     PrepareParams pre{};
-    pre.spd = spd; pre.spd_t = spd_t; pre.spd_offsets = p.spd_offsets; pre.cu_seqlens = p.cu_seqlens;
+    pre.spd = spd; pre.spd_t = spd_t; pre.spd_offsets = batch->n_graphs > 1 ? spd_offsets : nullptr; pre.cu_seqlens = p.cu_seqlens;
+    pre.maps = const_cast<uint8_t*>(p.maps);
+    pre.model = tspd;
     pre.out = (const __nv_bfloat16*)out; pre.out_f32 = out_f32; pre.dout = (const __nv_bfloat16*)dout; pre.lse = lse;
     pre.ext = ext;
     pre.dq_acc = (float4*)p.dq_acc;
@@ -1148,8 +1124,6 @@ extern "C" gt_status gt_biased_attn_bwd_step(const void* q, const void* k, const
     if ((st = encode_thd_map(&text, ws + cx.ext_off, n, n_heads, kExtCols)) != GT_OK) return st;
     if ((st = encode_spd_map(&tspd, ws + cx.spdt_off, n, 128)) != GT_OK) return st;
     BwdParams p{};
-    p.spd_tma = 1;
-    p.spd_t = ws + cx.spdt_off;
     p.bias = bias;
     p.dq_acc = dq_acc;
     p.db_acc = dbias_acc;

@@ -25,6 +25,29 @@ gt_status encode_spd_map(CUtensorMap* map, const uint8_t* spd, int32_t n, int32_
 // head, 128-byte swizzle (target of the backward kernel's TMA reduce-add).
 gt_status encode_dq_map(CUtensorMap* map, const float* dq_acc, int32_t n_total, int32_t n_heads, int32_t head_dim);
 
+// Tensor maps of the SPD blocks of a packed batch, whose sizes and offsets are known on the device only: map g is `model` (a map
+// of any size, from encode_spd_map) with graph g's base, dimensions and pitch put in.  One thread per graph; the reader of a
+// map acquires it with acquire_tensor_map before its first use.
+__device__ __forceinline__ void make_spd_map(uint8_t* map, const CUtensorMap& model, const uint8_t* block, int32_t n)
+{
+    const uint32_t ld = (uint32_t)((n + 15) & ~15);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ((uint4*)map)[i] = ((const uint4*)&model)[i];
+    asm volatile("tensormap.replace.tile.global_address.global.b1024.b64 [%0], %1;" ::"l"(map), "l"(block) : "memory");
+    asm volatile("tensormap.replace.tile.global_dim.global.b1024.b32 [%0], 0, %1;" ::"l"(map), "r"(ld) : "memory");
+    asm volatile("tensormap.replace.tile.global_dim.global.b1024.b32 [%0], 1, %1;" ::"l"(map), "r"(n) : "memory");
+    asm volatile("tensormap.replace.tile.global_stride.global.b1024.b64 [%0], 0, %1;" ::"l"(map), "l"((uint64_t)ld) : "memory");
+    asm volatile("fence.proxy.tensormap::generic.release.gpu;" ::: "memory");
+}
+__device__ __forceinline__ void acquire_tensor_map(const void* map)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
+}
+constexpr size_t kMapBytes = 128;
+// their place in a workspace whose address is a multiple of 16; none for a single graph
+inline size_t maps_bytes(int32_t n_graphs) { return n_graphs > 1 ? align_up((size_t)n_graphs * kMapBytes, 256) + kMapBytes : 0; }
+inline uint8_t* maps_at(uint8_t* region) { return (uint8_t*)align_up(reinterpret_cast<uintptr_t>(region), kMapBytes); }
+
 struct AttnArgsCheck {
     const void* ptrs[12];
     int n_ptrs;

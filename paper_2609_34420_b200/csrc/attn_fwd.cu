@@ -82,7 +82,8 @@ struct FwdParams {
     float* state_lse;          //   ([T,H,D] fp32, [H,T]); rows [state_q_begin, state_q_end) only
     int32_t state_q_begin;
     int32_t state_q_end;
-    int32_t spd_tma;           // 1: single graph, SPD tiles come by TMA; 0: cp.async loader warp
+    const uint8_t* maps;       // packed batch: tensor maps of the graphs' SPD blocks
+    int32_t spd_tma;           // 1: SPD tiles come by TMA; 0: packed batch without room for the maps, cp.async loader warp
     float c1;                  // log2(e) / sqrt(d)
 };
 
@@ -200,7 +201,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         prefetch_tensormap(&tmap_q);
         prefetch_tensormap(&tmap_k);
         prefetch_tensormap(&tmap_v);
-        if (p.spd_tma) prefetch_tensormap(&tmap_spd);
+        if (p.spd_tma && !p.maps) prefetch_tensormap(&tmap_spd);
     }
     if (warp == 1) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
     grid_wait();
@@ -216,7 +217,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // =========================== producer / MMA / SPD warps ===========================
         if constexpr (kHalves == 2) setmaxnreg_dec_32(); else setmaxnreg_dec_56();
         if (warp == 0) {
+            const void* spd_map = !kPartial && p.maps ? (const void*)(p.maps + (size_t)g * kMapBytes) : &tmap_spd;
             if (lane == 0) {
+                if (!kPartial && p.maps) acquire_tensor_map(spd_map);
                 mbar_arrive_expect_tx(bar(kBarQFull), kQTiles * L::kTileBytes);
                 for (int t = 0; t < kQTiles; ++t)
                     tma_load_3d(smem_u32(smem + L::kQ + t * L::kTileBytes), &tmap_q, bar(kBarQFull), 0, h,
@@ -235,7 +238,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     mbar_wait(bar(kBarSpdEmpty + ss), ((j / kSpdStages) & 1) ^ 1, abort_flag, p.status, 11);
                     if (lane == 0) {
                         mbar_arrive_expect_tx(bar(kBarSpdFull + ss), L::kSpdTileBytes);
-                        tma_load_2d(smem_u32(smem + L::kSpd + ss * L::kSpdTileBytes), &tmap_spd, bar(kBarSpdFull + ss), kv0, q0);
+                        tma_load_2d(smem_u32(smem + L::kSpd + ss * L::kSpdTileBytes), spd_map, bar(kBarSpdFull + ss), kv0, q0);
                     }
                 }
                 mbar_wait(bar(kBarVEmpty + vs), ((j / kVStages) & 1) ^ 1, abort_flag, p.status, 12);
@@ -729,6 +732,17 @@ int32_t chunk_rows(int32_t n, int32_t n_chunks)
     return (w + kKvTile - 1) / kKvTile * kKvTile;
 }
 
+__global__ void __launch_bounds__(128) fwd_maps_kernel(const __grid_constant__ CUtensorMap model, uint8_t* maps, const uint8_t* spd,
+                                                       const int64_t* spd_offsets, const int32_t* cu_seqlens, int32_t n_graphs)
+{
+    grid_wait();
+    grid_release();
+    const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (g >= n_graphs) return;
+    const int32_t n = cu_seqlens[g + 1] - cu_seqlens[g];
+    if (n > 0) make_spd_map(maps + (size_t)g * kMapBytes, model, spd + spd_offsets[g], n);
+}
+
 template <int D, bool kPartial>
 gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tspd,
                      const FwdParams& p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0)
@@ -762,8 +776,8 @@ gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint
 
 extern "C" size_t gt_biased_attn_fwd_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim)
 {
-    (void)batch; (void)n_heads; (void)head_dim;
-    return gt::kHeaderBytes;
+    (void)n_heads; (void)head_dim;
+    return gt::kHeaderBytes + (gt::validate_batch(batch) == GT_OK ? gt::maps_bytes(batch->n_graphs) : 0);
 }
 
 extern "C" gt_status gt_biased_attn_fwd(const void* q, const void* k, const void* v,
@@ -795,7 +809,11 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     CUtensorMap tspd = tq;                       // placeholder when the cp.async loader is used
     FwdParams p{};
     p.spd_tma = batch->n_graphs == 1 ? 1 : 0;
-    if (p.spd_tma && (st = encode_spd_map(&tspd, spd, batch->n_total, 256)) != GT_OK) return st;
+    if (batch->n_graphs > 1 && workspace_bytes >= gt_biased_attn_fwd_workspace(batch, n_heads, head_dim)) {
+        p.maps = maps_at((uint8_t*)workspace + kHeaderBytes);
+        p.spd_tma = 1;
+    }
+    if (p.spd_tma && (st = encode_spd_map(&tspd, spd, batch->max_seqlen, 256)) != GT_OK) return st;
     p.spd = spd;
     p.spd_offsets = batch->n_graphs > 1 ? spd_offsets : nullptr;
     p.cu_seqlens = batch->n_graphs > 1 ? batch->cu_seqlens : nullptr;
@@ -809,6 +827,11 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     p.n_buckets = max_dist + 2;
     p.c1 = kLog2e / sqrtf((float)head_dim);
     cudaStream_t s = (cudaStream_t)stream;
+    if (p.maps) {
+        st = launch_overlapped(fwd_maps_kernel, dim3((unsigned)(batch->n_graphs + 127) / 128), 128, 0, s, tspd, (uint8_t*)p.maps, spd,
+                               p.spd_offsets, p.cu_seqlens, batch->n_graphs);
+        if (st != GT_OK) return st;
+    }
     return head_dim == 64 ? launch_fwd<64, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s)
                           : launch_fwd<32, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s);
 }

@@ -67,7 +67,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
                                           uint32_t* status, uint32_t site)
 {
     if (mbar_try_wait(bar, parity)) return true;
-    for (uint32_t it = 0; it < kWaitIterations; ++it) {
+#pragma unroll 1
+    for (uint32_t it = 0; it < kWaitIterations; ++it) {      // (unrolled copies at every call site crowd the instruction cache)
         if (mbar_try_wait(bar, parity)) return true;
         if ((it & 255u) == 255u && *abort_flag) return false;
     }
