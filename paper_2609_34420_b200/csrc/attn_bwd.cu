@@ -53,6 +53,7 @@ constexpr int kHalf = 64;                   // queries per TMEM stage
 constexpr int kStages = 2;
 constexpr int kBwdThreads = 768;
 constexpr int kSoftmaxThreads = 512;
+constexpr int kPrivateBinLog = 9;           // a bin column per softmax thread
 constexpr int kMaxPrivateBinBuckets = 26;   // 2 KB of shared memory per bucket, between the 128 KB mark and the last two buffers
 constexpr int kExtCols = 16;                // bf16 per (query, head) row of folded terms
 constexpr int kExtTileBytes = kTile * kExtCols * 2;
@@ -68,6 +69,8 @@ struct BwdParams {
     int32_t n_total;
     int32_t n_heads;
     int32_t n_buckets;
+    int32_t bin_log;         // shared bins (more than kMaxPrivateBinBuckets buckets): log2 of the columns per bucket
+    int32_t early_release;   // let the next kernel start its set-up while this one runs
     const uint8_t* maps;     // packed batch: tensor maps of the graphs' SPD^T blocks (workspace); nullptr: single graph
     int32_t kv_row0;         // key rows [kv_row0, kv_row_end) of a graph are this launch's (chunked / step entry points)
     int32_t kv_row_end;
@@ -174,7 +177,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     float* s_bins = (float*)(smem + L::kBins);
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     volatile uint32_t* abort_flag = &misc[1];
-    const int n_bin_floats = kPrivateBins ? p.n_buckets * kSoftmaxThreads : p.n_buckets * 32;
+    const int bin_log = kPrivateBins ? kPrivateBinLog : p.bin_log;          // log2 of the columns per bucket
+    const int n_bin_floats = p.n_buckets << bin_log;
     uint8_t* const s_stg = smem + L::kBins + (((size_t)n_bin_floats * 4 + 1023) & ~(size_t)1023);
     uint8_t* const s_ds = s_stg + 16384;
 
@@ -207,7 +211,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (warp == 2) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
     for (int i = tid; i < n_bin_floats; i += kBwdThreads) s_bins[i] = 0.f;
     grid_wait();
-    grid_release();
+    if (p.early_release) grid_release();
     for (int i = tid; i < 256; i += kBwdThreads)
         s_bias[i] = p.bias[(size_t)h * p.n_buckets + min(i, p.n_buckets - 1)] * kLog2e;
     if (tid < 32) {
@@ -353,10 +357,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const bool kv_valid = kv0 + r < kv_lim;
         const uint64_t c1c1 = pack_f32x2(p.c1, p.c1);
         const float tbl = s_bias[lane];
-        float* my_bins = s_bins + (kPrivateBins ? st : lane);
+        const uint32_t bins_base = smem_u32(s_bins + (st & ((1 << bin_log) - 1)));
         // the thread's 32 bucket bytes: row r of the SPD^T tile, 16-byte chunks 2 grp and 2 grp + 1 (swizzled by r & 7)
         const uint32_t spd_off0 = r * 128 + (((2 * grp) ^ (r & 7)) << 4), spd_off1 = r * 128 + (((2 * grp + 1) ^ (r & 7)) << 4);
-        const uint32_t bins_base = smem_u32(my_bins);
         uint8_t* ds_row = s_ds + half * 16384 + r * 128;
 
         // K (warps 4-7) and V (warps 8-11) rows -> tensor memory, where they stay as the A operands of
@@ -446,13 +449,17 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     const int c = rnd * 16 + k;
                     unpack_f32x2(mul_f32x2(pack_f32x2(pr[c], pr[c + 1]), pack_u32x2(dp[k], dp[k + 1])), pr[c], pr[c + 1]);
                 }
-                // byte offset of bin b: b * stride * 4, formed by one funnel shift and one logic operation; with
-                // private bins that operation also ORs in the address of the thread's bin column (see the memory map)
-                constexpr int kLog = kPrivateBins ? 11 : 7;               // log2(kBinStride * 4)
-                auto bin_off = [&](int c) {
-                    const int sh = 8 * (c & 3) - kLog;
-                    const uint32_t x = sh >= 0 ? (bw[c >> 2] >> (sh >= 0 ? sh : 0)) : (bw[c >> 2] << (sh < 0 ? -sh : 0));
-                    return kPrivateBins ? ((x & (0xffu << kLog)) | bins_base) : (x & (0xffu << kLog));
+                // Address of an element's bin.  Private bins: the shifted bucket byte, by one funnel shift and one logic operation that
+                // also ORs in the address of the thread's bin column (see the memory map).
+                auto bin_addr = [&](int c) -> uint32_t {
+                    if constexpr (kPrivateBins) {
+                        constexpr int kLog = kPrivateBinLog + 2;
+                        const int sh = 8 * (c & 3) - kLog;
+                        const uint32_t x = sh >= 0 ? (bw[c >> 2] >> (sh >= 0 ? sh : 0)) : (bw[c >> 2] << (sh < 0 ? -sh : 0));
+                        return (x & (0xffu << kLog)) | bins_base;
+                    } else {
+                        return bins_base + (((bw[c >> 2] >> (8 * (c & 3))) & 0xffu) << (bin_log + 2));
+                    }
                 };
                 if (kPrivateBins) {
                     // read-modify-write of the thread's own bins, two elements at a time so that two loads are
@@ -460,7 +467,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
                     for (int k = 0; k < 16; k += 2) {
                         const int c = rnd * 16 + k;
-                        const uint32_t o0 = bin_off(c), o1 = bin_off(c + 1);
+                        const uint32_t o0 = bin_addr(c), o1 = bin_addr(c + 1);
                         float v0, v1;
                         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v0) : "r"(o0));
                         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v1) : "r"(o1));
@@ -471,7 +478,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     }
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) atomicAdd((float*)((uint8_t*)my_bins + bin_off(rnd * 16 + k)), pr[rnd * 16 + k]);
+                    for (int k = 0; k < 16; ++k)
+                        asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(bin_addr(rnd * 16 + k)), "f"(pr[rnd * 16 + k]) : "memory");
                 }
             };
             ds_round(0, dpa);
@@ -534,23 +542,14 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
         // ---------------- flush the bias-gradient bins ----------------
         named_barrier_sync(kNbFlush, kSoftmaxThreads);
-        if (kPrivateBins) {
-            // a warp per bucket: lanes add every 32nd column, then the warp adds its lanes (one thread walking all
-            // 512 columns of a bucket took 9 us per CTA, a third of the kernel on graphs of a thousand nodes)
-            for (int b = st >> 5; b < p.n_buckets; b += kSoftmaxThreads / 32) {
-                float a = 0.f;
+        // a warp per bucket: lanes add every 32nd column, then the warp adds its lanes (one thread walking all
+        // 512 columns of a bucket took 9 us per CTA, a third of the kernel on graphs of a thousand nodes)
+        for (int b = st >> 5; b < p.n_buckets; b += kSoftmaxThreads / 32) {
+            float a = 0.f;
+            for (int k = lane; k < (1 << bin_log); k += 32) a += s_bins[(b << bin_log) + k];
 #pragma unroll
-                for (int k = 0; k < kSoftmaxThreads / 32; ++k) a += s_bins[b * kSoftmaxThreads + k * 32 + lane];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-                if (lane == 0) atomicAdd(&p.db_acc[(size_t)h * p.n_buckets + b], (double)a);
-            }
-        } else {
-            for (int b = st; b < p.n_buckets; b += kSoftmaxThreads) {
-                float a = 0.f;
-                for (int k = 0; k < 32; ++k) a += s_bins[b * 32 + ((k + b) & 31)];
-                atomicAdd(&p.db_acc[(size_t)h * p.n_buckets + b], (double)a);
-            }
+            for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+            if (lane == 0) atomicAdd(&p.db_acc[(size_t)h * p.n_buckets + b], (double)a);
         }
     } else {
         // ================================ dQ reducer ================================
@@ -827,7 +826,7 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
 
 template <int D>
 gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
-                     const CUtensorMap& text, const CUtensorMap& tspd, const BwdParams& p,
+                     const CUtensorMap& text, const CUtensorMap& tspd, BwdParams p,
                      const gt_batch* batch, cudaStream_t s)
 {
     const int32_t kv_end = p.kv_row_end < batch->max_seqlen ? p.kv_row_end : batch->max_seqlen;
@@ -837,7 +836,13 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     gt_status st_map = encode_dq_map(&tdq, p.dq_acc, p.n_total, p.n_heads, D);
     if (st_map != GT_OK) return st_map;
     const bool priv = p.n_buckets <= kMaxPrivateBinBuckets;
-    const size_t smem = BwdSmem<D>::dynamic_bytes(priv ? p.n_buckets * kSoftmaxThreads : p.n_buckets * 32);
+    // As many columns per bucket as the private bins' space holds: two warps that meet in a column retry each other's adds.
+    p.bin_log = kPrivateBinLog;
+    while ((p.n_buckets << p.bin_log) > (kMaxPrivateBinBuckets << kPrivateBinLog)) --p.bin_log;
+    const size_t smem = BwdSmem<D>::dynamic_bytes(p.n_buckets << p.bin_log);
+    // With several waves of blocks the early start of the next kernel slows the dispatch of this one's (65 536 nodes: 36.5 ->
+    // 39.9 ms); with one it hides the next one's start.
+    p.early_release = (int64_t)grid.x * grid.y * grid.z <= sm_count();
     static_assert(kMaxPrivateBinBuckets <= 32, "private bins go with the shuffle lookup");
     auto kern = priv ? attn_bwd_kernel<D, true, true>
                      : (p.n_buckets <= 32 ? attn_bwd_kernel<D, false, true> : attn_bwd_kernel<D, false, false>);
