@@ -24,9 +24,11 @@ namespace gt {
 namespace {
 
 constexpr int kSorted = 256;           // batches of up to this many graphs are worked on by falling size
-constexpr int kBins = 34;              // hubs, then degrees 32 .. 0
+constexpr int kBins = 66;              // hubs, then degrees 64 .. 0
 constexpr uint16_t kListed = 0x8000;   // vertices are numbered below this
-constexpr int kHubDegree = 32;         // vertices with more out-edges than this are pulled by a whole warp
+// Vertices with more out-edges than this are pulled by a whole warp: some 150 instructions each, where 32 of them side by side
+// in one group cost 100 and 8 per pair of edges (a limit of 32: 11.4k clocks a level at 4 096 nodes, issue bound).
+constexpr int kHubDegree = 64;
 
 struct PullParams {
     const int32_t* row_ptr;
@@ -46,6 +48,9 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
 {
     using R = Rows<kT>;
     constexpr int W = R::kWords;
+    // Rows of one word stay in the vertices' order: a vertex' own row is then read out of order, which costs less than looking
+    // up every edge's position.  Wider rows lie by position (their out-of-order accesses cost 6 or 11 wavefronts, not 3.5).
+    constexpr bool kByPosition = W > 1;
     extern __shared__ __align__(16) uint8_t pull_smem[];
     __shared__ int s_graph, s_node0, s_n, s_first, s_list_words, s_bin[kBins];
     int* s_size = (int*)pull_smem;           // before the rows
@@ -101,7 +106,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
     uint8_t* nxt = cur + row_bytes;
     uint8_t* planes = nxt + row_bytes;
     uint16_t* order = (uint16_t*)(planes + (size_t)p.n_planes * row_bytes);          // vertex at position i (and kListed)
-    uint32_t* ginfo = (uint32_t*)((uint8_t*)order + pull_align(2 * (size_t)n));       // per group of 32 positions: list << 5 | pairs
+    uint32_t* ginfo = (uint32_t*)((uint8_t*)order + pull_align(2 * (size_t)n));       // per group of 32 positions: list << 6 | pairs
     uint32_t* hub_at = ginfo + pull_align(4 * (size_t)(n / 32 + 1)) / 4;               // staged: word at which a hub's list starts; else: the hubs
     const uint32_t used = (uint32_t)((uint8_t*)hub_at - pull_smem);
     // The edge list with 16-bit positions goes to shared memory where it fits behind the state; while it is laid out, the
@@ -119,8 +124,8 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
     __syncthreads();
     int n_hubs = 0;
     uint32_t* list = hub_at;                           // edge lists, behind hub_at
-    uint16_t* pos = (uint16_t*)nxt;                    // position of vertex v
-    uint16_t* eoff = pos + ((n + 7) & ~7);             // first edge of vertex v
+    uint16_t* pos = (uint16_t*)nxt;                    // position of vertex v (kByPosition)
+    uint16_t* eoff = pos + (kByPosition ? (n + 7) & ~7 : 0);             // first edge of vertex v
     const int skew = (int)(((uintptr_t)(p.col_idx + e_base) >> 2) & 3u);
     uint16_t* raw = eoff + ((n + 8) & ~7) + skew;      // columns (original ids), placed as the caller's list is in its vectors
     if (staged) {
@@ -173,7 +178,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
             if (v < n) key[v] = (uint32_t)bin << 16 | (uint32_t)rank;
         }
         __syncthreads();
-        if (warp == 0) {                              // exclusive scan of the bins (34)
+        if (warp == 0) {                              // exclusive scan of the bins
             int carry = 0;
             for (int b = 0; b < kBins; b += 32) {
                 const int cnt = b + lane < kBins ? s_bin[b + lane] : 0;
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
         for (int v = threadIdx.x; v < n; v += blockDim.x) {
             const uint32_t k = key[v];
             const int i = s_bin[k >> 16] + (int)(k & 0xffffu);
-            pos[v] = (uint16_t)i;
+            if (kByPosition) pos[v] = (uint16_t)i;
             order[i] = (uint16_t)v;
         }
         __syncthreads();
@@ -209,7 +214,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
                 const int v = i < n ? order[i] : 0;
                 const int pairs = i < n ? ((int)eoff[v + 1] - (int)eoff[v] + 1) / 2 : 0;
                 const int x = warp_scan(32 * pairs, lane);
-                if (i < n) ginfo[g0 + lane] = (uint32_t)(at + x - 32 * pairs) << 5 | (uint32_t)pairs;
+                if (i < n) ginfo[g0 + lane] = (uint32_t)(at + x - 32 * pairs) << 6 | (uint32_t)pairs;
                 at += __shfl_sync(0xffffffffu, x, 31);
             }
             if (lane == 0) s_list_words = at;
@@ -229,33 +234,33 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
             for (int k = 0; k < W; ++k) w[k] = 0u;
             for (int i = lane; i < ((deg + 1) & ~1); i += 32) {
                 const int u = i < deg ? raw[e0 + i] : v;
-                dst[i] = pos[u];
+                dst[i] = kByPosition ? pos[u] : (uint16_t)u;
                 R::add_target(u - t0, nt, w);
             }
             R::add_target(v - t0, nt, w);
 #pragma unroll
             for (int k = 0; k < W; ++k) w[k] = __reduce_or_sync(0xffffffffu, w[k]);
-            if (lane == 0) R::store(cur, h, w);
+            if (lane == 0) R::store(cur, kByPosition ? h : v, w);
         }
         for (int q = warp; n_hubs + 32 * q < n; q += n_warps) {
             const int i = n_hubs + 32 * q + lane;
             const int v = order[min(i, n - 1)];
             const int e0 = eoff[v], deg = i < n ? (int)eoff[v + 1] - e0 : 0;
             const uint32_t info = ginfo[q];
-            uint32_t* dst = list + (info >> 5) + lane;
+            uint32_t* dst = list + (info >> 6) + lane;
             uint32_t w[W];
 #pragma unroll
             for (int k = 0; k < W; ++k) w[k] = 0u;
             R::add_target(v - t0, nt, w);
-            for (int j = 0; j < (int)(info & 31u); ++j) {
+            for (int j = 0; j < (int)(info & 63u); ++j) {
                 const int u0 = 2 * j < deg ? raw[e0 + 2 * j] : v, u1 = 2 * j + 1 < deg ? raw[e0 + 2 * j + 1] : v;
-                dst[32 * j] = (uint32_t)pos[u0] | (uint32_t)pos[u1] << 16;
+                dst[32 * j] = kByPosition ? (uint32_t)pos[u0] | (uint32_t)pos[u1] << 16 : (uint32_t)u0 | (uint32_t)u1 << 16;
                 R::add_target(u0 - t0, nt, w);
                 R::add_target(u1 - t0, nt, w);
             }
-            if (i < n) R::store(cur, i, w);
+            if (i < n) R::store(cur, kByPosition ? i : v, w);
         }
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) s_tpos[t] = pos[t0 + t];
+        for (int t = threadIdx.x; t < nt; t += blockDim.x) s_tpos[t] = kByPosition ? pos[t0 + t] : (uint16_t)(t0 + t);
         __syncthreads();
     } else {                                           // the caller's list in place, vertices in their own order
         const int hub_cap = (int)((p.smem_bytes - used) / 4u);
@@ -286,7 +291,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
         __syncthreads();
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             uint32_t w[W], self[W];
-            R::load(cur, i, w);
+            R::load(cur, kByPosition ? i : (int)order[i], w);
 #pragma unroll
             for (int k = 0; k < W; ++k) self[k] = 0u;
             R::add_target((int)order[i] - t0, nt, self);
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
     }
     __syncthreads();
 
+    auto row_of = [&](int i) -> int { return kByPosition ? i : order[i] & (kListed - 1); };        // of position i
     // bits that position i gained at level `code`: into the code planes
     auto note = [&](int i, const uint32_t (&old)[W], const uint32_t (&acc)[W], int code) {
         uint32_t fresh[W], any = 0u;
@@ -325,8 +331,9 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
         uint32_t gained = 0u;
         for (int h = warp; h < n_hubs; h += n_warps) {
             const int i = staged ? h : (int)hub_at[h];
+            const int own_row = row_of(i);
             uint32_t old[W], acc[W];
-            R::load(src, i, old);
+            R::load(src, own_row, old);
             uint32_t miss = 0u;
 #pragma unroll
             for (int k = 0; k < W; ++k) { acc[k] = old[k]; miss |= live[k] & ~old[k]; }
@@ -347,13 +354,14 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
                 note(i, old, acc, code);
 #pragma unroll
                 for (int k = 0; k < W; ++k) gained |= acc[k] & ~old[k];
-                R::store(dst, i, acc);
+                R::store(dst, own_row, acc);
             }
         }
         for (int q = warp; q < n_groups; q += n_warps) {
             const int i = group0 + 32 * q + lane;
             uint32_t old[W], acc[W];
-            R::load(src, min(i, n - 1), old);
+            const int own_row = row_of(min(i, n - 1));
+            R::load(src, own_row, old);
             uint32_t miss = 0u;
 #pragma unroll
             for (int k = 0; k < W; ++k) { acc[k] = old[k]; miss |= live[k] & ~old[k]; }
@@ -361,9 +369,9 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
             if (staged) {
                 if (__any_sync(0xffffffffu, miss != 0u && own)) {
                     const uint32_t info = ginfo[q];
-                    const uint32_t* mine = list + (info >> 5) + lane;
+                    const uint32_t* mine = list + (info >> 6) + lane;
                     constexpr int kPairs = W == 4 ? 2 : 4;         // 4 or 8 rows in flight
-                    int left = (int)(info & 31u);
+                    int left = (int)(info & 63u);
                     for (; left >= kPairs; left -= kPairs, mine += 32 * kPairs) {
                         uint32_t u[kPairs], x[2 * kPairs][W];
 #pragma unroll
@@ -411,7 +419,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
                 note(i, old, acc, code);
 #pragma unroll
                 for (int k = 0; k < W; ++k) gained |= acc[k] & ~old[k];
-                R::store(dst, i, acc);
+                R::store(dst, own_row, acc);
             }
         }
         if constexpr (W == 1) {
@@ -437,7 +445,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
         __syncthreads();
         // every vertex inherits the rows of the targets it reaches; a closed row covers all targets inside it
         for (int v = threadIdx.x; v < n; v += blockDim.x)
-            if ((unsigned)((int)(order[v] & (kListed - 1)) - t0) >= (unsigned)nt) inherit<kT>(cur, v, s_tpos);
+            if ((unsigned)((kByPosition ? order[v] & (kListed - 1) : v) - t0) >= (unsigned)nt) inherit<kT>(cur, v, s_tpos);
         __syncthreads();
         open = pass(cur, cur, 0);
     }
@@ -457,7 +465,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
         uint8_t* row = out + (int64_t)v * ld + col;
         const int self = v - t0 - col;
         auto word = [&](const uint8_t* rows) -> uint32_t { return ((const uint32_t*)rows)[at]; };
-        const uint32_t reach = word(cur);
+        const uint32_t reach = kByPosition ? word(cur) : ((const uint32_t*)cur)[v];
         uint32_t seen = (unsigned)self < 32u ? 1u << R::bit(self) : 0u;
         uint32_t c[8];
 #pragma unroll
@@ -498,7 +506,7 @@ PullPlan spd_pull_plan(const gt_batch* b, int64_t nnz, int32_t max_dist)
     // turns out not to fit is read in place).
     const int64_t edges = b->n_graphs == 1 ? nnz : (int64_t)((double)nnz / b->n_total * n * 1.02) + 1;
     const int64_t hubs = edges / (kHubDegree + 1) < n ? edges / (kHubDegree + 1) : n;
-    const size_t list = 4 * (size_t)(hubs + 4) + 2 * ((size_t)edges + (b->n_graphs == 1 ? (size_t)n + 1088 : (size_t)n / 2 + 448));
+    const size_t list = 4 * (size_t)(hubs + 4) + 2 * ((size_t)edges + (b->n_graphs == 1 ? (size_t)n + 2112 : (size_t)n / 2 + 448));
     // Wider rows cost less per target (wavefronts above), narrower ones give more thread blocks: 128 and 64 targets are taken
     // while they leave two blocks per SM.
     for (int t = 128; t >= 32 && !pl.fits; t >>= 1) {
