@@ -97,10 +97,10 @@ gt_status gt_check(void* workspace, void* stream);
  * Workspace (gt_spd_build_workspace says how much): 256 bytes for graphs of up to about 5 000 nodes, whose whole traversal
  * state fits shared memory; a single graph of up to 22 000 nodes: its edge list once more (2 bytes per edge) and bit planes of
  * 4 bytes per node, bit of max_dist + 1 and thread block in flight (up to two per SM; 24 MB at 8 192 nodes); a single graph
- * from 14 500 nodes on at least what its bit-matrix traversal needs (the one used beyond 22 000 nodes): about 7 KB per node
- * for each of min(4, ceil(n/8192)) groups of thread blocks (seven bit matrices of 1 KB rows per group: visited, and one
- * frontier per level up to 5; later levels reuse two of them) plus 1 KB per 33 edges per group (rows for vertices with more
- * than 32 out-edges) and 16 bytes per 32 edges -- 2.0 GB at 65 536 nodes with 786 000 edges -- and a device that supports
+ * from 14 500 nodes on at least what its bit-matrix traversal needs (the one used beyond 22 000 nodes): about 8 KB per node
+ * for each of min(4, ceil(n/8192)) groups of thread blocks (eight bit matrices of 1 KB rows per group: visited, and one
+ * frontier per level up to 6; later levels reuse two of them) plus 1 KB per 33 edges per group (rows for vertices with more
+ * than 32 out-edges) and 16 bytes per 32 edges -- 2.2 GB at 65 536 nodes with 786 000 edges -- and a device that supports
  * cooperative launches; other batches with a larger graph: 4(G+1) + 4 n_total + 4 G bytes (per-graph offsets, and the
  * connected-component label of every node: the search of an undirected graph without a vertex of more than 64 out-edges
  * stops at level max_dist), and beyond 17 066 nodes 12 bytes per node of the largest graph for each of up to

@@ -386,7 +386,8 @@ constexpr int kDenseVecs = kDenseRowWords / 128;         // 16-byte vectors per 
 constexpr int kDenseChunk = 32;                          // out-edges per work item
 constexpr int kDenseBatch = 4;                           // work items a warp takes at a time
 constexpr int kDenseMaxGroups = 4;                       // CTA groups working on different column blocks at once
-constexpr int kDenseHist = 5;                            // levels whose frontier matrices are kept for the output pass (later levels blend into written rows)
+constexpr int kDenseHist = 6;                            // levels whose frontier matrices are kept for the output pass (later levels blend into written rows)
+constexpr size_t kDenseSyncBytes = (size_t)(256 + 4 * kDenseRowWords * 4) * kDenseMaxGroups;       // sync words, then live targets
 constexpr int kDensePlanes = kDenseHist + 1;             // frontier matrices per group (level 0 .. kDenseHist)
 constexpr int kDenseFlagWords = 8192;                    // row flags of a level kept as a bitmap in shared memory (graphs up to 262 144 vertices)
 constexpr uint32_t kGridWaitIterations = 1u << 24;
@@ -402,6 +403,7 @@ struct DenseParams {
     uint8_t* row_done;      // [n_max] every valid target of the block is visited
     int32_t* item_start;    // [n_max + 1] prefix sum of chunks per vertex (of the current graph)
     int4* item_rec;         // [n_items] {vertex, first edge, one past the last edge, chunks of the vertex} of a work item
+    uint32_t* live;         // [4][kDenseRowWords] targets that some vertex gained, by level mod 4
     uint32_t* sync;         // [0] barrier counter, [1] abort, [2..5] "some frontier bit" and [8..11] work counter, by level mod 4
     int32_t n_max;
     int32_t n_pad;          // n_max rounded up to 32: pitch of the flag arrays
@@ -541,17 +543,16 @@ __device__ __forceinline__ bool dense_grid_sync(uint32_t* sync, uint32_t& epoch,
     return s_ok != 0;
 }
 
-// the 16 output bytes of 16 targets: bytes whose bit is set in m16 take `code`, the others keep `old`
-__device__ __forceinline__ uint4 dense_blend16(uint4 old, uint32_t m16, uint32_t code4)
+// Within a word of 32 targets, target 4 k + j is bit 8 j + k (Rows in spd_pull.cuh): the byte lanes of (word >> k) & 0x01010101
+// are then four neighbouring output bytes.
+__device__ __forceinline__ uint32_t dense_bit(int32_t rel) { return rel >= 0 && rel < 32 ? 1u << ((rel & 3) * 8 + (rel >> 2)) : 0u; }
+// the first n of a word's targets
+__device__ __forceinline__ uint32_t dense_valid(int32_t n)
 {
-    uint32_t o[4] = {old.x, old.y, old.z, old.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t nib = (m16 >> (4 * j)) & 0xFu;
-        const uint32_t bm = ((nib * 0x00204081u) & 0x01010101u) * 0xFFu;      // bit i of the nibble -> byte i
-        o[j] = (o[j] & ~bm) | (code4 & bm);
-    }
-    return make_uint4(o[0], o[1], o[2], o[3]);
+    if (n >= 32) return 0xffffffffu;
+    if (n <= 0) return 0u;
+    const int k = n >> 2, r = n & 3;
+    return ((1u << k) - 1u) * 0x01010101u | ((0x00010101u >> (8 * (3 - r))) << k);
 }
 
 // bytes of a word (32 targets from t0) of an output row that the output pass has written: the bytes whose bit
@@ -561,11 +562,16 @@ __device__ __forceinline__ void dense_blend_word(uint8_t* row, int32_t t0, uint3
     const uint32_t code4 = code * 0x01010101u;
 #pragma unroll
     for (int hlf = 0; hlf < 2; ++hlf) {
-        const uint32_t m = (set >> (16 * hlf)) & 0xFFFFu;
-        if (m) {
-            uint4* ptr = (uint4*)(row + t0 + 16 * hlf);
-            *ptr = dense_blend16(__ldcg(ptr), m, code4);      // written by another SM in an earlier level
+        if (((set >> (4 * hlf)) & 0x0F0F0F0Fu) == 0u) continue;
+        uint4* ptr = (uint4*)(row + t0 + 16 * hlf);
+        const uint4 old = __ldcg(ptr);                           // written by another SM in an earlier level
+        uint32_t o[4] = {old.x, old.y, old.z, old.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t bm = ((set >> (4 * hlf + j)) & 0x01010101u) * 0xFFu;
+            o[j] = (o[j] & ~bm) | (code4 & bm);
         }
+        *ptr = make_uint4(o[0], o[1], o[2], o[3]);
     }
 }
 
@@ -586,6 +592,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
         d.vis += m * kDenseRowWords; d.fr += m * kDensePlanes * kDenseRowWords; d.acc += (size_t)grp * d.acc_rows * kDenseRowWords;
         d.acc_cnt += m; d.nonempty += (size_t)grp * d.n_pad * kDensePlanes; d.row_done += m;
         d.sync += grp * 64;
+        d.live += grp * 4 * kDenseRowWords;
     }
     const int lane = threadIdx.x & 31;
     const int gw = (int)((cta * blockDim.x + threadIdx.x) >> 5);
@@ -596,6 +603,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     const int32_t n_items = d.item_start[n];
     const uint32_t unreach = (uint32_t)(p.max_dist + 1);
     __shared__ uint32_t s_flags[kDenseFlagWords];
+    __shared__ __align__(16) uint32_t s_live[kDenseRowWords], s_gained[kDenseRowWords];
     const bool flags_in_smem = n <= kDenseFlagWords * 32;
     uint32_t epoch = 0;
     uint32_t step = 0;                         // levels over all column blocks: index of the rotating "any" flags
@@ -614,8 +622,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int32_t t0 = col0 + dense_word(lane, q, j) * 32;
-                const int32_t nv = n - t0;
-                const uint32_t vm = nv >= 32 ? 0xffffffffu : (nv <= 0 ? 0u : ((1u << nv) - 1u));
+                const uint32_t vm = dense_valid(n - t0);
                 acc[q][j] &= ~v[j] & vm;
                 if (acc[q][j]) {
                     if (blend) dense_blend_word(p.spd + (int64_t)s * ld, t0, acc[q][j], code);
@@ -624,6 +631,13 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 full = full && (((v[j] | acc[q][j]) & vm) == vm);
             }
             if (vec_new) *(uint4*)&vis_row[dense_word(lane, q, 0)] = make_uint4(v[0] | acc[q][0], v[1] | acc[q][1], v[2] | acc[q][2], v[3] | acc[q][3]);
+            if (vec_new) {                 // (most rows add no target that another row of this CTA has not gained)
+                const uint4 g4 = *(const uint4*)&s_gained[dense_word(lane, q, 0)];
+                const uint32_t g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (acc[q][j] & ~g[j]) atomicOr(&s_gained[dense_word(lane, q, j)], acc[q][j]);
+            }
             any_new = any_new || vec_new;
         }
         const bool row_new = __any_sync(0xffffffffu, any_new);
@@ -677,25 +691,16 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 for (int j = 0; j < 4; ++j) {
                     const int32_t t0 = col0 + dense_word(lane, q, j) * 32;
                     if (t0 >= (int32_t)ld) continue;
-                    const int32_t nv = n - t0, np = (int32_t)ld - t0, rel = s - t0;
-                    const uint32_t vm = nv >= 32 ? 0xffffffffu : (nv <= 0 ? 0u : ((1u << nv) - 1u));
-                    const uint32_t pm = (np >= 32 ? 0xffffffffu : ((1u << np) - 1u)) & ~vm;       // padding columns
-                    const uint32_t self = (rel >= 0 && rel < 32) ? (1u << rel) : 0u;
-                    const uint32_t miss = ~found[j] & ~self & vm;
+                    const uint32_t vm = dense_valid(n - t0), pm = ~vm;
+                    const uint32_t miss = ~found[j] & ~dense_bit(s - t0) & vm;
+                    uint32_t o[8];
+                    nibbles<false>(cb[0][j], cb[1][j], cb[2][j], cb[3][j], o);
 #pragma unroll
-                    for (int hlf = 0; hlf < 2; ++hlf) {
-                        if (t0 + 16 * hlf >= (int32_t)ld) continue;
-                        uint32_t o[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int sh = 16 * hlf + 4 * k;
-                            auto spread = [&](uint32_t w) { return (((w >> sh) & 0xFu) * 0x00204081u) & 0x01010101u; };   // bit i of the nibble -> byte i
-                            o[k] = spread(cb[0][j]) | (spread(cb[1][j]) << 1) | (spread(cb[2][j]) << 2) | (spread(cb[3][j]) << 3);
-                            o[k] |= spread(miss) * unreach;
-                            if (pm) o[k] |= spread(pm) * 255u;
-                        }
-                        *(uint4*)(row + t0 + 16 * hlf) = make_uint4(o[0], o[1], o[2], o[3]);
+                    for (int k = 0; k < 8; ++k) {
+                        o[k] |= ((miss >> k) & 0x01010101u) * unreach;
+                        if (pm) o[k] |= ((pm >> k) & 0x01010101u) * 255u;
                     }
+                    store_row_piece(row + t0, o, (int32_t)ld - t0);
                 }
             }
         }
@@ -710,8 +715,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 uint32_t bit[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int32_t rel = s - col0 - dense_word(lane, q, j) * 32;
-                    bit[j] = (rel >= 0 && rel < 32) ? (1u << rel) : 0u;
+                    bit[j] = dense_bit(s - col0 - dense_word(lane, q, j) * 32);
                 }
                 const uint4 b4 = make_uint4(bit[0], bit[1], bit[2], bit[3]);
                 *(uint4*)&d.vis[(size_t)s * kDenseRowWords + dense_word(lane, q, 0)] = b4;
@@ -733,6 +737,13 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
             uint32_t* fnext = d.fr + (size_t)pl_next * d.n_max * kDenseRowWords;
             const uint8_t* ne_cur = d.nonempty + (size_t)pl_cur * d.n_pad;
             uint8_t* ne_next = d.nonempty + (size_t)pl_next * d.n_pad;
+            // Targets that some vertex gained at the level before: no other target can be gained at this one (a path to it of this
+            // length contains one shorter by a hop), so a vertex that misses only others is done.  Without this the targets in
+            // tiny components keep every row open to the last level.
+            for (int w = (int)threadIdx.x; w < kDenseRowWords; w += (int)blockDim.x) {
+                s_live[w] = level == 1 ? 0xffffffffu : __ldcg(&d.live[((step - 1u) & 3u) * kDenseRowWords + w]);
+                s_gained[w] = 0u;
+            }
             // The flags of the current frontier as a bitmap in shared memory: an item looks up one per out-edge, and
             // at the first and last levels that look-up is all an item does.
             if (flags_in_smem) {
@@ -745,8 +756,8 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                         bits |= ((x[k] & 1u) | ((x[k] >> 7) & 2u) | ((x[k] >> 14) & 4u) | ((x[k] >> 21) & 8u)) << (4 * k);
                     s_flags[w] = bits;
                 }
-                __syncthreads();
             }
+            __syncthreads();
             // Items cost between one flag read and tens of KB of row reads, so warps take them in batches of four
             // from a counter (one per level, four in rotation) and ask for the next batch before working.  The
             // four items of a batch lie a quarter of the list apart: the chunks of one high-degree vertex are
@@ -759,48 +770,69 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 const int batch = __shfl_sync(0xffffffffu, batch_next, 0);
                 if (batch >= n_batches) break;
                 if (lane == 0) batch_next = (int)atomicAdd(counter, 1u);
-              int4 rec_next = d.item_rec[batch];
-              for (int item = batch; item < n_items; item += n_batches) {
-                const int4 rec = rec_next;                                  // one 16-byte record per item, fetched an item ahead
-                if (item + n_batches < n_items) rec_next = d.item_rec[item + n_batches];
-                const int s = rec.x;
-                const int32_t n_chunks = rec.w;
+                // Lane k looks item k of the batch over, so that a batch without work costs one chain of loads and not one per
+                // item (at most levels most items have none).
+                static_assert(kDenseChunk == 32 && kDenseBatch <= 32, "one edge per lane, one item per lane");
+                const int item = batch + lane * n_batches;
+                const bool valid = lane < kDenseBatch && item < n_items;
+                const int4 rec_mine = valid ? d.item_rec[item] : make_int4(0, 0, 0, 1);
+                const bool done = !valid || __ldcg(&d.row_done[rec_mine.x]) != 0;
+                uint32_t m_mine = 0u;                       // the neighbours whose frontier row has a bit set
+                {
+                    int32_t u[kDenseBatch];
+#pragma unroll
+                    for (int k = 0; k < kDenseBatch; ++k) {
+                        const int32_t e = __shfl_sync(0xffffffffu, rec_mine.y, k) + lane, e1 = __shfl_sync(0xffffffffu, done ? 0 : rec_mine.z, k);
+                        u[k] = e < e1 ? ci[e] : -1;
+                    }
+#pragma unroll
+                    for (int k = 0; k < kDenseBatch; ++k) {
+                        const bool hit = u[k] >= 0 && (flags_in_smem ? ((s_flags[u[k] >> 5] >> (u[k] & 31)) & 1u) : (uint32_t)__ldcg(&ne_cur[u[k]]));
+                        const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                        if (lane == k) m_mine = hits;
+                    }
+                }
+                // Without a neighbour's bit nothing can be new; the flag of the next row may be stale (planes in turn).  A split vertex
+                // that is not complete has all its chunks counted.
+                const bool idle = done || (m_mine == 0u && rec_mine.w == 1);
+                if (valid && idle && emitted) ne_next[rec_mine.x] = 0;
+                uint32_t todo = __ballot_sync(0xffffffffu, !idle);
+              while (todo) {
+                const int k_item = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const int s = __shfl_sync(0xffffffffu, rec_mine.x, k_item);
+                const int32_t n_chunks = __shfl_sync(0xffffffffu, rec_mine.w, k_item);
                 uint32_t acc[kDenseVecs][4];
 #pragma unroll
                 for (int q = 0; q < kDenseVecs; ++q)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) acc[q][j] = 0u;
                 uint32_t* vis_row = d.vis + (size_t)s * kDenseRowWords;
-                const bool done = __ldcg(&d.row_done[s]) != 0;
-                // a complete vertex whose row in the next-frontier buffer is already empty needs nothing at all
-                // (every chunk of a split vertex sees the same two flags, so they all skip together)
-                if (done && !__ldcg(&ne_next[s])) continue;
-                if (!done) {
-                    static_assert(kDenseChunk == 32, "one edge per lane");
-                    // the neighbours whose frontier row has a bit set; with none of them nothing can be new
-                    // here, and the visited row need not even be read (most items at the first and last levels)
-                    const int32_t e = rec.y + lane;
-                    int32_t u = e < rec.z ? ci[e] : -1;
-                    if (u >= 0 && !(flags_in_smem ? ((s_flags[u >> 5] >> (u & 31)) & 1u) : (uint32_t)__ldcg(&ne_cur[u]))) u = -1;
-                    uint32_t m = __ballot_sync(0xffffffffu, u >= 0);
-                    if (m == 0u && n_chunks == 1) {
-                        if (emitted && lane == 0) ne_next[s] = 0;      // planes in turn: the flag may be stale
-                        continue;
-                    }
+                {
+                    uint32_t m = __shfl_sync(0xffffffffu, m_mine, k_item);
+                    const int32_t e0 = __shfl_sync(0xffffffffu, rec_mine.y, k_item);
+                    const int32_t u = (m >> lane) & 1u ? ci[e0 + lane] : -1;
                     if (m) {
-                        // bits this vertex still misses: once the neighbours read so far cover them all, the rest
+                        // bits this vertex still misses and may gain: once the neighbours read so far cover them all, the rest
                         // of the edge list cannot add anything (at the dense levels a few rows are enough)
-                        uint32_t need[kDenseVecs][4];
+                        uint32_t need[kDenseVecs][4], open = 0u;
 #pragma unroll
                         for (int q = 0; q < kDenseVecs; ++q) {
                             const uint4 v4 = __ldcg((const uint4*)&vis_row[dense_word(lane, q, 0)]);
-                            const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
+                            const uint4 l4 = *(const uint4*)&s_live[dense_word(lane, q, 0)];
+                            need[q][0] = ~v4.x & l4.x; need[q][1] = ~v4.y & l4.y; need[q][2] = ~v4.z & l4.z; need[q][3] = ~v4.w & l4.w;
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                const int32_t nv = n - (col0 + dense_word(lane, q, j) * 32);
-                                const uint32_t vm = nv >= 32 ? 0xffffffffu : (nv <= 0 ? 0u : ((1u << nv) - 1u));
-                                need[q][j] = ~v[j] & vm;
+                                if (level == 1) need[q][j] &= dense_valid(n - (col0 + dense_word(lane, q, j) * 32));     // (later, no others are live)
+                                open |= need[q][j];
                             }
+                        }
+                        if (__all_sync(0xffffffffu, open == 0u)) {    // nothing to gain at this level or later
+                            if (n_chunks == 1) {
+                                if (lane == 0) { ne_next[s] = 0; d.row_done[s] = 1; }
+                                continue;
+                            }
+                            m = 0u;                                   // (every chunk of a split vertex has to be counted)
                         }
                         while (m) {                                   // two frontier rows (2 x 1 KB) in flight
                             const int b0 = __ffs(m) - 1;
@@ -862,12 +894,17 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 }
               }
             }
+            __syncthreads();
+            for (int w = (int)threadIdx.x; w < kDenseRowWords; w += (int)blockDim.x)
+                if (s_gained[w]) atomicOr(&d.live[(step & 3u) * kDenseRowWords + w], s_gained[w]);
             if (!dense_grid_sync(d.sync, epoch, p.header, n_ctas, d.barrier_extra, d.barrier_limit)) return;
             const uint32_t any = *(volatile uint32_t*)&d.sync[2 + flag_idx];
             if (cta == 0 && threadIdx.x == 0) {                 // next written two levels from now
                 d.sync[2 + ((step + 2u) & 3u)] = 0u;
                 d.sync[8 + ((step + 2u) & 3u)] = 0u;
             }
+            if (cta == 0)
+                for (int w = (int)threadIdx.x; w < kDenseRowWords; w += (int)blockDim.x) d.live[((step + 2u) & 3u) * kDenseRowWords + w] = 0u;
             ++step;
             if (!emitted && (!any || level == kDenseHist)) {
                 emit_rows(col0, level);
@@ -970,7 +1007,7 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
             pl.dense_off[4] = off; off += align_up(G * align_up(n, 32) * kDensePlanes, 256);
             pl.dense_off[5] = off; off += align_up(G * n, 256);
             pl.dense_off[6] = off; off += align_up((n + 1) * sizeof(int32_t), 256);
-            pl.dense_off[7] = off; off += 256 * kDenseMaxGroups;
+            pl.dense_off[7] = off; off += kDenseSyncBytes;
             // work items: one per vertex plus one per further chunk of out-edges
             pl.dense_off[8] = off; off += align_up((n + (size_t)(nnz > 0 ? nnz : 0) / kDenseChunk + 1) * sizeof(int4), 256);
             pl.dense_off[9] = off; off += align_up(n * sizeof(int32_t), 256);
@@ -1042,6 +1079,7 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
         d.row_done = ws + pl.dense_off[5];
         d.item_start = (int32_t*)(ws + pl.dense_off[6]);
         d.sync = (uint32_t*)(ws + pl.dense_off[7]);
+        d.live = d.sync + 64 * kDenseMaxGroups;
         d.item_rec = (int4*)(ws + pl.dense_off[8]);
         d.acc_row = (int32_t*)(ws + pl.dense_off[9]);
         d.acc_rows = pl.dense_acc_rows;
@@ -1053,7 +1091,7 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
         g_barrier_overcount = 0;
         // accumulator rows, their counters and the barrier words start at zero
         GT_CUDA_TRY(cudaMemsetAsync(ws + pl.dense_off[2], 0, pl.dense_off[4] - pl.dense_off[2], s));
-        GT_CUDA_TRY(cudaMemsetAsync(ws + pl.dense_off[7], 0, 256 * kDenseMaxGroups, s));
+        GT_CUDA_TRY(cudaMemsetAsync(ws + pl.dense_off[7], 0, kDenseSyncBytes, s));
         {
             // the block totals borrow the start of the item records, which are written afterwards
             const unsigned scan_blocks = (unsigned)((batch->n_total + kScanBlock - 1) / kScanBlock);

@@ -216,6 +216,19 @@ __device__ __forceinline__ void inherit(uint8_t* cur, int i, const uint16_t* tpo
     if (grew) R::store(cur, i, row);
 }
 
+// 32 output bytes of which the row's pitch (a multiple of 16) has room for `room`: a whole sector where it is aligned.
+__device__ __forceinline__ void store_row_piece(uint8_t* at, const uint32_t (&o)[8], int room)
+{
+    if (room >= 32 && ((uintptr_t)at & 31u) == 0) {
+        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(at), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                     "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                     : "memory");
+    } else {
+        *(uint4*)at = make_uint4(o[0], o[1], o[2], o[3]);
+        if (room > 16) *(uint4*)(at + 16) = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+}
+
 // One word of a row's code planes -> 32 output bytes at `row`, columns `col` and up of a block of nt valid targets and `cols`
 // columns inside the row pitch; columns past the last target are row padding.
 __device__ __forceinline__ void emit_word(const uint32_t (&c)[8], int n_planes, uint8_t* row, int col, int nt, int cols)
@@ -230,14 +243,7 @@ __device__ __forceinline__ void emit_word(const uint32_t (&c)[8], int n_planes, 
             if (past > 0) o[j] |= past >= 4 ? 0xffffffffu : 0xffffffffu << (8 * (4 - past));
         }
     }
-    if (col + 32 <= cols && ((uintptr_t)row & 31u) == 0) {
-        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(row), "r"(o[0]), "r"(o[1]), "r"(o[2]),
-                     "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
-                     : "memory");
-    } else {
-        *(uint4*)row = make_uint4(o[0], o[1], o[2], o[3]);
-        if (col + 16 < cols) *(uint4*)(row + 16) = make_uint4(o[4], o[5], o[6], o[7]);
-    }
+    store_row_piece(row, o, cols - col);
 }
 
 }  // namespace gt
