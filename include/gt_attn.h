@@ -95,9 +95,9 @@ gt_status gt_check(void* workspace, void* stream);
  * distinct from unreachable pairs (bucket max_dist+1).  Bit-exact and deterministic.
  * Out-of-range col_idx entries are undefined behaviour.
  * Workspace (gt_spd_build_workspace says how much): 256 bytes for graphs of up to about 5 000 nodes, whose whole traversal
- * state fits shared memory; a single graph of up to 22 000 nodes: its edge list once more (2 bytes per edge) and bit planes of
+ * state fits shared memory; a single graph of up to 19 000 nodes: its edge list once more (2 bytes per edge) and bit planes of
  * 4 bytes per node, bit of max_dist + 1 and thread block in flight (up to two per SM; 24 MB at 8 192 nodes); a single graph
- * from 14 500 nodes on at least what its bit-matrix traversal needs (the one used beyond 22 000 nodes): about 8 KB per node
+ * from 14 500 nodes on at least what its bit-matrix traversal needs (the one used beyond 19 000 nodes): about 8 KB per node
  * for each of min(4, ceil(n/8192)) groups of thread blocks (eight bit matrices of 1 KB rows per group: visited, and one
  * frontier per level up to 6; later levels reuse two of them) plus 1 KB per 33 edges per group (rows for vertices with more
  * than 32 out-edges) and 16 bytes per 32 edges -- 2.2 GB at 65 536 nodes with 786 000 edges -- and a device that supports

@@ -4,7 +4,7 @@
 // loading data (Sec. "Preliminaries"; the data-loading stall of the latency model).  Here
 // the index form of that bias is built on the GPU, by one of four kernels (make_plan below):
 //   graphs of up to about 5 000 nodes       pull in shared memory (spd_pull.cu)
-//   one graph of up to 22 000 nodes         the same with edge list and code planes in the workspace (spd_pull_large.cu)
+//   one graph of up to 19 000 nodes         the same with edge list and code planes in the workspace (spd_pull_large.cu)
 //   one larger graph                        bit matrices in the workspace (further down)
 //   batches with a larger graph             multi-source frontier push (here)
 //

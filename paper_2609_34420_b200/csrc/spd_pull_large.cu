@@ -1,5 +1,5 @@
 // gt_spd_build for a single graph whose reachability rows fit shared memory but whose edge list does not (about 5 000 to
-// 22 000 nodes): the pull of spd_pull.cu with the edge list and the code planes in the workspace.
+// 19 000 nodes): the pull of spd_pull.cu with the edge list and the code planes in the workspace.
 //
 // Two small kernels sort the vertices by degree and lay the edge list out once for all thread blocks: groups of 32 vertices
 // of (nearly) equal degree with their edges interleaved, 16-bit vertex numbers in pairs, so that a warp reads 128 coalesced
@@ -23,9 +23,9 @@ constexpr int kLargeHubDegree = 126;
 constexpr int kLargeBins = 128;            // hubs, then degrees 126 .. 0
 constexpr size_t kLargeSmemLimit = 222 * 1024;      // and 3 KB of static arrays
 constexpr int kTargets = 32;
-// Beyond this the bit-matrix build is the faster one (power law, degree 12: 20 000 nodes 1.14 against 1.23 ms, 28 000 nodes
-// 1.84 against 1.79 ms); the two row sets would fit up to 28 000 nodes.
-constexpr int32_t kLargeMaxNodes = 22000;
+// Beyond this the bit-matrix build is the faster one (power law, degree 12: 18 000 nodes 0.85 against 0.91 ms, 20 000 nodes
+// 1.13 against 1.04 ms; from 592 blocks of targets on there is a fifth round); the row sets would fit up to 28 000 nodes.
+constexpr int32_t kLargeMaxNodes = 18944;
 constexpr int kCachedHubs = 400;           // hubs whose numbers and lists' places are kept in shared memory
 
 struct LargeParams {

@@ -43,7 +43,7 @@ def test_a_graph_whose_edges_do_not_fit_beside_sparse_ones():
     check(wl.Workload("outlier", wl.pack_graphs(graphs), 1, 32, 6))
 
 
-@pytest.mark.parametrize("n,m,D", [(5600, 80000, 1), (6001, 90000, 5), (7000, 9000, 30), (14200, 60000, 20), (21999, 50000, 9)])
+@pytest.mark.parametrize("n,m,D", [(5600, 80000, 1), (6001, 90000, 5), (7000, 9000, 30), (14200, 60000, 20), (18941, 50000, 9)])
 def test_one_graph_with_lists_in_the_workspace(n, m, D):
     """Hubs beyond a group's degree (some more than are kept in shared memory), sparse directed graphs of many levels,
     the last target block ragged, two blocks per SM and one."""
