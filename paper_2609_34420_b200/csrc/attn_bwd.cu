@@ -71,6 +71,7 @@ struct BwdParams {
     int32_t n_buckets;
     int32_t bin_log;         // shared bins (more than kMaxPrivateBinBuckets buckets): log2 of the columns per bucket
     int32_t early_release;   // let the next kernel start its set-up while this one runs
+    const int4* list;        // packed batch: work list; block index = entry * heads + head (nullptr: grid of heads x tiles x graphs)
     const uint8_t* maps;     // packed batch: tensor maps of the graphs' SPD^T blocks (workspace); nullptr: single graph
     int32_t kv_row0;         // key rows [kv_row0, kv_row_end) of a graph are this launch's (chunked / step entry points)
     int32_t kv_row_end;
@@ -159,12 +160,22 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
-    const int h = blockIdx.x;
-    const int g = blockIdx.z;
+    int h = blockIdx.x, g = blockIdx.z, kv_tile = blockIdx.y;
+    int32_t node0 = 0, n_g = p.n_total;
     if (p.cu_seqlens) grid_wait();          // a single graph's blocks set up their barriers and tensor memory before they wait
-    const int32_t node0 = p.cu_seqlens ? p.cu_seqlens[g] : 0;
-    const int32_t n_g = p.cu_seqlens ? p.cu_seqlens[g + 1] - node0 : p.n_total;
-    const int32_t kv0 = p.kv_row0 + (int32_t)blockIdx.y * kTile;
+    if (p.list) {
+        const int4 entry = p.list[blockIdx.x / (unsigned)p.n_heads];
+        if (entry.x < 0) return;
+        h = (int)(blockIdx.x % (unsigned)p.n_heads);
+        g = entry.x;
+        kv_tile = entry.y;
+        node0 = entry.z;
+        n_g = entry.w;
+    } else if (p.cu_seqlens) {
+        node0 = p.cu_seqlens[g];
+        n_g = p.cu_seqlens[g + 1] - node0;
+    }
+    const int32_t kv0 = p.kv_row0 + kv_tile * kTile;
     const int32_t kv_lim = min(n_g, p.kv_row_end);
     if (kv0 >= kv_lim) return;
     const int32_t q_lo = p.q_row0, q_hi = min(n_g, p.q_row_end);
@@ -655,6 +666,7 @@ struct PrepareParams {
     const uint8_t* spd;
     uint8_t* spd_t;
     uint8_t* maps;             // packed batch: tensor maps of the spd_t blocks, made from `model`
+    int4* list;                // packed batch: work list of the main kernel, made by the last blocks
     const int64_t* spd_offsets;
     const int32_t* cu_seqlens;
     const __nv_bfloat16* out;
@@ -664,7 +676,7 @@ struct PrepareParams {
     uint4* ext;
     float4* dq_acc;            // cleared, unless nullptr (step entry points: the caller's sums)
     double* db_acc;            // cleared: [n_db]
-    int32_t n_total, n_heads, n_db;
+    int32_t n_total, n_graphs, n_heads, n_db;
     int32_t tiles;             // transpose tiles along a side of the largest graph
     uint32_t row_blocks;       // thread blocks that work on rows; the others transpose
     uint32_t last_bucket;
@@ -690,6 +702,11 @@ __global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const __gr
     grid_release();
     if (blockIdx.x >= p.row_blocks) {
         const uint32_t b = blockIdx.x - p.row_blocks, per_graph = (uint32_t)(p.tiles * p.tiles);
+        if (b >= per_graph * (uint32_t)p.n_graphs) {
+            const int32_t w = (int32_t)((b - per_graph * (uint32_t)p.n_graphs) * (kPrepareThreads / 32) + (threadIdx.x >> 5));
+            if (w < p.n_graphs) write_work_list<kTile>(p.list, p.n_total / kTile + p.n_graphs, p.cu_seqlens, p.n_graphs, w);
+            return;
+        }
         const int g = (int)(b / per_graph), r = (int)(b % per_graph);
         const int32_t n_g = p.cu_seqlens ? p.cu_seqlens[g + 1] - p.cu_seqlens[g] : p.n_total;
         const int32_t i0 = (r / p.tiles) * 128, j0 = (r % p.tiles) * 128;
@@ -770,13 +787,14 @@ __global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const __gr
     p.ext[2 * row + 1] = e1;
 }
 
-gt_status launch_prepare(PrepareParams p, int32_t head_dim, int32_t max_seqlen, int32_t n_graphs, cudaStream_t s)
+gt_status launch_prepare(PrepareParams p, int32_t head_dim, int32_t max_seqlen, cudaStream_t s)
 {
     const size_t rows = (size_t)p.n_total * p.n_heads, per_block = kPrepareRows;
     p.tiles = (max_seqlen + 127) / 128;
     p.row_blocks = (uint32_t)((rows + per_block - 1) / per_block);
     p.sqrt_d = sqrtf((float)head_dim);
-    const dim3 grid((unsigned)(p.row_blocks + (uint64_t)p.tiles * p.tiles * n_graphs));
+    const uint64_t list_blocks = p.list != nullptr ? (p.n_graphs + kPrepareThreads / 32 - 1) / (kPrepareThreads / 32) : 0;
+    const dim3 grid((unsigned)(p.row_blocks + (uint64_t)p.tiles * p.tiles * p.n_graphs + list_blocks));
     return head_dim == 64 ? launch_overlapped(bwd_prepare_kernel<64>, grid, kPrepareThreads, 0, s, p)
                           : launch_overlapped(bwd_prepare_kernel<32>, grid, kPrepareThreads, 0, s, p);
 }
@@ -807,7 +825,7 @@ __global__ void bwd_finalize_kernel(const float* __restrict__ dq_acc, __nv_bfloa
 }
 
 struct BwdWorkspace {
-    size_t db_off, ext_off, dq_off, maps_off, spdt_off, total;
+    size_t db_off, ext_off, dq_off, maps_off, list_off, spdt_off, total;
 };
 
 BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim, int32_t max_dist, int32_t n_chunks = 1)
@@ -818,7 +836,8 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
     w.ext_off = w.db_off + align_up((size_t)n_chunks * n_heads * (max_dist + 2) * sizeof(double), 256);
     w.dq_off = w.ext_off + align_up(rows * kExtCols * 2, 256);
     w.maps_off = w.dq_off + align_up(rows * head_dim * sizeof(float), 256);
-    w.spdt_off = w.maps_off + maps_bytes(b->n_graphs);
+    w.list_off = w.maps_off + maps_bytes(b->n_graphs);
+    w.spdt_off = w.list_off + list_bytes(b, kTile);
     // transposed SPD copy: at most sum n_g * round_up(n_g,16) <= n_total * round_up(max_seqlen,16) bytes
     w.total = w.spdt_off + align_up((size_t)b->n_total * (size_t)((b->max_seqlen + 15) & ~15), 256);
     return w;
@@ -831,7 +850,8 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
 {
     const int32_t kv_end = p.kv_row_end < batch->max_seqlen ? p.kv_row_end : batch->max_seqlen;
     if (kv_end <= p.kv_row0 || p.q_row_end <= p.q_row0) return GT_OK;      // empty key chunk / no queries
-    dim3 grid((unsigned)p.n_heads, (unsigned)((kv_end - p.kv_row0 + kTile - 1) / kTile), (unsigned)batch->n_graphs);
+    const dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kTile) * p.n_heads))
+                             : dim3((unsigned)p.n_heads, (unsigned)((kv_end - p.kv_row0 + kTile - 1) / kTile), (unsigned)batch->n_graphs);
     CUtensorMap tdq;
     gt_status st_map = encode_dq_map(&tdq, p.dq_acc, p.n_total, p.n_heads, D);
     if (st_map != GT_OK) return st_map;
@@ -915,7 +935,10 @@ static gt_status gt_bwd_run(const void* q, const void* k, const void* v, const v
     BwdParams p{};
     uint8_t* spd_t = ws + wsp.spdt_off;
     if ((st = encode_spd_map(&tspd, spd_t, batch->max_seqlen, 128)) != GT_OK) return st;
-    if (batch->n_graphs > 1) p.maps = maps_at(ws + wsp.maps_off);
+    if (batch->n_graphs > 1) {
+        p.maps = maps_at(ws + wsp.maps_off);
+        if (list_saves(batch, kTile, n_heads, 0)) p.list = (const int4*)(ws + wsp.list_off);
+    }
     p.cu_seqlens = batch->n_graphs > 1 ? batch->cu_seqlens : nullptr;
     p.bias = bias;
     p.dq_acc = (float*)(ws + wsp.dq_off);
@@ -933,6 +956,8 @@ static gt_status gt_bwd_run(const void* q, const void* k, const void* v, const v
     PrepareParams pre{};
     pre.spd = spd; pre.spd_t = spd_t; pre.spd_offsets = batch->n_graphs > 1 ? spd_offsets : nullptr; pre.cu_seqlens = p.cu_seqlens;
     pre.maps = const_cast<uint8_t*>(p.maps);
+    pre.list = const_cast<int4*>(p.list);
+    pre.n_graphs = batch->n_graphs;
     pre.model = tspd;
     pre.out = (const __nv_bfloat16*)out; pre.out_f32 = out_f32; pre.dout = (const __nv_bfloat16*)dout; pre.lse = lse;
     pre.ext = ext;
@@ -940,7 +965,7 @@ static gt_status gt_bwd_run(const void* q, const void* k, const void* v, const v
     pre.db_acc = p.db_acc;
     pre.n_total = batch->n_total; pre.n_heads = n_heads; pre.n_db = n_kv_chunks * n_db;
     pre.last_bucket = (uint32_t)(max_dist + 1);
-    if ((st = launch_prepare(pre, head_dim, batch->max_seqlen, batch->n_graphs, s)) != GT_OK) return st;
+    if ((st = launch_prepare(pre, head_dim, batch->max_seqlen, s)) != GT_OK) return st;
     CUtensorMap text;
     if ((st = encode_thd_map(&text, ext, batch->n_total, n_heads, kExtCols)) != GT_OK) return st;
     // key chunks of w = round_up(ceil(N / C), 128) rows, as in the chunked forward
@@ -1093,9 +1118,9 @@ extern "C" gt_status gt_biased_attn_bwd_step_prepare_ex(const void* out, const f
     pre.spd = spd; pre.spd_t = ws + cx.spdt_off;
     pre.out = (const __nv_bfloat16*)out; pre.out_f32 = out_f32; pre.dout = (const __nv_bfloat16*)dout; pre.lse = lse;
     pre.ext = (uint4*)(ws + cx.ext_off);
-    pre.n_total = batch->n_total; pre.n_heads = n_heads;
+    pre.n_total = batch->n_total; pre.n_graphs = 1; pre.n_heads = n_heads;
     pre.last_bucket = (uint32_t)(max_dist + 1);
-    return launch_prepare(pre, head_dim, batch->n_total, 1, s);
+    return launch_prepare(pre, head_dim, batch->n_total, s);
 }
 
 extern "C" gt_status gt_biased_attn_bwd_step(const void* q, const void* k, const void* v, const void* dout, const float* bias,

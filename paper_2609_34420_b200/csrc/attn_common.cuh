@@ -44,9 +44,44 @@ __device__ __forceinline__ void acquire_tensor_map(const void* map)
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
 }
 constexpr size_t kMapBytes = 128;
-// their place in a workspace whose address is a multiple of 16; none for a single graph
+// Their place in a workspace whose address is a multiple of 16; none for a single graph.
 inline size_t maps_bytes(int32_t n_graphs) { return n_graphs > 1 ? align_up((size_t)n_graphs * kMapBytes, 256) + kMapBytes : 0; }
 inline uint8_t* maps_at(uint8_t* region) { return (uint8_t*)align_up(reinterpret_cast<uintptr_t>(region), kMapBytes); }
+
+// Work list of a packed batch, whose sizes are on the device only: entry i = {graph, block of `rows` rows of it, the graph's first
+// row, its rows}; graph -1: unused.  A grid of (largest graph) x (graphs) launches a third to a half of its blocks for nothing where
+// sizes vary a lot, and those hold up the others (30 graphs of 128 to 4 096 nodes: forward 520 -> 504 us, backward 1 332 -> 1 275;
+// 64 of 512 to 2 048: 949 -> 945, 2 565 -> 2 518).  Up to kListSorted graphs come by falling size: the blocks that take longest start
+// first, which a few large graphs need (in batch order 510 and 1 303 us).  More graphs stay in the batch's order: the tail is short
+// anyway, and blocks of different lengths side by side hide each other's fill and drain (200 graphs of 64 to 1 000 nodes: 436 us in
+// order, 443 sorted).  A warp per graph writes its graph's entries and the unused ones behind them, with nothing to wait for.
+constexpr int kListSorted = 64;
+inline size_t list_entries(const gt_batch* b, int32_t rows) { return (size_t)(b->n_total / rows) + (size_t)b->n_graphs; }
+inline size_t list_bytes(const gt_batch* b, int32_t rows) { return b->n_graphs > 1 ? align_up(list_entries(b, rows) * sizeof(int4), 256) : 0; }
+// The grid without the list has more than `blocks` blocks more than the one with it (many graphs of one size need no list).
+inline bool list_saves(const gt_batch* b, int32_t rows, int32_t n_heads, size_t blocks)
+{
+    return (size_t)((b->max_seqlen + rows - 1) / rows) * (size_t)b->n_graphs * (size_t)n_heads > list_entries(b, rows) * (size_t)n_heads + blocks;
+}
+template <int kRows>
+__device__ __forceinline__ void write_work_list(int4* list, int32_t entries, const int32_t* __restrict__ cu_seqlens, int32_t n_graphs, int32_t g)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t c0 = cu_seqlens[g], n = cu_seqlens[g + 1] - c0, blocks = (n + kRows - 1) / kRows;
+    int32_t first = c0 / kRows + g, end = (c0 + n) / kRows + g + 1;      // in batch order: the next graph's first entry
+    if (n_graphs <= kListSorted) {
+        int32_t before = 0, all = 0;
+        for (int j = lane; j < n_graphs; j += 32) {
+            const int32_t other = cu_seqlens[j + 1] - cu_seqlens[j], b = (other + kRows - 1) / kRows;
+            before += other > n || (other == n && j < g) ? b : 0;
+            all += b;
+        }
+        first = __reduce_add_sync(0xffffffffu, before);
+        end = first + blocks == __reduce_add_sync(0xffffffffu, all) ? entries : first + blocks;
+    }
+    for (int32_t i = first + lane; i < end && i < entries; i += 32)
+        list[i] = i < first + blocks ? make_int4(g, i - first, c0, n) : make_int4(-1, 0, 0, 0);
+}
 
 struct AttnArgsCheck {
     const void* ptrs[12];

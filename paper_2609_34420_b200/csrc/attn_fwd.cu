@@ -83,6 +83,7 @@ struct FwdParams {
     int32_t state_q_begin;
     int32_t state_q_end;
     const uint8_t* maps;       // packed batch: tensor maps of the graphs' SPD blocks
+    const int4* list;          // packed batch: work list; block index = entry * heads + head (nullptr: grid of heads x blocks x graphs)
     int32_t spd_tma;           // 1: SPD tiles come by TMA; 0: packed batch without room for the maps, cp.async loader warp
     float c1;                  // log2(e) / sqrt(d)
 };
@@ -154,14 +155,25 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
-    const int h = blockIdx.x;
-    const int g = kPartial ? 0 : (int)blockIdx.z;
+    int h = blockIdx.x, g = kPartial ? 0 : (int)blockIdx.z;
+    int32_t q_block = (int32_t)blockIdx.y + p.q_block0;
     const int chunk = kPartial ? (int)blockIdx.z : 0;
 
     if (p.cu_seqlens) grid_wait();          // a single graph's blocks set up their barriers and tensor memory before they wait
-    const int32_t node0 = p.cu_seqlens ? p.cu_seqlens[g] : 0;
-    const int32_t n_g = p.cu_seqlens ? p.cu_seqlens[g + 1] - node0 : p.n_total;
-    const int32_t q0 = ((int32_t)blockIdx.y + p.q_block0) * kRowsPerCta;
+    int32_t node0 = 0, n_g = p.n_total;
+    if (!kPartial && p.list) {
+        const int4 entry = p.list[blockIdx.x / (unsigned)p.n_heads];
+        if (entry.x < 0) return;
+        h = (int)(blockIdx.x % (unsigned)p.n_heads);
+        g = entry.x;
+        q_block = entry.y;
+        node0 = entry.z;
+        n_g = entry.w;
+    } else if (p.cu_seqlens) {
+        node0 = p.cu_seqlens[g];
+        n_g = p.cu_seqlens[g + 1] - node0;
+    }
+    const int32_t q0 = q_block * kRowsPerCta;
     if (q0 >= n_g) return;
     const int64_t ld = (int64_t)((n_g + 15) & ~15);
     const uint8_t* spd_g = p.spd + (p.spd_offsets ? p.spd_offsets[g] : 0);
@@ -732,12 +744,24 @@ int32_t chunk_rows(int32_t n, int32_t n_chunks)
     return (w + kKvTile - 1) / kKvTile * kKvTile;
 }
 
-__global__ void __launch_bounds__(128) fwd_maps_kernel(const __grid_constant__ CUtensorMap model, uint8_t* maps, const uint8_t* spd,
-                                                       const int64_t* spd_offsets, const int32_t* cu_seqlens, int32_t n_graphs)
+constexpr size_t kListMinSaved = 128;     // thread blocks
+
+// Tensor maps of a packed batch, a thread per graph, behind its work list (unless `list` is null), a warp per graph.
+constexpr int kBatchThreads = 128;
+__global__ void __launch_bounds__(kBatchThreads) fwd_batch_kernel(const __grid_constant__ CUtensorMap model, uint8_t* maps, int4* list, int32_t entries,
+                                                                  const uint8_t* spd, const int64_t* spd_offsets, const int32_t* cu_seqlens, int32_t n_graphs)
 {
     grid_wait();
     grid_release();
-    const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    int32_t w = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (list != nullptr) {
+        if (w < n_graphs) {
+            write_work_list<kRowsPerCta>(list, entries, cu_seqlens, n_graphs, w);
+            return;
+        }
+        w -= n_graphs;
+    }
+    const int32_t g = w * 32 + (int32_t)(threadIdx.x & 31);
     if (g >= n_graphs) return;
     const int32_t n = cu_seqlens[g + 1] - cu_seqlens[g];
     if (n > 0) make_spd_map(maps + (size_t)g * kMapBytes, model, spd + spd_offsets[g], n);
@@ -755,7 +779,9 @@ gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     static std::atomic<uint64_t> granted[4] = {};
     const gt_status st = grant_smem(kern, granted[(p.n_buckets <= 32 ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0)], FwdSmem<D>::kDynamic);
     if (st != GT_OK) return st;
-    dim3 grid((unsigned)p.n_heads, (unsigned)(grid_y > 0 ? grid_y : (batch->max_seqlen + kRowsPerCta - 1) / kRowsPerCta), (unsigned)grid_z);
+    const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + kRowsPerCta - 1) / kRowsPerCta;
+    const dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kRowsPerCta) * p.n_heads))
+                             : dim3((unsigned)p.n_heads, (unsigned)row_blocks, (unsigned)grid_z);
     return launch_overlapped(kern, grid, kFwdThreads, FwdSmem<D>::kDynamic, s, tq, tk, tv, tspd, p);
 }
 
@@ -777,7 +803,7 @@ gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint
 extern "C" size_t gt_biased_attn_fwd_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim)
 {
     (void)n_heads; (void)head_dim;
-    return gt::kHeaderBytes + (gt::validate_batch(batch) == GT_OK ? gt::maps_bytes(batch->n_graphs) : 0);
+    return gt::kHeaderBytes + (gt::validate_batch(batch) == GT_OK ? gt::maps_bytes(batch->n_graphs) + gt::list_bytes(batch, gt::kRowsPerCta) : 0);
 }
 
 extern "C" gt_status gt_biased_attn_fwd(const void* q, const void* k, const void* v,
@@ -811,6 +837,9 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     p.spd_tma = batch->n_graphs == 1 ? 1 : 0;
     if (batch->n_graphs > 1 && workspace_bytes >= gt_biased_attn_fwd_workspace(batch, n_heads, head_dim)) {
         p.maps = maps_at((uint8_t*)workspace + kHeaderBytes);
+        // The list costs 1 us before the first block; that has to come back from the empty blocks that it saves.
+        if (list_saves(batch, kRowsPerCta, n_heads, kListMinSaved))
+            p.list = (const int4*)((uint8_t*)workspace + kHeaderBytes + maps_bytes(batch->n_graphs));
         p.spd_tma = 1;
     }
     if (p.spd_tma && (st = encode_spd_map(&tspd, spd, batch->max_seqlen, 256)) != GT_OK) return st;
@@ -828,8 +857,9 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     p.c1 = kLog2e / sqrtf((float)head_dim);
     cudaStream_t s = (cudaStream_t)stream;
     if (p.maps) {
-        st = launch_overlapped(fwd_maps_kernel, dim3((unsigned)(batch->n_graphs + 127) / 128), 128, 0, s, tspd, (uint8_t*)p.maps, spd,
-                               p.spd_offsets, p.cu_seqlens, batch->n_graphs);
+        const int32_t warps = (batch->n_graphs + 31) / 32 + (p.list ? batch->n_graphs : 0);
+        st = launch_overlapped(fwd_batch_kernel, dim3((unsigned)((warps * 32 + kBatchThreads - 1) / kBatchThreads)), kBatchThreads, 0, s, tspd,
+                               (uint8_t*)p.maps, (int4*)p.list, (int32_t)list_entries(batch, kRowsPerCta), spd, p.spd_offsets, p.cu_seqlens, batch->n_graphs);
         if (st != GT_OK) return st;
     }
     return head_dim == 64 ? launch_fwd<64, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s)

@@ -1,0 +1,48 @@
+"""The edges of the size rules by which the attention kernels choose their form, against the fp64 oracle
+(tolerances of the forward and backward parity tests, whose checks these call)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_34420_b200 import binding as gt
+from paper_2609_34420_b200 import workloads as wl
+
+from test_gpu_attn_bwd import check_backward
+from test_gpu_attn_fwd import check_forward, pytestmark  # noqa: F401  (GPU tests)
+
+
+def sizes(n_graphs, largest):
+    """One graph that dominates the grid of a batch; the others end at, before and behind the edges of 128 and 256 rows."""
+    rest = [1, 127, 128, 129, 255, 256, 257, 16, 300, 31]
+    return ([rest[i % len(rest)] for i in range(n_graphs // 2)] + [largest] + [rest[-1 - i % len(rest)] for i in range(n_graphs - n_graphs // 2 - 1)])
+
+
+# up to 64 graphs the work list is sorted, beyond that in batch order; 2 graphs: no list in the forward
+@pytest.mark.parametrize("n_graphs,largest,d", [(2, 257, 64), (40, 1500, 32), (64, 1281, 64), (65, 1281, 32), (97, 1024, 64)])
+def test_packed_batches_with_and_without_a_work_list(n_graphs, largest, d):
+    case, out, lse = check_forward(wl.small_workload(sizes(n_graphs, largest), 4, d, 6, seed=n_graphs, avg_degree=1.8))
+    # a workspace of the header alone: no tensor maps, no list, the SPD tiles come by 16-byte copies; same arithmetic
+    ws = torch.zeros(256, dtype=torch.uint8, device=case.q.device)
+    out2, lse2 = torch.full_like(out, float("nan")), torch.full_like(lse, float("nan"))
+    gt.gt_biased_attn_fwd(case.q, case.k, case.v, case.spd, case.bias, case.batch, case.w.max_dist, out2, lse2, ws)
+    gt.gt_check(ws)
+    assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("n_graphs,largest,d", [(2, 129, 32), (64, 700, 64), (65, 700, 32)])
+def test_packed_backward_work_list(n_graphs, largest, d):
+    check_backward(wl.small_workload(sizes(n_graphs, largest), 2, d, 6, seed=n_graphs, avg_degree=1.8))
+
+
+# private bin columns up to 26 buckets, then half as many columns per bucket at every doubling
+@pytest.mark.parametrize("buckets", [26, 27, 52, 53, 104, 105, 208, 209, 256])
+def test_bias_gradient_at_the_edges_of_the_bin_columns(buckets):
+    check_backward(wl.small_workload([260], 2, 64 if buckets % 2 else 32, buckets - 2, seed=buckets, avg_degree=1.1))
+
+
+def test_bias_gradient_reaches_every_bucket_of_a_path():
+    n, D = 400, 120
+    i = np.arange(n - 1)
+    w = wl.small_workload([n], 2, 64, D, seed=1)
+    w.batch = wl.pack_graphs([wl.csr_from_edges(n, i, i + 1, symmetric=True)])
+    check_backward(w)
