@@ -52,3 +52,9 @@ def test_one_graph_with_lists_in_the_workspace(n, m, D):
 
 def test_one_deep_undirected_graph_with_lists_in_the_workspace():
     one(wl.random_geometric(9000, 6.5, 4), 9)
+
+
+@pytest.mark.parametrize("n,m,D", [(18945, 46000, 11), (19200, 24000, 254), (19457, 400000, 2)])
+def test_one_graph_beyond_the_pull(n, m, D):
+    """The bit matrices at their smallest: more levels than level bits, a clip above them, rows that close early, isolated nodes."""
+    one(directed(n, m, n, hub_edges=5000, hubs=2), D)
