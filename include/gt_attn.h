@@ -178,8 +178,9 @@ void gt_test_hook_barrier_overcount(int32_t extra);
  * before the running max / sum are updated (Sec. GA-CP, item 3).  bf16 inputs, fp32
  * accumulation and softmax, bf16 `out` [T,H,d], fp32 `lse` [H,T].
  * bias: fp32 [n_heads, max_dist+2].
- * Workspace: 256 bytes, and for a packed batch 128 bytes per graph (descriptors of the SPD blocks) and 16 bytes per graph and per
- * 256 rows (a list of the work); a call that is handed the 256 bytes alone does without both, more slowly.
+ * Workspace: 256 bytes, 4 bytes per head and 256 rows (norms of the keys, for the fp32 output), and for a packed batch 128 bytes per
+ * graph (descriptors of the SPD blocks) and 16 bytes per graph and per 256 rows (a list of the work); a call that is handed the
+ * 256 bytes alone does without all of it, more slowly.
  * ------------------------------------------------------------------------------------- */
 size_t gt_biased_attn_fwd_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim);
 gt_status gt_biased_attn_fwd(const void* q, const void* k, const void* v,

@@ -58,6 +58,8 @@ constexpr int kCW = kHalves == 1 ? 32 : 16;   // columns per TMEM load
 constexpr int kChunks = kCols / kCW;
 static_assert(kChunks == 4, "the softmax pass is written for four chunks");
 constexpr float kSumThreshold = 1024.0f;      // tile row sum above which the reference maximum is raised
+constexpr int kNormRows = 256;                // precise variant: rows per entry of key_norms
+constexpr float kReach = 60.0f;               // precise variant: log2 of the largest P entry that needs no new reference
 
 struct FwdParams {
     const uint8_t* spd;
@@ -84,6 +86,8 @@ struct FwdParams {
     int32_t state_q_end;
     const uint8_t* maps;       // packed batch: tensor maps of the graphs' SPD blocks
     const int4* list;          // packed batch: work list; block index = entry * heads + head (nullptr: grid of heads x blocks x graphs)
+    const __nv_bfloat16* q;    // precise variant: for the rows' norms
+    const float* key_norms;    // precise variant: largest |k|^2 of every kNormRows rows, [H][blocks] (nullptr: always the classical way)
     int32_t spd_tma;           // 1: SPD tiles come by TMA; 0: packed batch without room for the maps, cp.async loader warp
     float c1;                  // log2(e) / sqrt(d)
 };
@@ -135,11 +139,29 @@ __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[N])
     if constexpr (N == 32) tmem_st32(taddr, r); else tmem_st16(taddr, r);
 }
 
+// Sum of the squares of eight bf16 values.
+__device__ __forceinline__ float square_sum(const uint4& v)
+{
+    float a = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t w = i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
+        const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xffff0000u);
+        a += lo * lo + hi * hi;
+    }
+    return a;
+}
+// Larger of two values that are not negative; NaN wins.
+__device__ __forceinline__ float norm_max(float a, float b) { return __uint_as_float(max(__float_as_uint(a) & 0x7fffffffu, __float_as_uint(b) & 0x7fffffffu)); }
+
 // kPrecise (the fp32-output entry point): P goes to the P V MMA as TWO bf16 terms, P = hi + lo with
 // lo = bf16(P - hi) (16 mantissa bits instead of 8), so that the output is accurate to fp32 accumulation
 // instead of to the 2^-9 relative rounding of a bf16 P.  The two terms of a 16-key chunk overwrite that
-// chunk's own score columns ([0,8) hi, [8,16) lo) as soon as the chunk has been read, which needs the
-// tile's maximum first: the precise variant always takes the classical two-pass way.
+// chunk's own score columns ([0,8) hi, [8,16) lo) as soon as the chunk has been read, so a tile cannot be
+// redone.  It may go the speculative way all the same where no score can overflow: |q_i| max|k_j| / sqrt(d) + max bias
+// bounds a row's scores, and while that is within 2^60 of the row's reference, P, l and O stay far inside the range
+// of fp32 and bf16, whose relative precision does not depend on the reference.  Rows (warps of 32) beyond it take the
+// maximum first, which costs a second pass over the scores.  8 192 nodes, 8 heads of 64: 386 -> 251 us, norms included.
 template <int D, bool kPartial, bool kShflBias, bool kPrecise = false>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
@@ -376,6 +398,28 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const float tbl = s_bias[lane];
         const uint64_t c1c1 = pack_f32x2(p.c1, p.c1);
 
+        // Precise variant: no score of this row exceeds |q| max|k| / sqrt(d) + max bias (log2 units; with room for rounding).
+        float limit = INFINITY;
+        if constexpr (kPrecise) {
+            if (p.key_norms != nullptr) {
+                const int32_t n_blocks = (p.n_total + kNormRows - 1) / kNormRows;
+                float kk = 0.f, qq = 0.f, bmax = -INFINITY;
+                for (int32_t b = node0 / kNormRows + lane; b <= (node0 + n_g - 1) / kNormRows; b += 32)
+                    kk = norm_max(kk, p.key_norms[(size_t)h * n_blocks + b]);
+                for (int i = lane; i < 256; i += 32) bmax = fmaxf(bmax, s_bias[i]);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    kk = norm_max(kk, __shfl_xor_sync(0xffffffffu, kk, off));
+                    bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
+                }
+                const int32_t row = node0 + min(q0 + t * kRowsPerTile + r, n_g - 1);
+                const uint4* src = (const uint4*)(p.q + ((size_t)row * p.n_heads + h) * D);
+#pragma unroll 2
+                for (int i = 0; i < D / 8; ++i) qq += square_sum(src[i]);
+                limit = sqrtf(qq * kk) * p.c1 * 1.001f + bmax + 1.0f;
+            }
+        }
+
         uint32_t sa[kCW], sb[kCW];              // score chunks, alternating
         uint4 wa[kCW / 16], wb[kCW / 16];       // their SPD bytes
         uint32_t tS = 0;                        // this thread's score columns of the current step
@@ -423,7 +467,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             uint32_t pk[kCols / 64][32];           // P of this thread's columns, bf16 pairs
             float tile_sum = 0.f;
             bool loaded = true;                    // chunk 0 is already on its way
-            bool exact = kPrecise || (j == 0);     // take the tile maximum first
+            bool exact = j == 0;                   // take the tile maximum first
+            // The precise variant's P overwrites the scores chunk by chunk, so a tile cannot be redone: it goes the speculative way
+            // only where the row's reference leaves no score out of reach (both column halves decide alike).
+            if constexpr (kPrecise) exact = exact || __any_sync(0xffffffffu, !(limit <= m + kReach));
 
             for (;;) {
                 if (exact) {
@@ -527,7 +574,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     unpack_f32x2(sum2, lo, hi);
                     tile_sum = lo + hi;
                 }
-                if (exact) break;
+                if (kPrecise || exact) break;
                 // reference too low for some row of this warp (pair of warps)?  Also catches inf / NaN.
                 const bool need = !(tile_sum <= kSumThreshold);
                 bool any_need;
@@ -746,6 +793,44 @@ int32_t chunk_rows(int32_t n, int32_t n_chunks)
 
 constexpr size_t kListMinSaved = 128;     // thread blocks
 
+// Largest |k|^2 of every kNormRows rows of a head: block (row block, head), D / 8 lanes per row.  Bound by its launch (8 192 rows,
+// 8 heads: 3 us for 8 MB).
+template <int D>
+__global__ void __launch_bounds__(256) key_norms_kernel(const uint4* __restrict__ k, float* __restrict__ norms, int32_t n_total, int32_t n_heads)
+{
+    constexpr int kLanes = D / 8, kRowsAtOnce = 256 / kLanes;
+    __shared__ float part[8];
+    grid_wait();
+    grid_release();
+    const int part_of_row = threadIdx.x % kLanes, first = blockIdx.x * kNormRows + threadIdx.x / kLanes;
+    uint4 v[kNormRows / kRowsAtOnce];
+#pragma unroll
+    for (int i = 0; i < kNormRows / kRowsAtOnce; ++i) {
+        const int row = first + i * kRowsAtOnce;
+        v[i] = row < n_total ? k[((size_t)row * n_heads + blockIdx.y) * kLanes + part_of_row] : make_uint4(0, 0, 0, 0);
+    }
+    float best = 0.f;
+#pragma unroll
+    for (int i = 0; i < kNormRows / kRowsAtOnce; ++i) {
+        float a = square_sum(v[i]);
+#pragma unroll
+        for (int off = kLanes / 2; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        best = norm_max(best, a);
+    }
+#pragma unroll
+    for (int off = 16; off >= kLanes; off >>= 1) best = norm_max(best, __shfl_xor_sync(0xffffffffu, best, off));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) best = norm_max(best, part[w]);
+        norms[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = best;
+    }
+}
+
+inline size_t norms_bytes(const gt_batch* b, int32_t n_heads) { return (size_t)((b->n_total + kNormRows - 1) / kNormRows) * (size_t)n_heads * sizeof(float); }
+// Precise forward: a tile saves half its softmax time (1 us) from the second one of a graph on; the norms cost about 3 us.
+constexpr int32_t kNormsMinNodes = 513;
+
 // Tensor maps of a packed batch, a thread per graph, behind its work list (unless `list` is null), a warp per graph.
 constexpr int kBatchThreads = 128;
 __global__ void __launch_bounds__(kBatchThreads) fwd_batch_kernel(const __grid_constant__ CUtensorMap model, uint8_t* maps, int4* list, int32_t entries,
@@ -802,8 +887,9 @@ gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint
 
 extern "C" size_t gt_biased_attn_fwd_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim)
 {
-    (void)n_heads; (void)head_dim;
-    return gt::kHeaderBytes + (gt::validate_batch(batch) == GT_OK ? gt::maps_bytes(batch->n_graphs) + gt::list_bytes(batch, gt::kRowsPerCta) : 0);
+    (void)head_dim;
+    if (gt::validate_batch(batch) != GT_OK || n_heads < 1) return gt::kHeaderBytes;
+    return gt::kHeaderBytes + gt::maps_bytes(batch->n_graphs) + gt::list_bytes(batch, gt::kRowsPerCta) + gt::norms_bytes(batch, n_heads);
 }
 
 extern "C" gt_status gt_biased_attn_fwd(const void* q, const void* k, const void* v,
@@ -835,7 +921,8 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     CUtensorMap tspd = tq;                       // placeholder when the cp.async loader is used
     FwdParams p{};
     p.spd_tma = batch->n_graphs == 1 ? 1 : 0;
-    if (batch->n_graphs > 1 && workspace_bytes >= gt_biased_attn_fwd_workspace(batch, n_heads, head_dim)) {
+    const bool room = workspace_bytes >= gt_biased_attn_fwd_workspace(batch, n_heads, head_dim);
+    if (batch->n_graphs > 1 && room) {
         p.maps = maps_at((uint8_t*)workspace + kHeaderBytes);
         // The list costs 1 us before the first block; that has to come back from the empty blocks that it saves.
         if (list_saves(batch, kRowsPerCta, n_heads, kListMinSaved))
@@ -856,6 +943,15 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     p.n_buckets = max_dist + 2;
     p.c1 = kLog2e / sqrtf((float)head_dim);
     cudaStream_t s = (cudaStream_t)stream;
+    if (out_f32 != nullptr && room && batch->max_seqlen >= kNormsMinNodes) {
+        float* norms = (float*)((uint8_t*)workspace + kHeaderBytes + maps_bytes(batch->n_graphs) + list_bytes(batch, kRowsPerCta));
+        const dim3 grid((unsigned)((batch->n_total + kNormRows - 1) / kNormRows), (unsigned)n_heads);
+        st = head_dim == 64 ? launch_overlapped(key_norms_kernel<64>, grid, 256, 0, s, (const uint4*)k, norms, batch->n_total, n_heads)
+                            : launch_overlapped(key_norms_kernel<32>, grid, 256, 0, s, (const uint4*)k, norms, batch->n_total, n_heads);
+        if (st != GT_OK) return st;
+        p.q = (const __nv_bfloat16*)q;
+        p.key_norms = norms;
+    }
     if (p.maps) {
         const int32_t warps = (batch->n_graphs + 31) / 32 + (p.list ? batch->n_graphs : 0);
         st = launch_overlapped(fwd_batch_kernel, dim3((unsigned)((warps * 32 + kBatchThreads - 1) / kBatchThreads)), kBatchThreads, 0, s, tspd,

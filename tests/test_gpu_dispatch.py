@@ -7,8 +7,9 @@ import torch
 from paper_2609_34420_b200 import binding as gt
 from paper_2609_34420_b200 import workloads as wl
 
+from gpu_util import DeviceCase, rel_l2, to_f64
 from test_gpu_attn_bwd import check_backward
-from test_gpu_attn_fwd import check_forward, pytestmark  # noqa: F401  (GPU tests)
+from test_gpu_attn_fwd import LSE_MAX_ABS, check_forward, oracle_forward, pytestmark  # noqa: F401  (GPU tests)
 
 
 def sizes(n_graphs, largest):
@@ -46,3 +47,22 @@ def test_bias_gradient_reaches_every_bucket_of_a_path():
     w = wl.small_workload([n], 2, 64, D, seed=1)
     w.batch = wl.pack_graphs([wl.csr_from_edges(n, i, i + 1, symmetric=True)])
     check_backward(w)
+
+
+# 512 nodes: every tile takes its maximum first; beyond that only the tiles whose scores may be out of reach of the row's
+# reference.  Inputs of 3 standard deviations and wide bias tables put some rows on either side.
+@pytest.mark.parametrize("sizes_,d,D,std,spread", [([512], 64, 5, 1.0, 1.0), ([513], 32, 5, 1.0, 1.0), ([1100], 64, 60, 2.0, 12.0),
+                                                   ([1100], 64, 20, 3.0, 1.0), ([900], 32, 254, 3.0, 30.0), ([700, 3, 1300, 256], 64, 9, 3.0, 4.0)])
+def test_precise_forward_with_tiles_in_and_out_of_reach(sizes_, d, D, std, spread):
+    w = wl.small_workload(sizes_, 2, d, D, seed=sum(sizes_) + D, avg_degree=1.3, qkv_std=std)
+    w.tensors().bias[:] *= spread
+    case = DeviceCase(w)
+    out, lse, out32 = case.forward_ex()
+    ro, rl = oracle_forward(case)
+    # two bf16 terms of P: 2^-17 of each entry; scores of up to 100 in fp32: 100 * 2^-22 of each entry
+    assert rel_l2(to_f64(out32), ro) <= 1e-4 and np.abs(to_f64(lse) - rl).max() <= LSE_MAX_ABS
+    ws = torch.zeros(256, dtype=torch.uint8, device=case.q.device)       # no room for the norms: maximum first everywhere
+    out32b = torch.full_like(out32, float("nan"))
+    gt.gt_biased_attn_fwd_ex(case.q, case.k, case.v, case.spd, case.bias, case.batch, w.max_dist, out, lse, out32b, ws)
+    gt.gt_check(ws)
+    assert rel_l2(to_f64(out32b), ro) <= 1e-4
