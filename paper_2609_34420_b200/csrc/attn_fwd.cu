@@ -51,8 +51,6 @@ constexpr int kKStages = 2;
 constexpr int kVStages = 2;
 constexpr int kSpdStages = 3;
 constexpr int kHalves = 2;                    // softmax threads per query row (column halves)
-constexpr int kSoftmaxWarps = 8 * kHalves;
-constexpr int kFwdThreads = 128 + 32 * kSoftmaxWarps;
 constexpr int kCols = kKvTile / kHalves;      // score columns per softmax thread
 constexpr int kCW = kHalves == 1 ? 32 : 16;   // columns per TMEM load
 constexpr int kChunks = kCols / kCW;
@@ -162,13 +160,17 @@ __device__ __forceinline__ float norm_max(float a, float b) { return __uint_as_f
 // bounds a row's scores, and while that is within 2^60 of the row's reference, P, l and O stay far inside the range
 // of fp32 and bf16, whose relative precision does not depend on the reference.  Rows (warps of 32) beyond it take the
 // maximum first, which costs a second pass over the scores.  8 192 nodes, 8 heads of 64: 386 -> 251 us, norms included.
-template <int D, bool kPartial, bool kShflBias, bool kPrecise = false>
-__global__ void __launch_bounds__(kFwdThreads, 1)
+// kTiles = 1: thread blocks of one 128-row query tile and eight softmax warps, for grids that would leave half
+// of the SMs idle or more (rows_per_block).  Two score buffers then: with three, a warp could be two key tiles ahead of another.
+template <int D, bool kPartial, bool kShflBias, bool kPrecise = false, int kTiles = kQTiles>
+__global__ void __launch_bounds__(128 + 256 * kTiles, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_spd,
                 const FwdParams p)
 {
     using L = FwdSmem<D>;
+    constexpr int kRows = kRowsPerTile * kTiles, kThreads = 128 + 256 * kTiles, kBuffers = kTiles + 1;
+    static_assert(kHalves == 2);
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment by pointer arithmetic on the __shared__ array itself, so that every derived
     // pointer keeps its shared address space (integer round trips would turn the accesses generic)
@@ -195,7 +197,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         node0 = p.cu_seqlens[g];
         n_g = p.cu_seqlens[g + 1] - node0;
     }
-    const int32_t q0 = q_block * kRowsPerCta;
+    const int32_t q0 = q_block * kRows;
     if (q0 >= n_g) return;
     const int64_t ld = (int64_t)((n_g + 15) & ~15);
     const uint8_t* spd_g = p.spd + (p.spd_offsets ? p.spd_offsets[g] : 0);
@@ -205,7 +207,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     if (kPartial && n_kv == 0) {            // empty chunk: weight zero in the merge
         grid_wait();
-        for (int i = tid; i < kRowsPerCta; i += kFwdThreads) {
+        for (int i = tid; i < kRows; i += kThreads) {
             int q = q0 + i;
             if (q < n_g) {
                 p.part_lse[((size_t)chunk * p.n_heads + h) * p.n_total + q] = -INFINITY;
@@ -227,7 +229,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         mbar_init(bar(kBarQFull), 1);
         for (int s = 0; s < kKStages; ++s) { mbar_init(bar(kBarKFull + s), 1); mbar_init(bar(kBarKEmpty + s), 1); }
         for (int s = 0; s < kVStages; ++s) { mbar_init(bar(kBarVFull + s), 1); mbar_init(bar(kBarVEmpty + s), 1); }
-        for (int s = 0; s < kSpdStages; ++s) { mbar_init(bar(kBarSpdFull + s), p.spd_tma ? 1 : 32); mbar_init(bar(kBarSpdEmpty + s), kSoftmaxWarps); }
+        for (int s = 0; s < kSpdStages; ++s) { mbar_init(bar(kBarSpdFull + s), p.spd_tma ? 1 : 32); mbar_init(bar(kBarSpdEmpty + s), 8 * kTiles); }
         for (int b = 0; b < 3; ++b) { mbar_init(bar(kBarSFull + b), 1); mbar_init(bar(kBarBufFree + b), 1); }
         for (int t = 0; t < 4; ++t) mbar_init(bar(kBarPFull + t), 4 * kHalves);     // one arrival per warp
         for (int t = 0; t < 4; ++t) mbar_init(bar(kBarODone + t), 1);
@@ -240,7 +242,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (warp == 1) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
     grid_wait();
     grid_release();
-    for (int i = tid; i < 256; i += kFwdThreads)
+    for (int i = tid; i < 256; i += kThreads)
         s_bias[i] = p.bias[(size_t)h * p.n_buckets + min(i, p.n_buckets - 1)] * kLog2e;
     tc_fence_before();
     __syncthreads();
@@ -249,13 +251,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     if (warp < 4) {
         // =========================== producer / MMA / SPD warps ===========================
-        if constexpr (kHalves == 2) setmaxnreg_dec_32(); else setmaxnreg_dec_56();
+        if constexpr (kTiles == 2) setmaxnreg_dec_32();
         if (warp == 0) {
             const void* spd_map = !kPartial && p.maps ? (const void*)(p.maps + (size_t)g * kMapBytes) : &tmap_spd;
             if (lane == 0) {
                 if (!kPartial && p.maps) acquire_tensor_map(spd_map);
-                mbar_arrive_expect_tx(bar(kBarQFull), kQTiles * L::kTileBytes);
-                for (int t = 0; t < kQTiles; ++t)
+                mbar_arrive_expect_tx(bar(kBarQFull), kTiles * L::kTileBytes);
+                for (int t = 0; t < kTiles; ++t)
                     tma_load_3d(smem_u32(smem + L::kQ + t * L::kTileBytes), &tmap_q, bar(kBarQFull), 0, h,
                                 node0 + q0 + t * kRowsPerTile);
             }
@@ -271,7 +273,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (p.spd_tma) {
                     mbar_wait(bar(kBarSpdEmpty + ss), ((j / kSpdStages) & 1) ^ 1, abort_flag, p.status, 11);
                     if (lane == 0) {
-                        mbar_arrive_expect_tx(bar(kBarSpdFull + ss), L::kSpdTileBytes);
+                        mbar_arrive_expect_tx(bar(kBarSpdFull + ss), kRows * kKvTile);
                         tma_load_2d(smem_u32(smem + L::kSpd + ss * L::kSpdTileBytes), spd_map, bar(kBarSpdFull + ss), kv0, q0);
                     }
                 }
@@ -294,9 +296,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 const int ks = j % kKStages;
                 mbar_wait(bar(kBarKFull + ks), (j / kKStages) & 1, abort_flag, p.status, 22);
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    const int step = 2 * j + t, b = step % 3;
-                    if (step >= 3) mbar_wait(bar(kBarBufFree + b), (step / 3 - 1) & 1, abort_flag, p.status, 23);
+                for (int t = 0; t < kTiles; ++t) {
+                    const int step = kTiles * j + t, b = step % kBuffers;
+                    if (step >= kBuffers) mbar_wait(bar(kBarBufFree + b), (step / kBuffers - 1) & 1, abort_flag, p.status, 23);
                     tc_fence_after();
                     if (elect_one()) {
                         const uint64_t da = advance_desc(desc_q0, t * L::kTileBytes);
@@ -305,7 +307,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         for (int k = 0; k < D / 16; ++k)
                             mma_ss(tm + b * 128, advance_desc(da, k * 32), advance_desc(db, k * 32), idesc_s, k > 0);
                         mma_commit(bar(kBarSFull + b));
-                        if (t == 1) mma_commit(bar(kBarKEmpty + ks));
+                        if (t == kTiles - 1) mma_commit(bar(kBarKEmpty + ks));
                     }
                     __syncwarp();
                 }
@@ -321,8 +323,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 const uint64_t dv = advance_desc(desc_v0, vs * L::kTileBytes);
                 const uint32_t acc0 = j > 0 ? 1u : 0u;
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    const int b = (2 * j + t) % 3;
+                for (int t = 0; t < kTiles; ++t) {
+                    const int b = (kTiles * j + t) % kBuffers;
                     mbar_wait(bar(kBarPFull + 2 * t + (j & 1)), (j >> 1) & 1, abort_flag, p.status, 24);
                     tc_fence_after();
                     if (elect_one()) {
@@ -341,7 +343,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         }
                         mma_commit(bar(kBarODone + 2 * t + (j & 1)));
                         mma_commit(bar(kBarBufFree + b));
-                        if (t == 1) mma_commit(bar(kBarVEmpty + vs));
+                        if (t == kTiles - 1) mma_commit(bar(kBarVEmpty + vs));
                     }
                     __syncwarp();
                 }
@@ -355,21 +357,21 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const uint32_t dst_even = (uint32_t)(lr * 128 + ((cc ^ lr) << 4)), dst_odd = (uint32_t)(lr * 128 + ((cc ^ (4 + lr)) << 4));
             const uint8_t* lane_src = spd_g + (int64_t)(q0 + lr) * ld + cc * 16;
             const uint32_t step = 4u * (uint32_t)ld;      // every copy's address is base + (constant round) * step: no dependent chain
-            const int32_t rows_valid = min(kRowsPerCta, n_g - q0);
+            const int32_t rows_valid = min(kRows, n_g - q0);
             for (int j = 0; j < n_kv; ++j) {
                 const int s2 = j % kSpdStages;
                 mbar_wait(bar(kBarSpdEmpty + s2), ((j / kSpdStages) & 1) ^ 1, abort_flag, p.status, 30);
                 const int32_t kv0 = kv_begin + j * kKvTile;
                 const uint32_t dst0 = smem_u32(smem + L::kSpd + s2 * L::kSpdTileBytes);
                 const uint8_t* src = lane_src + kv0;
-                if (rows_valid == kRowsPerCta && (int64_t)kv0 + kKvTile <= ld) {
+                if (rows_valid == kRows && (int64_t)kv0 + kKvTile <= ld) {
 #pragma unroll 16
-                    for (int i = 0; i < kRowsPerCta / 4; ++i)
+                    for (int i = 0; i < kRows / 4; ++i)
                         cp_async_16(dst0 + i * 512 + ((i & 1) ? dst_odd : dst_even), src + (uint64_t)step * (uint32_t)i, 16u);
                 } else {
                     const int32_t lim = ((int64_t)kv0 + cc * 16 < ld) ? rows_valid - lr : 0;     // rounds 4 i < lim are in range
 #pragma unroll 8
-                    for (int i = 0; i < kRowsPerCta / 4; ++i) {
+                    for (int i = 0; i < kRows / 4; ++i) {
                         const bool valid = 4 * i < lim;
                         cp_async_16(dst0 + i * 512 + ((i & 1) ? dst_odd : dst_even), valid ? src + (uint64_t)step * (uint32_t)i : spd_g, valid ? 16u : 0u);
                     }
@@ -379,7 +381,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
     } else {
         // =================================== softmax warps ===================================
-        if constexpr (kHalves == 2) setmaxnreg_inc_112(); else setmaxnreg_inc_224();
+        if constexpr (kTiles == 2) setmaxnreg_inc_112();
         const int sw = warp - 4;
         const int t = sw / (4 * kHalves);
         const int hf = (sw >> 2) & (kHalves - 1);
@@ -450,9 +452,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         };
         // first chunk of key tile j: fetched at the end of tile j-1, behind the P store
         auto begin_tile = [&](int j) {
-            const int step = 2 * j + t, b = step % 3;
+            const int step = kTiles * j + t, b = step % kBuffers;
             tS = tmem + b * 128 + hf * kCols + lane_off;
-            mbar_wait(bar(kBarSFull + b), (step / 3) & 1, abort_flag, p.status, 40);
+            mbar_wait(bar(kBarSFull + b), (step / kBuffers) & 1, abort_flag, p.status, 40);
             tc_fence_after();
             mbar_wait(bar(kBarSpdFull + (j % kSpdStages)), (j / kSpdStages) & 1, abort_flag, p.status, 41);
             srow = smem + L::kSpd + (j % kSpdStages) * L::kSpdTileBytes + (t * 128 + r) * 128;
@@ -852,22 +854,35 @@ __global__ void __launch_bounds__(kBatchThreads) fwd_batch_kernel(const __grid_c
     if (n > 0) make_spd_map(maps + (size_t)g * kMapBytes, model, spd + spd_offsets[g], n);
 }
 
+// Rows per thread block.  One tile where the grid of two would leave at least half of the SMs idle: the softmax of a tile is bound
+// by its SM's issue slots and exponentials, so two SMs with a tile each are faster than one with both: 1 000 nodes, 8 heads of 64:
+// 19.5 -> 13.8 us; 2 048 nodes 31.8 -> 23.0; 4 096 nodes, 4 heads: 56.4 -> 40.3; up to 256 nodes no difference.
+inline int32_t rows_per_block(const gt_batch* b, int32_t n_heads)
+{
+    return (int64_t)((b->max_seqlen + kRowsPerTile - 1) / kRowsPerTile) * b->n_graphs * n_heads <= sm_count() ? kRowsPerTile : kRowsPerCta;
+}
+
 template <int D, bool kPartial>
 gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tspd,
                      const FwdParams& p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0)
 {
-    auto kern = p.n_buckets <= 32 ? attn_fwd_kernel<D, kPartial, true> : attn_fwd_kernel<D, kPartial, false>;
+    const bool shfl = p.n_buckets <= 32;
+    const int32_t rows = kPartial ? kRowsPerCta : rows_per_block(batch, p.n_heads);
+    auto kern = shfl ? attn_fwd_kernel<D, kPartial, true> : attn_fwd_kernel<D, kPartial, false>;
     if constexpr (!kPartial) {
-        if (p.out_f32 != nullptr)
-            kern = p.n_buckets <= 32 ? attn_fwd_kernel<D, false, true, true> : attn_fwd_kernel<D, false, false, true>;
+        if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true> : attn_fwd_kernel<D, false, false, true>;
+        if (rows == kRowsPerTile) {
+            kern = shfl ? attn_fwd_kernel<D, false, true, false, 1> : attn_fwd_kernel<D, false, false, false, 1>;
+            if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1> : attn_fwd_kernel<D, false, false, true, 1>;
+        }
     }
-    static std::atomic<uint64_t> granted[4] = {};
-    const gt_status st = grant_smem(kern, granted[(p.n_buckets <= 32 ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0)], FwdSmem<D>::kDynamic);
+    static std::atomic<uint64_t> granted[8] = {};
+    const gt_status st = grant_smem(kern, granted[(shfl ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0) + (rows == kRowsPerTile ? 4 : 0)], FwdSmem<D>::kDynamic);
     if (st != GT_OK) return st;
-    const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + kRowsPerCta - 1) / kRowsPerCta;
+    const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + rows - 1) / rows;
     const dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kRowsPerCta) * p.n_heads))
                              : dim3((unsigned)p.n_heads, (unsigned)row_blocks, (unsigned)grid_z);
-    return launch_overlapped(kern, grid, kFwdThreads, FwdSmem<D>::kDynamic, s, tq, tk, tv, tspd, p);
+    return launch_overlapped(kern, grid, 128 + 2 * rows, FwdSmem<D>::kDynamic, s, tq, tk, tv, tspd, p);
 }
 
 gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint8_t* spd, const int64_t* spd_offsets,
@@ -920,16 +935,17 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     if ((st = encode_thd_map(&tv, v, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
     CUtensorMap tspd = tq;                       // placeholder when the cp.async loader is used
     FwdParams p{};
+    const int32_t rows = rows_per_block(batch, n_heads);
     p.spd_tma = batch->n_graphs == 1 ? 1 : 0;
     const bool room = workspace_bytes >= gt_biased_attn_fwd_workspace(batch, n_heads, head_dim);
     if (batch->n_graphs > 1 && room) {
         p.maps = maps_at((uint8_t*)workspace + kHeaderBytes);
         // The list costs 1 us before the first block; that has to come back from the empty blocks that it saves.
-        if (list_saves(batch, kRowsPerCta, n_heads, kListMinSaved))
+        if (rows == kRowsPerCta && list_saves(batch, kRowsPerCta, n_heads, kListMinSaved))
             p.list = (const int4*)((uint8_t*)workspace + kHeaderBytes + maps_bytes(batch->n_graphs));
         p.spd_tma = 1;
     }
-    if (p.spd_tma && (st = encode_spd_map(&tspd, spd, batch->max_seqlen, 256)) != GT_OK) return st;
+    if (p.spd_tma && (st = encode_spd_map(&tspd, spd, batch->max_seqlen, rows)) != GT_OK) return st;
     p.spd = spd;
     p.spd_offsets = batch->n_graphs > 1 ? spd_offsets : nullptr;
     p.cu_seqlens = batch->n_graphs > 1 ? batch->cu_seqlens : nullptr;

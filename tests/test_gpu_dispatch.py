@@ -66,3 +66,11 @@ def test_precise_forward_with_tiles_in_and_out_of_reach(sizes_, d, D, std, sprea
     gt.gt_biased_attn_fwd_ex(case.q, case.k, case.v, case.spd, case.bias, case.batch, w.max_dist, out, lse, out32b, ws)
     gt.gt_check(ws)
     assert rel_l2(to_f64(out32b), ro) <= 1e-4
+
+
+# one 128-row query tile per thread block up to 148 of them, two beyond: ragged graphs on either side of the line
+@pytest.mark.parametrize("n", [128, 257, 300, 513])
+@pytest.mark.parametrize("beyond", [0, 1])
+def test_one_and_two_query_tiles_per_block(n, beyond):
+    tiles = -(-n // 128)
+    check_forward(wl.small_workload([n], 148 // tiles + beyond, 32 if n % 2 else 64, 5, seed=n + beyond, avg_degree=2.0))
