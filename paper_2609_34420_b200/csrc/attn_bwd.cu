@@ -71,6 +71,7 @@ struct BwdParams {
     int32_t n_buckets;
     int32_t bin_log;         // shared bins (more than kMaxPrivateBinBuckets buckets): log2 of the columns per bucket
     int32_t early_release;   // let the next kernel start its set-up while this one runs
+    int32_t split;           // thread blocks (a cluster) that share the queries of a key tile; 1: no cluster
     const int4* list;        // packed batch: work list; block index = entry * heads + head (nullptr: grid of heads x tiles x graphs)
     const uint8_t* maps;     // packed batch: tensor maps of the graphs' SPD^T blocks (workspace); nullptr: single graph
     int32_t kv_row0;         // key rows [kv_row0, kv_row_end) of a graph are this launch's (chunked / step entry points)
@@ -140,7 +141,23 @@ struct BwdSmem {
 __device__ __forceinline__ void setmaxnreg_inc_96() { asm volatile("setmaxnreg.inc.sync.aligned.u32 96;"); }
 __device__ __forceinline__ void setmaxnreg_dec_48() { asm volatile("setmaxnreg.dec.sync.aligned.u32 48;"); }
 
-template <int D, bool kPrivateBins, bool kShflBias>
+// All threads of the cluster's blocks that have not returned.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// 16 bytes at a shared address of the cluster's block `rank`
+__device__ __forceinline__ float4 ld_cluster_float4(uint32_t addr, uint32_t rank)
+{
+    float4 v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+
+// kSplit: blocks of a cluster share the queries of a key tile (BwdParams::split); a form of its own, because the code for it costs
+// the others 1 % even where it is not reached.
+template <int D, bool kPrivateBins, bool kShflBias, bool kSplit>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_do,
@@ -152,7 +169,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     extern __shared__ uint8_t smem_raw[];
     // pointers are derived from the __shared__ array itself, so that they keep the shared address space
     uint8_t* smem = smem_raw;
-    if (smem_u32(smem_raw) != kSmemWindowBase) {      // the address arithmetic of the bins assumes this window base
+    // The address arithmetic of the bins assumes this window base (in a cluster, the block's rank stands in bits 24 and up, which it leaves alone).
+    if ((smem_u32(smem_raw) & 0xffffffu) != kSmemWindowBase) {
         if (threadIdx.x == 0 && atomicCAS(p.status, 0u, (uint32_t)GT_ERR_CUDA) == 0u) p.status[1] = 199;
         return;
     }
@@ -161,6 +179,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int warp = tid >> 5;
     const int lane = tid & 31;
     int h = blockIdx.x, g = blockIdx.z, kv_tile = blockIdx.y;
+    const int rank = kSplit ? (int)blockIdx.x % p.split : 0;
+    if constexpr (kSplit) h = (int)blockIdx.x / p.split;
     int32_t node0 = 0, n_g = p.n_total;
     if (p.cu_seqlens) grid_wait();          // a single graph's blocks set up their barriers and tensor memory before they wait
     if (p.list) {
@@ -178,9 +198,17 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int32_t kv0 = p.kv_row0 + kv_tile * kTile;
     const int32_t kv_lim = min(n_g, p.kv_row_end);
     if (kv0 >= kv_lim) return;
-    const int32_t q_lo = p.q_row0, q_hi = min(n_g, p.q_row_end);
+    int32_t q_lo = p.q_row0, q_hi = min(n_g, p.q_row_end);
     if (q_hi <= q_lo) return;
-    const int32_t n_q = (q_hi - q_lo + kTile - 1) / kTile;
+    int32_t n_q = (q_hi - q_lo + kTile - 1) / kTile, sharers = 1;      // sharers: blocks of the cluster that have queries
+    if constexpr (kSplit) {
+        const int32_t per = (n_q + p.split - 1) / p.split;
+        sharers = (n_q + per - 1) / per;
+        if (rank >= sharers) return;                                  // (the cluster's barriers wait for blocks that are still there)
+        q_lo += rank * per * kTile;
+        q_hi = min(q_hi, q_lo + per * kTile);
+        n_q = (q_hi - q_lo + kTile - 1) / kTile;
+    }
 
     uint64_t* bars = (uint64_t*)(smem + L::kBars);
     uint32_t* misc = (uint32_t*)(smem + L::kMisc);
@@ -527,7 +555,11 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if constexpr (kOC == 32) tmem_ld32(tacc, o); else tmem_ld16(tacc, o);
             tmem_wait_ld();
             float* acc_base = half == 0 ? p.dv_acc : p.dk_acc;
-            if (kv_valid && acc_base != nullptr) {
+            if (kSplit && sharers > 1) {              // to the block's own shared memory (the Q / dO stages: every MMA is done), added up below
+                uint4* part = (uint4*)(smem + L::kQ) + (half * (D / 4) + ch * (kOC / 4)) * 128 + r;
+#pragma unroll
+                for (int k = 0; k < kOC / 4; ++k) part[k * 128] = make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+            } else if (kv_valid && acc_base != nullptr) {
                 // step entry point: this launch's share is added to the caller's unscaled fp32 sums (a key row belongs
                 // to one CTA of the launch, launches are ordered by the stream: plain read-modify-write)
                 float4* dst = (float4*)(acc_base + ((size_t)(node0 + kv0 + r) * p.n_heads + h) * D + ch * kOC);
@@ -610,6 +642,27 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     if (*abort_flag) __nanosleep(200000);
     if (warp == 2) tmem_dealloc(tmem, 512);
+    if (kSplit && sharers > 1) {
+        // dV and dK of the key tile: every block adds up its share of the rows over all blocks' sums, through shared memory.
+        cluster_sync();
+        constexpr int kPieces = 2 * (D / 4) * 128;        // of four channels of a row: dV, then dK
+        const int per = (kPieces + sharers - 1) / sharers;
+        for (int i = rank * per + tid; i < min(kPieces, (rank + 1) * per); i += kBwdThreads) {
+            const int row = i & 127, c4 = (i >> 7) % (D / 4), half = i / (kPieces / 2);
+            const uint32_t at = smem_u32(smem + L::kQ) + (uint32_t)i * 16u;
+            float4 a = ld_cluster_float4(at, 0);
+            for (int k = 1; k < sharers; ++k) {
+                const float4 b = ld_cluster_float4(at, (uint32_t)k);
+                a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+            }
+            if (kv0 + row < kv_lim) {
+                const float mul = half == 0 ? 1.0f : p.scale;
+                __nv_bfloat16* dst = (half == 0 ? p.dv : p.dk) + ((size_t)(node0 + kv0 + row) * p.n_heads + h) * D + c4 * 4;
+                *(uint2*)dst = make_uint2(pack_bf16x2(a.x * mul, a.y * mul), pack_bf16x2(a.z * mul, a.w * mul));
+            }
+        }
+        cluster_sync();                                   // no block leaves while another reads its sums
+    }
 }
 
 // spd_t[j][i] = min(spd[i][j], last_bucket) for one 128 x 128 byte tile of a graph block (same offsets and pitch as the
@@ -843,6 +896,36 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
     return w;
 }
 
+// Thread blocks that share the queries of a key tile: as many as let the whole grid run at once, of a cluster size of which the
+// device holds enough at a time (a cluster's blocks lie in one group of SMs).  A query tile takes 1.3 us (with the shared bins of many
+// buckets four times that), the cluster and its sums 2 us: from four query tiles on, or two.
+// Whole call, 8 heads of 64 if not said otherwise: 1 000 nodes 29.8 -> 24.9 us (4 heads: 29.8 -> 21.5), 1 200 nodes, 4 heads 33.4 ->
+// 24.2, 2 048 nodes, 4 heads 47.5 -> 34.7, 300 nodes, 4 heads of 32, 256 buckets 47.0 -> 32.3; 512 nodes no difference.
+constexpr int kMaxSplit = 4;
+constexpr int32_t kMinSplitTiles = 4;
+template <typename Kernel>
+int32_t query_split(Kernel kern, std::atomic<int32_t> (&max_clusters)[kMaxSplit + 1], int64_t blocks, int32_t n_q, size_t smem)
+{
+    for (int32_t split = kMaxSplit; split > 1; --split) {
+        if (blocks * split > sm_count() || n_q < split) continue;
+        int32_t fit = max_clusters[split].load(std::memory_order_relaxed);
+        if (fit == 0) {                                    // (asked once; the largest shared memory, whose blocks have an SM each anyway)
+            cudaLaunchAttribute attr{};
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = (unsigned)split; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)split); cfg.blockDim = dim3(kBwdThreads); cfg.dynamicSmemBytes = smem;
+            cfg.attrs = &attr; cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+            fit = n > 0 ? n : -1;
+            max_clusters[split].store(fit, std::memory_order_relaxed);
+        }
+        if (blocks <= fit) return split;
+    }
+    return 1;
+}
+
 template <int D>
 gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
                      const CUtensorMap& text, const CUtensorMap& tspd, BwdParams p,
@@ -850,7 +933,7 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
 {
     const int32_t kv_end = p.kv_row_end < batch->max_seqlen ? p.kv_row_end : batch->max_seqlen;
     if (kv_end <= p.kv_row0 || p.q_row_end <= p.q_row0) return GT_OK;      // empty key chunk / no queries
-    const dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kTile) * p.n_heads))
+    dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kTile) * p.n_heads))
                              : dim3((unsigned)p.n_heads, (unsigned)((kv_end - p.kv_row0 + kTile - 1) / kTile), (unsigned)batch->n_graphs);
     CUtensorMap tdq;
     gt_status st_map = encode_dq_map(&tdq, p.dq_acc, p.n_total, p.n_heads, D);
@@ -862,14 +945,30 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     const size_t smem = BwdSmem<D>::dynamic_bytes(p.n_buckets << p.bin_log);
     // With several waves of blocks the early start of the next kernel slows the dispatch of this one's (65 536 nodes: 36.5 ->
     // 39.9 ms); with one it hides the next one's start.
-    p.early_release = (int64_t)grid.x * grid.y * grid.z <= sm_count();
+    p.early_release = (int64_t)grid.x * grid.y * grid.z <= sm_count();      // (a split grid fits, too)
     static_assert(kMaxPrivateBinBuckets <= 32, "private bins go with the shuffle lookup");
-    auto kern = priv ? attn_bwd_kernel<D, true, true>
-                     : (p.n_buckets <= 32 ? attn_bwd_kernel<D, false, true> : attn_bwd_kernel<D, false, false>);
-    static std::atomic<uint64_t> granted[3] = {};
-    const gt_status st = grant_smem(kern, granted[priv ? 0 : (p.n_buckets <= 32 ? 1 : 2)], kMaxSmemBytes);
+    const int form = priv ? 0 : (p.n_buckets <= 32 ? 1 : 2);
+    void (*const forms[3][2])(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, BwdParams) = {
+        {attn_bwd_kernel<D, true, true, false>, attn_bwd_kernel<D, true, true, true>},
+        {attn_bwd_kernel<D, false, true, false>, attn_bwd_kernel<D, false, true, true>},
+        {attn_bwd_kernel<D, false, false, false>, attn_bwd_kernel<D, false, false, true>}};
+    static std::atomic<uint64_t> granted[3][2] = {};
+    static std::atomic<int32_t> max_clusters[3][kMaxSplit + 1] = {};
+    p.split = 1;
+    if (p.dk_acc == nullptr && p.list == nullptr) {
+        const int32_t q_end = p.q_row_end < batch->max_seqlen ? p.q_row_end : batch->max_seqlen;
+        const int32_t n_q = (q_end - p.q_row0 + kTile - 1) / kTile;
+        if (n_q >= (priv ? kMinSplitTiles : kMinSplitTiles / 2)) {
+            const gt_status st = grant_smem(forms[form][1], granted[form][1], kMaxSmemBytes);
+            if (st != GT_OK) return st;
+            p.split = query_split(forms[form][1], max_clusters[form], (int64_t)grid.x * grid.y * grid.z, n_q, smem);
+            grid.x *= (unsigned)p.split;
+        }
+    }
+    auto kern = forms[form][p.split > 1];
+    const gt_status st = grant_smem(kern, granted[form][p.split > 1], kMaxSmemBytes);
     if (st != GT_OK) return st;
-    return launch_overlapped(kern, grid, kBwdThreads, smem, s, tq, tk, tv, tdo, text, tspd, tdq, p);
+    return launch_overlapped_cluster(kern, grid, kBwdThreads, smem, p.split, s, tq, tk, tv, tdo, text, tspd, tdq, p);
 }
 
 }  // namespace

@@ -7,6 +7,7 @@
 #include <stdlib.h>
 
 #include <atomic>
+#include <utility>
 
 #include "../../include/gt_attn.h"
 
@@ -50,21 +51,30 @@ inline gt_status validate_batch(const gt_batch* b)
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-template <class... Params, class... Args>
-inline gt_status launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem_bytes, cudaStream_t stream, Args&&... args)
+template <typename... Params, typename... Args>
+inline gt_status launch_overlapped_cluster(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem_bytes, int cluster, cudaStream_t stream,
+                                           Args&&... args)
 {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     GT_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...));
     return GT_OK;
+}
+template <typename... Params, typename... Args>
+inline gt_status launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem_bytes, cudaStream_t stream, Args&&... args)
+{
+    return launch_overlapped_cluster(kernel, grid, threads, smem_bytes, 1, stream, std::forward<Args>(args)...);
 }
 
 // Lets a kernel use up to `bytes` of dynamic shared memory, once per device: `granted` is that kernel's own (a bit per device),

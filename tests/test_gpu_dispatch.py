@@ -74,3 +74,21 @@ def test_precise_forward_with_tiles_in_and_out_of_reach(sizes_, d, D, std, sprea
 def test_one_and_two_query_tiles_per_block(n, beyond):
     tiles = -(-n // 128)
     check_forward(wl.small_workload([n], 148 // tiles + beyond, 32 if n % 2 else 64, 5, seed=n + beyond, avg_degree=2.0))
+
+
+# a key tile's queries shared by a cluster of 2, 3 or 4 blocks (private and shared bins), a share that is empty (5 tiles by 4),
+# graphs of a batch with fewer tiles than blocks, and the first size without
+@pytest.mark.parametrize("sizes_,heads,d,D", [([385], 37, 32, 6), ([513], 7, 64, 6), ([640], 9, 64, 6), ([641], 8, 32, 24), ([900], 9, 64, 6),
+                                              ([129], 2, 64, 60), ([300], 4, 32, 254), ([500, 500, 500], 2, 64, 9), ([512, 1], 4, 32, 9)])
+def test_backward_with_shared_key_tiles(sizes_, heads, d, D):
+    check_backward(wl.small_workload(sizes_, heads, d, D, seed=sum(sizes_) + D, avg_degree=2.0))
+
+
+@pytest.mark.parametrize("chunks", [1, 3])
+def test_chunked_backward_with_shared_key_tiles(chunks):
+    w = wl.small_workload([700], 4, 64, 6, seed=chunks, avg_degree=2.0, directed=True)
+    case, _ = check_backward(w)
+    out, lse = case.forward()
+    whole = case.backward(out, lse)
+    for got, want in zip(case.backward_chunked(out, lse, chunks)[:4], whole):       # sums in another order, results rounded to bf16
+        assert rel_l2(to_f64(got), to_f64(want)) <= 5e-3
