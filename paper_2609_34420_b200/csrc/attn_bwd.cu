@@ -141,20 +141,6 @@ struct BwdSmem {
 __device__ __forceinline__ void setmaxnreg_inc_96() { asm volatile("setmaxnreg.inc.sync.aligned.u32 96;"); }
 __device__ __forceinline__ void setmaxnreg_dec_48() { asm volatile("setmaxnreg.dec.sync.aligned.u32 48;"); }
 
-// All threads of the cluster's blocks that have not returned.
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-// 16 bytes at a shared address of the cluster's block `rank`
-__device__ __forceinline__ float4 ld_cluster_float4(uint32_t addr, uint32_t rank)
-{
-    float4 v;
-    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr), "r"(rank) : "memory");
-    return v;
-}
-
 // kSplit: blocks of a cluster share the queries of a key tile (BwdParams::split); a form of its own, because the code for it costs
 // the others 1 % even where it is not reached.
 template <int D, bool kPrivateBins, bool kShflBias, bool kSplit>
@@ -896,35 +882,11 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
     return w;
 }
 
-// Thread blocks that share the queries of a key tile: as many as let the whole grid run at once, of a cluster size of which the
-// device holds enough at a time (a cluster's blocks lie in one group of SMs).  A query tile takes 1.3 us (with the shared bins of many
-// buckets four times that), the cluster and its sums 2 us: from four query tiles on, or two.
+// Thread blocks that share the queries of a key tile (cluster_split): a query tile takes 1.3 us (with the shared bins of many
+// buckets four times that), the cluster and its sums 2 us, so from four query tiles on, or two.
 // Whole call, 8 heads of 64 if not said otherwise: 1 000 nodes 29.8 -> 24.9 us (4 heads: 29.8 -> 21.5), 1 200 nodes, 4 heads 33.4 ->
 // 24.2, 2 048 nodes, 4 heads 47.5 -> 34.7, 300 nodes, 4 heads of 32, 256 buckets 47.0 -> 32.3; 512 nodes no difference.
-constexpr int kMaxSplit = 4;
 constexpr int32_t kMinSplitTiles = 4;
-template <typename Kernel>
-int32_t query_split(Kernel kern, std::atomic<int32_t> (&max_clusters)[kMaxSplit + 1], int64_t blocks, int32_t n_q, size_t smem)
-{
-    for (int32_t split = kMaxSplit; split > 1; --split) {
-        if (blocks * split > sm_count() || n_q < split) continue;
-        int32_t fit = max_clusters[split].load(std::memory_order_relaxed);
-        if (fit == 0) {                                    // (asked once; the largest shared memory, whose blocks have an SM each anyway)
-            cudaLaunchAttribute attr{};
-            attr.id = cudaLaunchAttributeClusterDimension;
-            attr.val.clusterDim.x = (unsigned)split; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)split); cfg.blockDim = dim3(kBwdThreads); cfg.dynamicSmemBytes = smem;
-            cfg.attrs = &attr; cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-            fit = n > 0 ? n : -1;
-            max_clusters[split].store(fit, std::memory_order_relaxed);
-        }
-        if (blocks <= fit) return split;
-    }
-    return 1;
-}
 
 template <int D>
 gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
@@ -953,7 +915,7 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
         {attn_bwd_kernel<D, false, true, false>, attn_bwd_kernel<D, false, true, true>},
         {attn_bwd_kernel<D, false, false, false>, attn_bwd_kernel<D, false, false, true>}};
     static std::atomic<uint64_t> granted[3][2] = {};
-    static std::atomic<int32_t> max_clusters[3][kMaxSplit + 1] = {};
+    static ClusterFit max_clusters[3];
     p.split = 1;
     if (p.dk_acc == nullptr && p.list == nullptr) {
         const int32_t q_end = p.q_row_end < batch->max_seqlen ? p.q_row_end : batch->max_seqlen;
@@ -961,7 +923,7 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
         if (n_q >= (priv ? kMinSplitTiles : kMinSplitTiles / 2)) {
             const gt_status st = grant_smem(forms[form][1], granted[form][1], kMaxSmemBytes);
             if (st != GT_OK) return st;
-            p.split = query_split(forms[form][1], max_clusters[form], (int64_t)grid.x * grid.y * grid.z, n_q, smem);
+            p.split = cluster_split(forms[form][1], kBwdThreads, smem, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, n_q);
             grid.x *= (unsigned)p.split;
         }
     }

@@ -84,6 +84,7 @@ struct FwdParams {
     int32_t state_q_end;
     const uint8_t* maps;       // packed batch: tensor maps of the graphs' SPD blocks
     const int4* list;          // packed batch: work list; block index = entry * heads + head (nullptr: grid of heads x blocks x graphs)
+    int32_t split;             // one query tile: thread blocks (a cluster) that share its keys
     const __nv_bfloat16* q;    // precise variant: for the rows' norms
     const float* key_norms;    // precise variant: largest |k|^2 of every kNormRows rows, [H][blocks] (nullptr: always the classical way)
     int32_t spd_tma;           // 1: SPD tiles come by TMA; 0: packed batch without room for the maps, cp.async loader warp
@@ -161,7 +162,7 @@ __device__ __forceinline__ float norm_max(float a, float b) { return __uint_as_f
 // of fp32 and bf16, whose relative precision does not depend on the reference.  Rows (warps of 32) beyond it take the
 // maximum first, which costs a second pass over the scores.  8 192 nodes, 8 heads of 64: 386 -> 251 us, norms included.
 // kTiles = 1: thread blocks of one 128-row query tile and eight softmax warps, for grids that would leave half
-// of the SMs idle or more (rows_per_block).  Two score buffers then: with three, a warp could be two key tiles ahead of another.
+// of the SMs idle or more (rows_per_block); a cluster of them may share the keys (FwdParams::split).  Two score buffers then: with three, a warp could be two key tiles ahead of another.
 template <int D, bool kPartial, bool kShflBias, bool kPrecise = false, int kTiles = kQTiles>
 __global__ void __launch_bounds__(128 + 256 * kTiles, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
@@ -182,6 +183,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     int h = blockIdx.x, g = kPartial ? 0 : (int)blockIdx.z;
     int32_t q_block = (int32_t)blockIdx.y + p.q_block0;
     const int chunk = kPartial ? (int)blockIdx.z : 0;
+    constexpr bool kShared = kTiles == 1 && !kPartial;       // blocks of a cluster may share the keys
+    const int rank = kShared ? (int)blockIdx.x % p.split : 0;
+    if constexpr (kShared) h = (int)blockIdx.x / p.split;
 
     if (p.cu_seqlens) grid_wait();          // a single graph's blocks set up their barriers and tensor memory before they wait
     int32_t node0 = 0, n_g = p.n_total;
@@ -201,8 +205,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (q0 >= n_g) return;
     const int64_t ld = (int64_t)((n_g + 15) & ~15);
     const uint8_t* spd_g = p.spd + (p.spd_offsets ? p.spd_offsets[g] : 0);
-    const int32_t kv_begin = kPartial ? (p.use_ranges ? p.range_begin[chunk] : chunk * p.kv_chunk_rows) : 0;
-    const int32_t kv_end = kPartial ? (p.use_ranges ? p.range_end[chunk] : min(n_g, kv_begin + p.kv_chunk_rows)) : n_g;
+    int32_t kv_begin = kPartial ? (p.use_ranges ? p.range_begin[chunk] : chunk * p.kv_chunk_rows) : 0;
+    int32_t kv_end = kPartial ? (p.use_ranges ? p.range_end[chunk] : min(n_g, kv_begin + p.kv_chunk_rows)) : n_g;
+    int sharers = 1;                        // blocks of the cluster that have keys
+    if constexpr (kShared) {
+        const int32_t tiles = (n_g + kKvTile - 1) / kKvTile, per = (tiles + p.split - 1) / p.split;
+        sharers = (tiles + per - 1) / per;
+        if (rank >= sharers) return;        // (the cluster's barriers wait for blocks that are still there)
+        kv_begin = rank * per * kKvTile;
+        kv_end = min(n_g, kv_begin + per * kKvTile);
+    }
     const int32_t n_kv = kv_end > kv_begin ? (kv_end - kv_begin + kKvTile - 1) / kKvTile : 0;
 
     if (kPartial && n_kv == 0) {            // empty chunk: weight zero in the merge
@@ -616,7 +628,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int32_t q = q0 + t * kRowsPerTile + r;
         const float inv_l = 1.0f / l;
         const float lse_nat = (m + log2f(l)) * kLn2;
-        if (kPartial && p.state_o != nullptr) {
+        if (kShared && sharers > 1) {
+            // This block's share of O, not normalised, and its m and l, to its own shared memory (over K and V: every MMA is done).
+#pragma unroll
+            for (int c = 0; c < kOC / kOP; ++c) {
+                uint32_t o[kOP];
+                tmem_ld<kOP>(tO + c * kOP, o);
+                tmem_wait_ld();
+                uint4* part = (uint4*)(smem + L::kK) + ((hf * kOC + c * kOP) / 4) * 128 + r;
+#pragma unroll
+                for (int i = 0; i < kOP / 4; ++i) part[i * 128] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+            }
+            if (hf == 0) *(float2*)(smem + L::kXchg + 512 * 4 + r * 8) = make_float2(m, l);
+        } else if (kPartial && p.state_o != nullptr) {
             // Merge into the carried state: lse' = log(e^lse0 + e^lse), o' = e^(lse0-lse') o0 + e^(lse-lse') o.
             const bool mine = q >= p.state_q_begin && q < p.state_q_end;
             float* lse_ptr = p.state_lse + (size_t)h * p.n_total + q;
@@ -695,6 +719,43 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     if (*abort_flag) __nanosleep(200000);    // let copies that may still be in flight land
     if (warp == 1) tmem_dealloc(tmem, 512);
+    if (kShared && sharers > 1) {
+        // Every block merges its part of the rows' channels from all blocks' shares.
+        cluster_sync();
+        constexpr int kPieces = (D / 4) * 128;           // of four channels of a row
+        const int per = (kPieces + sharers - 1) / sharers;
+        for (int i = rank * per + tid; i < min(kPieces, (rank + 1) * per); i += kThreads) {
+            const int row = i & 127, c4 = i >> 7;
+            const uint32_t at = smem_u32(smem + L::kK) + (uint32_t)i * 16u, at_ml = smem_u32(smem + L::kXchg) + 512u * 4u + (uint32_t)row * 8u;
+            float2 ml[kMaxSplit];
+            float mx = -INFINITY;
+#pragma unroll
+            for (int k = 0; k < kMaxSplit; ++k) {
+                ml[k] = k < sharers ? ld_cluster_float2(at_ml, (uint32_t)k) : make_float2(-INFINITY, 0.f);
+                mx = fmaxf(mx, ml[k].x);
+            }
+            float den = 0.f;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < kMaxSplit; ++k) {
+                if (ml[k].x == -INFINITY && mx != -INFINITY) continue;       // no such block, or nothing to attend to among its keys
+                if (k >= sharers) continue;
+                const float w = ex2_approx(ml[k].x - mx);                    // references are whole numbers: a power of two
+                const float4 b = ld_cluster_float4(at, (uint32_t)k);
+                den += w * ml[k].y;
+                a.x += w * b.x; a.y += w * b.y; a.z += w * b.z; a.w += w * b.w;
+            }
+            const int32_t q = q0 + row;
+            if (q >= n_g) continue;
+            const float inv = 1.0f / den;
+            a.x *= inv; a.y *= inv; a.z *= inv; a.w *= inv;
+            const size_t to = ((size_t)(node0 + q) * p.n_heads + h) * D + c4 * 4;
+            *(uint2*)(p.out + to) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+            if (kPrecise && p.out_f32 != nullptr) *(float4*)(p.out_f32 + to) = a;
+            if (c4 == 0) p.lse[(size_t)h * p.n_total + node0 + q] = (mx + log2f(den)) * kLn2;
+        }
+        cluster_sync();                                  // no block leaves while another reads its share
+    }
 }
 
 // Merge of per-chunk partials: lse = log sum_c exp(lse_c), out = sum_c exp(lse_c - lse) out_c.
@@ -862,9 +923,14 @@ inline int32_t rows_per_block(const gt_batch* b, int32_t n_heads)
     return (int64_t)((b->max_seqlen + kRowsPerTile - 1) / kRowsPerTile) * b->n_graphs * n_heads <= sm_count() ? kRowsPerTile : kRowsPerCta;
 }
 
+// Blocks that share a query tile's keys (cluster_split): a key tile takes 1.2 us, the cluster and the merge 3 us.  1 000 nodes, heads
+// of 64: 8 heads 13.9 -> 12.6 us, 4 heads 13.7 -> 10.8; 2 048 nodes, 4 heads 22.3 -> 17.1; 512 nodes, 8 heads 10.5 -> 10.7; 8 graphs of
+// 500 nodes, 2 heads 11.6 -> 12.2: from six key tiles on.
+constexpr int32_t kMinSplitTiles = 6;
+
 template <int D, bool kPartial>
 gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tspd,
-                     const FwdParams& p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0)
+                     FwdParams p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0)
 {
     const bool shfl = p.n_buckets <= 32;
     const int32_t rows = kPartial ? kRowsPerCta : rows_per_block(batch, p.n_heads);
@@ -877,12 +943,19 @@ gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
         }
     }
     static std::atomic<uint64_t> granted[8] = {};
-    const gt_status st = grant_smem(kern, granted[(shfl ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0) + (rows == kRowsPerTile ? 4 : 0)], FwdSmem<D>::kDynamic);
+    static ClusterFit max_clusters[4];
+    const int form = (shfl ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0);
+    const gt_status st = grant_smem(kern, granted[form + (rows == kRowsPerTile ? 4 : 0)], FwdSmem<D>::kDynamic);
     if (st != GT_OK) return st;
     const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + rows - 1) / rows;
-    const dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kRowsPerCta) * p.n_heads))
-                             : dim3((unsigned)p.n_heads, (unsigned)row_blocks, (unsigned)grid_z);
-    return launch_overlapped(kern, grid, 128 + 2 * rows, FwdSmem<D>::kDynamic, s, tq, tk, tv, tspd, p);
+    dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kRowsPerCta) * p.n_heads))
+                       : dim3((unsigned)p.n_heads, (unsigned)row_blocks, (unsigned)grid_z);
+    p.split = 1;
+    const int32_t tiles = (batch->max_seqlen + kKvTile - 1) / kKvTile;
+    if (rows == kRowsPerTile && tiles >= kMinSplitTiles)
+        p.split = cluster_split(kern, 128 + 2 * rows, FwdSmem<D>::kDynamic, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, tiles);
+    grid.x *= (unsigned)p.split;
+    return launch_overlapped_cluster(kern, grid, 128 + 2 * rows, FwdSmem<D>::kDynamic, p.split, s, tq, tk, tv, tspd, p);
 }
 
 gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint8_t* spd, const int64_t* spd_offsets,

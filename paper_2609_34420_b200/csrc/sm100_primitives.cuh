@@ -336,5 +336,27 @@ __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
     return r;
 }
 
+// All threads of the cluster's blocks that have not returned.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// 16 bytes at a shared address of the cluster's block `rank`
+__device__ __forceinline__ float4 ld_cluster_float4(uint32_t addr, uint32_t rank)
+{
+    float4 v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ float2 ld_cluster_float2(uint32_t addr, uint32_t rank)
+{
+    float2 v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %2, %3;\n\tld.shared::cluster.v2.f32 {%0, %1}, [a];\n\t}"
+                 : "=f"(v.x), "=f"(v.y) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+
 }  // namespace sm100
 }  // namespace gt

@@ -92,3 +92,16 @@ def test_chunked_backward_with_shared_key_tiles(chunks):
     whole = case.backward(out, lse)
     for got, want in zip(case.backward_chunked(out, lse, chunks)[:4], whole):       # sums in another order, results rounded to bf16
         assert rel_l2(to_f64(got), to_f64(want)) <= 5e-3
+
+
+# a query tile's keys shared by a cluster of 2, 3 or 4 blocks: the first size with it, a share that is empty (9 and 10 tiles by 4: 3
+# each), one key in the last tile, graphs of a batch with fewer tiles than blocks, wide bias tables (shares of different references)
+@pytest.mark.parametrize("sizes_,heads,d,D,spread", [([641], 4, 64, 6, 1.0), ([700], 4, 32, 6, 12.0), ([1200], 3, 64, 60, 12.0), ([1025], 5, 64, 20, 1.0),
+                                                     ([1100], 7, 32, 6, 12.0), ([800, 1, 300], 2, 64, 6, 1.0)])
+def test_forward_with_shared_query_tiles(sizes_, heads, d, D, spread):
+    w = wl.small_workload(sizes_, heads, d, D, seed=sum(sizes_) + D, avg_degree=1.5)
+    w.tensors().bias[:] *= spread
+    case, out, lse = check_forward(w)
+    out_p, lse_p, out32 = case.forward_ex()
+    ro, _ = oracle_forward(case)
+    assert rel_l2(to_f64(out32), ro) <= 1e-4 and (lse_p - lse).abs().max().item() <= LSE_MAX_ABS
