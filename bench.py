@@ -232,10 +232,14 @@ def run_cuda(args) -> int:
         if marks is not None:
             marks[4].record()
 
-    # spd: setup + component pre-pass + BFS, or for a single graph beyond the shared-memory state setup + two item-scan
-    # kernels + item table + bit-matrix BFS; fwd; bwd: transpose, pre-pass, main, finalize; chunked: partial + merge
-    dense_spd = single and b.max_seqlen >= 14500          # the library's switch to the bit-matrix build
-    kernels_per_step = (5 if dense_spd else 3) + 1 + 4 + (2 if single else 0)
+    # spd: one pull kernel where it needs no workspace beyond the header; a larger single graph: order, lists and pull, or beyond
+    # 18 944 nodes setup, two item scans, item table and bit-matrix BFS; a larger batch: setup, components, BFS.
+    # fwd: (a batch's maps and work list,) main; bwd: prepare, main, finalize; chunked: partial, merge
+    dense_spd = single and b.max_seqlen > 18944           # the library's switch to the bit-matrix build
+    spd_kernel = ("spd_pull_kernel" if ws_spd.numel() <= 256 else "spd_dense_kernel" if dense_spd else
+                  "spd_large_pull_kernel" if single else "spd_bfs_kernel")
+    spd_launches = 1 if spd_kernel == "spd_pull_kernel" else (5 if dense_spd else 3)
+    kernels_per_step = spd_launches + (1 if single else 2) + 3 + (2 if single else 0)
 
     for _ in range(max(args.warmup, 0)):
         step()
@@ -396,7 +400,7 @@ def run_cuda(args) -> int:
                         "bwd_ms": ft["codes_bwd_ms"], "bwd_tflops": tf(ft["bwd_flops"], ft["codes_bwd_ms"]),
                         "fp32_path_fwd_ms": ft["fp32_fwd_ms"], "fp32_path_bwd_ms": ft["fp32_bwd_ms"],
                         "note": "outside the timed step; categorical features as a code matrix through the tensor-core kernels "
-                                "(forward with the fp32 output), next to the fp32 path on the CUDA cores that serves any features"}
+                                "(forward with the fp32 output), next to the path that serves any features"}
 
     # ---- end to end through the C ABI with host buffers (pinned), copies inside the timed region ----
     host_in = {name: x.cpu().pin_memory() for name, x in
@@ -479,7 +483,7 @@ def run_cuda(args) -> int:
         "flops_per_launch": f_bwd, "ms_per_launch": bwd_kernel_ms,
         "timing": "CUDA events recorded by the library around the kernel's launch inside every timed step (mean over the steps)",
         "ms_per_call": bwd_ms, "frac_of_call": bwd_tflops / peak_tf,
-        "call_note": "gt_biased_attn_bwd also runs the SPD transpose, the per-query pre-pass, two zero fills and the final conversion",
+        "call_note": "gt_biased_attn_bwd also runs the preparation (SPD transpose, per-query terms, zero fills) and the final conversion",
     }
     fwd_tflops_ = f_fwd / (fwd_ms * 1e-3) / 1e12
     roofline_fwd = {
@@ -489,7 +493,7 @@ def run_cuda(args) -> int:
         "traffic": FWD_KERNEL_DRAM_BYTES_PER_N2 * sum_n2, "flops_per_launch": f_fwd, "ms_per_launch": fwd_ms,
     }
     roofline_spd = {
-        "kernel": "spd_dense_kernel" if dense_spd else "spd_bfs_kernel", "bound": "hbm", "achieved": spd_alg_bytes / (spd_ms * 1e-3) / 1e9,
+        "kernel": spd_kernel, "bound": "hbm", "achieved": spd_alg_bytes / (spd_ms * 1e-3) / 1e9,
         "peak": float(peaks["hbm_gbs"]), "unit": "GB/s",
         "frac": spd_alg_bytes / (spd_ms * 1e-3) / 1e9 / float(peaks["hbm_gbs"]), "peak_kind": f"hbm_gbs of {peak_kind}",
         "bytes_per_launch": spd_alg_bytes, "ms_per_launch": spd_ms,

@@ -6,8 +6,8 @@
 WORKLOAD is one of the named workloads (tiny_er256, ba4096, powerlaw16k, powerlaw64k,
 varlen_rgg64) or plN for a power-law graph of N nodes (H=8, d=64, max_dist=24).  A small,
 self-contained timing command line for one entry point at a time.  featN times the feature-bias
-variant on N nodes (H=8, d=64) with VECTORS distinct feature vectors (default 12): the fp32 path on
-the CUDA cores, and the code matrix through the tensor-core kernels of the bucket form.
+variant on N nodes (H=8, d=64) with VECTORS distinct feature vectors (default 12): the path for any
+features, and the code matrix through the tensor-core kernels of the bucket form.
 """
 from __future__ import annotations
 
@@ -80,8 +80,8 @@ def feature_timings(n: int, reps: int, n_vec: int, cuda_core_path: bool = True) 
 def feature_case(n: int, reps: int, n_vec: int) -> int:
     r = feature_timings(n, reps, n_vec)
     tf = lambda flops, ms: flops / ms / 1e9
-    print(f"feature fwd (CUDA cores) {r['fp32_fwd_ms']:.3f} ms  {tf(r['fwd_flops'], r['fp32_fwd_ms']):.1f} TFLOP/s")
-    print(f"feature bwd (CUDA cores) {r['fp32_bwd_ms']:.3f} ms  {tf(r['bwd_flops'], r['fp32_bwd_ms']):.1f} TFLOP/s")
+    print(f"feature fwd (any) {r['fp32_fwd_ms']:.3f} ms  {tf(r['fwd_flops'], r['fp32_fwd_ms']):.1f} TFLOP/s")
+    print(f"feature bwd (any) {r['fp32_bwd_ms']:.3f} ms  {tf(r['bwd_flops'], r['fp32_bwd_ms']):.1f} TFLOP/s")
     print(f"feature encode {r['encode_ms']:.3f} ms  {n * n * 5 / r['encode_ms'] / 1e6:.1f} GB/s  ({r['codes']} codes)")
     print(f"feature fwd (codes, fp32 output too) {r['codes_fwd_ms']:.3f} ms  {tf(r['fwd_flops'], r['codes_fwd_ms']):.1f} TFLOP/s")
     print(f"feature bwd (codes) {r['codes_bwd_ms']:.3f} ms  {tf(r['bwd_flops'], r['codes_bwd_ms']):.1f} TFLOP/s")
