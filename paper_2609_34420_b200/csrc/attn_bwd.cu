@@ -882,11 +882,12 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
     return w;
 }
 
-// Thread blocks that share the queries of a key tile (cluster_split): a query tile takes 1.3 us (with the shared bins of many
-// buckets four times that), the cluster and its sums 2 us, so from four query tiles on, or two.
+// Thread blocks that share the queries of a key tile (cluster_split): fill and drain take as long as three query tiles, the cluster
+// and its sums as one (a quarter of that with the shared bins of many buckets, whose tiles take four times as long).
 // Whole call, 8 heads of 64 if not said otherwise: 1 000 nodes 29.8 -> 24.9 us (4 heads: 29.8 -> 21.5), 1 200 nodes, 4 heads 33.4 ->
-// 24.2, 2 048 nodes, 4 heads 47.5 -> 34.7, 300 nodes, 4 heads of 32, 256 buckets 47.0 -> 32.3; 512 nodes no difference.
-constexpr int32_t kMinSplitTiles = 4;
+// 24.2, 2 048 nodes, 4 heads 47.5 -> 34.7, 300 nodes, 4 heads of 32, 256 buckets 47.0 -> 32.3; 512 nodes no difference.  Last waves
+// of few blocks: 2 500 nodes 105 -> 99, 3 000 128.5 -> 118, 8 192 602 -> 581, 6 000 nodes, 4 heads 237 -> 207.
+constexpr float kFixedTiles = 3.0f, kClusterTiles = 1.0f;
 
 template <int D>
 gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
@@ -905,9 +906,6 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     p.bin_log = kPrivateBinLog;
     while ((p.n_buckets << p.bin_log) > (kMaxPrivateBinBuckets << kPrivateBinLog)) --p.bin_log;
     const size_t smem = BwdSmem<D>::dynamic_bytes(p.n_buckets << p.bin_log);
-    // With several waves of blocks the early start of the next kernel slows the dispatch of this one's (65 536 nodes: 36.5 ->
-    // 39.9 ms); with one it hides the next one's start.
-    p.early_release = (int64_t)grid.x * grid.y * grid.z <= sm_count();      // (a split grid fits, too)
     static_assert(kMaxPrivateBinBuckets <= 32, "private bins go with the shuffle lookup");
     const int form = priv ? 0 : (p.n_buckets <= 32 ? 1 : 2);
     void (*const forms[3][2])(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, BwdParams) = {
@@ -920,13 +918,16 @@ gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     if (p.dk_acc == nullptr && p.list == nullptr) {
         const int32_t q_end = p.q_row_end < batch->max_seqlen ? p.q_row_end : batch->max_seqlen;
         const int32_t n_q = (q_end - p.q_row0 + kTile - 1) / kTile;
-        if (n_q >= (priv ? kMinSplitTiles : kMinSplitTiles / 2)) {
-            const gt_status st = grant_smem(forms[form][1], granted[form][1], kMaxSmemBytes);
-            if (st != GT_OK) return st;
-            p.split = cluster_split(forms[form][1], kBwdThreads, smem, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, n_q);
-            grid.x *= (unsigned)p.split;
-        }
+        const float unit = priv ? 1.0f : 0.25f;
+        const gt_status st = grant_smem(forms[form][1], granted[form][1], kMaxSmemBytes);
+        if (st != GT_OK) return st;
+        p.split = cluster_split(forms[form][1], kBwdThreads, smem, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, n_q,
+                                unit * kFixedTiles, unit * kClusterTiles);
+        grid.x *= (unsigned)p.split;
     }
+    // With several waves of blocks the early start of the next kernel slows the dispatch of this one's (65 536 nodes: 36.5 ->
+    // 39.9 ms); with one it hides the next one's start.
+    p.early_release = (int64_t)grid.x * grid.y * grid.z <= sm_count();
     auto kern = forms[form][p.split > 1];
     const gt_status st = grant_smem(kern, granted[form][p.split > 1], kMaxSmemBytes);
     if (st != GT_OK) return st;

@@ -83,38 +83,53 @@ __device__ __forceinline__ void write_work_list(int4* list, int32_t entries, con
         list[i] = i < first + blocks ? make_int4(g, i - first, c0, n) : make_int4(-1, 0, 0, 0);
 }
 
-// Blocks of a cluster that share the work of one: as many (up to kMaxSplit, and one per tile of that work) as let the whole grid
-// run at once, of a cluster size of which the device holds enough at a time (a cluster's blocks lie in one group of SMs).
+// Clusters of `split` blocks that the device holds at a time (a cluster's blocks lie in one group of SMs), -1: none.
 constexpr int kMaxSplit = 4;
-struct ClusterFit { std::atomic<int32_t> n[kMaxSplit + 1] = {}; };       // clusters at a time, by size; 0: not asked yet
+struct ClusterFit { std::atomic<int32_t> n[kMaxSplit + 1] = {}; };       // by size; 0: not asked yet
 template <typename Kernel>
-int32_t cluster_split(Kernel kern, int threads, size_t smem, ClusterFit& fits, int64_t blocks, int32_t tiles)
+int32_t clusters_at_a_time(Kernel kern, int threads, size_t smem, ClusterFit& fits, int32_t split)
 {
-    for (int32_t split = kMaxSplit; split > 1; --split) {
-        if (blocks * split > sm_count() || tiles < split) continue;
-        int32_t fit = fits.n[split].load(std::memory_order_relaxed);
-        if (fit == 0) {                                    // (whatever the shared memory, these kernels' blocks have an SM each)
-            cudaLaunchAttribute attr{};
-            attr.id = cudaLaunchAttributeClusterDimension;
-            attr.val.clusterDim.x = (unsigned)split;
-            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)split);
-            cfg.blockDim = dim3((unsigned)threads);
-            cfg.dynamicSmemBytes = smem;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-                cudaGetLastError();
-                n = 0;
-            }
-            fit = n > 0 ? n : -1;
-            fits.n[split].store(fit, std::memory_order_relaxed);
-        }
-        if (blocks <= fit) return split;
+    if (split == 1) return sm_count();                     // (whatever the shared memory, these kernels' blocks have an SM each)
+    int32_t fit = fits.n[split].load(std::memory_order_relaxed);
+    if (fit != 0) return fit;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)split;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)split);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
     }
-    return 1;
+    fit = n > 0 ? n : -1;
+    fits.n[split].store(fit, std::memory_order_relaxed);
+    return fit;
+}
+
+// Blocks of a cluster that share the work of one: where `blocks` of `tiles` tiles each end soonest, taking a tile as the unit of time,
+// `fixed` for a block's fill and drain and `shared` for what a cluster costs on top.  The grid runs in waves, so that a last wave
+// of few blocks may end sooner in shares, too.  Sharing has to promise 5 %.
+template <typename Kernel>
+int32_t cluster_split(Kernel kern, int threads, size_t smem, ClusterFit& fits, int64_t blocks, int32_t tiles, float fixed, float shared)
+{
+    int32_t best = 1;
+    float least = 0.95f * (float)((blocks + sm_count() - 1) / sm_count()) * ((float)tiles + fixed);
+    for (int32_t split = 2; split <= kMaxSplit && split <= tiles; ++split) {
+        const int32_t fit = clusters_at_a_time(kern, threads, smem, fits, split);
+        if (fit <= 0) continue;
+        const float time = (float)((blocks + fit - 1) / fit) * ((float)((tiles + split - 1) / split) + fixed + shared);
+        if (time < least) {
+            least = time;
+            best = split;
+        }
+    }
+    return best;
 }
 
 struct AttnArgsCheck {

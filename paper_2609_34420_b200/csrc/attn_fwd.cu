@@ -923,7 +923,7 @@ inline int32_t rows_per_block(const gt_batch* b, int32_t n_heads)
     return (int64_t)((b->max_seqlen + kRowsPerTile - 1) / kRowsPerTile) * b->n_graphs * n_heads <= sm_count() ? kRowsPerTile : kRowsPerCta;
 }
 
-// Blocks that share a query tile's keys (cluster_split): a key tile takes 1.2 us, the cluster and the merge 3 us.  1 000 nodes, heads
+// Blocks that share a query tile's keys (cluster_split): a key tile takes 1.2 us, the cluster and the merge 2 to 3 us.  1 000 nodes, heads
 // of 64: 8 heads 13.9 -> 12.6 us, 4 heads 13.7 -> 10.8; 2 048 nodes, 4 heads 22.3 -> 17.1; 512 nodes, 8 heads 10.5 -> 10.7; 8 graphs of
 // 500 nodes, 2 heads 11.6 -> 12.2: from six key tiles on.
 constexpr int32_t kMinSplitTiles = 6;
@@ -953,7 +953,7 @@ gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     p.split = 1;
     const int32_t tiles = (batch->max_seqlen + kKvTile - 1) / kKvTile;
     if (rows == kRowsPerTile && tiles >= kMinSplitTiles)
-        p.split = cluster_split(kern, 128 + 2 * rows, FwdSmem<D>::kDynamic, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, tiles);
+        p.split = cluster_split(kern, 128 + 2 * rows, FwdSmem<D>::kDynamic, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, tiles, 3.0f, 2.0f);
     grid.x *= (unsigned)p.split;
     return launch_overlapped_cluster(kern, grid, 128 + 2 * rows, FwdSmem<D>::kDynamic, p.split, s, tq, tk, tv, tspd, p);
 }
