@@ -883,11 +883,12 @@ BwdWorkspace bwd_workspace(const gt_batch* b, int32_t n_heads, int32_t head_dim,
 }
 
 // Thread blocks that share the queries of a key tile (cluster_split): fill and drain take as long as three query tiles, the cluster
-// and its sums as one (a quarter of that with the shared bins of many buckets, whose tiles take four times as long).
+// and its sums as one to two (a quarter of that with the shared bins of many buckets, whose tiles take four times as long).
 // Whole call, 8 heads of 64 if not said otherwise: 1 000 nodes 29.8 -> 24.9 us (4 heads: 29.8 -> 21.5), 1 200 nodes, 4 heads 33.4 ->
 // 24.2, 2 048 nodes, 4 heads 47.5 -> 34.7, 300 nodes, 4 heads of 32, 256 buckets 47.0 -> 32.3; 512 nodes no difference.  Last waves
-// of few blocks: 2 500 nodes 105 -> 99, 3 000 128.5 -> 118, 8 192 602 -> 581, 6 000 nodes, 4 heads 237 -> 207.
-constexpr float kFixedTiles = 3.0f, kClusterTiles = 1.0f;
+// of few blocks: 3 000 nodes 128.5 -> 118, 6 000 nodes, 4 heads 237 -> 207.  With one tile for the cluster, 8 192 nodes went from 602
+// to 581 on an idle device, but from 573 to 583 behind a forward, whose blocks free the SMs one by one: two keeps away from that.
+constexpr float kFixedTiles = 3.0f, kClusterTiles = 2.0f;
 
 template <int D>
 gt_status launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,

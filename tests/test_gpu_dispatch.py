@@ -80,7 +80,7 @@ def test_one_and_two_query_tiles_per_block(n, beyond):
 # graphs of a batch with fewer tiles than blocks, and the first size without
 @pytest.mark.parametrize("sizes_,heads,d,D", [([385], 37, 32, 6), ([513], 7, 64, 6), ([640], 9, 64, 6), ([641], 8, 32, 24), ([900], 9, 64, 6),
                                               ([129], 2, 64, 60), ([300], 4, 32, 254), ([500, 500, 500], 2, 64, 9), ([512, 1], 4, 32, 9),
-                                              ([2500], 8, 32, 6)])       # (the last: 160 blocks, two waves or shares of two)
+                                              ([3000], 8, 32, 6)])       # (the last: 192 blocks, two waves or three of shares)
 def test_backward_with_shared_key_tiles(sizes_, heads, d, D):
     check_backward(wl.small_workload(sizes_, heads, d, D, seed=sum(sizes_) + D, avg_degree=2.0))
 
