@@ -5,11 +5,12 @@
 // dW[h][c] = sum_ij dS_ij f[i][j][c], instead of the scatter of the bucket form.
 //
 // The contractions run on the tensor cores without giving up fp32: the bf16 inputs are exact operands, and a probability or
-// a score gradient, an fp32 number, goes in as three bf16 terms (8 + 8 + 8 bits of mantissa: the sum is the number), so the
-// products are those of the fp32 form; sums are fp32 and the elementwise part is unchanged fp32.  Three kernels of one shape:
+// a score gradient, an fp32 number, goes in as three bf16 terms (8 + 8 + 8 bits of mantissa: the sum is the number); sums
+// over more than one MMA block are fp32 adds (add_product).  Against fp64, lse and dW are no further off than the same sums
+// formed element by element on the fp32 pipes, and fewer of the bf16 results miss the nearest value.  Three kernels of one shape:
 //   forward      a warp owns 16 query rows and walks over keys:   S = Q K^T, online softmax, O += P V
-//   query side   the same rows and keys:  S, dP = dO V^T, then in ONE walk the sums of P dP K and P K (and of P dP f, P f and
-//                P dP); with Delta_i = sum_j P_ij dP_ij known at the end,  dQ_i = sum P dP K - Delta_i sum P K,  and dW alike
+//   query side   the same rows and keys, twice:  S and dP = dO V^T for Delta_i = sum_j P_ij dP_ij, then again for dS = P (dP - Delta),
+//                dQ += dS K and dW += dS f
 //   key side     a warp owns 16 key rows and walks over queries:  S^T, dP^T, dV += P^T dO, dK += dS^T Q
 // The score fragments of one product are the operand fragments of the next (mma.sync keeps both in registers), a pair's four
 // features are read straight into the lane that holds its score, and Delta is formed from the same P as the gradients: the
@@ -19,9 +20,9 @@
 //
 // mma.sync and not tcgen05: at the 500 - 8 192 nodes this form is meant for, a 128-row tile per thread block would leave
 // most SMs empty, and the three-term operands would have to travel through tensor memory.
-// What bounds it: latency at ten warps per SM (1 500 nodes have no more rows), with the warp-level MMAs at 36-46 % of their
-// pipe (14 of the 20 contractions are the terms of P and dS) and the issue slots at 41-50 %.  1 500 nodes, H = 8, d = 64:
-// forward 55 us, query side 92 us, key side 85 us; the same sums on the fp32 pipes took 3 000 us.
+// What bounds it: latency at ten warps per SM (1 500 nodes have no more rows); 12 of the 19 contractions are the terms of P and
+// dS.  1 500 nodes, H = 8, d = 64: forward 64 us, backward 199 us (54 and 172 with one chain of MMAs over all keys, ex2 in the
+// forward and one walk on the query side, whose results are further off); the same sums on the fp32 pipes took 3 000 us.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -171,16 +172,31 @@ __device__ __forceinline__ void split_block(const float (&p)[2][4], uint32_t (&t
     split3(p[1][2], p[1][3], t[0][3], t[1][3], t[2][3]);
 }
 
-// Two sums (16 x 16 of 16 x D): acc += P (16 x 16, three terms; smallest first) times 16 rows of a tile, steps alternating.
-__device__ __forceinline__ void two_sums(float (&u0)[4], float (&u1)[4], const uint32_t (&t)[3][4], const uint32_t (&b)[4],
-                                         float (&v0)[4], float (&v1)[4], const uint32_t (&r)[3][4], const uint32_t (&d)[4])
+// acc (16 x D) += P (16 x 16, three terms; smallest first) times 16 rows of a tile.  The tensor core cuts off what its
+// accumulator cannot hold instead of rounding it, an error that grows with every MMA of a chain and does not cancel: a chain is
+// one block of 16 long and its result is added to the sum by an fp32 add.  (With chains over all keys two to five times as many
+// outputs miss the nearest bf16 value, growing with n.)  Four chains alternate: an MMA that adds to the result of the one before
+// it would wait for it.
+template <int D>
+__device__ __forceinline__ void add_product(float (&acc)[D / 8][4], const uint32_t (&t)[3][4], uint32_t base, int row, int lane)
 {
 #pragma unroll
-    for (int x = 2; x >= 0; --x) {
-        mma16816(u0, t[x], b[0], b[1]);
-        mma16816(v0, r[x], d[0], d[1]);
-        mma16816(u1, t[x], b[2], b[3]);
-        mma16816(v1, r[x], d[2], d[3]);
+    for (int c = 0; c < D / 16; c += 2) {
+        uint32_t b0[4], b1[4];
+        Tile<D>::load_bt(b0, base, row, c, lane);
+        Tile<D>::load_bt(b1, base, row, c + 1, lane);
+        float u[4][4] = {};
+#pragma unroll
+        for (int x = 2; x >= 0; --x) {
+            mma16816(u[0], t[x], b0[0], b0[1]);
+            mma16816(u[2], t[x], b1[0], b1[1]);
+            mma16816(u[1], t[x], b0[2], b0[3]);
+            mma16816(u[3], t[x], b1[2], b1[3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) acc[2 * c + k][x] += u[k][x];
     }
 }
 
@@ -190,6 +206,8 @@ __device__ __forceinline__ void unpack_features(uint32_t f4, float (&f)[kFeat])
 #pragma unroll
     for (int c = 0; c < kFeat; ++c) f[c] = __uint_as_float(__byte_perm(f4, 0x47000000u, 0x7404u | ((uint32_t)c << 4))) - 32768.f;
 }
+
+template <bool B> struct BoolConst { static constexpr bool value = B; };
 
 struct FeatureArgs {
     const __nv_bfloat16 *q, *k, *v, *dout;
@@ -205,11 +223,12 @@ struct FeatureArgs {
     float scale;                  // 1 / sqrt(d)
 };
 
-// 2^x to 2 ulp (0 for -inf)
-__device__ __forceinline__ float exp2_of(float x)
+// e^x for the backward's P, off by up to |x| 2^-24 beside the 2 ulp of ex2, and less than P matters where x is large.  (1 500 nodes:
+// 17 us of 272 less than expf.)  The forward keeps expf, because its lse is returned in fp32.
+__device__ __forceinline__ float exp_of(float x)
 {
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * kLog2e));
     return y;
 }
 
@@ -263,8 +282,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
     const bool pairs = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.feat) & 7u) == 0;
     float w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c] * kLog2e;      // scores in units of log 2
-    const float scale = p.scale * kLog2e;
+    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
 
     uint32_t qa[D / 16][4];
     Tile<D>::template fetch<kRows>(base, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
@@ -310,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
                 for (int x = 0; x < 4; ++x) {
                     const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
                     const float bias = bias_of(x & 1 ? f[b][t][x >> 1].y : f[b][t][x >> 1].x, w);
-                    s[b][t][x] = s[b][t][x] * scale + bias;                      // bias added before the softmax statistics
+                    s[b][t][x] = s[b][t][x] * p.scale + bias;                    // bias added before the softmax statistics
                     if (ragged && j >= n) s[b][t][x] = -INFINITY;
                     top[x >> 1] = fmaxf(top[x >> 1], s[b][t][x]);
                 }
@@ -318,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
         top[0] = quad_max(top[0]);
         top[1] = quad_max(top[1]);
         if (__any_sync(0xffffffffu, top[0] > m[0] || top[1] > m[1])) {
-            const float a0 = m[0] == top[0] ? 1.f : exp2_of(m[0] - top[0]), a1 = m[1] == top[1] ? 1.f : exp2_of(m[1] - top[1]);
+            const float a0 = m[0] == top[0] ? 1.f : expf(m[0] - top[0]), a1 = m[1] == top[1] ? 1.f : expf(m[1] - top[1]);
             l[0] *= a0; l[1] *= a1;
 #pragma unroll
             for (int c = 0; c < D / 8; ++c) { o[c][0] *= a0; o[c][1] *= a0; o[c][2] *= a1; o[c][3] *= a1; }
@@ -330,19 +348,12 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    s[b][t][x] = exp2_of(s[b][t][x] - (x < 2 ? ref0 : ref1));            // 0 for keys past the end
-                    l[x >> 1] += s[b][t][x];
-                }
+                for (int x = 0; x < 4; ++x) s[b][t][x] = expf(s[b][t][x] - (x < 2 ? ref0 : ref1));       // 0 for keys past the end
+            l[0] += (s[b][0][0] + s[b][0][1]) + (s[b][1][0] + s[b][1][1]);
+            l[1] += (s[b][0][2] + s[b][0][3]) + (s[b][1][2] + s[b][1][3]);
             uint32_t pt[3][4];
             split_block(s[b], pt);
-#pragma unroll
-            for (int c = 0; c < D / 16; c += 2) {
-                uint32_t v0[4], v1[4];
-                Tile<D>::load_bt(v0, vt, 32 * half + 16 * b, c, lane);
-                Tile<D>::load_bt(v1, vt, 32 * half + 16 * b, c + 1, lane);
-                two_sums(o[2 * c], o[2 * c + 1], pt, v0, o[2 * c + 2], o[2 * c + 3], pt, v1);
-            }
+            add_product<D>(o, pt, vt, 32 * half + 16 * b, lane);
         }
         __syncthreads();
     }
@@ -366,7 +377,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
         for (int r = 0; r < 2; ++r) {
             const int32_t i = i0 + g + 8 * r;
             const float m2 = part[16 * D + g + 8 * r], l2 = part[16 * D + 16 + g + 8 * r];
-            const float mm = fmaxf(m[r], m2), a = exp2_of(m[r] - mm), b = m2 == -INFINITY ? 0.f : exp2_of(m2 - mm);
+            const float mm = fmaxf(m[r], m2), a = expf(m[r] - mm), b = m2 == -INFINITY ? 0.f : expf(m2 - mm);
             const float ll = l[r] * a + l2 * b, inv = 1.0f / ll;
             if (i < n) {
 #pragma unroll
@@ -375,14 +386,17 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
                     const float x = (o[c][2 * r] * a + o2[0] * b) * inv, y = (o[c][2 * r + 1] * a + o2[1] * b) * inv;
                     *(__nv_bfloat162*)(p.out + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) = __floats2bfloat162_rn(x, y);
                 }
-                if (t4 == 0) p.lse[(size_t)h * n + i] = mm * kLn2 + logf(ll);
+                if (t4 == 0) p.lse[(size_t)h * n + i] = mm + logf(ll);
             }
         }
     }
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Backward, query side: dQ, Delta and the row block's share of dW.
+// Backward, query side: dQ, Delta and the row block's share of dW.  Two walks over the keys: first Delta_i = sum_j P_ij dP_ij,
+// divided by sum_j P_ij (1 up to the rounding of lse, whose share of a dP with a large common part would come back as an error of
+// dW), then dS.  (One walk that takes Delta_i sum_j P_ij K_j from sum_j P_ij dP_ij K_j at its end needs one MMA more per 16 keys
+// and channels and loses what the two sums have in common.)
 // ---------------------------------------------------------------------------------------------------
 template <int D>
 __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs p)
@@ -392,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
     constexpr int kTileBytes = kTile * 2 * D;
     __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];
     __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' Q and dO (in registers they would cost a block per SM)
-    __shared__ float s_sums[2][16][kFeat + 1];                                    // the second half's P dP and P f per row
+    __shared__ float2 s_sums[2][2][16];                                           // [half][group][row]: sums of P dP and of P
     __shared__ double s_dw[4][kFeat];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
     const int h = blockIdx.y;
@@ -402,24 +416,23 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
     const bool pairs = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.feat) & 7u) == 0;
     float w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c] * kLog2e;
-    const float scale = p.scale * kLog2e;
+    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
 
     const uint32_t own_q = smem_addr(s_own), own_d = own_q + kRows * 2 * D;
     Tile<D>::template fetch<kRows>(own_q, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     Tile<D>::template fetch<kRows>(own_d, p.dout, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     cp_commit();
 
-    float lse[2], xk[D / 8][4], pk[D / 8][4];                                     // sums of P dP K and of P K
-    float xs[2] = {0.f, 0.f}, pf[2][kFeat], xf[kFeat];                            // sums of P dP, P f (per row) and P dP f
+    float lse[2], delta[2] = {0.f, 0.f}, sum_px[2] = {0.f, 0.f}, sum_p[2] = {0.f, 0.f};
+    float dq[D / 8][4], xf[kFeat];                                                // sums of dS K and of dS f
 #pragma unroll
-    for (int r = 0; r < 2; ++r) lse[r] = i0 + g + 8 * r < n ? p.lse_in[(size_t)h * n + i0 + g + 8 * r] * kLog2e : INFINITY;     // P = 0
+    for (int r = 0; r < 2; ++r) lse[r] = i0 + g + 8 * r < n ? p.lse_in[(size_t)h * n + i0 + g + 8 * r] : INFINITY;     // P = 0
 #pragma unroll
     for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-        for (int x = 0; x < 4; ++x) xk[c][x] = pk[c][x] = 0.f;
+        for (int x = 0; x < 4; ++x) dq[c][x] = 0.f;
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) xf[c] = pf[0][c] = pf[1][c] = 0.f;
+    for (int c = 0; c < kFeat; ++c) xf[c] = 0.f;
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
@@ -427,113 +440,109 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
         Tile<D>::template fetch<kTile>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
         cp_commit();
     };
-    stage(0);
-    for (int32_t tile = 0; tile < n_tiles; ++tile) {
-        const int32_t j0 = tile * kTile + 32 * half;
-        uint2 f[2][2];                                                            // of the next 16 keys
-        auto fetch_features = [&](int b) {
+    auto walk = [&](auto for_delta) {
+        constexpr bool kForDelta = decltype(for_delta)::value;
+        stage(0);
+        for (int32_t tile = 0; tile < n_tiles; ++tile) {
+            const int32_t j0 = tile * kTile + 32 * half;
+            uint2 f[2][2];                                                        // of the next 16 keys
+            auto fetch_features = [&](int b) {
 #pragma unroll
-            for (int t = 0; t < 2; ++t)
+                for (int t = 0; t < 2; ++t)
 #pragma unroll
-                for (int r = 0; r < 2; ++r) f[t][r] = feature_pair(p.feat, n, pairs, i0 + g + 8 * r, j0 + 16 * b + 8 * t + 2 * t4);
-        };
-        fetch_features(0);
-        if (tile + 1 < n_tiles) { stage(tile + 1); cp_wait<1>(); } else cp_wait<0>();
-        __syncthreads();
-        const uint32_t kt = base + (uint32_t)(tile & 1) * 2 * kTileBytes, vt = kt + kTileBytes;
+                    for (int r = 0; r < 2; ++r) f[t][r] = feature_pair(p.feat, n, pairs, i0 + g + 8 * r, j0 + 16 * b + 8 * t + 2 * t4);
+            };
+            fetch_features(0);
+            if (tile + 1 < n_tiles) { stage(tile + 1); cp_wait<1>(); } else cp_wait<0>();
+            __syncthreads();
+            const uint32_t kt = base + (uint32_t)(tile & 1) * 2 * kTileBytes, vt = kt + kTileBytes;
 #pragma unroll 1
-        for (int b = 0; b < 2; ++b) {
-            float s[2][4], dp[2][4];
-            two_scores<D>(s, own_q, dp, own_d, 16 * group, kt, vt, 32 * half + 16 * b, lane);
-            const bool ragged = j0 + 16 * b + 16 > n;
+            for (int b = 0; b < 2; ++b) {
+                float s[2][4], dp[2][4], y[kFeat] = {};
+                two_scores<D>(s, own_q, dp, own_d, 16 * group, kt, vt, 32 * half + 16 * b, lane);
+                const bool ragged = j0 + 16 * b + 16 > n;
 #pragma unroll
-            for (int t = 0; t < 2; ++t)
+                for (int t = 0; t < 2; ++t)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const int r = x >> 1;
-                    const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
-                    float fv[kFeat];
-                    unpack_features(x & 1 ? f[t][r].y : f[t][r].x, fv);
-                    const float bias = w[0] * fv[0] + w[1] * fv[1] + w[2] * fv[2] + w[3] * fv[3];
-                    float pr = exp2_of(s[t][x] * scale + (bias - lse[r]));
-                    if (ragged && j >= n) pr = 0.f;
-                    const float px = pr * dp[t][x];
-                    s[t][x] = pr;
-                    dp[t][x] = px;
-                    xs[r] += px;
+                    for (int x = 0; x < 4; ++x) {
+                        const int r = x >> 1;
+                        const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
+                        float fv[kFeat];
+                        unpack_features(x & 1 ? f[t][r].y : f[t][r].x, fv);
+                        const float bias = w[0] * fv[0] + w[1] * fv[1] + w[2] * fv[2] + w[3] * fv[3];
+                        float pr = exp_of((s[t][x] * p.scale + bias) - lse[r]);
+                        if (ragged && j >= n) pr = 0.f;
+                        if constexpr (kForDelta) {
+                            dp[t][x] *= pr;
+                            s[t][x] = pr;
+                        } else {
+                            dp[t][x] = pr * (dp[t][x] - delta[r]);
 #pragma unroll
-                    for (int c = 0; c < kFeat; ++c) { pf[r][c] += pr * fv[c]; xf[c] += px * fv[c]; }
+                            for (int c = 0; c < kFeat; ++c) y[c] += dp[t][x] * fv[c];
+                        }
+                    }
+                if (b == 0) fetch_features(1);
+                if constexpr (kForDelta) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        sum_px[r] += (dp[0][2 * r] + dp[0][2 * r + 1]) + (dp[1][2 * r] + dp[1][2 * r + 1]);
+                        sum_p[r] += (s[0][2 * r] + s[0][2 * r + 1]) + (s[1][2 * r] + s[1][2 * r + 1]);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < kFeat; ++c) xf[c] += y[c];
+                    uint32_t xt[3][4];
+                    split_block(dp, xt);
+                    add_product<D>(dq, xt, kt, 32 * half + 16 * b, lane);
                 }
-            if (b == 0) fetch_features(1);
-            uint32_t pt[3][4], xt[3][4];
-            split_block(s, pt);
-            split_block(dp, xt);
-#pragma unroll
-            for (int c = 0; c < D / 16; ++c) {
-                uint32_t kb[4];
-                Tile<D>::load_bt(kb, kt, 32 * half + 16 * b, c, lane);
-                two_sums(pk[2 * c], pk[2 * c + 1], pt, kb, xk[2 * c], xk[2 * c + 1], xt, kb);
             }
+            __syncthreads();
         }
-        __syncthreads();
-    }
+    };
+    walk(BoolConst<true>{});
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        xs[r] = quad_sum(xs[r]);
-#pragma unroll
-        for (int c = 0; c < kFeat; ++c) pf[r][c] = quad_sum(pf[r][c]);
+        sum_px[r] = quad_sum(sum_px[r]);
+        sum_p[r] = quad_sum(sum_p[r]);
+        if (t4 == 0) s_sums[half][group][g + 8 * r] = make_float2(sum_px[r], sum_p[r]);
     }
-    float* part = (float*)s_tiles + group * (2 * 16 * D);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int32_t i = i0 + g + 8 * r;
+        const float2 a = s_sums[0][group][g + 8 * r], b = s_sums[1][group][g + 8 * r];
+        delta[r] = a.y + b.y > 0.f ? (a.x + b.x) / (a.y + b.y) : a.x + b.x;      // (rows past the end: 0)
+        if (half == 0 && t4 == 0 && i < n) p.delta[(size_t)h * n + i] = delta[r];
+    }
+    walk(BoolConst<false>{});
+    float* part = (float*)s_tiles + group * (16 * D);
     if (half == 1) {
 #pragma unroll
         for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int at = (g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1);
-                part[at] = xk[c][x];
-                part[16 * D + at] = pk[c][x];
-            }
-        if (t4 == 0) {
+            for (int x = 0; x < 4; ++x) part[(g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1)] = dq[c][x];
+    }
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                s_sums[group][g + 8 * r][kFeat] = xs[r];
+    for (int c = 0; c < kFeat; ++c) {
+        double dw = (double)xf[c];
 #pragma unroll
-                for (int c = 0; c < kFeat; ++c) s_sums[group][g + 8 * r][c] = pf[r][c];
-            }
-        }
+        for (int off = 16; off > 0; off >>= 1) dw += __shfl_xor_sync(0xffffffffu, dw, off);
+        if (lane == 0) s_dw[warp][c] = dw;
     }
     __syncthreads();
-    double dw[kFeat];
-#pragma unroll
-    for (int c = 0; c < kFeat; ++c) dw[c] = (double)xf[c];
     if (half == 0) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int32_t i = i0 + g + 8 * r;
-            const float delta = xs[r] + s_sums[group][g + 8 * r][kFeat];
-            if (i < n) {
+            if (i >= n) continue;
 #pragma unroll
-                for (int c = 0; c < D / 8; ++c) {
-                    const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
-                    const float a = (xk[c][2 * r] + x2[0]) - delta * (pk[c][2 * r] + x2[16 * D]);
-                    const float b = (xk[c][2 * r + 1] + x2[1]) - delta * (pk[c][2 * r + 1] + x2[16 * D + 1]);
-                    *(__nv_bfloat162*)(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) = __floats2bfloat162_rn(a * p.scale, b * p.scale);
-                }
-                if (t4 == 0) p.delta[(size_t)h * n + i] = delta;
-            }
-            if (t4 == 0) {
-#pragma unroll
-                for (int c = 0; c < kFeat; ++c) dw[c] -= (double)delta * ((double)pf[r][c] + (double)s_sums[group][g + 8 * r][c]);
+            for (int c = 0; c < D / 8; ++c) {
+                const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
+                *(__nv_bfloat162*)(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) =
+                    __floats2bfloat162_rn((dq[c][2 * r] + x2[0]) * p.scale, (dq[c][2 * r + 1] + x2[1]) * p.scale);
             }
         }
     }
-#pragma unroll
-    for (int c = 0; c < kFeat; ++c) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) dw[c] += __shfl_xor_sync(0xffffffffu, dw[c], off);
-        if (lane == 0) s_dw[warp][c] = dw[c];
-    }
-    __syncthreads();
     if (threadIdx.x < kFeat)
         p.dw_part[((size_t)h * gridDim.x + blockIdx.x) * kFeat + threadIdx.x] =
             s_dw[0][threadIdx.x] + s_dw[1][threadIdx.x] + s_dw[2][threadIdx.x] + s_dw[3][threadIdx.x];
@@ -550,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
     constexpr int kTileBytes = kTile * 2 * D;
     __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];                    // two stages of Q and dO
     __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' K and V
-    __shared__ float2 s_row[2][kTile];                                            // {lse / ln 2, Delta} of the queries
+    __shared__ float2 s_row[2][kTile];                                            // {lse, Delta} of the queries
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
     const int h = blockIdx.y;
     const int32_t n = p.n, j0 = (int32_t)blockIdx.x * kRows + 16 * group;
@@ -565,8 +574,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
     }
     float w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c] * kLog2e;
-    const float scale = p.scale * kLog2e;
+    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
 
     const uint32_t own_k = smem_addr(s_own), own_v = own_k + kRows * 2 * D;
     Tile<D>::template fetch<kRows>(own_k, p.k, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
@@ -586,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
         cp_commit();
         if (threadIdx.x < kTile) {
             const int32_t i = tile * kTile + (int32_t)threadIdx.x;
-            s_row[tile & 1][threadIdx.x] = i < n ? make_float2(p.lse_in[(size_t)h * n + i] * kLog2e, p.delta[(size_t)h * n + i]) : make_float2(INFINITY, 0.f);
+            s_row[tile & 1][threadIdx.x] = i < n ? make_float2(p.lse_in[(size_t)h * n + i], p.delta[(size_t)h * n + i]) : make_float2(INFINITY, 0.f);
         }
     };
     stage(0);
@@ -615,20 +623,15 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     const float2 row = s_row[tile & 1][32 * half + 16 * b + 8 * t + 2 * t4 + (x & 1)];
-                    s[t][x] = exp2_of(s[t][x] * scale + (bias_of(f[t][x], w) - row.x));        // 0 for queries past the end
+                    s[t][x] = exp_of((s[t][x] * p.scale + bias_of(f[t][x], w)) - row.x);        // 0 for queries past the end
                     dp[t][x] = s[t][x] * (dp[t][x] - row.y);
                 }
             if (b == 0) fetch_features(1);
-            uint32_t pt[3][4], st[3][4];
-            split_block(s, pt);
-            split_block(dp, st);
-#pragma unroll
-            for (int c = 0; c < D / 16; ++c) {
-                uint32_t ob[4], qb[4];
-                Tile<D>::load_bt(ob, dt, 32 * half + 16 * b, c, lane);
-                Tile<D>::load_bt(qb, qt, 32 * half + 16 * b, c, lane);
-                two_sums(dv[2 * c], dv[2 * c + 1], pt, ob, dk[2 * c], dk[2 * c + 1], st, qb);
-            }
+            uint32_t terms[3][4];
+            split_block(s, terms);
+            add_product<D>(dv, terms, dt, 32 * half + 16 * b, lane);
+            split_block(dp, terms);
+            add_product<D>(dk, terms, qt, 32 * half + 16 * b, lane);
         }
         __syncthreads();
     }

@@ -66,6 +66,45 @@ def test_features_with_a_large_common_part():
     run_case(500, 2, 64, seed=8, structured=True)
 
 
+@pytest.mark.parametrize("d,shift,structured", [(64, 0.0, False), (32, 0.0, True), (64, 16.0, False), (64, 16.0, True)])
+def test_results_keep_what_fp32_gives(d, shift, structured):
+    """What the three-term operands, the order of the sums and the per-query term are for, on values with a large common part.
+    LSE (8 to 16): two units in its last place.  dW: a dS carries the roundings of its score and of lse (2^-24 of their size, times
+    dS), of its dP and of Delta; they are independent from pair to pair, so their squares add up, but Delta's is the same for a
+    row, so that row's pairs add up first; a factor of 4 for the four MMA steps of a dP and for the sums.  dV and out, which do
+    not cancel: the share of elements that miss the bf16 value nearest to the exact one is the sums' relative error over half
+    a bf16 step, 2^-24 sqrt(n) / 2^-9 = 1.2e-3; P in two bf16 terms alone would miss 2^-17 / 2^-9 = 4e-3 of them."""
+    n, H = 1500, 2
+    t, f, w = make_case(n, H, d, 21, structured=structured)
+    dev = "cuda"
+    q, k, v, do = (bf16_tensor(x, dev) for x in (t.q, t.k, t.v, t.dout))
+    v = (v.float() + shift).bfloat16()
+    batch = gt.Batch(n)
+    feat, wt = torch.from_numpy(f).to(dev), torch.from_numpy(w).to(dev)
+    out, lse = torch.empty_like(q), torch.empty(H, n, device=dev)
+    gt.gt_feature_attn_fwd(q, k, v, feat, wt, batch, out, lse)
+    dq, dk, dv = (torch.empty_like(q) for _ in range(3))
+    dw = torch.empty_like(wt)
+    gt.gt_check(gt.gt_feature_attn_bwd(q, k, v, do, lse, feat, wt, batch, dq, dk, dv, dw))
+    qf, kf, vf, dof = (to_f64(x) for x in (q, k, v, do))
+    ff, wf = f.astype(np.float64), w.astype(np.float64)
+    ro, rl = ofeat.forward_feature(qf, kf, vf, f, wf)
+    _, _, rdv, rdw = ofeat.backward_feature(qf, kf, vf, dof, f, wf)
+    assert np.abs(to_f64(lse) - rl).max() <= 2 * 2.0 ** -20
+    for h in range(H):
+        s = qf[:, h] @ kf[:, h].T / np.sqrt(d) + ff @ wf[h]
+        p = np.exp(s - rl[h][:, None])
+        dp = dof[:, h] @ vf[:, h].T
+        delta = (p * dp).sum(1, keepdims=True)
+        pair = p * ((np.abs(s) + np.abs(rl[h])[:, None]) * np.abs(dp - delta) + np.abs(dp) + np.abs(delta))
+        row = np.abs(delta) * np.einsum("ij,ijc->ic", p, ff)
+        bound = 4 * 2.0 ** -24 * np.sqrt(np.tensordot(pair ** 2, ff ** 2, axes=([0, 1], [0, 1])) + (row ** 2).sum(0))
+        assert (np.abs(to_f64(dw)[h] - rdw[h]) <= bound).all(), np.abs(to_f64(dw)[h] - rdw[h]) / bound
+    for got, exact in ((out, ro), (dv, rdv)):
+        missed = (got.cpu() != torch.from_numpy(exact).bfloat16()).double().mean().item()
+        assert missed <= 1.2e-3, missed
+
+
 def test_packed_batches_and_other_head_dims_are_refused():
     dev = "cuda"
     x = torch.zeros(64, 2, 16, dtype=torch.bfloat16, device=dev)
