@@ -716,8 +716,9 @@ struct PrepareParams {
     float4* dq_acc;            // cleared, unless nullptr (step entry points: the caller's sums)
     double* db_acc;            // cleared: [n_db]
     int32_t n_total, n_graphs, n_heads, n_db;
-    int32_t tiles;             // transpose tiles along a side of the largest graph
-    uint32_t row_blocks;       // thread blocks that work on rows; the others transpose
+    uint32_t row_blocks;       // thread blocks that work on rows
+    uint32_t tile_blocks;      // thread blocks that transpose: tile_cols for every row of tiles of every graph
+    uint32_t tile_cols;        // thread blocks side by side on a row of tiles
     uint32_t last_bucket;
     float sqrt_d;
     CUtensorMap model;
@@ -729,7 +730,8 @@ struct PrepareParams {
 // -Delta with Delta = sum_c dO[t,h,c] O[t,h,c], zeros elsewhere; and the rows of the fp32 dQ accumulator are cleared.  A
 // thread owns a row and adds its products in channel order (a row whose softmax has one key then has dP = Delta to the bit);
 // the rows reach it through shared memory, because 32 lanes that each walk along a row of their own ask the L1 for every line
-// eight times.  The other blocks transpose the SPD matrix.
+// eight times.  The other blocks transpose the SPD matrix, a row of tiles of a graph each or a share of it (tile_cols): a block for
+// every tile of the largest graph, for every graph, can be more blocks than a grid holds.
 // 64 graphs of 512-2 048 nodes, H = 16, d = 64: 197 us in two fills and two kernels before.
 constexpr int kPrepareRows = 128;
 template <int D>
@@ -740,19 +742,27 @@ __global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const __gr
     grid_wait();
     grid_release();
     if (blockIdx.x >= p.row_blocks) {
-        const uint32_t b = blockIdx.x - p.row_blocks, per_graph = (uint32_t)(p.tiles * p.tiles);
-        if (b >= per_graph * (uint32_t)p.n_graphs) {
-            const int32_t w = (int32_t)((b - per_graph * (uint32_t)p.n_graphs) * (kPrepareThreads / 32) + (threadIdx.x >> 5));
+        const uint32_t b = blockIdx.x - p.row_blocks;
+        if (b >= p.tile_blocks) {
+            const int32_t w = (int32_t)((b - p.tile_blocks) * (kPrepareThreads / 32) + (threadIdx.x >> 5));
             if (w < p.n_graphs) write_work_list<kTile>(p.list, p.n_total / kTile + p.n_graphs, p.cu_seqlens, p.n_graphs, w);
             return;
         }
-        const int g = (int)(b / per_graph), r = (int)(b % per_graph);
-        const int32_t n_g = p.cu_seqlens ? p.cu_seqlens[g + 1] - p.cu_seqlens[g] : p.n_total;
-        const int32_t i0 = (r / p.tiles) * 128, j0 = (r % p.tiles) * 128;
-        if (i0 >= n_g || j0 >= n_g) return;
-        if (r == 0 && threadIdx.x == 0 && p.maps != nullptr)
+        const int32_t first = (int32_t)(b % p.tile_cols);
+        int32_t g = 0, row = (int32_t)(b / p.tile_cols), n_g = p.n_total;
+        if (p.cu_seqlens) {
+            g = graph_of_entry<kTile>(p.cu_seqlens, p.n_graphs, row);
+            const int32_t c0 = p.cu_seqlens[g];
+            n_g = p.cu_seqlens[g + 1] - c0;
+            row -= c0 / kTile + g;
+        }
+        if (row * kTile >= n_g) return;
+        if (row == 0 && first == 0 && threadIdx.x == 0 && p.maps != nullptr)
             make_spd_map(p.maps + (size_t)g * kMapBytes, p.model, p.spd_t + p.spd_offsets[g], n_g);
-        transpose_tile(p.spd, p.spd_t, n_g, p.spd_offsets ? p.spd_offsets[g] : 0, i0, j0, p.last_bucket, (uint32_t*)s_rows);
+        for (int32_t col = first; col * kTile < n_g; col += (int32_t)p.tile_cols) {
+            if (col != first) __syncthreads();
+            transpose_tile(p.spd, p.spd_t, n_g, p.spd_offsets ? p.spd_offsets[g] : 0, row * kTile, col * kTile, p.last_bucket, (uint32_t*)s_rows);
+        }
         return;
     }
     const size_t n_rows = (size_t)p.n_total * p.n_heads, row0 = (size_t)blockIdx.x * kPrepareRows;
@@ -826,14 +836,21 @@ __global__ void __launch_bounds__(kPrepareThreads) bwd_prepare_kernel(const __gr
     p.ext[2 * row + 1] = e1;
 }
 
+constexpr uint32_t kMaxTileBlocks = 1u << 18;
+
 gt_status launch_prepare(PrepareParams p, int32_t head_dim, int32_t max_seqlen, cudaStream_t s)
 {
     const size_t rows = (size_t)p.n_total * p.n_heads, per_block = kPrepareRows;
-    p.tiles = (max_seqlen + 127) / 128;
     p.row_blocks = (uint32_t)((rows + per_block - 1) / per_block);
+    // A block per tile while that is no more than kMaxTileBlocks (65 536 nodes), beyond that as many blocks per row of tiles as give them.
+    const uint32_t tiles = (uint32_t)((max_seqlen + kTile - 1) / kTile);
+    const uint32_t rows_of_tiles = p.cu_seqlens ? (uint32_t)(p.n_total / kTile + p.n_graphs) : tiles;
+    const uint32_t fit = kMaxTileBlocks / rows_of_tiles;
+    p.tile_cols = fit < 1 ? 1 : (fit < tiles ? fit : tiles);
+    p.tile_blocks = rows_of_tiles * p.tile_cols;
     p.sqrt_d = sqrtf((float)head_dim);
     const uint64_t list_blocks = p.list != nullptr ? (p.n_graphs + kPrepareThreads / 32 - 1) / (kPrepareThreads / 32) : 0;
-    const dim3 grid((unsigned)(p.row_blocks + (uint64_t)p.tiles * p.tiles * p.n_graphs + list_blocks));
+    const dim3 grid((unsigned)(p.row_blocks + p.tile_blocks + list_blocks));
     return head_dim == 64 ? launch_overlapped(bwd_prepare_kernel<64>, grid, kPrepareThreads, 0, s, p)
                           : launch_overlapped(bwd_prepare_kernel<32>, grid, kPrepareThreads, 0, s, p);
 }

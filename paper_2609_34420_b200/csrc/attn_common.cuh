@@ -83,6 +83,22 @@ __device__ __forceinline__ void write_work_list(int4* list, int32_t entries, con
         list[i] = i < first + blocks ? make_int4(g, i - first, c0, n) : make_int4(-1, 0, 0, 0);
 }
 
+// The graph that entry `entry` belongs to in the batch's order, where graph g's entries begin at cu_seqlens[g] / kRows + g; by whole warps.
+template <int kRows>
+__device__ __forceinline__ int32_t graph_of_entry(const int32_t* __restrict__ cu_seqlens, int32_t n_graphs, int32_t entry)
+{
+    const int lane = threadIdx.x & 31;
+    int32_t lo = 0, n = n_graphs;                          // it is one of [lo, lo + n)
+    while (n > 1) {
+        const int32_t step = (n + 31) / 32, x = lane * step;
+        const bool begins = x < n && cu_seqlens[lo + x] / kRows + lo + x <= entry;
+        const int32_t last = __popc(__ballot_sync(0xffffffffu, begins)) - 1;       // (lane 0's begins)
+        lo += last * step;
+        n = min(step, n - last * step);
+    }
+    return lo;
+}
+
 // Clusters of `split` blocks that the device holds at a time (a cluster's blocks lie in one group of SMs), -1: none.
 constexpr int kMaxSplit = 4;
 struct ClusterFit { std::atomic<int32_t> n[kMaxSplit + 1] = {}; };       // by size; 0: not asked yet

@@ -106,3 +106,42 @@ def test_forward_with_shared_query_tiles(sizes_, heads, d, D, spread):
     out_p, lse_p, out32 = case.forward_ex()
     ro, _ = oracle_forward(case)
     assert rel_l2(to_f64(out32), ro) <= 1e-4 and (lse_p - lse).abs().max().item() <= LSE_MAX_ABS
+
+
+def test_backward_of_a_large_graph_among_many_of_one_node():
+    """32 769 graphs whose largest has 256 x 256 tiles to transpose: a block for every tile of the largest graph and every graph
+    would be more than a grid holds.  The large graph's gradients are those of the graph by itself (sums of dQ in another order,
+    results rounded to bf16); a single node passes dout on to dv and has no other gradient."""
+    n, G, before, d, D, dev = 32768, 32769, 20000, 32, 6, "cuda"
+    lengths = np.ones(G, np.int64)
+    lengths[before] = n
+    cu = np.concatenate([[0], np.cumsum(lengths)])
+    sizes_ = lengths * ((lengths + 15) // 16 * 16)
+    off = np.concatenate([[0], np.cumsum(sizes_)])
+    T = int(cu[-1])
+    gen = torch.Generator(device=dev).manual_seed(5)
+    q, k, v, do = (torch.randn(T, 1, d, device=dev, generator=gen).bfloat16() for _ in range(4))
+    spd = torch.randint(0, D + 2, (int(off[-1]),), device=dev, generator=gen, dtype=torch.uint8)
+    bias = torch.randn(1, D + 2, device=dev, generator=gen)
+
+    def run(batch, q, k, v, do, spd):
+        out, lse = torch.empty_like(q), torch.empty(1, q.shape[0], device=dev)
+        gt.gt_check(gt.gt_biased_attn_fwd(q, k, v, spd, bias, batch, D, out, lse))
+        grads = [torch.full_like(q, float("nan")) for _ in range(3)] + [torch.full_like(bias, float("nan"))]
+        gt.gt_check(gt.gt_biased_attn_bwd(q, k, v, out, do, lse, spd, bias, batch, D, *grads))
+        return [out] + grads
+
+    packed = gt.Batch(T, G, n, torch.tensor(cu, dtype=torch.int32, device=dev), torch.tensor(off[:-1], dtype=torch.int64, device=dev))
+    big = slice(before, before + n)
+    single = torch.cat([torch.arange(before), torch.arange(before + n, T)]).to(dev)
+    _, dq, dk, dv, _ = run(packed, q, k, v, do, spd)
+    # P of a single key is 1 up to its rounding to bf16 (2^-9), and so are out and dP - Delta relative to v and dP
+    assert ((dv[single] - do[single]).abs() <= do[single].abs() * 2.0 ** -7).all()
+    assert max(x[single].float().abs().max().item() for x in (dq, dk)) <= 2.0 ** -8 * 4 * d
+    do[single] = 0                                         # (these residues would add up in dbias)
+    out, dq, dk, dv, db = run(packed, q, k, v, do, spd)
+    alone = run(gt.Batch(n), *(x[big].contiguous() for x in (q, k, v, do)), spd[int(off[before]):int(off[before + 1])].clone())
+    for got, want in zip((out, dq, dk, dv), alone):
+        assert rel_l2(to_f64(got[big]), to_f64(want)) <= 5e-3
+    assert rel_l2(to_f64(db), to_f64(alone[4])) <= 1e-3
+    assert all(not x[single].any() for x in (dq, dk, dv))
