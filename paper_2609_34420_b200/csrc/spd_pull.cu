@@ -13,7 +13,7 @@
 // completed by in-place passes over the rows, sped up by closing the block's targets under each other: target t's own row
 // says which targets follow from t, so after a transitive closure of those kT rows every vertex inherits the closed row of
 // each target it reaches.  That only adds what is reachable, and the passes run until one changes nothing, so it is exact
-// for any directed graph; on an undirected graph one or two passes do what took a level per hop before.
+// for any directed graph.  What is still open after kPlainRounds of them (graphs hundreds of edges across) is left to finish_far.
 //
 // What bounds it: the shared-memory pipe in the level passes (a gathered row costs the bank conflicts of 32 random rows:
 // 3.5 wavefronts for 32 lanes of 4 bytes, 6.2 of 8, 10.6 of 16: wider rows cost less per target), and the stores of the
@@ -29,6 +29,9 @@ constexpr uint16_t kListed = 0x8000;   // vertices are numbered below this
 // Vertices with more out-edges than this are pulled by a whole warp: some 150 instructions each, where 32 of them side by side
 // in one group cost 100 and 8 per pair of edges (a limit of 32: 11.4k clocks a level at 4 096 nodes, issue bound).
 constexpr int kHubDegree = 64;
+
+// Rounds of the search for what is farther than max_dist, after which finish_far takes over, and its rounds before it asks for the components.
+constexpr int kPlainRounds = 40, kFarComponents = 8;
 
 struct PullParams {
     const int32_t* row_ptr;
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
         open = pass(cur, nxt, level);
         uint8_t* t = cur; cur = nxt; nxt = t;
     }
-    while (open) {
+    for (int round = 0; round < kPlainRounds && open; ++round) {
         if (warp == 0) close_targets<kT>(cur, s_tpos, nt, full, lane);
         __syncthreads();
         // every vertex inherits the rows of the targets it reaches; a closed row covers all targets inside it
@@ -477,6 +480,13 @@ __global__ void __launch_bounds__(1024, 1) spd_pull_kernel(PullParams p)
 #pragma unroll
         for (int b = 0; b < 8; ++b) c[b] |= (far & (0u - ((far_code >> b) & 1u))) | (none & (0u - ((none_code >> b) & 1u)));
         emit_word(c, p.n_planes, row, col, nt, cols);
+    }
+    if (open) {
+        __shared__ FarState s_far;
+        __syncthreads();
+        if (threadIdx.x == 0) s_far = {out, ld, grp, p.col_idx, nullptr, nullptr, node0, n, t0, nt, none_code, kFarComponents};
+        __syncthreads();
+        finish_far<kT>(pull_smem, s_far);
     }
 }
 

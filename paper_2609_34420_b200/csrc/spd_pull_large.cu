@@ -28,6 +28,8 @@ constexpr int kTargets = 32;
 constexpr int32_t kLargeMaxNodes = 18944;
 constexpr int kCachedHubs = 400;           // hubs whose numbers and lists' places are kept in shared memory
 
+constexpr int kPlainRounds = 3, kFarComponents = 1;         // as in spd_pull.cu; a round takes 6 to 25 us here
+
 struct LargeParams {
     const int32_t* row_ptr;
     const int32_t* col_idx;
@@ -36,7 +38,8 @@ struct LargeParams {
     uint32_t* hub_at;         // first word of a hub's list, and one past the last hub's
     uint32_t* list;
     uint32_t* planes;         // [grid][n_planes][n_pad]
-    uint32_t* counts;         // [0] hubs
+    uint32_t* counts;         // [0] hubs, [1] `component` is there
+    uint16_t* component;      // [n] root of a vertex' component (finish_far), once a block has needed it
     uint8_t* spd;
     int32_t n;
     int32_t n_pad;
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(1024, 1) spd_large_order_kernel(LargeParams p)
             if (h + lane < n_hubs) p.hub_at[h + lane] = (uint32_t)(at + x - words);
             at += __shfl_sync(0xffffffffu, x, 31);
         }
-        if (lane == 0) { p.hub_at[n_hubs] = (uint32_t)at; p.counts[0] = (uint32_t)n_hubs; }
+        if (lane == 0) { p.hub_at[n_hubs] = (uint32_t)at; p.counts[0] = (uint32_t)n_hubs; p.counts[1] = 0u; }
         for (int g0 = 0; n_hubs + 32 * g0 < n; g0 += 32) {
             const int i = n_hubs + 32 * (g0 + lane);
             const int pairs = i < n ? (sorted[i] + 1) / 2 : 0, x = warp_scan(32 * pairs, lane);
@@ -153,7 +156,7 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
 {
     using R = Rows<kTargets>;
     extern __shared__ __align__(16) uint8_t large_smem[];
-    __shared__ uint32_t s_live[3], s_hub_at[kCachedHubs + 1];
+    __shared__ uint32_t s_live[3], s_hub_at[kCachedHubs + 1], s_unfinished[(kLargeMaxNodes / kTargets + 31) / 32];      // a bit per turn of the block
     __shared__ uint16_t s_tpos[kTargets], s_hub[kCachedHubs];
     grid_wait();
     grid_release();
@@ -169,6 +172,7 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
     const int64_t ld = (int64_t)((n + 15) & ~15);
     const uint32_t far_code = (uint32_t)p.max_dist, none_code = (uint32_t)p.max_dist + 1u;
     if (threadIdx.x < 3) s_live[threadIdx.x] = 0u;
+    if (threadIdx.x < sizeof(s_unfinished) / 4) s_unfinished[threadIdx.x] = 0u;
     for (int h = threadIdx.x; h <= min(n_hubs, kCachedHubs); h += blockDim.x) {
         s_hub_at[h] = p.hub_at[h];
         if (h < min(n_hubs, kCachedHubs)) s_hub[h] = order[h];
@@ -314,7 +318,7 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
             uint32_t* t = cur; cur = nxt; nxt = t;
             last = level;
         }
-        while (open) {
+        for (int round = 0; round < kPlainRounds && open; ++round) {
             if (warp == 0) close_targets<kTargets>((uint8_t*)cur, s_tpos, nt, full, lane);
             __syncthreads();
             for (int v = threadIdx.x; v < n; v += blockDim.x)
@@ -322,6 +326,7 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
             __syncthreads();
             open = pass(std::false_type{}, cur, cur, 0);
         }
+        if (open && threadIdx.x == 0) s_unfinished[t0 / kTargets / (int)gridDim.x / 32] |= 1u << (t0 / kTargets / (int)gridDim.x % 32);
 
         __threadfence();                                   // the reductions on the planes, before they are read
         __syncthreads();
@@ -340,6 +345,17 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
             for (int b = 0; b < 8; ++b) c[b] |= (far & (0u - ((far_code >> b) & 1u))) | (none & (0u - ((none_code >> b) & 1u)));
             emit_word(c, p.n_planes, out + (int64_t)v * ld, 0, nt, cols);
         }
+    }
+    __syncthreads();
+    for (int turns = 0, t0 = (int)blockIdx.x * kTargets; t0 < p.n; ++turns, t0 += (int)gridDim.x * kTargets) {
+        if (!((s_unfinished[turns / 32] >> (turns % 32)) & 1u)) continue;
+        __shared__ FarState s_far;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            s_far = {p.spd + t0, (int64_t)((p.n + 15) & ~15), p.row_ptr, p.col_idx, &p.counts[1], p.component, 0, p.n, t0, min(kTargets, p.n - t0),
+                     (uint32_t)p.max_dist + 1u, kFarComponents};
+        __syncthreads();
+        finish_far<kTargets>(large_smem, s_far);
     }
 }
 
@@ -364,6 +380,7 @@ PullLargePlan spd_pull_large_plan(const gt_batch* b, int64_t nnz, int32_t max_di
     pl.info_off = off; off += align_up(4 * (n / 32 + 2), 256);
     pl.hub_off = off; off += align_up(4 * ((size_t)nnz / (kLargeHubDegree + 1) + 2), 256);
     pl.list_off = off; off += align_up(2 * ((size_t)nnz + n + 32 * (kLargeHubDegree + 2)) + 256, 256);
+    pl.component_off = off; off += align_up(2 * n, 256);
     pl.plane_off = off; off += 4 * (size_t)pl.blocks * (size_t)pull_planes(max_dist) * (size_t)pl.n_pad;
     pl.total_bytes = off;
     return pl;
@@ -382,6 +399,7 @@ gt_status spd_pull_large_launch(const PullLargePlan& pl, const int32_t* row_ptr,
     p.list = (uint32_t*)(ws + pl.list_off);
     p.planes = (uint32_t*)(ws + pl.plane_off);
     p.counts = (uint32_t*)ws + 4;
+    p.component = (uint16_t*)(ws + pl.component_off);
     p.spd = spd;
     p.n = batch->n_total;
     p.n_pad = pl.n_pad;

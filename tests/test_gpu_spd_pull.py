@@ -58,3 +58,51 @@ def test_one_deep_undirected_graph_with_lists_in_the_workspace():
 def test_one_graph_beyond_the_pull(n, m, D):
     """The bit matrices at their smallest: more levels than level bits, a clip above them, rows that close early, isolated nodes."""
     one(directed(n, m, n, hub_edges=5000, hubs=2), D)
+
+
+def shuffled(csr, seed):
+    rp, ci = csr
+    n = len(rp) - 1
+    to = np.random.Generator(np.random.PCG64(seed)).permutation(n)
+    return wl.csr_from_edges(n, to[np.repeat(np.arange(n), np.diff(rp))], to[ci], symmetric=False)
+
+
+def long_ways(n, kind, seed):
+    """Graphs hundreds to thousands of edges across."""
+    i = np.arange(n)
+    if kind == "ring":
+        return wl.csr_from_edges(n, i, (i + 1) % n, symmetric=True)
+    if kind == "directed ring":
+        return shuffled(wl.csr_from_edges(n, i, (i + 1) % n, symmetric=False), seed)
+    if kind == "one way":                    # a path with some of its reverse edges missing: components of edges both ways, in a row
+        both = wl.csr_from_edges(n, np.concatenate([i[:-1], i[1:]]), np.concatenate([i[1:], i[:-1]]), symmetric=False)
+        src, dst = np.repeat(i, np.diff(both[0])), both[1]
+        keep = (src < dst) | (src % 37 != 0)
+        return shuffled(wl.csr_from_edges(n, src[keep], dst[keep], symmetric=False), seed)
+    if kind == "two hubs":                   # a path whose middle part hangs on two vertices with more edges than are searched for a reverse
+        m, leaves = n // 2, np.arange(100)
+        src = np.concatenate([i[:m - 1], np.full(100, m // 2), np.full(100, m // 2 + 1)])
+        dst = np.concatenate([i[1:m], m + leaves, m + 100 + leaves])
+        return shuffled(wl.csr_from_edges(n, src, dst, symmetric=True), seed)
+    side = int(n ** 0.5)                     # a grid whose edges lead right and down
+    v = np.arange(side * side).reshape(side, side)
+    return shuffled(wl.csr_from_edges(n, np.concatenate([v[:, :-1].ravel(), v[:-1].ravel()]), np.concatenate([v[:, 1:].ravel(), v[1:].ravel()]),
+                                      symmetric=False), seed)
+
+
+KINDS = ("ring", "directed ring", "one way", "two hubs", "grid")
+
+
+@pytest.mark.parametrize("total,D", [(9000, 1), (25000, 6), (48000, 40)])       # rows of 32, 64 and 128 targets
+def test_long_ways_in_a_batch(total, D):
+    graphs, at = [], 0
+    while sum(len(g[0]) - 1 for g in graphs) < total:
+        graphs.append(long_ways(700 + 61 * at % 450, KINDS[at % len(KINDS)], at))
+        at += 1
+    check(wl.Workload("far", wl.pack_graphs(graphs), 1, 32, D))
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n", [3300, 6100, 14300])       # edge list in shared memory; in the workspace, two blocks per SM and one
+def test_long_ways_in_one_graph(n, kind):
+    one(long_ways(n, kind, n), 5)
