@@ -18,7 +18,8 @@
  *    buffer; the library allocates and frees no device memory.  Scratch comes from a
  *    caller-provided workspace whose size is obtained from the matching *_workspace()
  *    query (host function, no GPU work).  Workspace and all tensor base pointers must be
- *    16-byte aligned.
+ *    16-byte aligned.  (gt_feature_attn_* also take bf16 tensors, gt_feature_encode `codes` and gt_spd_build `spd_out` and
+ *    blocks at any address that their elements allow, more slowly; gt_spd_build not where it uses bit matrices.)
  *  - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls only
  *    enqueue work and return; they never synchronise.  Errors detected on the host are
  *    returned immediately.  Errors detected on the device (a bounded wait that ran out)

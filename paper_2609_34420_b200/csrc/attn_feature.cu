@@ -26,6 +26,8 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <initializer_list>
+
 #include "attn_common.cuh"
 
 namespace gt {
@@ -87,8 +89,8 @@ struct Tile {
         const int x = D == 64 ? (row & 7) : ((row >> 1) & 3);
         return base + (uint32_t)(row * kRowBytes + ((chunk ^ x) * 16));
     }
-    // rows [r0, r0 + kCount) of head h of a [n, H, D] tensor; rows past n are zero
-    template <int kCount>
+    // rows [r0, r0 + kCount) of head h of a [n, H, D] tensor; rows past n are zero.  kAligned: the tensor begins at a multiple of 16 bytes
+    template <int kCount, bool kAligned>
     static __device__ __forceinline__ void fetch(uint32_t base, const __nv_bfloat16* __restrict__ x, int32_t n, int32_t n_heads, int32_t h, int32_t r0)
     {
         constexpr int kChunks = D / 8;
@@ -96,7 +98,16 @@ struct Tile {
         for (int e = 0; e < kCount * kChunks / kThreads; ++e) {
             const int i = e * kThreads + (int)threadIdx.x, r = i / kChunks, c = i % kChunks;
             const bool ok = r0 + r < n;
-            cp16(at(base, r, c), x + ((size_t)(ok ? r0 + r : 0) * n_heads + h) * D + c * 8, ok);
+            const __nv_bfloat16* src = x + ((size_t)(ok ? r0 + r : 0) * n_heads + h) * D + c * 8;
+            if constexpr (kAligned) {
+                cp16(at(base, r, c), src, ok);
+            } else {
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    w[k] = ok ? (uint32_t)((const uint16_t*)src)[2 * k] | (uint32_t)((const uint16_t*)src)[2 * k + 1] << 16 : 0u;
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at(base, r, c)), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+            }
         }
     }
     // A fragments (16 rows from `row`, all of D)
@@ -209,6 +220,18 @@ __device__ __forceinline__ void unpack_features(uint32_t f4, float (&f)[kFeat])
 
 template <bool B> struct BoolConst { static constexpr bool value = B; };
 
+// Two neighbouring results.
+template <bool kAligned>
+__device__ __forceinline__ void store_pair(__nv_bfloat16* to, float a, float b)
+{
+    if constexpr (kAligned) {
+        *(__nv_bfloat162*)to = __floats2bfloat162_rn(a, b);
+    } else {
+        to[0] = __float2bfloat16_rn(a);
+        to[1] = __float2bfloat16_rn(b);
+    }
+}
+
 struct FeatureArgs {
     const __nv_bfloat16 *q, *k, *v, *dout;
     const uint32_t* feat;         // the four features of a pair as one word, [n][n]
@@ -267,7 +290,7 @@ __device__ __forceinline__ float quad_max(float x)
 // ---------------------------------------------------------------------------------------------------
 // Forward: a warp owns 16 query rows and one half of the keys.
 // ---------------------------------------------------------------------------------------------------
-template <int D>
+template <int D, bool kAligned>
 __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 {
     grid_wait();
@@ -285,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
     for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
 
     uint32_t qa[D / 16][4];
-    Tile<D>::template fetch<kRows>(base, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows, kAligned>(base, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     cp_commit();
     cp_wait<0>();
     __syncthreads();
@@ -300,8 +323,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
-        Tile<D>::template fetch<kTile>(at, p.k, n, p.n_heads, h, tile * kTile);
-        Tile<D>::template fetch<kTile>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile, kAligned>(at, p.k, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile, kAligned>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
         cp_commit();
     };
     stage(0);
@@ -384,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
                 for (int c = 0; c < D / 8; ++c) {
                     const float* o2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
                     const float x = (o[c][2 * r] * a + o2[0] * b) * inv, y = (o[c][2 * r + 1] * a + o2[1] * b) * inv;
-                    *(__nv_bfloat162*)(p.out + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) = __floats2bfloat162_rn(x, y);
+                    store_pair<kAligned>(p.out + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4, x, y);
                 }
                 if (t4 == 0) p.lse[(size_t)h * n + i] = mm + logf(ll);
             }
@@ -398,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 // dW), then dS.  (One walk that takes Delta_i sum_j P_ij K_j from sum_j P_ij dP_ij K_j at its end needs one MMA more per 16 keys
 // and channels and loses what the two sums have in common.)
 // ---------------------------------------------------------------------------------------------------
-template <int D>
+template <int D, bool kAligned>
 __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs p)
 {
     grid_wait();
@@ -419,8 +442,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
     for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
 
     const uint32_t own_q = smem_addr(s_own), own_d = own_q + kRows * 2 * D;
-    Tile<D>::template fetch<kRows>(own_q, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
-    Tile<D>::template fetch<kRows>(own_d, p.dout, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows, kAligned>(own_q, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows, kAligned>(own_d, p.dout, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     cp_commit();
 
     float lse[2], delta[2] = {0.f, 0.f}, sum_px[2] = {0.f, 0.f}, sum_p[2] = {0.f, 0.f};
@@ -436,8 +459,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
-        Tile<D>::template fetch<kTile>(at, p.k, n, p.n_heads, h, tile * kTile);
-        Tile<D>::template fetch<kTile>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile, kAligned>(at, p.k, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile, kAligned>(at + kTileBytes, p.v, n, p.n_heads, h, tile * kTile);
         cp_commit();
     };
     auto walk = [&](auto for_delta) {
@@ -538,8 +561,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
 #pragma unroll
             for (int c = 0; c < D / 8; ++c) {
                 const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
-                *(__nv_bfloat162*)(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4) =
-                    __floats2bfloat162_rn((dq[c][2 * r] + x2[0]) * p.scale, (dq[c][2 * r + 1] + x2[1]) * p.scale);
+                store_pair<kAligned>(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4, (dq[c][2 * r] + x2[0]) * p.scale, (dq[c][2 * r + 1] + x2[1]) * p.scale);
             }
         }
     }
@@ -551,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
 // ---------------------------------------------------------------------------------------------------
 // Backward, key side: dK and dV (and, by the first block of a head, the sum of the row blocks' shares of dW).
 // ---------------------------------------------------------------------------------------------------
-template <int D>
+template <int D, bool kAligned>
 __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs p)
 {
     grid_wait();
@@ -577,8 +599,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
     for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
 
     const uint32_t own_k = smem_addr(s_own), own_v = own_k + kRows * 2 * D;
-    Tile<D>::template fetch<kRows>(own_k, p.k, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
-    Tile<D>::template fetch<kRows>(own_v, p.v, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows, kAligned>(own_k, p.k, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
+    Tile<D>::template fetch<kRows, kAligned>(own_v, p.v, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     cp_commit();
 
     float dk[D / 8][4], dv[D / 8][4];
@@ -589,8 +611,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
-        Tile<D>::template fetch<kTile>(at, p.q, n, p.n_heads, h, tile * kTile);
-        Tile<D>::template fetch<kTile>(at + kTileBytes, p.dout, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile, kAligned>(at, p.q, n, p.n_heads, h, tile * kTile);
+        Tile<D>::template fetch<kTile, kAligned>(at + kTileBytes, p.dout, n, p.n_heads, h, tile * kTile);
         cp_commit();
         if (threadIdx.x < kTile) {
             const int32_t i = tile * kTile + (int32_t)threadIdx.x;
@@ -656,8 +678,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
             for (int c = 0; c < D / 8; ++c) {
                 const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
                 const size_t at = ((size_t)j * p.n_heads + h) * D + 8 * c + 2 * t4;
-                *(__nv_bfloat162*)(p.dk + at) = __floats2bfloat162_rn((dk[c][2 * r] + x2[0]) * p.scale, (dk[c][2 * r + 1] + x2[1]) * p.scale);
-                *(__nv_bfloat162*)(p.dv + at) = __floats2bfloat162_rn(dv[c][2 * r] + x2[16 * D], dv[c][2 * r + 1] + x2[16 * D + 1]);
+                store_pair<kAligned>(p.dk + at, (dk[c][2 * r] + x2[0]) * p.scale, (dk[c][2 * r + 1] + x2[1]) * p.scale);
+                store_pair<kAligned>(p.dv + at, dv[c][2 * r] + x2[16 * D], dv[c][2 * r + 1] + x2[16 * D + 1]);
             }
         }
     }
@@ -672,6 +694,19 @@ gt_status check_feature_common(const gt_batch* batch, int32_t n_heads, int32_t h
     if (batch->n_graphs != 1 || n_heads > 65535) return GT_ERR_UNSUPPORTED;
     return GT_OK;
 }
+
+// What the pointers have in common: 16: vectors and bf16 pairs; 2: element by element; 1: not a bf16 tensor.
+unsigned alignment(std::initializer_list<const void*> tensors)
+{
+    uintptr_t bits = 16;
+    for (const void* t : tensors) bits |= reinterpret_cast<uintptr_t>(t);
+    return (bits & 15u) == 0 ? 16u : ((bits & 1u) == 0 ? 2u : 1u);
+}
+
+// launches kernel<head_dim, aligned>
+#define FEATURE_LAUNCH(kernel, grid, s, p)                                                                                            \
+    (head_dim == 64 ? launch_overlapped(aligned ? kernel<64, true> : kernel<64, false>, grid, kThreads, 0, s, p)                     \
+                    : launch_overlapped(aligned ? kernel<32, true> : kernel<32, false>, grid, kThreads, 0, s, p))
 
 size_t dw_part_bytes(int32_t n, int32_t n_heads)
 {
@@ -690,6 +725,9 @@ extern "C" gt_status gt_feature_attn_fwd(const void* q, const void* k, const voi
     if (st != GT_OK) return st;
     if (!q || !k || !v || !features || !weights || !out || !lse) return GT_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(features) & 3u) != 0) return GT_ERR_INVALID_ARG;
+    const unsigned bytes = alignment({q, k, v, out});
+    if (bytes < 2) return GT_ERR_INVALID_ARG;
+    const bool aligned = bytes == 16;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
     FeatureArgs p{};
     p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v;
@@ -701,7 +739,7 @@ extern "C" gt_status gt_feature_attn_fwd(const void* q, const void* k, const voi
     p.n_heads = n_heads;
     p.scale = 1.0f / sqrtf((float)head_dim);
     const dim3 grid((unsigned)((p.n + kRows - 1) / kRows), (unsigned)n_heads);
-    return launch_overlapped(head_dim == 64 ? feature_fwd_kernel<64> : feature_fwd_kernel<32>, grid, kThreads, 0, (cudaStream_t)stream, p);
+    return FEATURE_LAUNCH(feature_fwd_kernel, grid, (cudaStream_t)stream, p);
 }
 
 extern "C" size_t gt_feature_attn_bwd_workspace(const gt_batch* batch, int32_t n_heads)
@@ -721,6 +759,9 @@ extern "C" gt_status gt_feature_attn_bwd(const void* q, const void* k, const voi
     if (st != GT_OK) return st;
     if (!q || !k || !v || !dout || !lse || !features || !weights || !dq || !dk || !dv || !dweights) return GT_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(features) & 3u) != 0) return GT_ERR_INVALID_ARG;
+    const unsigned bytes = alignment({q, k, v, dout, dq, dk, dv});
+    if (bytes < 2) return GT_ERR_INVALID_ARG;
+    const bool aligned = bytes == 16;
     if (workspace == nullptr || workspace_bytes < gt_feature_attn_bwd_workspace(batch, n_heads) || misaligned16(workspace)) return GT_ERR_WORKSPACE;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
     uint8_t* ws = (uint8_t*)workspace;
@@ -738,7 +779,7 @@ extern "C" gt_status gt_feature_attn_bwd(const void* q, const void* k, const voi
     p.scale = 1.0f / sqrtf((float)head_dim);
     const dim3 grid((unsigned)((p.n + kRows - 1) / kRows), (unsigned)n_heads);
     cudaStream_t s = (cudaStream_t)stream;
-    st = launch_overlapped(head_dim == 64 ? feature_bwd_q_kernel<64> : feature_bwd_q_kernel<32>, grid, kThreads, 0, s, p);
+    st = FEATURE_LAUNCH(feature_bwd_q_kernel, grid, s, p);
     if (st != GT_OK) return st;
-    return launch_overlapped(head_dim == 64 ? feature_bwd_kv_kernel<64> : feature_bwd_kv_kernel<32>, grid, kThreads, 0, s, p);
+    return FEATURE_LAUNCH(feature_bwd_kv_kernel, grid, s, p);
 }

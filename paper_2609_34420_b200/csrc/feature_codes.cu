@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(512) feature_encode_kernel(const uint32_t* __r
     const uint32_t segs = (uint32_t)(ld + 511) / 512;
     const uint64_t items = (uint64_t)n * segs;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+    const bool words = (reinterpret_cast<uintptr_t>(codes) & 3) == 0;
     const bool aligned = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(f) & 15) == 0;
     for (uint64_t it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += warps) {
         const int32_t i = (int32_t)(it / segs), j0 = (int32_t)(it % segs) * 512 + 4 * lane;
@@ -191,7 +192,10 @@ __global__ void __launch_bounds__(512) feature_encode_kernel(const uint32_t* __r
                 if (j + 1 < n) out = (out & ~0xff00u) | code_of(v[k].y) << 8;
                 if (j + 2 < n) out = (out & ~0xff0000u) | code_of(v[k].z) << 16;
             }
-            *(uint32_t*)(codes + (size_t)i * ld + j) = out;
+            uint8_t* to = codes + (size_t)i * ld + j;
+            if (words) *(uint32_t*)to = out;
+            else
+                for (int b = 0; b < 4; ++b) to[b] = (uint8_t)(out >> (8 * b));
         }
     }
 }

@@ -1050,6 +1050,7 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
                                batch->n_graphs > 1 ? spd_offsets : nullptr, batch, max_dist, spd_out, s);
     if (pl.large.fits && !(pl.dense && g_barrier_overcount))
         return spd_pull_large_launch(pl.large, row_ptr, col_idx, nnz, batch, max_dist, spd_out, workspace, s);
+    if (pl.dense && misaligned16(spd_out)) return GT_ERR_INVALID_ARG;      // (it reads and writes 16 bytes at a time; the others take any address)
     uint8_t* ws = (uint8_t*)workspace;
     SpdParams p{};
     p.row_ptr = row_ptr;

@@ -374,6 +374,18 @@ __device__ __forceinline__ void store_row_piece(uint8_t* at, const uint32_t (&o)
         if (room > 16) *(uint4*)(at + 16) = make_uint4(o[4], o[5], o[6], o[7]);
     }
 }
+// The same in a matrix that begins anywhere (gt_spd_validate takes one).  Unrolled: an index into o would put it in local memory, which
+// slows all of a kernel down by 8 %.
+__device__ __forceinline__ void store_row_piece_anywhere(uint8_t* at, const uint32_t (&o)[8], int room)
+{
+    if (((uintptr_t)at & 15u) == 0) {
+        store_row_piece(at, o, room);
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+        if (j < 16 || room > 16) at[j] = (uint8_t)(o[j / 4] >> (8 * (j % 4)));
+}
 
 struct FarState {
     uint8_t* out;                 // column t0 of row 0
@@ -409,6 +421,16 @@ __device__ __forceinline__ void finish_far(uint8_t* smem, const FarState& p)
     auto bytes_of = [&](int at, uint32_t (&o)[8]) {
         const uint8_t* piece = p.out + (int64_t)(at / W) * p.ld + 32 * (at % W);
         const bool first = 32 * (at % W) < p.nt, second = 32 * (at % W) + 16 < p.nt;
+        if (((uintptr_t)piece & 15u) != 0) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                o[j] = 0u;
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (j < 4 ? first : second) o[j] |= (uint32_t)piece[4 * j + b] << (8 * b);
+            }
+            return;
+        }
         const uint4 a = first ? *(const uint4*)piece : make_uint4(0u, 0u, 0u, 0u), b = second ? *(const uint4*)(piece + 16) : make_uint4(0u, 0u, 0u, 0u);
         o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
         o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
@@ -480,7 +502,7 @@ __device__ __forceinline__ void finish_far(uint8_t* smem, const FarState& p)
             o[b] -= far;
             any |= far;
         }
-        if (any) store_row_piece(p.out + (int64_t)(at / W) * p.ld + 32 * (at % W), o, (int)min(p.ld - p.t0 - 32 * (at % W), (int64_t)32));
+        if (any) store_row_piece_anywhere(p.out + (int64_t)(at / W) * p.ld + 32 * (at % W), o, (int)min(p.ld - p.t0 - 32 * (at % W), (int64_t)32));
     }
     __syncthreads();
 }
@@ -499,7 +521,7 @@ __device__ __forceinline__ void emit_word(const uint32_t (&c)[8], int n_planes, 
             if (past > 0) o[j] |= past >= 4 ? 0xffffffffu : 0xffffffffu << (8 * (4 - past));
         }
     }
-    store_row_piece(row, o, cols - col);
+    store_row_piece_anywhere(row, o, cols - col);
 }
 
 }  // namespace gt

@@ -79,3 +79,70 @@ def test_argument_errors_are_codes_not_launches():
                               workspace=torch.zeros(512, dtype=torch.uint8, device="cuda"))
     assert e.value.status == 3                              # GT_ERR_WORKSPACE
     torch.cuda.synchronize()
+
+
+def shifted(t, by):
+    """The same tensor, `by` elements behind an aligned address."""
+    store = torch.zeros(t.numel() + by, dtype=t.dtype, device=t.device)
+    view = store[by:].view(t.shape)
+    view.copy_(t)
+    return view
+
+
+@pytest.mark.parametrize("d", [32, 64])
+@pytest.mark.parametrize("by", [1, 2])
+def test_feature_attention_takes_tensors_at_any_element(d, by):
+    n, H, dev = 150, 2, "cuda"
+    gen = torch.Generator(device=dev).manual_seed(d + by)
+    q, k, v, do = (torch.randn(n, H, d, device=dev, generator=gen).bfloat16() for _ in range(4))
+    feat = torch.randint(0, 256, (n, n, 4), device=dev, generator=gen, dtype=torch.uint8)
+    w = torch.randn(H, 4, device=dev, generator=gen) * 0.01
+
+    def run(move):
+        a = [move(x) for x in (q, k, v, do)]
+        out, dq, dk, dv = (move(torch.full_like(q, float("nan"))) for _ in range(4))
+        lse, dw = torch.empty(H, n, device=dev), torch.empty_like(w)
+        gt.gt_feature_attn_fwd(a[0], a[1], a[2], feat, w, gt.Batch(n), out, lse)
+        gt.gt_check(gt.gt_feature_attn_bwd(*a, lse, feat, w, gt.Batch(n), dq, dk, dv, dw))
+        return out, lse, dq, dk, dv, dw
+
+    for got, want in zip(run(lambda x: shifted(x, by)), run(lambda x: x)):
+        assert torch.equal(got, want)
+    odd = torch.zeros(2 * q.numel() + 1, dtype=torch.uint8, device=dev)[1:]            # refused on the host, nothing is launched
+    st = gt.lib().gt_feature_attn_fwd(odd.data_ptr(), k.data_ptr(), v.data_ptr(), feat.data_ptr(), w.data_ptr(), gt.Batch(n)._c_pair()[1], H, d,
+                                      q.data_ptr(), torch.empty(H, n, device=dev).data_ptr(), None)
+    assert st == 1
+
+
+def test_codes_are_written_at_any_address():
+    n, dev = 37, "cuda"
+    f = torch.randint(0, 3, (n, n, 4), device=dev, dtype=torch.uint8)
+    vectors = torch.empty(256, dtype=torch.int32, device=dev)
+    out = []
+    for by in (0, 1, 2):
+        codes = shifted(torch.full((n * 48,), 77, dtype=torch.uint8, device=dev), by)
+        gt.gt_check(gt.gt_feature_encode(f, gt.Batch(n), codes, vectors))
+        out.append(codes.clone())
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("by", [1, 8, 18])
+def test_distances_are_written_at_any_address(by):
+    """A ragged batch of blocks of 128 targets with a ring that is finished by shortcuts, single graphs of both pull kernels; the bit
+    matrices, which work on 16 bytes at a time, refuse it on the host."""
+    from gpu_util import device_batch, device_csr
+    i = np.arange(900)
+    ring = wl.csr_from_edges(900, i, (i + 1) % 900, symmetric=True)
+    wide = [wl.random_geometric(900 + 5 * j, 5.0, j) for j in range(42)] + [ring]
+    for graphs in ([wl.erdos_renyi(70, 0.05, 3)], [ring], wide, [wl.erdos_renyi(6001, 0.0016, 4)]):
+        b = wl.pack_graphs(graphs)
+        bt = device_batch(b)
+        rp, ci = device_csr(b)
+        out = shifted(torch.full((b.spd_bytes,), 77, dtype=torch.uint8, device="cuda"), by)
+        gt.gt_check(gt.gt_spd_build(rp, ci, bt, 6, out))
+        np.testing.assert_array_equal(out.cpu().numpy(), ospd.spd_packed(b.row_ptr, b.col_idx, b.cu_seqlens, 6))
+    b = wl.pack_graphs([wl.erdos_renyi(19000, 0.0001, 5)])
+    rp, ci = device_csr(b)
+    with pytest.raises(gt.GtError) as e:
+        gt.gt_spd_build(rp, ci, device_batch(b), 6, shifted(torch.zeros(b.spd_bytes, dtype=torch.uint8, device="cuda"), by))
+    assert e.value.status == 1
