@@ -174,9 +174,17 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return t.data_ptr()
 
 
-def _stream() -> int:
-    """Handle of torch's current stream on the current device (without making a Stream object for it)."""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+def _public_stream() -> int:
+    """Handle of torch's current stream on the current device."""
+    return torch.cuda.current_stream().cuda_stream
+
+
+# torch's own entry points give the handle without making a Stream object; where a version lacks them, the public call does.
+try:
+    _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    _stream = lambda: _raw_stream(_device())      # noqa: E731
+except AttributeError:
+    _stream = _public_stream
 
 
 def _raise(status: int, where: str) -> None:
