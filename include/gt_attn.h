@@ -19,7 +19,7 @@
  *    caller-provided workspace whose size is obtained from the matching *_workspace()
  *    query (host function, no GPU work).  Workspace and all tensor base pointers must be
  *    16-byte aligned.  (gt_feature_attn_* also take bf16 tensors, gt_feature_encode `codes` and gt_spd_build `spd_out` and
- *    blocks at any address that their elements allow, more slowly; gt_spd_build not where it uses bit matrices.)
+ *    blocks at any address that their elements allow, more slowly; gt_spd_build not for a single graph beyond 18 944 nodes.)
  *  - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls only
  *    enqueue work and return; they never synchronise.  Errors detected on the host are
  *    returned immediately.  Errors detected on the device (a bounded wait that ran out)
@@ -96,9 +96,10 @@ gt_status gt_check(void* workspace, void* stream);
  * distinct from unreachable pairs (bucket max_dist+1).  Bit-exact and deterministic.
  * Out-of-range col_idx entries are undefined behaviour.
  * Workspace (gt_spd_build_workspace says how much): 256 bytes for graphs of up to about 5 000 nodes, whose whole traversal
- * state fits shared memory; a single graph of up to 19 000 nodes: its edge list once more (2 bytes per edge) and bit planes of
- * 4 bytes per node, bit of max_dist + 1 and thread block in flight (up to two per SM; 24 MB at 8 192 nodes); a single graph
- * from 14 500 nodes on at least what its bit-matrix traversal needs (the one used beyond 19 000 nodes): about 8 KB per node
+ * state fits shared memory; a single graph of up to 18 944 nodes: its edge list once more (2 bytes per edge) and bit planes of
+ * 4 bytes per node, bit of max_dist + 1 and thread block in flight (up to two per SM; 24 MB at 8 192 nodes; below 14 500 nodes a
+ * call that is handed 4 n_total + 1 024 bytes does without, more slowly); a larger single graph, or one of 14 500 nodes or
+ * more with over 32 edges per node, what the bit matrices of its traversal need: about 8 KB per node
  * for each of min(4, ceil(n/8192)) groups of thread blocks (eight bit matrices of 1 KB rows per group: visited, and one
  * frontier per level up to 6; later levels reuse two of them) plus 1 KB per 33 edges per group (rows for vertices with more
  * than 32 out-edges) and 16 bytes per 32 edges -- 2.2 GB at 65 536 nodes with 786 000 edges -- and a device that supports
@@ -163,7 +164,7 @@ gt_status gt_spd_validate_count(void* workspace, void* stream, int64_t* count_ho
  * gt_test_hook_barrier_overcount -- test hook of the device-timeout path (no counterpart in the
  * paper).  Every device-side wait of this library is bounded; one that runs out makes its kernel
  * return and gt_check() report GT_ERR_DEVICE_TIMEOUT.  After gt_test_hook_barrier_overcount(k), k > 0,
- * the NEXT bit-matrix build of this process (gt_spd_build on a single graph of 14 500 nodes or more) waits
+ * the NEXT bit-matrix build of this process (gt_spd_build on a single graph of more than 18 944 nodes) waits
  * at its grid barriers for k arrivals more than there are thread blocks, with a shortened limit, so the
  * wait runs out within a second; the kernel issues no asynchronous copies, so nothing is in flight when
  * it returns, the context stays usable and the next build is normal.  The output of the hooked build

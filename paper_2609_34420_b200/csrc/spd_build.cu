@@ -952,7 +952,7 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
     pl.pull = spd_pull_plan(b, nnz, max_dist);
     if (pl.pull.fits) { pl.total_bytes = kHeaderBytes; return pl; }
     if (!in_place) pl.large = spd_pull_large_plan(b, nnz, max_dist);
-    if (pl.large.fits && b->n_total < kDenseMinNodes) { pl.total_bytes = pl.large.total_bytes; return pl; }
+    if (pl.large.fits) { pl.total_bytes = pl.large.total_bytes; return pl; }
     size_t state = spd_state_bytes(b->max_seqlen);
     pl.smem_state = state <= kSmemStateLimit;
     pl.threads = b->max_seqlen <= 1024 ? 256 : (b->max_seqlen <= 4096 ? 512 : 1024);
@@ -1016,7 +1016,6 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
             cudaGetLastError();
         }
     }
-    if (pl.large.total_bytes > pl.total_bytes) pl.total_bytes = pl.large.total_bytes;      // room for both: the test hook asks for the bit matrices
     return pl;
 }
 
@@ -1042,13 +1041,14 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
     if (batch->n_graphs > 1 && spd_offsets == nullptr) return GT_ERR_INVALID_ARG;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
     SpdPlan pl = make_plan(batch, nnz, max_dist, in_place);
+    if (workspace_bytes < pl.total_bytes && !in_place) pl = make_plan(batch, nnz, max_dist, true);      // what does with less, more slowly
     if (workspace == nullptr || workspace_bytes < pl.total_bytes || misaligned16(workspace)) return GT_ERR_WORKSPACE;
 
     cudaStream_t s = (cudaStream_t)stream;
     if (pl.pull.fits)
         return spd_pull_launch(pl.pull, row_ptr, col_idx, batch->n_graphs > 1 ? batch->cu_seqlens : nullptr,
                                batch->n_graphs > 1 ? spd_offsets : nullptr, batch, max_dist, spd_out, s);
-    if (pl.large.fits && !(pl.dense && g_barrier_overcount))
+    if (pl.large.fits)
         return spd_pull_large_launch(pl.large, row_ptr, col_idx, nnz, batch, max_dist, spd_out, workspace, s);
     if (pl.dense && misaligned16(spd_out)) return GT_ERR_INVALID_ARG;      // (it reads and writes 16 bytes at a time; the others take any address)
     uint8_t* ws = (uint8_t*)workspace;

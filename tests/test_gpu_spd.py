@@ -102,8 +102,7 @@ def test_undirected_graphs_deeper_than_max_dist_stop_at_the_clip_level():
 
 @pytest.mark.parametrize("n,D", [(3000, 3), (5000, 12), (12000, 6)])
 def test_deep_undirected_single_graph(n, D):
-    """Random geometric graph near its connectivity threshold: many levels, several components.  (At 12 000 nodes the
-    graph's CSR no longer fits beside the labels in the component pre-pass's shared memory and is read in place.)"""
+    """Random geometric graph near its connectivity threshold: many levels, several components."""
     w = wl.Workload("rgg", wl.pack_graphs([wl.random_geometric(n, 5.0, 11)]), 1, 32, D)
     check(w)
 
@@ -128,21 +127,58 @@ def test_named_workloads(name):
 
 
 def test_single_graph_beyond_the_shared_memory_state_matches_and_is_deterministic():
-    """A single graph of 14 500 nodes or more takes the bit-matrix build."""
+    """A single graph of more than 18 944 nodes takes the bit-matrix build."""
     w = wl.Workload("pl20k", wl.pack_graphs([wl.chung_lu_power_law(20000, 8.0, 2.1, 3)]), 1, 32, 10)
     a = check(w)
     b = gpu_spd(w).cpu().numpy()
     np.testing.assert_array_equal(a, b)
 
 
-@pytest.mark.parametrize("n", [14499, 14500, 16001])
+@pytest.mark.parametrize("n", [14499, 14500, 16001, 18944, 18945])
 def test_single_graphs_around_the_switch_to_the_bit_matrix_build(n):
-    """14 499 nodes: multi-source BFS with the state in shared memory; 14 500 and 16 001: bit-matrix build with a
-    ragged second column block.  Directed, so that the matrix is asymmetric."""
+    """Up to 18 944 nodes: the pull with its lists in the workspace; 18 945: bit-matrix build with a ragged third column
+    block.  Directed, so that the matrix is asymmetric."""
     rng = np.random.Generator(np.random.PCG64(n))
     m = 4 * n
     csr = wl.csr_from_edges(n, rng.integers(0, n - 50, m), rng.integers(0, n - 20, m), symmetric=False)
     check(wl.Workload("switch", wl.pack_graphs([csr]), 1, 32, 7))
+
+
+def _packed_with(big, seed):
+    return wl.pack_graphs([wl.random_directed(40, 2.0, seed), big, wl.erdos_renyi(300, 0.01, seed)])
+
+
+@pytest.mark.parametrize("kind", ["deep", "one reverse edge missing", "hub", "directed", "deep, list read in place"])
+def test_packed_batch_with_a_graph_beyond_the_pull(kind):
+    """Between the pull's limit and 17 066 nodes the batch runs the multi-source BFS with its words in shared memory.  Deep undirected
+    graphs stop at level max_dist by their components (at 13 000 nodes the edge list does not fit beside the labels and is read in
+    place); one missing reverse edge or a hub of more than 64 edges makes them search to the end."""
+    n = {"hub": 7000, "directed": 17000, "deep, list read in place": 13000}.get(kind, 6500)
+    big = wl.random_geometric(n, 6.0, 7)
+    if kind == "one reverse edge missing":
+        src, dst = np.repeat(np.arange(n), np.diff(big[0])), big[1]
+        at = int(np.flatnonzero(src > dst)[1000])
+        big = _csr(n, np.delete(src, at), np.delete(dst, at))
+    elif kind == "hub":
+        src, dst = np.repeat(np.arange(n), np.diff(big[0])), big[1]
+        far = np.arange(100, 6900, 68)
+        big = _csr(n, np.concatenate([src, np.full(100, 5), far]), np.concatenate([dst, far, np.full(100, 5)]))
+    elif kind == "directed":
+        big = wl.random_directed(n, 2.5, 8)
+    check(wl.Workload("packed_push", _packed_with(big, 3), 1, 32, 7))
+
+
+@pytest.mark.parametrize("n,D", [(6500, 5), (14000, 9)])
+def test_static_build_beyond_the_pull(n, D):
+    """Without a workspace a single graph beyond the shared-memory pull runs the multi-source BFS, undirected and directed."""
+    from gpu_util import device_batch, device_csr
+    from paper_2609_34420_b200 import binding as gt
+    for csr in (wl.random_geometric(n, 6.0, 2), wl.random_directed(n, 3.0, 4)):
+        b = wl.pack_graphs([csr])
+        rp, ci = device_csr(b)
+        out = torch.full((b.spd_bytes,), 0xEE, dtype=torch.uint8, device="cuda")
+        gt.gt_spd_build_static(rp, ci, device_batch(b), D, out)
+        np.testing.assert_array_equal(out.cpu().numpy(), ospd.spd_packed(b.row_ptr, b.col_idx, b.cu_seqlens, D))
 
 
 def test_packed_batch_with_a_graph_beyond_the_shared_memory_state():
@@ -182,7 +218,7 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
     and the same workspace then serves a normal, bit-exact build."""
     from gpu_util import device_batch, device_csr
     from paper_2609_34420_b200 import binding as gt
-    w = wl.Workload("pl18k", wl.pack_graphs([wl.chung_lu_power_law(18000, 6.0, 2.1, 9)]), 1, 32, 8)
+    w = wl.Workload("pl19k", wl.pack_graphs([wl.chung_lu_power_law(19000, 6.0, 2.1, 9)]), 1, 32, 8)
     bt = device_batch(w.batch)
     rp, ci = device_csr(w.batch)
     out = torch.empty(w.batch.spd_bytes, dtype=torch.uint8, device="cuda")
@@ -197,6 +233,24 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
     gt.gt_check(ws)
     exp = ospd.spd_packed(w.batch.row_ptr, w.batch.col_idx, w.batch.cu_seqlens, w.max_dist)
     np.testing.assert_array_equal(out.cpu().numpy(), exp)
+
+
+def test_a_workspace_is_no_larger_than_its_build_needs_and_a_small_one_will_do():
+    """Single graphs of 14 500 to 18 944 nodes with few edges are pulled, with code planes of 4 bytes per node and bit in the workspace and
+    not bit matrices of hundreds of megabytes.  Below 14 500 nodes a workspace without room for the planes is served, too."""
+    from gpu_util import device_batch, device_csr
+    from paper_2609_34420_b200 import binding as gt
+    w = wl.Workload("pull", wl.pack_graphs([wl.chung_lu_power_law(18000, 6.0, 2.1, 9)]), 1, 32, 8)
+    assert gt.gt_spd_build_workspace(device_batch(w.batch), int(w.batch.col_idx.size), 8) <= 4 * 4 * 18016 * 296 + (4 << 20)
+    w = wl.Workload("push", wl.pack_graphs([wl.random_directed(9000, 6.0, 9)]), 1, 32, 8)
+    bt = device_batch(w.batch)
+    rp, ci = device_csr(w.batch)
+    out = torch.empty(w.batch.spd_bytes, dtype=torch.uint8, device="cuda")
+    ws = torch.zeros(4 * 9000 + 1024, dtype=torch.uint8, device="cuda")
+    assert ws.numel() < gt.gt_spd_build_workspace(bt, int(ci.numel()), 8)
+    gt.gt_spd_build(rp, ci, bt, 8, out, ws)
+    gt.gt_check(ws)
+    np.testing.assert_array_equal(out.cpu().numpy(), ospd.spd_packed(w.batch.row_ptr, w.batch.col_idx, w.batch.cu_seqlens, 8))
 
 
 def test_spd_validate_counts_entries_that_name_no_bucket():
