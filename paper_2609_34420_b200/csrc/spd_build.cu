@@ -925,7 +925,6 @@ uint32_t g_barrier_overcount = 0;
 constexpr size_t kCompSmemBytes = 200 * 1024;     // shared memory of the component pre-pass (graphs whose labels do not fit skip it)
 size_t spd_state_bytes(int32_t max_seqlen) { return (size_t)3 * (size_t)max_seqlen * sizeof(uint32_t); }
 constexpr size_t kSmemStateLimit = 200 * 1024;
-constexpr int32_t kDenseMinNodes = 14500;
 
 struct SpdPlan {
     PullPlan pull;             // used where it fits

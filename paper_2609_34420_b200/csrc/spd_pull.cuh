@@ -29,6 +29,8 @@ struct PullLargePlan {
     int32_t n_pad;            // pitch of a code plane, in words
 };
 
+constexpr int32_t kDenseMinNodes = 14500;          // a single graph from here on that is not pulled takes the bit matrices
+
 PullLargePlan spd_pull_large_plan(const gt_batch* batch, int64_t nnz, int32_t max_dist);
 
 gt_status spd_pull_large_launch(const PullLargePlan& plan, const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,

@@ -26,6 +26,11 @@ constexpr int kTargets = 32;
 // Beyond this the bit-matrix build is the faster one (power law, degree 12: 18 000 nodes 0.85 against 0.91 ms, 20 000 nodes
 // 1.13 against 1.04 ms; from 592 blocks of targets on there is a fifth round); the row sets would fit up to 28 000 nodes.
 constexpr int32_t kLargeMaxNodes = 18944;
+// Many edges per vertex: beyond kDenseDegree the bit matrices are the faster ones where they are the alternative (Erdos-Renyi / power law:
+// 16 000 nodes, degree 25 687 against 778 us / 804 against 710, degree 50 974 against 822 / 1 140 against 680; 18 900 nodes, degree
+// 50 1 223 against 1 282 / 1 370 against 976); where the push is, beyond kLargeHubDegree, when every vertex is pulled by a warp (9 000
+// nodes, degree 100 400 against 933 us, degree 200 1 767 against 1 267).
+constexpr int kDenseDegree = 32;
 constexpr int kCachedHubs = 400;           // hubs whose numbers and lists' places are kept in shared memory
 
 constexpr int kPlainRounds = 3, kFarComponents = 1;         // as in spd_pull.cu; a round takes 6 to 25 us here
@@ -359,6 +364,17 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
     }
 }
 
+size_t static_smem()
+{
+    static const size_t bytes = [] {
+        cudaFuncAttributes a{};
+        if (cudaFuncGetAttributes(&a, spd_large_pull_kernel) == cudaSuccess) return a.sharedSizeBytes;
+        cudaGetLastError();
+        return (size_t)4096;
+    }();
+    return bytes;
+}
+
 }  // namespace
 
 PullLargePlan spd_pull_large_plan(const gt_batch* b, int64_t nnz, int32_t max_dist)
@@ -366,10 +382,11 @@ PullLargePlan spd_pull_large_plan(const gt_batch* b, int64_t nnz, int32_t max_di
     PullLargePlan pl{};
     const size_t n = (size_t)b->n_total;
     const size_t rows = 2 * pull_align(4 * n);
-    if (b->n_graphs != 1 || b->n_total > kLargeMaxNodes || nnz >= (1 << 26)) return pl;
+    if (b->n_graphs != 1 || b->n_total > kLargeMaxNodes || nnz >= (1 << 26) || nnz > (int64_t)b->n_total * (b->n_total < kDenseMinNodes ? kLargeHubDegree : kDenseDegree)) return pl;
     pl.fits = true;
-    // Two blocks of 512 threads per SM, whose phases overlap, where two pairs of row sets fit; else one of 1 024.
-    const bool two = rows <= kLargeSmemLimit / 2;
+    // Two blocks of 512 threads per SM, whose phases overlap, where two pairs of row sets fit (up to 14 126 nodes), with the static
+    // arrays and the 1 KB that the device keeps of a block's shared memory; else one of 1 024.
+    const bool two = 2 * (rows + static_smem() + 1024) <= 228 * 1024;
     pl.threads = two ? 512 : 1024;
     const size_t want = (size_t)sm_count() * (two ? 2 : 1), have = (n + kTargets - 1) / kTargets;
     pl.blocks = (unsigned)(have < want ? have : want);

@@ -43,11 +43,18 @@ def test_a_graph_whose_edges_do_not_fit_beside_sparse_ones():
     check(wl.Workload("outlier", wl.pack_graphs(graphs), 1, 32, 6))
 
 
-@pytest.mark.parametrize("n,m,D", [(5600, 80000, 1), (6001, 90000, 5), (7000, 9000, 30), (14200, 60000, 20), (18941, 50000, 9)])
+@pytest.mark.parametrize("n,m,D", [(5600, 80000, 1), (6001, 90000, 5), (7000, 9000, 30), (14100, 60000, 20), (14128, 60000, 20), (14200, 60000, 20),
+                                   (18941, 50000, 9)])
 def test_one_graph_with_lists_in_the_workspace(n, m, D):
     """Hubs beyond a group's degree (some more than are kept in shared memory), sparse directed graphs of many levels,
-    the last target block ragged, two blocks per SM and one."""
+    the last target block ragged, two blocks per SM (up to 14 126 nodes) and one."""
     one(directed(n, m, n, hub_edges=300, hubs=450 if n == 6001 else 2), D)
+
+
+@pytest.mark.parametrize("n,degree", [(5600, 128), (14500, 33)])
+def test_one_graph_with_too_many_edges_for_lists_in_the_workspace(n, degree):
+    """More than 126 edges per vertex: the push; more than 32 from 14 500 nodes on: the bit matrices."""
+    one(directed(n, n * degree, n), 3)
 
 
 def test_one_deep_undirected_graph_with_lists_in_the_workspace():
