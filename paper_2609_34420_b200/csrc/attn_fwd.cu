@@ -52,7 +52,7 @@ constexpr int kVStages = 2;
 constexpr int kSpdStages = 3;
 constexpr int kHalves = 2;                    // softmax threads per query row (column halves)
 constexpr int kCols = kKvTile / kHalves;      // score columns per softmax thread
-constexpr int kCW = kHalves == 1 ? 32 : 16;   // columns per TMEM load
+constexpr int kCW = 16;                       // columns per TMEM load
 constexpr int kChunks = kCols / kCW;
 static_assert(kChunks == 4, "the softmax pass is written for four chunks");
 constexpr float kSumThreshold = 1024.0f;      // tile row sum above which the reference maximum is raised
@@ -172,7 +172,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 {
     using L = FwdSmem<D>;
     constexpr int kRows = kRowsPerTile * kTiles, kThreads = 128 + 256 * kTiles, kBuffers = kTiles + 1;
-    static_assert(kHalves == 2);
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment by pointer arithmetic on the __shared__ array itself, so that every derived
     // pointer keeps its shared address space (integer round trips would turn the accesses generic)
@@ -517,11 +516,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tmem_wait_ld(); max_chunk(3, sb, wb);
                     loaded = false;
                     float mt = fmaxf(mx0, mx1);
-                    if constexpr (kHalves == 2) {
-                        xchg[hf * 128 + r] = mt;
-                        named_barrier_sync(pair_bar, 64);
-                        mt = fmaxf(mt, xchg[(hf ^ 1) * 128 + r]);
-                    }
+                    xchg[hf * 128 + r] = mt;
+                    named_barrier_sync(pair_bar, 64);
+                    mt = fmaxf(mt, xchg[(hf ^ 1) * 128 + r]);
                     const float m_new = fmaxf(m, ceilf(mt));
                     const float alpha = ex2_approx(m - m_new);
                     l *= alpha;
@@ -592,10 +589,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (kPrecise || exact) break;
                 // reference too low for some row of this warp (pair of warps)?  Also catches inf / NaN.
                 const bool need = !(tile_sum <= kSumThreshold);
-                bool any_need;
-                if constexpr (kHalves == 2) any_need = named_barrier_or(pair_bar, 64, need);
-                else any_need = __any_sync(0xffffffffu, need);
-                if (!any_need) break;
+                if (!named_barrier_or(pair_bar, 64, need)) break;
                 exact = true;
             }
             __syncwarp();
@@ -621,11 +615,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // ---- epilogue: O / l, LSE ----
         mbar_wait(bar(kBarODone + 2 * t + ((n_kv - 1) & 1)), ((n_kv - 1) >> 1) & 1, abort_flag, p.status, 43);
         tc_fence_after();
-        if constexpr (kHalves == 2) {
-            xchg[256 + hf * 128 + r] = l;
-            named_barrier_sync(pair_bar, 64);
-            l += xchg[256 + (hf ^ 1) * 128 + r];
-        }
+        xchg[256 + hf * 128 + r] = l;
+        named_barrier_sync(pair_bar, 64);
+        l += xchg[256 + (hf ^ 1) * 128 + r];
         const int32_t q = q0 + t * kRowsPerTile + r;
         const float inv_l = 1.0f / l;
         const float lse_nat = (m + log2f(l)) * kLn2;

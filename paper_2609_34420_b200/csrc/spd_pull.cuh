@@ -47,8 +47,6 @@ inline int pull_planes(int32_t max_dist)           // bits of the largest code, 
     return planes;
 }
 
-constexpr int kLeaders = 1;
-
 template <int kT>
 struct Rows {
     static constexpr int kWords = kT / 32;
@@ -110,16 +108,16 @@ __device__ __forceinline__ int warp_scan(int x, int lane)
     return x;
 }
 
-// Close the targets' rows under each other, a strongly connected set at a time.  With a leader a, C = all that its row
-// leads to and B = all targets whose rows lead to a; every target of both has exactly the row C.  One warp holds the
-// rows; a few leaders are enough (the passes below finish what is left).
+// Close the targets' rows under each other around the target a with the longest row.  C = all that its row leads to, B = all
+// targets whose rows lead to a; every target of both, a strongly connected set, has exactly the row C.  One warp holds the rows; the
+// passes finish what is left (eight such sets at a time took longer).
 template <int kT>
 __device__ __forceinline__ void close_targets(uint8_t* cur, const uint16_t* tpos, int nt, const uint32_t (&full)[Rows<kT>::kWords], int lane)
 {
     using R = Rows<kT>;
     constexpr int W = R::kWords;
     constexpr int kPer = kT / 32;                  // targets per lane
-    uint32_t row[kPer][W], todo[W];
+    uint32_t row[kPer][W];
     int bits[kPer];
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
@@ -129,59 +127,49 @@ __device__ __forceinline__ void close_targets(uint8_t* cur, const uint16_t* tpos
         for (int k = 0; k < W; ++k) row[j][k] = 0u;
         if (t < nt) R::load(cur, tpos[t], row[j]);
     }
+    unsigned best = 0u;                                      // the longest row: size << 7 | target
 #pragma unroll
-    for (int k = 0; k < W; ++k) todo[k] = full[k];
-    for (int leader = 0; leader < kLeaders; ++leader) {
-        unsigned best = 0u;                                      // the longest row that is left: size << 7 | target
+    for (int j = 0; j < kPer; ++j) {
+        const uint32_t m = bits[j] < 32 ? 1u << bits[j] : 0u;
+        int size = 0;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
+        for (int k = 0; k < W; ++k) size += __popc(row[j][k]);
+        if (full[j] & m) best = max(best, (unsigned)size << 7 | (unsigned)(lane + 32 * j));
+    }
+    best = __reduce_max_sync(0xffffffffu, best);
+    if (best == 0u) return;
+    const int lead = (int)(best & 127u);
+    uint32_t c[W], back[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) c[k] = back[k] = (lead >> 5) == k ? 1u << R::bit(lead & (kT - 1)) : 0u;
+    for (bool grew = true; grew;) {
+        uint32_t x[W], y[W], fresh = 0u;
+#pragma unroll
+        for (int k = 0; k < W; ++k) x[k] = y[k] = 0u;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {                     // target lane + 32 j sits in word j
             const uint32_t m = bits[j] < 32 ? 1u << bits[j] : 0u;
-            int size = 0;
-#pragma unroll
-            for (int k = 0; k < W; ++k) size += __popc(row[j][k]);
-            if (todo[j] & m) best = max(best, (unsigned)size << 7 | (unsigned)(lane + 32 * j));
-        }
-        best = __reduce_max_sync(0xffffffffu, best);
-        if (best == 0u) break;
-        const int lead = (int)(best & 127u);
-        uint32_t c[W], back[W];
-#pragma unroll
-        for (int k = 0; k < W; ++k) c[k] = back[k] = (lead >> 5) == k ? 1u << R::bit(lead & (kT - 1)) : 0u;
-        for (bool grew = true; grew;) {
-            uint32_t x[W], y[W], fresh = 0u;
-#pragma unroll
-            for (int k = 0; k < W; ++k) x[k] = y[k] = 0u;
-#pragma unroll
-            for (int j = 0; j < kPer; ++j) {                     // target lane + 32 j sits in word j
-                const uint32_t m = bits[j] < 32 ? 1u << bits[j] : 0u;
-                uint32_t leads = 0u;
-#pragma unroll
-                for (int k = 0; k < W; ++k) {
-                    if (c[j] & m) x[k] |= row[j][k];
-                    leads |= row[j][k] & back[k];
-                }
-                if (leads) y[j] |= m;
-            }
+            uint32_t leads = 0u;
 #pragma unroll
             for (int k = 0; k < W; ++k) {
-                x[k] = __reduce_or_sync(0xffffffffu, x[k]) | c[k];
-                y[k] = __reduce_or_sync(0xffffffffu, y[k]) | back[k];
-                fresh |= (x[k] ^ c[k]) | (y[k] ^ back[k]);
-                c[k] = x[k]; back[k] = y[k];
+                if (c[j] & m) x[k] |= row[j][k];
+                leads |= row[j][k] & back[k];
             }
-            grew = fresh != 0u;
+            if (leads) y[j] |= m;
         }
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const uint32_t m = bits[j] < 32 ? 1u << bits[j] : 0u;
-            if (c[j] & back[j] & m) {
-#pragma unroll
-                for (int k = 0; k < W; ++k) row[j][k] = c[k];
-                R::store(cur, tpos[lane + 32 * j], c);
-            }
+        for (int k = 0; k < W; ++k) {
+            x[k] = __reduce_or_sync(0xffffffffu, x[k]) | c[k];
+            y[k] = __reduce_or_sync(0xffffffffu, y[k]) | back[k];
+            fresh |= (x[k] ^ c[k]) | (y[k] ^ back[k]);
+            c[k] = x[k]; back[k] = y[k];
         }
+        grew = fresh != 0u;
+    }
 #pragma unroll
-        for (int k = 0; k < W; ++k) todo[k] &= ~(c[k] & back[k]);
+    for (int j = 0; j < kPer; ++j) {
+        const uint32_t m = bits[j] < 32 ? 1u << bits[j] : 0u;
+        if (c[j] & back[j] & m) R::store(cur, tpos[lane + 32 * j], c);
     }
 }
 
