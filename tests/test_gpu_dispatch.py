@@ -76,10 +76,11 @@ def test_one_and_two_query_tiles_per_block(n, beyond):
     check_forward(wl.small_workload([n], 148 // tiles + beyond, 32 if n % 2 else 64, 5, seed=n + beyond, avg_degree=2.0))
 
 
-# a key tile's queries shared by a cluster of 2, 3 or 4 blocks (private and shared bins), a share that is empty (5 tiles by 4),
-# graphs of a batch with fewer tiles than blocks, and the first size without
+# a key tile's queries shared by a cluster of 2, 3 or 4 blocks (private and shared bins), batches without a work list whose last graph
+# has fewer tiles than the cluster has blocks (two and three blocks leave at once), one that takes the list, and the first size without
 @pytest.mark.parametrize("sizes_,heads,d,D", [([385], 37, 32, 6), ([513], 7, 64, 6), ([640], 9, 64, 6), ([641], 8, 32, 24), ([900], 9, 64, 6),
-                                              ([129], 2, 64, 60), ([300], 4, 32, 254), ([500, 500, 500], 2, 64, 9), ([512, 1], 4, 32, 9),
+                                              ([129], 2, 64, 60), ([300], 4, 32, 254), ([500, 500, 500], 2, 64, 9), ([512, 512, 256], 2, 64, 9),
+                                              ([512, 512, 128], 2, 32, 40), ([512, 1], 4, 32, 9),
                                               ([3000], 8, 32, 6)])       # (the last: 192 blocks, two waves or three of shares)
 def test_backward_with_shared_key_tiles(sizes_, heads, d, D):
     check_backward(wl.small_workload(sizes_, heads, d, D, seed=sum(sizes_) + D, avg_degree=2.0))
@@ -95,8 +96,8 @@ def test_chunked_backward_with_shared_key_tiles(chunks):
         assert rel_l2(to_f64(got), to_f64(want)) <= 5e-3
 
 
-# a query tile's keys shared by a cluster of 2, 3 or 4 blocks: the first size with it, a share that is empty (9 and 10 tiles by 4: 3
-# each), one key in the last tile, graphs of a batch with fewer tiles than blocks, wide bias tables (shares of different references)
+# a query tile's keys shared by a cluster of 2, 3 or 4 blocks: the first size with it, shares of 3 tiles by which the last block has
+# fewer, one key in the last tile, graphs of a batch with fewer tiles than blocks, wide bias tables (shares of different references)
 @pytest.mark.parametrize("sizes_,heads,d,D,spread", [([641], 4, 64, 6, 1.0), ([700], 4, 32, 6, 12.0), ([1200], 3, 64, 60, 12.0), ([1025], 5, 64, 20, 1.0),
                                                      ([1100], 7, 32, 6, 12.0), ([800, 1, 300], 2, 64, 6, 1.0)])
 def test_forward_with_shared_query_tiles(sizes_, heads, d, D, spread):

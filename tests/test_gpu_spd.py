@@ -168,7 +168,7 @@ def test_packed_batch_with_a_graph_beyond_the_pull(kind):
     check(wl.Workload("packed_push", _packed_with(big, 3), 1, 32, 7))
 
 
-@pytest.mark.parametrize("n,D", [(6500, 5), (14000, 9)])
+@pytest.mark.parametrize("n,D", [(9000, 5), (14000, 9)])
 def test_static_build_beyond_the_pull(n, D):
     """Without a workspace a single graph beyond the shared-memory pull runs the multi-source BFS, undirected and directed."""
     from gpu_util import device_batch, device_csr
