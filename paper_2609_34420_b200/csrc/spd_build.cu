@@ -374,9 +374,8 @@ __global__ void __launch_bounds__(1024, kSmemState ? 1 : 2) spd_bfs_kernel(SpdPa
 // warps that OR into an accumulator row, and the last one to finish finalises the vertex.  Items are
 // handed out in batches from a counter.  Rows of empty frontiers are not read, complete vertices are
 // skipped, and a vertex stops reading neighbours once everything it still misses is covered.
-// Distances are written as the bits appear: the 32 output bytes of a word are read (only if some of
-// them were final already), blended and written back; unreachable pairs and padding follow at the
-// end of a column block.  Cost model: per level and column block nnz x 1 KB of row reads (L2 / HBM),
+// The frontiers of the first levels are kept, and one pass writes their distances and everything else
+// of a column block; later levels blend their distances into the bytes that are there.  Cost model: per level and column block nnz x 1 KB of row reads (L2 / HBM),
 // so a graph of large diameter is slow here (levels x blocks barriers) - the kernel is meant for the
 // small-world graphs of the paper's workloads.
 // ------------------------------------------------------------------------------------------
