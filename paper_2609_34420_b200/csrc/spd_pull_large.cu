@@ -8,8 +8,8 @@
 // rows: an edge whose head lies in the block is the pair.  The code planes are read and written where they are first needed
 // only (level 1, 2, 4, .. open a plane) and by the lane that owns the vertex, coalesced, from L2.
 //
-// What bounds it: the issue slots (75 % busy at 14 000 nodes: some hundred instructions per group of 32 vertices besides
-// those of its edges), then the bank conflicts of the row gathers, 3.5 wavefronts for 32 edges (spd_pull.cu).  Power-law
+// What bounds it: the issue slots (some hundred instructions per group of 32 vertices besides those of its edges), then the
+// bank conflicts of the row gathers, 3.5 wavefronts for 32 edges (spd_pull.cu).  Power-law
 // graphs of degree 12 against the frontier push that served them before: 12 000 nodes 915 -> 417 us, 14 400 nodes 1 395 ->
 // 632 us; against the bit-matrix build 16 384 nodes 920 -> 738 us; a graph of degree 10 and 8 192 nodes 374 -> 163 us.
 #include <type_traits>
@@ -385,7 +385,8 @@ PullLargePlan spd_pull_large_plan(const gt_batch* b, int64_t nnz, int32_t max_di
     if (b->n_graphs != 1 || b->n_total > kLargeMaxNodes || nnz >= (1 << 26) || nnz > (int64_t)b->n_total * (b->n_total < kDenseMinNodes ? kLargeHubDegree : kDenseDegree)) return pl;
     pl.fits = true;
     // Two blocks of 512 threads per SM, whose phases overlap, where two pairs of row sets fit (up to 14 126 nodes), with the static
-    // arrays and the 1 KB that the device keeps of a block's shared memory; else one of 1 024.
+    // arrays and the 1 KB that the device keeps of a block's shared memory; else one of 1 024 (14 160 nodes, degree 12: 709 us with one
+    // of 512, 555 with one of 1 024; 14 140 nodes 607 and 491).
     const bool two = 2 * (rows + static_smem() + 1024) <= 228 * 1024;
     pl.threads = two ? 512 : 1024;
     const size_t want = (size_t)sm_count() * (two ? 2 : 1), have = (n + kTargets - 1) / kTargets;
