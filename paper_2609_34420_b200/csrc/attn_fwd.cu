@@ -20,12 +20,13 @@
 //               row = TMEM lane, 64 score elements per thread).
 //
 // Softmax is single pass and speculative: a key tile is exponentiated against the row's current
-// reference maximum without looking at the tile's own maximum first; the row sum of the tile tells
-// afterwards whether the reference was too low (sum above a threshold, or not finite), and only then
-// the tile is redone the classical way (maximum, rescale of l and O, exponentials).  The first key
-// tile always takes the classical way.  References only ever grow, and they are integers in log2
-// units, so rescale factors are exact powers of two and the bf16 mantissa of a P entry does not
-// depend on how the keys are tiled or chunked.
+// reference without looking at the tile's own maximum first; the row sum of the tile tells
+// afterwards whether the reference was out of reach (sum above a threshold, or not finite, or the first tile's
+// below its reciprocal), and only then the tile is redone the classical way (maximum, rescale of l and O,
+// exponentials).  References are integers in log2 units, so rescale factors are exact powers of two and the
+// bf16 mantissa of a P entry does not depend on the reference, nor on how the keys are tiled or chunked.  They start
+// at 0 (scores are mostly within some powers of two of 1), where nothing has to be subtracted: 4 096 nodes, 8 heads of 64:
+// 60.2 -> 59.4 us, 64 graphs of 512-2 048 nodes, 16 heads: 1 068 -> 1 033 (with the first tile's maximum taken first before).
 //
 // TMEM columns: three score buffers [0,128) [128,256) [256,384) used in rotation by the steps
 // (key tile j, query tile t) -> buffer (2j+t) mod 3, so that the S MMA of a step never waits for a
@@ -55,9 +56,9 @@ constexpr int kCols = kKvTile / kHalves;      // score columns per softmax threa
 constexpr int kCW = 16;                       // columns per TMEM load
 constexpr int kChunks = kCols / kCW;
 static_assert(kChunks == 4, "the softmax pass is written for four chunks");
-constexpr float kSumThreshold = 1024.0f;      // tile row sum above which the reference maximum is raised
+constexpr float kSumThreshold = 0x1p24f;       // tile row sum above which the reference is raised (the first tile's: lowered below 1 / it)
 constexpr int kNormRows = 256;                // precise variant: rows per entry of key_norms
-constexpr float kReach = 60.0f;               // precise variant: log2 of the largest P entry that needs no new reference
+constexpr float kReach = 60.0f;               // precise variant: log2 of the largest P entry that needs no new reference (and of the smallest at first)
 
 struct FwdParams {
     const uint8_t* spd;
@@ -404,7 +405,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t tO = tmem + 384 + t * 64 + hf * kOC + lane_off;
         const uint32_t pair_bar = kNbPair + t * 4 + (warp & 3);
         float* xchg = (float*)(smem + L::kXchg) + t * 512;
-        float m = -INFINITY, l = 0.f;
+        float m = 0.f, l = 0.f;
+        bool shifted = false;                   // the reference of this warp's rows may differ from 0
 
         // lane b of every softmax warp keeps table entry b (scaled by log2 e); entries past the
         // table repeat the last one.  With at most 32 buckets a score's bias is fetched by a
@@ -413,24 +415,27 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint64_t c1c1 = pack_f32x2(p.c1, p.c1);
 
         // Precise variant: no score of this row exceeds |q| max|k| / sqrt(d) + max bias (log2 units; with room for rounding).
-        float limit = INFINITY;
+        float limit = INFINITY, low = -INFINITY;             // ... and none is below `low`
         if constexpr (kPrecise) {
             if (p.key_norms != nullptr) {
                 const int32_t n_blocks = (p.n_total + kNormRows - 1) / kNormRows;
-                float kk = 0.f, qq = 0.f, bmax = -INFINITY;
+                float kk = 0.f, qq = 0.f, bmax = -INFINITY, bmin = INFINITY;
                 for (int32_t b = node0 / kNormRows + lane; b <= (node0 + n_g - 1) / kNormRows; b += 32)
                     kk = norm_max(kk, p.key_norms[(size_t)h * n_blocks + b]);
-                for (int i = lane; i < 256; i += 32) bmax = fmaxf(bmax, s_bias[i]);
+                for (int i = lane; i < 256; i += 32) { bmax = fmaxf(bmax, s_bias[i]); bmin = fminf(bmin, s_bias[i]); }
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {
                     kk = norm_max(kk, __shfl_xor_sync(0xffffffffu, kk, off));
                     bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
+                    bmin = fminf(bmin, __shfl_xor_sync(0xffffffffu, bmin, off));
                 }
                 const int32_t row = node0 + min(q0 + t * kRowsPerTile + r, n_g - 1);
                 const uint4* src = (const uint4*)(p.q + ((size_t)row * p.n_heads + h) * D);
 #pragma unroll 2
                 for (int i = 0; i < D / 8; ++i) qq += square_sum(src[i]);
-                limit = sqrtf(qq * kk) * p.c1 * 1.001f + bmax + 1.0f;
+                limit = sqrtf(qq * kk) * p.c1 * 1.001f + 1.0f;
+                low = bmin - limit;
+                limit += bmax;
             }
         }
 
@@ -481,10 +486,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             uint32_t pk[kCols / 64][32];           // P of this thread's columns, bf16 pairs
             float tile_sum = 0.f;
             bool loaded = true;                    // chunk 0 is already on its way
-            bool exact = j == 0;                   // take the tile maximum first
+            bool exact = false;                    // take the tile maximum first
             // The precise variant's P overwrites the scores chunk by chunk, so a tile cannot be redone: it goes the speculative way
             // only where the row's reference leaves no score out of reach (both column halves decide alike).
-            if constexpr (kPrecise) exact = exact || __any_sync(0xffffffffu, !(limit <= m + kReach));
+            if constexpr (kPrecise) exact = __any_sync(0xffffffffu, !(limit <= m + kReach) || (j == 0 && !(low >= -kReach)));
 
             for (;;) {
                 if (exact) {
@@ -519,7 +524,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     xchg[hf * 128 + r] = mt;
                     named_barrier_sync(pair_bar, 64);
                     mt = fmaxf(mt, xchg[(hf ^ 1) * 128 + r]);
-                    const float m_new = fmaxf(m, ceilf(mt));
+                    const float m_new = j == 0 ? ceilf(mt) : fmaxf(m, ceilf(mt));
                     const float alpha = ex2_approx(m - m_new);
                     l *= alpha;
                     if (j > 0) {
@@ -536,12 +541,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         }
                     }
                     m = m_new;
+                    shifted = true;
                 }
 
                 // ---- P = 2^(s c1 + bias - m), row sum ----
                 const uint64_t neg_m = pack_f32x2(-m, -m);
                 uint64_t sum2 = pack_f32x2(0.f, 0.f);
-                auto exp_chunk = [&](int c, const uint32_t (&sr)[kCW], const uint4 (&ws)[kCW / 16], auto rag) {
+                auto exp_chunk = [&](int c, const uint32_t (&sr)[kCW], const uint4 (&ws)[kCW / 16], auto rag, auto ref) {
                     [[maybe_unused]] uint32_t hl[kCW];   // precise variant: hi terms of the chunk, then its lo terms
 #pragma unroll
                     for (int q = 0; q < kCW / 8; ++q) {
@@ -551,8 +557,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
                             float lo, hi;
-                            unpack_f32x2(add_f32x2(fma_f32x2(pack_u32x2(sr[q * 8 + 2 * i], sr[q * 8 + 2 * i + 1]), c1c1,
-                                                             pack_f32x2(bb[2 * i], bb[2 * i + 1])), neg_m), lo, hi);
+                            uint64_t x = fma_f32x2(pack_u32x2(sr[q * 8 + 2 * i], sr[q * 8 + 2 * i + 1]), c1c1, pack_f32x2(bb[2 * i], bb[2 * i + 1]));
+                            if constexpr (decltype(ref)::value) x = add_f32x2(x, neg_m);
+                            unpack_f32x2(x, lo, hi);
                             if constexpr (decltype(rag)::value) {
                                 const int col = c * kCW + q * 8 + 2 * i;
                                 if (col >= valid) lo = -INFINITY;
@@ -572,14 +579,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     }
                     if constexpr (kPrecise) tmem_st<kCW>(tS + c * kCW, hl);      // over the chunk's own score columns (already in registers)
                 };
-                auto exp_pass = [&](auto rag) {
+                auto exp_pass = [&](auto rag, auto ref) {
                     if (!loaded) load_chunk(0, sa, wa);
-                    tmem_wait_ld(); load_chunk(1, sb, wb); exp_chunk(0, sa, wa, rag);
-                    tmem_wait_ld(); load_chunk(2, sa, wa); exp_chunk(1, sb, wb, rag);
-                    tmem_wait_ld(); load_chunk(3, sb, wb); exp_chunk(2, sa, wa, rag);
-                    tmem_wait_ld(); exp_chunk(3, sb, wb, rag);
+                    tmem_wait_ld(); load_chunk(1, sb, wb); exp_chunk(0, sa, wa, rag, ref);
+                    tmem_wait_ld(); load_chunk(2, sa, wa); exp_chunk(1, sb, wb, rag, ref);
+                    tmem_wait_ld(); load_chunk(3, sb, wb); exp_chunk(2, sa, wa, rag, ref);
+                    tmem_wait_ld(); exp_chunk(3, sb, wb, rag, ref);
                 };
-                if (ragged) exp_pass(BoolTag<true>{}); else exp_pass(BoolTag<false>{});
+                if (ragged) exp_pass(BoolTag<true>{}, BoolTag<true>{});
+                else if (shifted) exp_pass(BoolTag<false>{}, BoolTag<true>{});
+                else exp_pass(BoolTag<false>{}, BoolTag<false>{});
                 loaded = false;
                 {
                     float lo, hi;
@@ -587,8 +596,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tile_sum = lo + hi;
                 }
                 if (kPrecise || exact) break;
-                // reference too low for some row of this warp (pair of warps)?  Also catches inf / NaN.
-                const bool need = !(tile_sum <= kSumThreshold);
+                // Reference too low (the first: too high) for some row of this warp (pair of warps)?  Also catches inf / NaN.  A half without
+                // valid columns has nothing to say.
+                const bool need = !(tile_sum <= kSumThreshold) || (j == 0 && valid > 0 && !(tile_sum >= 1.0f / kSumThreshold));
                 if (!named_barrier_or(pair_bar, 64, need)) break;
                 exact = true;
             }
