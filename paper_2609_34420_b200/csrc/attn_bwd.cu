@@ -234,8 +234,32 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         if (!p.maps) prefetch_tensormap(&tmap_spd);
     }
     if (warp == 2) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
-    for (int i = tid; i < n_bin_floats; i += kBwdThreads) s_bins[i] = 0.f;
+    // The first tiles are on their way while the block is still setting up: the thread that set up the barriers is the one that loads.
+    // (64 graphs of 512-2 048 nodes, 16 heads: 2 804 -> 2 784 us.)
+    const void* spd_map = p.maps ? (const void*)(p.maps + (size_t)g * kMapBytes) : &tmap_spd;
+    auto load_q_do = [&](int i) {
+        const int s = i & 1;
+        const int32_t row = node0 + q_lo + i * kTile;
+        mbar_arrive_expect_tx(bar(kBarQdoFull + s), 2 * L::kTileBytes + kExtTileBytes);
+        tma_load_3d(smem_u32(smem + L::kQ + s * L::kStageBytes), &tmap_q, bar(kBarQdoFull + s), 0, h, row);
+        tma_load_3d(smem_u32(smem + L::kDo + s * L::kStageBytes), &tmap_do, bar(kBarQdoFull + s), 0, h, row);
+        tma_load_3d(smem_u32(smem + L::kExt + s * kExtTileBytes), &tmap_ext, bar(kBarQdoFull + s), 0, h, row);
+    };
+    auto load_spd = [&](int i) {
+        mbar_arrive_expect_tx(bar(kBarSpdFull), L::kSpdBytes);
+        tma_load_2d(smem_u32(smem + L::kSpd), spd_map, bar(kBarSpdFull), q_lo + i * kTile, kv0);
+    };
+    if (warp > 0)
+        for (int i = tid - 32; i < n_bin_floats; i += kBwdThreads - 32) s_bins[i] = 0.f;
     grid_wait();
+    if (tid == 0) {
+        mbar_arrive_expect_tx(bar(kBarKvFull), 2 * L::kTileBytes);
+        tma_load_3d(smem_u32(smem + L::kK), &tmap_k, bar(kBarKvFull), 0, h, node0 + kv0);
+        tma_load_3d(smem_u32(smem + L::kV), &tmap_v, bar(kBarKvFull), 0, h, node0 + kv0);
+        load_q_do(0);
+        if (p.maps) acquire_tensor_map(spd_map);
+        load_spd(0);
+    }
     if (p.early_release) grid_release();
     for (int i = tid; i < 256; i += kBwdThreads)
         s_bias[i] = p.bias[(size_t)h * p.n_buckets + min(i, p.n_buckets - 1)] * kLog2e;
@@ -259,29 +283,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         setmaxnreg_dec_40();
         if (warp == 0) {
             // ------------------------------ TMA producer ------------------------------
-            const void* spd_map = p.maps ? (const void*)(p.maps + (size_t)g * kMapBytes) : &tmap_spd;
-            if (lane == 0) {
-                if (p.maps) acquire_tensor_map(spd_map);
-                mbar_arrive_expect_tx(bar(kBarKvFull), 2 * L::kTileBytes);
-                tma_load_3d(smem_u32(smem + L::kK), &tmap_k, bar(kBarKvFull), 0, h, node0 + kv0);
-                tma_load_3d(smem_u32(smem + L::kV), &tmap_v, bar(kBarKvFull), 0, h, node0 + kv0);
-            }
-            for (int i = 0; i < n_q; ++i) {
-                const int s = i & 1;
-                mbar_wait(bar(kBarStageEmpty + s), ((i >> 1) & 1) ^ 1, abort_flag, p.status, 110);
-                if (lane == 0) {
-                    const int32_t row = node0 + q_lo + i * kTile;
-                    mbar_arrive_expect_tx(bar(kBarQdoFull + s), 2 * L::kTileBytes + kExtTileBytes);
-                    tma_load_3d(smem_u32(smem + L::kQ + s * L::kStageBytes), &tmap_q, bar(kBarQdoFull + s), 0, h, row);
-                    tma_load_3d(smem_u32(smem + L::kDo + s * L::kStageBytes), &tmap_do, bar(kBarQdoFull + s), 0, h, row);
-                    tma_load_3d(smem_u32(smem + L::kExt + s * kExtTileBytes), &tmap_ext, bar(kBarQdoFull + s), 0, h, row);
-                }
+            for (int i = 1; i < n_q; ++i) {
+                mbar_wait(bar(kBarStageEmpty + (i & 1)), ((i >> 1) & 1) ^ 1, abort_flag, p.status, 110);
+                if (lane == 0) load_q_do(i);
                 __syncwarp();
-                if (i > 0) mbar_wait(bar(kBarSpdEmpty), (i - 1) & 1, abort_flag, p.status, 111);
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(bar(kBarSpdFull), L::kSpdBytes);
-                    tma_load_2d(smem_u32(smem + L::kSpd), spd_map, bar(kBarSpdFull), q_lo + i * kTile, kv0);
-                }
+                mbar_wait(bar(kBarSpdEmpty), (i - 1) & 1, abort_flag, p.status, 111);
+                if (lane == 0) load_spd(i);
                 __syncwarp();
             }
         } else if (warp == 1 || warp == 3) {
