@@ -532,7 +532,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     named_barrier_sync(pair_bar, 64);
                     mt = fmaxf(mt, xchg[(hf ^ 1) * 128 + r]);
                     const float m_new = j == 0 ? ceilf(mt) : fmaxf(m, ceilf(mt));
-                    const float alpha = ex2_approx(m - m_new);
+                    const float alpha = j == 0 ? 0.f : ex2_approx(m - m_new);      // (there is nothing yet; a first reference far below 0 would give infinity)
                     l *= alpha;
                     if (j > 0) {
                         mbar_wait(bar(kBarODone + 2 * t + ((j - 1) & 1)), ((j - 1) >> 1) & 1, abort_flag, p.status, 42);

@@ -146,3 +146,13 @@ def test_backward_of_a_large_graph_among_many_of_one_node():
         assert rel_l2(to_f64(got[big]), to_f64(want)) <= 5e-3
     assert rel_l2(to_f64(db), to_f64(alone[4])) <= 1e-3
     assert all(not x[single].any() for x in (dq, dk, dv))
+
+
+# The softmax reference starts at 0: scores far above and far below it, a first tile far below the others, a first tile masked out.
+@pytest.mark.parametrize("n,shift,masked", [(300, 60.0, False), (300, -60.0, False), (129, -17.0, False), (700, 17.0, False), (300, 0.0, True), (520, -90.0, True)])
+def test_scores_far_from_the_first_reference(n, shift, masked):
+    w = wl.small_workload([n], 2, 64, 6, seed=n, avg_degree=1.2)
+    w.tensors().bias[:] += shift
+    if masked:                                   # unreachable pairs weigh nothing; vertex 0 .. 127 reach each other only
+        w.tensors().bias[:, 7] = -1e30
+    check_forward(w)
