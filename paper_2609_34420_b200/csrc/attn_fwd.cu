@@ -864,6 +864,30 @@ int32_t chunk_rows(int32_t n, int32_t n_chunks)
     return (w + kKvTile - 1) / kKvTile * kKvTile;
 }
 
+// Parts that a chunked forward takes its chunks in.  A thread block walks through the consecutive chunks of a part with the softmax
+// state on the chip, as from one ring step to the next; parts go through memory as partial results and are merged.  One part unless
+// more of them fill the grid's last wave better.  A 256 x 128 tile takes 1.55 us, a block's fill and drain 7, the merge 3 and its bytes
+// (written and read, 5 TB/s).  Every chunk a part of its own, as it was -> now, 8 heads of 64: 4 096 nodes, 8 chunks 113.6 -> 59.8 us; 30 000 nodes,
+// 8 chunks 3 104 -> 2 612; 4 heads: 10 000 nodes, 2 chunks 221 us as it was, and 264 in one part.
+int32_t chunk_parts(int32_t n, int32_t n_heads, int32_t head_dim, int32_t n_chunks)
+{
+    const int64_t blocks = (int64_t)((n + kRowsPerCta - 1) / kRowsPerCta) * n_heads;
+    const int32_t tiles = chunk_rows(n, n_chunks) / kKvTile;
+    int32_t best = 1;
+    double least = 0.0;
+    for (int32_t parts = 1; parts <= n_chunks && parts <= 64; ++parts) {
+        const int32_t per = (n_chunks + parts - 1) / parts;
+        if ((n_chunks + per - 1) / per != parts) continue;                 // (the same as fewer parts)
+        double us = (double)((blocks * parts + sm_count() - 1) / sm_count()) * (1.55 * per * tiles + 7.0);
+        if (parts > 1) us += 3.0 + 8e-6 / 5.0 * parts * (double)n * n_heads * head_dim;
+        if (parts == 1 || us < 0.95 * least) {
+            best = parts;
+            least = us;
+        }
+    }
+    return best;
+}
+
 constexpr size_t kListMinSaved = 128;     // thread blocks
 
 // Largest |k|^2 of every kNormRows rows of a head: block (row block, head), D / 8 lanes per row.  Bound by its launch (8 192 rows,
@@ -1088,6 +1112,10 @@ extern "C" gt_status gt_biased_attn_fwd_chunked(const void* q, const void* k, co
     const size_t need = gt_biased_attn_fwd_chunked_workspace(batch, n_heads, head_dim, n_kv_chunks);
     if (workspace == nullptr || workspace_bytes < need || misaligned16(workspace)) return GT_ERR_WORKSPACE;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
+    const int32_t parts = lse_chunks != nullptr ? n_kv_chunks                         // each chunk's own lse is wanted
+                          : rows_per_block(batch, n_heads) == kRowsPerTile ? 1 : chunk_parts(batch->n_total, n_heads, head_dim, n_kv_chunks);
+    if (parts == 1 && lse_chunks == nullptr)
+        return gt_biased_attn_fwd_ex(q, k, v, spd, nullptr, bias, batch, n_heads, head_dim, max_dist, out, lse, nullptr, workspace, workspace_bytes, stream);
     CUtensorMap tq, tk, tv;
     if ((st = encode_thd_map(&tq, q, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
     if ((st = encode_thd_map(&tk, k, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
@@ -1106,20 +1134,20 @@ extern "C" gt_status gt_biased_attn_fwd_chunked(const void* q, const void* k, co
     p.n_total = batch->n_total;
     p.n_heads = n_heads;
     p.n_buckets = max_dist + 2;
-    p.kv_chunk_rows = chunk_rows(batch->n_total, n_kv_chunks);
+    p.kv_chunk_rows = chunk_rows(batch->n_total, n_kv_chunks) * ((n_kv_chunks + parts - 1) / parts);
     p.c1 = kLog2e / sqrtf((float)head_dim);
     cudaStream_t s = (cudaStream_t)stream;
-    st = head_dim == 64 ? launch_fwd<64, true>(tq, tk, tv, tspd, p, batch, n_kv_chunks, s)
-                        : launch_fwd<32, true>(tq, tk, tv, tspd, p, batch, n_kv_chunks, s);
+    st = head_dim == 64 ? launch_fwd<64, true>(tq, tk, tv, tspd, p, batch, parts, s)
+                        : launch_fwd<32, true>(tq, tk, tv, tspd, p, batch, parts, s);
     if (st != GT_OK) return st;
     const size_t n_thr = rows * (head_dim / 4);
     const unsigned blocks = (unsigned)((n_thr + 255) / 256);
     if (head_dim == 64)
         st = launch_overlapped(chunk_merge_kernel<64>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
-                                                      batch->n_total, n_heads, n_kv_chunks);
+                                                      batch->n_total, n_heads, parts);
     else
         st = launch_overlapped(chunk_merge_kernel<32>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
-                                                      batch->n_total, n_heads, n_kv_chunks);
+                                                      batch->n_total, n_heads, parts);
     return st;
 }
 

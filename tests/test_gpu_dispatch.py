@@ -156,3 +156,18 @@ def test_scores_far_from_the_first_reference(n, shift, masked):
     if masked:                                   # unreachable pairs weigh nothing; vertex 0 .. 127 reach each other only
         w.tensors().bias[:, 7] = -1e30
     check_forward(w)
+
+
+# Without the chunks' own lse: all of them in one part, in some parts, each a part of its own.
+@pytest.mark.parametrize("n,heads,d,chunks", [(1000, 4, 64, 3), (5000, 4, 64, 5), (10000, 4, 32, 2), (9000, 4, 64, 8)])
+def test_chunked_forward_in_parts(n, heads, d, chunks):
+    dev, gen = torch.device("cuda"), torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(n, heads, d, device=dev, generator=gen).bfloat16() for _ in range(3))
+    spd = torch.randint(0, 8, (n * wl.round_up(n, 16),), device=dev, generator=gen, dtype=torch.uint8)
+    bias = torch.randn(heads, 8, device=dev, generator=gen)
+    batch = gt.Batch(n)
+    out, out_c, lse, lse_c = torch.empty_like(q), torch.empty_like(q), torch.empty(heads, n, device=dev), torch.empty(heads, n, device=dev)
+    gt.gt_check(gt.gt_biased_attn_fwd(q, k, v, spd, bias, batch, 6, out, lse))
+    gt.gt_check(gt.gt_biased_attn_fwd_chunked(q, k, v, spd, bias, batch, 6, out_c, lse_c, chunks))
+    assert rel_l2(to_f64(out_c), to_f64(out)) <= 1e-3
+    assert (lse - lse_c).abs().max().item() <= LSE_MAX_ABS
