@@ -21,7 +21,9 @@
 // mma.sync and not tcgen05: at the 500 - 8 192 nodes this form is meant for, a 128-row tile per thread block would leave
 // most SMs empty, and the three-term operands would have to travel through tensor memory.
 // What bounds it: latency at ten warps per SM (1 500 nodes have no more rows); 12 of the 19 contractions are the terms of P and
-// dS.  1 500 nodes, H = 8, d = 64: forward 64 us, backward 199 us (54 and 172 with one chain of MMAs over all keys, ex2 in the
+// dS.  What bounds it: the latency of an element's chain of instructions at two and a half warps per scheduler (issue slots 45 %, tensor
+// pipe 33-42 % busy); fp32 arithmetic goes by pairs (one instruction, the same results), and a chain's first MMA adds to zero.
+// 1 500 nodes, H = 8, d = 64: forward 60 us, backward 195 us (64 and 199 element by element; 54 and 172 with one chain of MMAs over all keys, ex2 in the
 // forward and one walk on the query side, whose results are further off); the same sums on the fp32 pipes took 3 000 us.
 #include <cuda_bf16.h>
 #include <math.h>
@@ -29,9 +31,12 @@
 #include <initializer_list>
 
 #include "attn_common.cuh"
+#include "sm100_primitives.cuh"
 
 namespace gt {
 namespace {
+
+using namespace sm100;
 
 constexpr int kFeat = 4;              // bias features per node pair
 constexpr int kRows = 32;             // rows of a thread block: two groups of 16
@@ -45,6 +50,13 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the same on an empty accumulator
+__device__ __forceinline__ void mma16816_first(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+                 : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 __device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t addr)
 {
@@ -63,20 +75,22 @@ template <int kLeft>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kLeft) : "memory"); }
 
 // Two fp32 numbers as three pairs of bf16 whose sum they are.
-__device__ __forceinline__ void split3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo)
+__device__ __forceinline__ void split3(uint64_t x, uint32_t& hi, uint32_t& mid, uint32_t& lo)
 {
-    auto pack = [](float a, float b) {
+    auto pack = [](uint64_t v) {
+        float a, b;
+        unpack_f32x2(v, a, b);
         uint32_t r;
         asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
         return r;
     };
-    hi = pack(x0, x1);
-    x0 -= __uint_as_float(hi << 16);
-    x1 -= __uint_as_float(hi & 0xffff0000u);
-    mid = pack(x0, x1);
-    x0 -= __uint_as_float(mid << 16);
-    x1 -= __uint_as_float(mid & 0xffff0000u);
-    lo = pack(x0, x1);
+    auto rest = [](uint64_t v, uint32_t term) {
+        return fma_f32x2(pack_u32x2(term << 16, term & 0xffff0000u), pack_f32x2(-1.f, -1.f), v);
+    };
+    hi = pack(x);
+    x = rest(x, hi);
+    mid = pack(x);
+    lo = pack(rest(x, mid));
 }
 
 // A tile of rows of D bf16 in shared memory: 16-byte chunks, XOR-swizzled so that eight rows of one chunk column lie in
@@ -133,20 +147,18 @@ template <int D>
 __device__ __forceinline__ void scores(float (&s)[2][2][4], const uint32_t (&a)[D / 16][4], uint32_t base, int row, int lane)
 {
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-        for (int t = 0; t < 2; ++t)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) s[b][t][x] = 0.f;
-#pragma unroll
     for (int k = 0; k < D / 16; ++k) {
         uint32_t b[4], c[4];
         Tile<D>::load_b(b, base, row, k, lane);
         Tile<D>::load_b(c, base, row + 16, k, lane);
-        mma16816(s[0][0], a[k], b[0], b[1]);
-        mma16816(s[0][1], a[k], b[2], b[3]);
-        mma16816(s[1][0], a[k], c[0], c[1]);
-        mma16816(s[1][1], a[k], c[2], c[3]);
+        auto step = [&](auto mma) {
+            mma(s[0][0], a[k], b[0], b[1]);
+            mma(s[0][1], a[k], b[2], b[3]);
+            mma(s[1][0], a[k], c[0], c[1]);
+            mma(s[1][1], a[k], c[2], c[3]);
+        };
+        if (k == 0) step(mma16816_first);
+        else step(mma16816);
     }
 }
 
@@ -157,30 +169,28 @@ __device__ __forceinline__ void two_scores(float (&s)[2][4], uint32_t own_s, flo
                                            uint32_t base_s, uint32_t base_u, int row, int lane)
 {
 #pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) s[t][x] = u[t][x] = 0.f;
-#pragma unroll
     for (int k = 0; k < D / 16; ++k) {
         uint32_t a[4], b[4], c[4], d[4];
         ldm4(a, Tile<D>::at(own_s, own_row + (lane & 15), 2 * k + (lane >> 4)));
         Tile<D>::load_b(b, base_s, row, k, lane);
         ldm4(c, Tile<D>::at(own_u, own_row + (lane & 15), 2 * k + (lane >> 4)));
         Tile<D>::load_b(d, base_u, row, k, lane);
-        mma16816(s[0], a, b[0], b[1]);
-        mma16816(u[0], c, d[0], d[1]);
-        mma16816(s[1], a, b[2], b[3]);
-        mma16816(u[1], c, d[2], d[3]);
+        auto step = [&](auto mma) {
+            mma(s[0], a, b[0], b[1]);
+            mma(u[0], c, d[0], d[1]);
+            mma(s[1], a, b[2], b[3]);
+            mma(u[1], c, d[2], d[3]);
+        };
+        if (k == 0) step(mma16816_first);
+        else step(mma16816);
     }
 }
 
-// a 16 x 16 block of fp32 in score fragments -> its three bf16 operand fragments
-__device__ __forceinline__ void split_block(const float (&p)[2][4], uint32_t (&t)[3][4])
+// a 16 x 16 block of fp32 in score fragments (pairs of neighbouring columns) -> its three bf16 operand fragments
+__device__ __forceinline__ void split_block(const uint64_t (&p)[2][2], uint32_t (&t)[3][4])
 {
-    split3(p[0][0], p[0][1], t[0][0], t[1][0], t[2][0]);
-    split3(p[0][2], p[0][3], t[0][1], t[1][1], t[2][1]);
-    split3(p[1][0], p[1][1], t[0][2], t[1][2], t[2][2]);
-    split3(p[1][2], p[1][3], t[0][3], t[1][3], t[2][3]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) split3(p[k >> 1][k & 1], t[0][k], t[1][k], t[2][k]);
 }
 
 // acc (16 x D) += P (16 x 16, three terms; smallest first) times 16 rows of a tile.  The tensor core cuts off what its
@@ -189,33 +199,44 @@ __device__ __forceinline__ void split_block(const float (&p)[2][4], uint32_t (&t
 // outputs miss the nearest bf16 value, growing with n.)  Four chains alternate: an MMA that adds to the result of the one before
 // it would wait for it.
 template <int D>
-__device__ __forceinline__ void add_product(float (&acc)[D / 8][4], const uint32_t (&t)[3][4], uint32_t base, int row, int lane)
+__device__ __forceinline__ void add_product(uint64_t (&acc)[D / 8][2], const uint32_t (&t)[3][4], uint32_t base, int row, int lane)
 {
 #pragma unroll
     for (int c = 0; c < D / 16; c += 2) {
         uint32_t b0[4], b1[4];
         Tile<D>::load_bt(b0, base, row, c, lane);
         Tile<D>::load_bt(b1, base, row, c + 1, lane);
-        float u[4][4] = {};
+        float u[4][4];
 #pragma unroll
         for (int x = 2; x >= 0; --x) {
-            mma16816(u[0], t[x], b0[0], b0[1]);
-            mma16816(u[2], t[x], b1[0], b1[1]);
-            mma16816(u[1], t[x], b0[2], b0[3]);
-            mma16816(u[3], t[x], b1[2], b1[3]);
+            auto step = [&](auto mma) {
+                mma(u[0], t[x], b0[0], b0[1]);
+                mma(u[2], t[x], b1[0], b1[1]);
+                mma(u[1], t[x], b0[2], b0[3]);
+                mma(u[3], t[x], b1[2], b1[3]);
+            };
+            if (x == 2) step(mma16816_first);
+            else step(mma16816);
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) acc[2 * c + k][x] += u[k][x];
+        for (int k = 0; k < 4; ++k) {
+            acc[2 * c + k][0] = add_f32x2(acc[2 * c + k][0], pack_f32x2(u[k][0], u[k][1]));
+            acc[2 * c + k][1] = add_f32x2(acc[2 * c + k][1], pack_f32x2(u[k][2], u[k][3]));
+        }
     }
 }
 
-__device__ __forceinline__ void unpack_features(uint32_t f4, float (&f)[kFeat])
+__device__ __forceinline__ uint64_t both(float x) { return pack_f32x2(x, x); }
+
+// The features of two pairs.  Byte -> fp32 without the conversion pipe: 2^15 + b has b in its mantissa's second byte, and 2^15
+// comes off exactly.
+__device__ __forceinline__ void unpack_features(uint32_t f4, uint32_t g4, uint64_t (&f)[kFeat])
 {
-    // byte -> fp32 without the conversion pipe: 2^15 + b has b in its mantissa's second byte, and 2^15 comes off exactly
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) f[c] = __uint_as_float(__byte_perm(f4, 0x47000000u, 0x7404u | ((uint32_t)c << 4))) - 32768.f;
+    for (int c = 0; c < kFeat; ++c) {
+        const uint32_t pick = 0x7404u | ((uint32_t)c << 4);
+        f[c] = add_f32x2(pack_u32x2(__byte_perm(f4, 0x47000000u, pick), __byte_perm(g4, 0x47000000u, pick)), both(-32768.f));
+    }
 }
 
 template <bool B> struct BoolConst { static constexpr bool value = B; };
@@ -246,13 +267,26 @@ struct FeatureArgs {
     float scale;                  // 1 / sqrt(d)
 };
 
-// e^x for the backward's P, off by up to |x| 2^-24 beside the 2 ulp of ex2, and less than P matters where x is large.  (1 500 nodes:
-// 17 us of 272 less than expf.)  The forward keeps expf, because its lse is returned in fp32.
-__device__ __forceinline__ float exp_of(float x)
+__device__ __forceinline__ float ex2(float x)
 {
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * kLog2e));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+__device__ __forceinline__ uint64_t ex2_pair(uint64_t x)
+{
+    float a, b;
+    unpack_f32x2(x, a, b);
+    return pack_f32x2(ex2(a), ex2(b));
+}
+// e^x for the backward's P, off by up to |x| 2^-24 beside the 2 ulp of ex2, and less than P matters where x is large.
+__device__ __forceinline__ uint64_t exp_of(uint64_t x) { return ex2_pair(mul_f32x2(x, both(kLog2e))); }
+// The forward keeps expf, because its lse is returned in fp32.
+__device__ __forceinline__ uint64_t expf_pair(uint64_t x)
+{
+    float a, b;
+    unpack_f32x2(x, a, b);
+    return pack_f32x2(expf(a), expf(b));
 }
 
 // words of pairs (i, j) and (i, j + 1), j even; out of range: 0
@@ -269,11 +303,9 @@ __device__ __forceinline__ uint2 feature_pair(const uint32_t* __restrict__ feat,
     }
     return r;
 }
-__device__ __forceinline__ float bias_of(uint32_t f4, const float (&w)[kFeat])
+__device__ __forceinline__ uint64_t bias_of(const uint64_t (&f)[kFeat], const uint64_t (&w)[kFeat])
 {
-    float f[kFeat];
-    unpack_features(f4, f);
-    return w[0] * f[0] + w[1] * f[1] + w[2] * f[2] + w[3] * f[3];
+    return fma_f32x2(w[3], f[3], fma_f32x2(w[2], f[2], fma_f32x2(w[1], f[1], mul_f32x2(w[0], f[0]))));
 }
 // sum over the four lanes that share a fragment row
 __device__ __forceinline__ float quad_sum(float x)
@@ -303,9 +335,10 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
     const int g = lane >> 2, t4 = lane & 3;
     const uint32_t base = smem_addr(s_tiles);
     const bool pairs = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.feat) & 7u) == 0;
-    float w[kFeat];
+    uint64_t w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
+    for (int c = 0; c < kFeat; ++c) w[c] = both(p.weights[h * kFeat + c]);
+    const uint64_t scale = both(p.scale);
 
     uint32_t qa[D / 16][4];
     Tile<D>::template fetch<kRows, kAligned>(base, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
@@ -315,11 +348,10 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
     Tile<D>::load_a(qa, base, 16 * group, lane);
     __syncthreads();
 
-    float o[D / 8][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+    uint64_t o[D / 8][2];
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
 #pragma unroll
-    for (int c = 0; c < D / 8; ++c)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) o[c][x] = 0.f;
+    for (int c = 0; c < D / 8; ++c) o[c][0] = o[c][1] = 0ull;
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
@@ -348,12 +380,15 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
-                    const float bias = bias_of(x & 1 ? f[b][t][x >> 1].y : f[b][t][x >> 1].x, w);
-                    s[b][t][x] = s[b][t][x] * p.scale + bias;                    // bias added before the softmax statistics
-                    if (ragged && j >= n) s[b][t][x] = -INFINITY;
-                    top[x >> 1] = fmaxf(top[x >> 1], s[b][t][x]);
+                for (int r = 0; r < 2; ++r) {
+                    const int32_t j = j0 + 16 * b + 8 * t + 2 * t4;
+                    uint64_t fv[kFeat];
+                    unpack_features(f[b][t][r].x, f[b][t][r].y, fv);
+                    float(&s2)[2] = *(float(*)[2])&s[b][t][2 * r];
+                    unpack_f32x2(fma_f32x2(pack_f32x2(s2[0], s2[1]), scale, bias_of(fv, w)), s2[0], s2[1]);     // bias added before the softmax statistics
+                    if (ragged && j >= n) s2[0] = -INFINITY;
+                    if (ragged && j + 1 >= n) s2[1] = -INFINITY;
+                    top[r] = fmaxf(top[r], fmaxf(s2[0], s2[1]));
                 }
         }
         top[0] = quad_max(top[0]);
@@ -362,20 +397,27 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
             const float a0 = m[0] == top[0] ? 1.f : expf(m[0] - top[0]), a1 = m[1] == top[1] ? 1.f : expf(m[1] - top[1]);
             l[0] *= a0; l[1] *= a1;
 #pragma unroll
-            for (int c = 0; c < D / 8; ++c) { o[c][0] *= a0; o[c][1] *= a0; o[c][2] *= a1; o[c][3] *= a1; }
+            for (int c = 0; c < D / 8; ++c) { o[c][0] = mul_f32x2(o[c][0], both(a0)); o[c][1] = mul_f32x2(o[c][1], both(a1)); }
             m[0] = top[0]; m[1] = top[1];
         }
-        const float ref0 = m[0] == -INFINITY ? 0.f : m[0], ref1 = m[1] == -INFINITY ? 0.f : m[1];     // a half without keys so far
+        uint64_t less[2];                                                        // minus the reference (0: a half without keys so far)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) less[r] = both(m[r] == -INFINITY ? 0.f : -m[r]);
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
+            uint64_t pr[2][2];                                                   // 0 for keys past the end
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) s[b][t][x] = expf(s[b][t][x] - (x < 2 ? ref0 : ref1));       // 0 for keys past the end
-            l[0] += (s[b][0][0] + s[b][0][1]) + (s[b][1][0] + s[b][1][1]);
-            l[1] += (s[b][0][2] + s[b][0][3]) + (s[b][1][2] + s[b][1][3]);
+                for (int r = 0; r < 2; ++r) pr[t][r] = expf_pair(add_f32x2(pack_f32x2(s[b][t][2 * r], s[b][t][2 * r + 1]), less[r]));
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                float x, y;
+                unpack_f32x2(add_f32x2(pr[0][r], pr[1][r]), x, y);
+                l[r] += x + y;
+            }
             uint32_t pt[3][4];
-            split_block(s[b], pt);
+            split_block(pr, pt);
             add_product<D>(o, pt, vt, 32 * half + 16 * b, lane);
         }
         __syncthreads();
@@ -388,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 #pragma unroll
         for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-            for (int x = 0; x < 4; ++x) part[(g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1)] = o[c][x];
+            for (int r = 0; r < 2; ++r) *(uint64_t*)&part[(g + 8 * r) * D + 8 * c + 2 * t4] = o[c][r];
         if (t4 == 0) {
 #pragma unroll
             for (int r = 0; r < 2; ++r) { part[16 * D + g + 8 * r] = m[r]; part[16 * D + 16 + g + 8 * r] = l[r]; }
@@ -406,7 +448,10 @@ __global__ void __launch_bounds__(kThreads, 3) feature_fwd_kernel(FeatureArgs p)
 #pragma unroll
                 for (int c = 0; c < D / 8; ++c) {
                     const float* o2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
-                    const float x = (o[c][2 * r] * a + o2[0] * b) * inv, y = (o[c][2 * r + 1] * a + o2[1] * b) * inv;
+                    float x, y;
+                    unpack_f32x2(o[c][r], x, y);
+                    x = (x * a + o2[0] * b) * inv;
+                    y = (y * a + o2[1] * b) * inv;
                     store_pair<kAligned>(p.out + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4, x, y);
                 }
                 if (t4 == 0) p.lse[(size_t)h * n + i] = mm + logf(ll);
@@ -437,9 +482,10 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
     const int g = lane >> 2, t4 = lane & 3;
     const uint32_t base = smem_addr(s_tiles);
     const bool pairs = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.feat) & 7u) == 0;
-    float w[kFeat];
+    uint64_t w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
+    for (int c = 0; c < kFeat; ++c) w[c] = both(p.weights[h * kFeat + c]);
+    const uint64_t scale = both(p.scale);
 
     const uint32_t own_q = smem_addr(s_own), own_d = own_q + kRows * 2 * D;
     Tile<D>::template fetch<kRows, kAligned>(own_q, p.q, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
@@ -447,15 +493,13 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
     cp_commit();
 
     float lse[2], delta[2] = {0.f, 0.f}, sum_px[2] = {0.f, 0.f}, sum_p[2] = {0.f, 0.f};
-    float dq[D / 8][4], xf[kFeat];                                                // sums of dS K and of dS f
+    uint64_t dq[D / 8][2], xf[kFeat];                                             // sums of dS K and of dS f (even and odd columns)
 #pragma unroll
     for (int r = 0; r < 2; ++r) lse[r] = i0 + g + 8 * r < n ? p.lse_in[(size_t)h * n + i0 + g + 8 * r] : INFINITY;     // P = 0
 #pragma unroll
-    for (int c = 0; c < D / 8; ++c)
+    for (int c = 0; c < D / 8; ++c) dq[c][0] = dq[c][1] = 0ull;
 #pragma unroll
-        for (int x = 0; x < 4; ++x) dq[c][x] = 0.f;
-#pragma unroll
-    for (int c = 0; c < kFeat; ++c) xf[c] = 0.f;
+    for (int c = 0; c < kFeat; ++c) xf[c] = 0ull;
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
@@ -481,41 +525,44 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
             const uint32_t kt = base + (uint32_t)(tile & 1) * 2 * kTileBytes, vt = kt + kTileBytes;
 #pragma unroll 1
             for (int b = 0; b < 2; ++b) {
-                float s[2][4], dp[2][4], y[kFeat] = {};
+                float s[2][4], dp[2][4];
+                uint64_t y[kFeat] = {}, px[2][2], pr[2][2];
                 two_scores<D>(s, own_q, dp, own_d, 16 * group, kt, vt, 32 * half + 16 * b, lane);
                 const bool ragged = j0 + 16 * b + 16 > n;
 #pragma unroll
                 for (int t = 0; t < 2; ++t)
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const int r = x >> 1;
-                        const int32_t j = j0 + 16 * b + 8 * t + 2 * t4 + (x & 1);
-                        float fv[kFeat];
-                        unpack_features(x & 1 ? f[t][r].y : f[t][r].x, fv);
-                        const float bias = w[0] * fv[0] + w[1] * fv[1] + w[2] * fv[2] + w[3] * fv[3];
-                        float pr = exp_of((s[t][x] * p.scale + bias) - lse[r]);
-                        if (ragged && j >= n) pr = 0.f;
+                    for (int r = 0; r < 2; ++r) {
+                        const int32_t j = j0 + 16 * b + 8 * t + 2 * t4;
+                        uint64_t fv[kFeat];
+                        unpack_features(f[t][r].x, f[t][r].y, fv);
+                        const uint64_t x = fma_f32x2(pack_f32x2(s[t][2 * r], s[t][2 * r + 1]), scale, bias_of(fv, w));
+                        pr[t][r] = exp_of(add_f32x2(x, both(-lse[r])));
+                        if (ragged && j + 1 >= n) pr[t][r] &= j >= n ? 0ull : 0xffffffffull;
+                        const uint64_t d = pack_f32x2(dp[t][2 * r], dp[t][2 * r + 1]);
                         if constexpr (kForDelta) {
-                            dp[t][x] *= pr;
-                            s[t][x] = pr;
+                            px[t][r] = mul_f32x2(d, pr[t][r]);
                         } else {
-                            dp[t][x] = pr * (dp[t][x] - delta[r]);
+                            px[t][r] = mul_f32x2(pr[t][r], add_f32x2(d, both(-delta[r])));
 #pragma unroll
-                            for (int c = 0; c < kFeat; ++c) y[c] += dp[t][x] * fv[c];
+                            for (int c = 0; c < kFeat; ++c) y[c] = fma_f32x2(px[t][r], fv[c], y[c]);
                         }
                     }
                 if (b == 0) fetch_features(1);
                 if constexpr (kForDelta) {
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
-                        sum_px[r] += (dp[0][2 * r] + dp[0][2 * r + 1]) + (dp[1][2 * r] + dp[1][2 * r + 1]);
-                        sum_p[r] += (s[0][2 * r] + s[0][2 * r + 1]) + (s[1][2 * r] + s[1][2 * r + 1]);
+                        float a, c;
+                        unpack_f32x2(add_f32x2(px[0][r], px[1][r]), a, c);
+                        sum_px[r] += a + c;
+                        unpack_f32x2(add_f32x2(pr[0][r], pr[1][r]), a, c);
+                        sum_p[r] += a + c;
                     }
                 } else {
 #pragma unroll
-                    for (int c = 0; c < kFeat; ++c) xf[c] += y[c];
+                    for (int c = 0; c < kFeat; ++c) xf[c] = add_f32x2(xf[c], y[c]);
                     uint32_t xt[3][4];
-                    split_block(dp, xt);
+                    split_block(px, xt);
                     add_product<D>(dq, xt, kt, 32 * half + 16 * b, lane);
                 }
             }
@@ -543,11 +590,13 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
 #pragma unroll
         for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-            for (int x = 0; x < 4; ++x) part[(g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1)] = dq[c][x];
+            for (int r = 0; r < 2; ++r) *(uint64_t*)&part[(g + 8 * r) * D + 8 * c + 2 * t4] = dq[c][r];
     }
 #pragma unroll
     for (int c = 0; c < kFeat; ++c) {
-        double dw = (double)xf[c];
+        float even, odd;
+        unpack_f32x2(xf[c], even, odd);
+        double dw = (double)even + (double)odd;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) dw += __shfl_xor_sync(0xffffffffu, dw, off);
         if (lane == 0) s_dw[warp][c] = dw;
@@ -561,7 +610,9 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_q_kernel(FeatureArgs 
 #pragma unroll
             for (int c = 0; c < D / 8; ++c) {
                 const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
-                store_pair<kAligned>(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4, (dq[c][2 * r] + x2[0]) * p.scale, (dq[c][2 * r + 1] + x2[1]) * p.scale);
+                float x, y;
+                unpack_f32x2(dq[c][r], x, y);
+                store_pair<kAligned>(p.dq + ((size_t)i * p.n_heads + h) * D + 8 * c + 2 * t4, (x + x2[0]) * p.scale, (y + x2[1]) * p.scale);
             }
         }
     }
@@ -581,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
     constexpr int kTileBytes = kTile * 2 * D;
     __shared__ __align__(128) uint8_t s_tiles[4 * kTileBytes];                    // two stages of Q and dO
     __shared__ __align__(128) uint8_t s_own[2 * kRows * 2 * D];                   // the rows' K and V
-    __shared__ float2 s_row[2][kTile];                                            // {lse, Delta} of the queries
+    __shared__ __align__(16) float s_lse[2][kTile], s_delta[2][kTile];            // minus lse and minus Delta of the queries
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 1, half = warp & 1;
     const int h = blockIdx.y;
     const int32_t n = p.n, j0 = (int32_t)blockIdx.x * kRows + 16 * group;
@@ -594,20 +645,19 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
         for (int off = 16; off >= 4; off >>= 1) dw += __shfl_xor_sync(0xffffffffu, dw, off);
         if (lane < kFeat) p.dweights[h * kFeat + lane] = (float)dw;
     }
-    float w[kFeat];
+    uint64_t w[kFeat];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) w[c] = p.weights[h * kFeat + c];
+    for (int c = 0; c < kFeat; ++c) w[c] = both(p.weights[h * kFeat + c]);
+    const uint64_t scale = both(p.scale);
 
     const uint32_t own_k = smem_addr(s_own), own_v = own_k + kRows * 2 * D;
     Tile<D>::template fetch<kRows, kAligned>(own_k, p.k, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     Tile<D>::template fetch<kRows, kAligned>(own_v, p.v, n, p.n_heads, h, (int32_t)blockIdx.x * kRows);
     cp_commit();
 
-    float dk[D / 8][4], dv[D / 8][4];
+    uint64_t dk[D / 8][2], dv[D / 8][2];
 #pragma unroll
-    for (int c = 0; c < D / 8; ++c)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) dk[c][x] = dv[c][x] = 0.f;
+    for (int c = 0; c < D / 8; ++c) dk[c][0] = dk[c][1] = dv[c][0] = dv[c][1] = 0ull;
     const int32_t n_tiles = (n + kTile - 1) / kTile;
     auto stage = [&](int32_t tile) {
         const uint32_t at = base + (uint32_t)(tile & 1) * 2 * kTileBytes;
@@ -616,7 +666,8 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
         cp_commit();
         if (threadIdx.x < kTile) {
             const int32_t i = tile * kTile + (int32_t)threadIdx.x;
-            s_row[tile & 1][threadIdx.x] = i < n ? make_float2(p.lse_in[(size_t)h * n + i], p.delta[(size_t)h * n + i]) : make_float2(INFINITY, 0.f);
+            s_lse[tile & 1][threadIdx.x] = i < n ? -p.lse_in[(size_t)h * n + i] : -INFINITY;
+            s_delta[tile & 1][threadIdx.x] = i < n ? -p.delta[(size_t)h * n + i] : 0.f;
         }
     };
     stage(0);
@@ -639,20 +690,26 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
 #pragma unroll 1
         for (int b = 0; b < 2; ++b) {
             float s[2][4], dp[2][4];
+            uint64_t pr[2][2], ds[2][2];
             two_scores<D>(s, own_k, dp, own_v, 16 * group, qt, dt, 32 * half + 16 * b, lane);
 #pragma unroll
-            for (int t = 0; t < 2; ++t)
+            for (int t = 0; t < 2; ++t) {
+                const int i = 32 * half + 16 * b + 8 * t + 2 * t4;
+                const uint64_t lse = *(const uint64_t*)&s_lse[tile & 1][i], delta = *(const uint64_t*)&s_delta[tile & 1][i];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const float2 row = s_row[tile & 1][32 * half + 16 * b + 8 * t + 2 * t4 + (x & 1)];
-                    s[t][x] = exp_of((s[t][x] * p.scale + bias_of(f[t][x], w)) - row.x);        // 0 for queries past the end
-                    dp[t][x] = s[t][x] * (dp[t][x] - row.y);
+                for (int r = 0; r < 2; ++r) {
+                    uint64_t fv[kFeat];
+                    unpack_features(f[t][2 * r], f[t][2 * r + 1], fv);
+                    const uint64_t x = fma_f32x2(pack_f32x2(s[t][2 * r], s[t][2 * r + 1]), scale, bias_of(fv, w));
+                    pr[t][r] = exp_of(add_f32x2(x, lse));                         // 0 for queries past the end
+                    ds[t][r] = mul_f32x2(pr[t][r], add_f32x2(pack_f32x2(dp[t][2 * r], dp[t][2 * r + 1]), delta));
                 }
+            }
             if (b == 0) fetch_features(1);
             uint32_t terms[3][4];
-            split_block(s, terms);
+            split_block(pr, terms);
             add_product<D>(dv, terms, dt, 32 * half + 16 * b, lane);
-            split_block(dp, terms);
+            split_block(ds, terms);
             add_product<D>(dk, terms, qt, 32 * half + 16 * b, lane);
         }
         __syncthreads();
@@ -662,10 +719,10 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
 #pragma unroll
         for (int c = 0; c < D / 8; ++c)
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int at = (g + 8 * (x >> 1)) * D + 8 * c + 2 * t4 + (x & 1);
-                part[at] = dk[c][x];
-                part[16 * D + at] = dv[c][x];
+            for (int r = 0; r < 2; ++r) {
+                const int at = (g + 8 * r) * D + 8 * c + 2 * t4;
+                *(uint64_t*)&part[at] = dk[c][r];
+                *(uint64_t*)&part[16 * D + at] = dv[c][r];
             }
     }
     __syncthreads();
@@ -678,8 +735,11 @@ __global__ void __launch_bounds__(kThreads, 3) feature_bwd_kv_kernel(FeatureArgs
             for (int c = 0; c < D / 8; ++c) {
                 const float* x2 = part + (g + 8 * r) * D + 8 * c + 2 * t4;
                 const size_t at = ((size_t)j * p.n_heads + h) * D + 8 * c + 2 * t4;
-                store_pair<kAligned>(p.dk + at, (dk[c][2 * r] + x2[0]) * p.scale, (dk[c][2 * r + 1] + x2[1]) * p.scale);
-                store_pair<kAligned>(p.dv + at, dv[c][2 * r] + x2[16 * D], dv[c][2 * r + 1] + x2[16 * D + 1]);
+                float x, y;
+                unpack_f32x2(dk[c][r], x, y);
+                store_pair<kAligned>(p.dk + at, (x + x2[0]) * p.scale, (y + x2[1]) * p.scale);
+                unpack_f32x2(dv[c][r], x, y);
+                store_pair<kAligned>(p.dv + at, x + x2[16 * D], y + x2[16 * D + 1]);
             }
         }
     }
