@@ -234,13 +234,14 @@ def run_cuda(args) -> int:
             marks[4].record()
 
     # spd: one pull kernel where it needs no workspace beyond the header; a larger single graph: order, lists and pull, or beyond
-    # 18 944 nodes setup, two item scans, item table and bit-matrix BFS; a larger batch: setup, components, BFS.
-    # fwd: (a batch's maps and work list,) main; bwd: prepare, main, finalize; chunked: partial, merge
+    # 18 944 nodes two item scans, item table and bit-matrix BFS, from 32 768 to 65 536 nodes with the choice of a core (seven kernels),
+    # a second form of the BFS and two of the expansion; a larger batch: setup, components, BFS.
+    # fwd: (a batch's maps and work list,) main; bwd: prepare, main, finalize; chunked: main (in parts: partial, merge)
     dense_spd = single and b.max_seqlen > 18944           # the library's switch to the bit-matrix build
     spd_kernel = ("spd_pull_kernel" if ws_spd.numel() <= 256 else "spd_dense_kernel" if dense_spd else
                   "spd_large_pull_kernel" if single else "spd_bfs_kernel")
-    spd_launches = 1 if spd_kernel == "spd_pull_kernel" else (5 if dense_spd else 3)
-    kernels_per_step = spd_launches + (1 if single else 2) + 3 + (2 if single else 0)
+    spd_launches = 1 if spd_kernel == "spd_pull_kernel" else ((14 if 32768 <= b.max_seqlen <= 65536 else 4) if dense_spd else 3)
+    kernels_per_step = spd_launches + (1 if single else 2) + 3 + (1 if single else 0)
 
     for _ in range(max(args.warmup, 0)):
         step()

@@ -20,11 +20,11 @@
 //
 // mma.sync and not tcgen05: at the 500 - 8 192 nodes this form is meant for, a 128-row tile per thread block would leave
 // most SMs empty, and the three-term operands would have to travel through tensor memory.
-// What bounds it: latency at ten warps per SM (1 500 nodes have no more rows); 12 of the 19 contractions are the terms of P and
-// dS.  What bounds it: the latency of an element's chain of instructions at two and a half warps per scheduler (issue slots 45 %, tensor
-// pipe 33-42 % busy); fp32 arithmetic goes by pairs (one instruction, the same results), and a chain's first MMA adds to zero.
-// 1 500 nodes, H = 8, d = 64: forward 60 us, backward 195 us (64 and 199 element by element; 54 and 172 with one chain of MMAs over all keys, ex2 in the
-// forward and one walk on the query side, whose results are further off); the same sums on the fp32 pipes took 3 000 us.
+// What bounds it: the latency of an element's chain of instructions at ten warps per SM (1 500 nodes have no more rows; issue slots
+// 45 %, tensor pipe 33-42 % busy).  12 of the 19 contractions are the terms of P and dS; fp32 arithmetic goes by pairs of neighbouring
+// columns (one instruction, the same results), and a chain's first MMA adds to zero.  1 500 nodes, H = 8, d = 64: forward 60 us,
+// backward 195 us (64 and 199 element by element; 54 and 172 with one chain of MMAs over all keys, ex2 in the forward and one walk on
+// the query side, whose results are further off); the same sums on the fp32 pipes took 3 000 us.
 #include <cuda_bf16.h>
 #include <math.h>
 

@@ -19,6 +19,7 @@
 // written once, unreachable pairs of graphs deeper than max_dist twice, so the HBM traffic is the matrix plus the CSR.
 // The frontier / next / visited words live in shared memory when 12 bytes per vertex fit, otherwise in an L2-resident slice
 // of the workspace.
+#include "spd_core.cuh"
 #include "spd_pull.cuh"
 
 namespace gt {
@@ -375,7 +376,8 @@ __global__ void __launch_bounds__(1024, kSmemState ? 1 : 2) spd_bfs_kernel(SpdPa
 // handed out in batches from a counter.  Rows of empty frontiers are not read, complete vertices are
 // skipped, and a vertex stops reading neighbours once everything it still misses is covered.
 // The frontiers of the first levels are kept, and one pass writes their distances and everything else
-// of a column block; later levels blend their distances into the bytes that are there.  Cost model: per level and column block nnz x 1 KB of row reads (L2 / HBM),
+// of a column block; later levels blend their distances into the bytes that are there.  From 32 768 to 65 536 vertices the targets
+// that follow from others are left out (spd_core.cu), and the expansion reads the frontiers in place of that pass.  Cost model: per level and column block nnz x 1 KB of row reads (L2 / HBM),
 // so a graph of large diameter is slow here (levels x blocks barriers) - the kernel is meant for the
 // small-world graphs of the paper's workloads.
 // ------------------------------------------------------------------------------------------
@@ -384,29 +386,32 @@ constexpr int kDenseRowWords = kDenseBlockBits / 32;     // 256 words = 1 KB per
 constexpr int kDenseVecs = kDenseRowWords / 128;         // 16-byte vectors per lane and row
 constexpr int kDenseChunk = 32;                          // out-edges per work item
 constexpr int kDenseBatch = 4;                           // work items a warp takes at a time
-constexpr int kDenseMaxGroups = 4;                       // CTA groups working on different column blocks at once
-constexpr int kDenseHist = 6;                            // levels whose frontier matrices are kept for the output pass (later levels blend into written rows)
-constexpr size_t kDenseSyncBytes = (size_t)(256 + 4 * kDenseRowWords * 4) * kDenseMaxGroups;       // sync words, then live targets
-constexpr int kDensePlanes = kDenseHist + 1;             // frontier matrices per group (level 0 .. kDenseHist)
+constexpr int kDenseMaxGroups = 4;                       // CTA groups working on different column blocks at once (one more where only a core is searched for)
+constexpr int kDensePlanes = 7;                          // levels whose frontier matrices are kept, with blocks of 8192 (more with narrower ones): the output
+                                                         // pass reads them, later levels blend into written rows
+constexpr size_t kDenseSyncBytes = (size_t)(256 + 4 * kDenseRowWords * 4) * kCoreMaxGroups;        // sync words, then live targets
 constexpr int kDenseFlagWords = 8192;                    // row flags of a level kept as a bitmap in shared memory (graphs up to 262 144 vertices)
 constexpr uint32_t kGridWaitIterations = 1u << 24;
 
 struct DenseParams {
-    uint32_t* vis;          // [n_max][kDenseRowWords]
-    uint32_t* fr;           // [kDensePlanes][n_max][kDenseRowWords] frontier of level l in plane l (later levels: planes 0 / 1 in turn)
-    uint32_t* acc;          // [acc_rows][kDenseRowWords] accumulator rows of split vertices (all zero between uses)
+    uint32_t* vis;          // [n_max][row words]
+    uint32_t* fr;           // [planes][n_max][row words] frontier of level l in plane l - 1 (levels beyond the planes: 0 / 1 in turn)
+    uint32_t* acc;          // [acc_rows][row words] accumulator rows of split vertices (all zero between uses)
     int32_t* acc_row;       // [n_max] accumulator row of a split vertex (vertices with more than kDenseChunk out-edges)
     int32_t acc_rows;       // accumulator rows per CTA group
     uint32_t* acc_cnt;      // [n_max] finished chunks of a split vertex
-    uint8_t* nonempty;      // [kDensePlanes][n_pad] the row of that plane is valid and has a bit set (rows without the flag are never read)
+    uint8_t* nonempty;      // [kCoreMaxLevels][n_pad] the row of that plane is valid and has a bit set (rows without the flag are never read)
+    uint32_t* slots;        // [kCoreMaxLevels][n_pad] where the row is, of a level without a plane of its own (core only)
     uint8_t* row_done;      // [n_max] every valid target of the block is visited
     int32_t* item_start;    // [n_max + 1] prefix sum of chunks per vertex (of the current graph)
     int4* item_rec;         // [n_items] {vertex, first edge, one past the last edge, chunks of the vertex} of a work item
     uint32_t* live;         // [4][kDenseRowWords] targets that some vertex gained, by level mod 4
-    uint32_t* sync;         // [0] barrier counter, [1] abort, [2..5] "some frontier bit" and [8..11] work counter, by level mod 4
+    uint32_t* sync;         // [0] barrier counter, [1] abort, [2..5] "some frontier bit", [8..11] work counter and [12..15] rows taken of the pool, by level mod 4
     int32_t n_max;
     int32_t n_pad;          // n_max rounded up to 32: pitch of the flag arrays
     int32_t n_groups;       // CTA groups that work on different column blocks at the same time (own state each)
+    CoreInfo* core;         // which targets are searched for; nullptr: all
+    const int32_t* column;  // [n_max] column of a vertex as a target, -1: none (where *core says so)
     uint32_t barrier_extra; // test hook: arrivals the grid barrier waits for beyond the thread blocks that exist (normally 0)
     uint32_t barrier_limit; // polls of the barrier word before a thread block gives up
 };
@@ -578,18 +583,29 @@ __device__ __forceinline__ void dense_blend_word(uint8_t* row, int32_t t0, uint3
 // vector q of all lanes together is a contiguous 512-byte piece of the row
 __device__ __forceinline__ int dense_word(int lane, int q, int j) { return q * 128 + lane * 4 + j; }
 
+// kCore: only the targets that *d.core names are searched for, with rows of what length they need (1 % to 10 % on top where all are).
+// Of the two launched kernels the one that it does not say so returns.
+template <bool kCore>
 __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DenseParams d)
 {
+    if ((d.core != nullptr && d.core->reduced != 0) != kCore) return;
     // CTA group g (CTAs g, g + G, ...) works on column blocks g, g + G, ... with its own bit matrices, flags
     // and barrier: while one group waits for its slowest warp at a level barrier, the CTAs of the other groups
     // on the same SMs keep the memory system busy.
+    const int block_bits = kCore ? d.core->block_bits : kDenseBlockBits;
+    const int row_words = kCore ? block_bits / 32 : kDenseRowWords;
+    // Levels that have a plane each; only few rows gain anything at later ones, and in a search for a core those take rows of a
+    // pool in turn, until it might overflow (pool_rows: room for one level's rows in full at its beginning).
+    const int n_planes = kCore ? d.core->n_planes : kDensePlanes, n_direct = kCore ? d.core->n_direct : kDensePlanes;
+    if (kCore) d.n_groups = d.core->n_groups;
     const int grp = (int)blockIdx.x % d.n_groups;
     const int cta = (int)blockIdx.x / d.n_groups;                                   // index within the group
     const uint32_t n_ctas = ((uint32_t)gridDim.x - (uint32_t)grp + (uint32_t)d.n_groups - 1u) / (uint32_t)d.n_groups;
     {
         const size_t m = (size_t)grp * d.n_max;
-        d.vis += m * kDenseRowWords; d.fr += m * kDensePlanes * kDenseRowWords; d.acc += (size_t)grp * d.acc_rows * kDenseRowWords;
-        d.acc_cnt += m; d.nonempty += (size_t)grp * d.n_pad * kDensePlanes; d.row_done += m;
+        d.vis += m * row_words; d.fr += m * n_planes * row_words; d.acc += (size_t)grp * d.acc_rows * row_words;
+        d.acc_cnt += m; d.nonempty += (size_t)grp * d.n_pad * kCoreMaxLevels; d.row_done += m;
+        d.slots += (size_t)grp * d.n_pad * kCoreMaxLevels;
         d.sync += grp * 64;
         d.live += grp * 4 * kDenseRowWords;
     }
@@ -598,30 +614,39 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     const int n_gw = (int)((n_ctas * blockDim.x) >> 5);
     const int32_t n = p.n_total;
     const int64_t ld = (int64_t)((n + 15) & ~15);
+    const int32_t n_cols = kCore ? d.core->n_cols : n;                              // targets, and what is written of a row
+    const int32_t out_cols = kCore ? (n_cols + 15) & ~15 : (int32_t)ld;
+    auto column = [&](int v) -> int32_t { return kCore ? d.column[v] : v; };
+    // a lane's vector q of a row (below) is inside the row
+    auto inside = [&](int q) -> bool { return !kCore || q * 128 + ((int)threadIdx.x & 31) * 4 < row_words; };
     const int32_t* __restrict__ ci = p.col_idx;
     const int32_t n_items = d.item_start[n];
     const uint32_t unreach = (uint32_t)(p.max_dist + 1);
-    __shared__ uint32_t s_flags[kDenseFlagWords];
+    __shared__ __align__(16) uint32_t s_flags[kDenseFlagWords];
     __shared__ __align__(16) uint32_t s_live[kDenseRowWords], s_gained[kDenseRowWords];
     const bool flags_in_smem = n <= kDenseFlagWords * 32;
+    // one item at a time where a warp has few (a batch is one chain of loads after the other)
+    const int batch_items = kCore ? min(kDenseBatch, max(1, n_items / (4 * n_gw))) : kDenseBatch;
     uint32_t epoch = 0;
+    uint32_t pool_used = 0;                    // rows of the pool that the levels so far hold
     uint32_t step = 0;                         // levels over all column blocks: index of the rotating "any" flags
 
     // finalise vertex s for this level: new bits (left in acc), visited, next frontier row, flags.  While the
     // levels still have a plane each (blend == false) no output byte is written here: the output pass reads the
     // planes once.  Later levels blend their bytes into the rows that pass has written.
-    auto finalise = [&](int s, uint32_t (&acc)[kDenseVecs][4], int32_t col0, uint32_t* vis_row, uint32_t* next_row,
+    auto finalise = [&](int s, uint32_t (&acc)[kDenseVecs][4], int32_t col0, uint32_t* vis_row, uint32_t* next, uint32_t* next_slot,
                         uint8_t* next_nonempty, uint32_t code, uint32_t flag_idx, bool blend) {
         bool any_new = false, full = true;
 #pragma unroll
         for (int q = 0; q < kDenseVecs; ++q) {
+            if (!inside(q)) continue;
             const uint4 v4 = __ldcg((const uint4*)&vis_row[dense_word(lane, q, 0)]);   // written by other SMs earlier: from L2
             const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
             bool vec_new = false;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int32_t t0 = col0 + dense_word(lane, q, j) * 32;
-                const uint32_t vm = dense_valid(n - t0);
+                const uint32_t vm = dense_valid(n_cols - t0);
                 acc[q][j] &= ~v[j] & vm;
                 if (acc[q][j]) {
                     if (blend) dense_blend_word(p.spd + (int64_t)s * ld, t0, acc[q][j], code);
@@ -642,9 +667,15 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
         const bool row_new = __any_sync(0xffffffffu, any_new);
         const bool row_full = __all_sync(0xffffffffu, full);
         if (row_new) {                 // the whole row, zeros included: a flagged row is read in full
+            uint32_t at = (uint32_t)s;
+            if (kCore && next_slot != nullptr) {
+                if (lane == 0) { at = pool_used + atomicAdd(&d.sync[12 + flag_idx], 1u); next_slot[s] = at; }
+                at = __shfl_sync(0xffffffffu, at, 0);
+            }
+            uint32_t* next_row = next + (size_t)at * row_words;
 #pragma unroll
             for (int q = 0; q < kDenseVecs; ++q)
-                *(uint4*)&next_row[dense_word(lane, q, 0)] = make_uint4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+                if (inside(q)) *(uint4*)&next_row[dense_word(lane, q, 0)] = make_uint4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
         }
         if (lane == 0) {
             next_nonempty[s] = row_new ? 1 : 0;
@@ -657,13 +688,15 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     // of levels 1..n_levels (a pair is in at most one of them): its level, clamped; 0 on the diagonal; the
     // unreachable code where no plane has the pair (later levels, if any, overwrite that); 255 in the padding.
     auto emit_rows = [&](int32_t col0, int n_levels) {
-        static_assert(kDenseHist <= 15, "four bit slices hold the level codes");
+        static_assert(kDensePlanes <= 15 && kCoreMaxLevels <= 15, "four bit slices hold the level codes");
         for (int s = gw; s < n; s += n_gw) {
             uint8_t* row = p.spd + (int64_t)s * ld;
-            const uint32_t fl = (lane >= 1 && lane <= n_levels) ? (uint32_t)__ldcg(&d.nonempty[(size_t)lane * d.n_pad + s]) : 0u;
+            const uint32_t fl = (lane >= 1 && lane <= n_levels) ? (uint32_t)__ldcg(&d.nonempty[(size_t)(lane - 1) * d.n_pad + s]) : 0u;
             const uint32_t valid = __ballot_sync(0xffffffffu, fl != 0u);
+            const int32_t own = column(s);
 #pragma unroll
             for (int q = 0; q < kDenseVecs; ++q) {
+                if (!inside(q)) continue;
                 uint32_t cb[4][4], found[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) { found[j] = 0u; cb[0][j] = cb[1][j] = cb[2][j] = cb[3][j] = 0u; }
@@ -672,9 +705,13 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                     m &= m - 1;
                     int l1 = 0;
                     if (m) { l1 = __ffs(m) - 1; m &= m - 1; }
-                    const uint4 x = __ldcg((const uint4*)&d.fr[((size_t)l0 * d.n_max + s) * kDenseRowWords + dense_word(lane, q, 0)]);
+                    auto row_of = [&](int l) -> const uint32_t* {
+                        const size_t at = !kCore || l <= n_direct ? (size_t)(l - 1) * d.n_max + s : (size_t)n_direct * d.n_max + __ldcg(&d.slots[(size_t)(l - 1) * d.n_pad + s]);
+                        return d.fr + at * row_words + dense_word(lane, q, 0);
+                    };
+                    const uint4 x = __ldcg((const uint4*)row_of(l0));
                     uint4 y = make_uint4(0u, 0u, 0u, 0u);
-                    if (l1) y = __ldcg((const uint4*)&d.fr[((size_t)l1 * d.n_max + s) * kDenseRowWords + dense_word(lane, q, 0)]);
+                    if (l1) y = __ldcg((const uint4*)row_of(l1));
                     const uint32_t c0 = (uint32_t)min(l0, p.max_dist), c1 = (uint32_t)min(l1, p.max_dist);
                     const uint32_t xw[4] = {x.x, x.y, x.z, x.w}, yw[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
@@ -689,9 +726,9 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int32_t t0 = col0 + dense_word(lane, q, j) * 32;
-                    if (t0 >= (int32_t)ld) continue;
-                    const uint32_t vm = dense_valid(n - t0), pm = ~vm;
-                    const uint32_t miss = ~found[j] & ~dense_bit(s - t0) & vm;
+                    if (t0 >= out_cols) continue;
+                    const uint32_t vm = dense_valid(n_cols - t0), pm = ~vm;
+                    const uint32_t miss = ~found[j] & ~dense_bit(own - t0) & vm;
                     uint32_t o[8];
                     nibbles<false>(cb[0][j], cb[1][j], cb[2][j], cb[3][j], o);
 #pragma unroll
@@ -699,43 +736,48 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                         o[k] |= ((miss >> k) & 0x01010101u) * unreach;
                         if (pm) o[k] |= ((pm >> k) & 0x01010101u) * 255u;
                     }
-                    store_row_piece(row + t0, o, (int32_t)ld - t0);
+                    store_row_piece(row + t0, o, out_cols - t0);
                 }
             }
         }
     };
 
-    for (int32_t col0 = grp * kDenseBlockBits; col0 < (int32_t)ld; col0 += d.n_groups * kDenseBlockBits) {
+    for (int32_t col0 = grp * block_bits; col0 < out_cols; col0 += d.n_groups * block_bits) {
         // ---- level 0 of this column block: every vertex has reached itself ----
         for (int s = gw; s < n; s += n_gw) {
-            const bool mine = s >= col0 && s < col0 + kDenseBlockBits;
+            const int32_t own = column(s) - col0;
 #pragma unroll
             for (int q = 0; q < kDenseVecs; ++q) {
                 uint32_t bit[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    bit[j] = dense_bit(s - col0 - dense_word(lane, q, j) * 32);
+                    bit[j] = dense_bit(own - dense_word(lane, q, j) * 32);
                 }
-                const uint4 b4 = make_uint4(bit[0], bit[1], bit[2], bit[3]);
-                *(uint4*)&d.vis[(size_t)s * kDenseRowWords + dense_word(lane, q, 0)] = b4;
-                if (mine) *(uint4*)&d.fr[(size_t)s * kDenseRowWords + dense_word(lane, q, 0)] = b4;      // plane 0
+                if (inside(q)) *(uint4*)&d.vis[(size_t)s * row_words + dense_word(lane, q, 0)] = make_uint4(bit[0], bit[1], bit[2], bit[3]);
             }
-            if (lane < kDensePlanes) d.nonempty[(size_t)lane * d.n_pad + s] = (lane == 0 && mine) ? 1 : 0;
+            if (lane < kCoreMaxLevels) d.nonempty[(size_t)lane * d.n_pad + s] = 0;
             if (lane == 0) d.row_done[s] = 0;
         }
         if (!dense_grid_sync(d.sync, epoch, p.header, n_ctas, d.barrier_extra, d.barrier_limit)) return;
 
         bool emitted = false;                  // the output pass of this column block has run
+        int last_kept = 0;                     // levels that it has read
         for (int level = 1;; ++level) {
             const uint32_t code = (uint32_t)min(level, p.max_dist);
             const uint32_t flag_idx = step & 3u;
-            // level l <= kDenseHist writes plane l; later levels take planes 0 and 1 in turn (free after the output pass)
-            const int pl_cur = level - 1 <= kDenseHist ? level - 1 : ((level - kDenseHist) & 1);
-            const int pl_next = level <= kDenseHist ? level : ((level - kDenseHist - 1) & 1);
-            const uint32_t* fcur = d.fr + (size_t)pl_cur * d.n_max * kDenseRowWords;
-            uint32_t* fnext = d.fr + (size_t)pl_next * d.n_max * kDenseRowWords;
-            const uint8_t* ne_cur = d.nonempty + (size_t)pl_cur * d.n_pad;
-            uint8_t* ne_next = d.nonempty + (size_t)pl_next * d.n_pad;
+            // Level l <= n_direct writes plane l - 1, further ones up to the output pass write rows of the pool; the levels behind it take
+            // planes 0 and 1 in turn, which are free then.  Level 1 reads the edges only.
+            const bool late = kCore && !emitted && level > n_direct, from_pool = kCore && level - 1 > n_direct && (!emitted || level - 1 == last_kept);
+            const int turn = (level - last_kept) & 1;
+            const int pl_cur = emitted && level - 1 > last_kept ? turn : (from_pool ? n_direct : max(level - 2, 0));
+            const int pl_next = emitted ? turn ^ 1 : min(level - 1, n_direct);
+            const int fl_cur = emitted && level - 1 > last_kept ? turn : max(level - 2, 0), fl_next = emitted ? turn ^ 1 : level - 1;
+            const uint32_t* fcur = d.fr + (size_t)pl_cur * d.n_max * row_words;
+            const uint32_t* slot_cur = from_pool ? d.slots + (size_t)(level - 2) * d.n_pad : nullptr;
+            uint32_t* fnext = d.fr + (size_t)pl_next * d.n_max * row_words;
+            uint32_t* slot_next = late ? d.slots + (size_t)(level - 1) * d.n_pad : nullptr;
+            const uint8_t* ne_cur = d.nonempty + (size_t)fl_cur * d.n_pad;
+            uint8_t* ne_next = d.nonempty + (size_t)fl_next * d.n_pad;
             // Targets that some vertex gained at the level before: no other target can be gained at this one (a path to it of this
             // length contains one shorter by a hop), so a vertex that misses only others is done.  Without this the targets in
             // tiny components keep every row open to the last level.
@@ -745,7 +787,10 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
             }
             // The flags of the current frontier as a bitmap in shared memory: an item looks up one per out-edge, and
             // at the first and last levels that look-up is all an item does.
-            if (flags_in_smem) {
+            static_assert(kDenseFlagWords >= 512 / 32 * kDenseRowWords, "a row per warp at level 1");
+            if (level == 1)
+                for (int w = (int)threadIdx.x; w < 512 / 32 * kDenseRowWords; w += (int)blockDim.x) s_flags[w] = 0u;
+            if (flags_in_smem && level > 1) {
                 for (int w = (int)threadIdx.x; w < (n + 31) / 32; w += (int)blockDim.x) {
                     const uint4 a = __ldcg((const uint4*)(ne_cur + 32 * (size_t)w)), b = __ldcg((const uint4*)(ne_cur + 32 * (size_t)w + 16));
                     const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -762,7 +807,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
             // four items of a batch lie a quarter of the list apart: the chunks of one high-degree vertex are
             // neighbours in the list and would otherwise queue up in one warp.
             uint32_t* counter = &d.sync[8 + flag_idx];
-            const int n_batches = (n_items + kDenseBatch - 1) / kDenseBatch;
+            const int n_batches = (n_items + batch_items - 1) / batch_items;
             int batch_next = 0;
             if (lane == 0) batch_next = (int)atomicAdd(counter, 1u);
             for (;;) {
@@ -773,7 +818,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 // item (at most levels most items have none).
                 static_assert(kDenseChunk == 32 && kDenseBatch <= 32, "one edge per lane, one item per lane");
                 const int item = batch + lane * n_batches;
-                const bool valid = lane < kDenseBatch && item < n_items;
+                const bool valid = lane < batch_items && item < n_items;
                 const int4 rec_mine = valid ? d.item_rec[item] : make_int4(0, 0, 0, 1);
                 const bool done = !valid || __ldcg(&d.row_done[rec_mine.x]) != 0;
                 uint32_t m_mine = 0u;                       // the neighbours whose frontier row has a bit set
@@ -786,7 +831,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                     }
 #pragma unroll
                     for (int k = 0; k < kDenseBatch; ++k) {
-                        const bool hit = u[k] >= 0 && (flags_in_smem ? ((s_flags[u[k] >> 5] >> (u[k] & 31)) & 1u) : (uint32_t)__ldcg(&ne_cur[u[k]]));
+                        const bool hit = u[k] >= 0 && (level == 1 ? (uint32_t)((uint32_t)(column(u[k]) - col0) < (uint32_t)block_bits) : flags_in_smem ? ((s_flags[u[k] >> 5] >> (u[k] & 31)) & 1u) : (uint32_t)__ldcg(&ne_cur[u[k]]));
                         const uint32_t hits = __ballot_sync(0xffffffffu, hit);
                         if (lane == k) m_mine = hits;
                     }
@@ -806,23 +851,25 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 for (int q = 0; q < kDenseVecs; ++q)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) acc[q][j] = 0u;
-                uint32_t* vis_row = d.vis + (size_t)s * kDenseRowWords;
+                uint32_t* vis_row = d.vis + (size_t)s * row_words;
                 {
                     uint32_t m = __shfl_sync(0xffffffffu, m_mine, k_item);
                     const int32_t e0 = __shfl_sync(0xffffffffu, rec_mine.y, k_item);
-                    const int32_t u = (m >> lane) & 1u ? ci[e0 + lane] : -1;
+                    int32_t u = (m >> lane) & 1u ? ci[e0 + lane] : -1;
                     if (m) {
                         // bits this vertex still misses and may gain: once the neighbours read so far cover them all, the rest
                         // of the edge list cannot add anything (at the dense levels a few rows are enough)
                         uint32_t need[kDenseVecs][4], open = 0u;
 #pragma unroll
                         for (int q = 0; q < kDenseVecs; ++q) {
+                            need[q][0] = need[q][1] = need[q][2] = need[q][3] = 0u;
+                            if (!inside(q)) continue;
                             const uint4 v4 = __ldcg((const uint4*)&vis_row[dense_word(lane, q, 0)]);
                             const uint4 l4 = *(const uint4*)&s_live[dense_word(lane, q, 0)];
                             need[q][0] = ~v4.x & l4.x; need[q][1] = ~v4.y & l4.y; need[q][2] = ~v4.z & l4.z; need[q][3] = ~v4.w & l4.w;
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                if (level == 1) need[q][j] &= dense_valid(n - (col0 + dense_word(lane, q, j) * 32));     // (later, no others are live)
+                                if (level == 1) need[q][j] &= dense_valid(n_cols - (col0 + dense_word(lane, q, j) * 32));     // (later, no others are live)
                                 open |= need[q][j];
                             }
                         }
@@ -833,6 +880,22 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                             }
                             m = 0u;                                   // (every chunk of a split vertex has to be counted)
                         }
+                        if (level == 1) {                             // the neighbours themselves, put together in the warp's row of s_flags
+                            uint32_t* mine = s_flags + ((int)threadIdx.x >> 5) * kDenseRowWords;
+                            const int32_t target = u >= 0 && m ? column(u) - col0 : 0;
+                            if (u >= 0 && m) atomicOr(&mine[target >> 5], dense_bit(target & 31));
+                            __syncwarp();
+#pragma unroll
+                            for (int q = 0; q < kDenseVecs; ++q) {
+                                const uint4 a4 = *(const uint4*)&mine[dense_word(lane, q, 0)];
+                                acc[q][0] = a4.x; acc[q][1] = a4.y; acc[q][2] = a4.z; acc[q][3] = a4.w;
+                            }
+                            __syncwarp();
+                            if (u >= 0 && m) mine[target >> 5] = 0u;
+                            __syncwarp();
+                            m = 0u;
+                        }
+                        if (kCore && slot_cur != nullptr && u >= 0) u = (int32_t)__ldcg(&slot_cur[u]);
                         while (m) {                                   // two frontier rows (2 x 1 KB) in flight
                             const int b0 = __ffs(m) - 1;
                             m &= m - 1;
@@ -840,15 +903,17 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                             int u1 = -1;
                             if (m) { const int b1 = __ffs(m) - 1; m &= m - 1; u1 = __shfl_sync(0xffffffffu, u, b1); }
                             uint4 x[kDenseVecs], y[kDenseVecs];
-                            const uint32_t* r0 = fcur + (size_t)u0 * kDenseRowWords;
+                            const uint32_t* r0 = fcur + (size_t)u0 * row_words;
 #pragma unroll
-                            for (int q = 0; q < kDenseVecs; ++q) x[q] = __ldcg((const uint4*)&r0[dense_word(lane, q, 0)]);
-#pragma unroll
-                            for (int q = 0; q < kDenseVecs; ++q) y[q] = make_uint4(0u, 0u, 0u, 0u);
+                            for (int q = 0; q < kDenseVecs; ++q) {
+                                x[q] = y[q] = make_uint4(0u, 0u, 0u, 0u);
+                                if (inside(q)) x[q] = __ldcg((const uint4*)&r0[dense_word(lane, q, 0)]);
+                            }
                             if (u1 >= 0) {
-                                const uint32_t* r1 = fcur + (size_t)u1 * kDenseRowWords;
+                                const uint32_t* r1 = fcur + (size_t)u1 * row_words;
 #pragma unroll
-                                for (int q = 0; q < kDenseVecs; ++q) y[q] = __ldcg((const uint4*)&r1[dense_word(lane, q, 0)]);
+                                for (int q = 0; q < kDenseVecs; ++q)
+                                    if (inside(q)) y[q] = __ldcg((const uint4*)&r1[dense_word(lane, q, 0)]);
                             }
 #pragma unroll
                             for (int q = 0; q < kDenseVecs; ++q) {
@@ -864,11 +929,10 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                         }
                     }
                 }
-                uint32_t* next_row = fnext + (size_t)s * kDenseRowWords;
                 if (n_chunks == 1) {
-                    finalise(s, acc, col0, vis_row, next_row, ne_next, code, flag_idx, emitted);
+                    finalise(s, acc, col0, vis_row, fnext, slot_next, ne_next, code, flag_idx, emitted);
                 } else {
-                    uint32_t* acc_row = d.acc + (size_t)d.acc_row[s] * kDenseRowWords;
+                    uint32_t* acc_row = d.acc + (size_t)d.acc_row[s] * row_words;
 #pragma unroll
                     for (int q = 0; q < kDenseVecs; ++q)
 #pragma unroll
@@ -883,12 +947,13 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                         __threadfence();
 #pragma unroll
                         for (int q = 0; q < kDenseVecs; ++q) {
+                            if (!inside(q)) continue;
                             const uint4 a4 = __ldcg((const uint4*)&acc_row[dense_word(lane, q, 0)]);
                             acc[q][0] = a4.x; acc[q][1] = a4.y; acc[q][2] = a4.z; acc[q][3] = a4.w;
                             if (a4.x | a4.y | a4.z | a4.w) *(uint4*)&acc_row[dense_word(lane, q, 0)] = make_uint4(0u, 0u, 0u, 0u);
                         }
                         if (lane == 0) d.acc_cnt[s] = 0u;
-                        finalise(s, acc, col0, vis_row, next_row, ne_next, code, flag_idx, emitted);
+                        finalise(s, acc, col0, vis_row, fnext, slot_next, ne_next, code, flag_idx, emitted);
                     }
                 }
               }
@@ -898,14 +963,24 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 if (s_gained[w]) atomicOr(&d.live[(step & 3u) * kDenseRowWords + w], s_gained[w]);
             if (!dense_grid_sync(d.sync, epoch, p.header, n_ctas, d.barrier_extra, d.barrier_limit)) return;
             const uint32_t any = *(volatile uint32_t*)&d.sync[2 + flag_idx];
+            if (late) pool_used += *(volatile uint32_t*)&d.sync[12 + flag_idx];
             if (cta == 0 && threadIdx.x == 0) {                 // next written two levels from now
                 d.sync[2 + ((step + 2u) & 3u)] = 0u;
                 d.sync[8 + ((step + 2u) & 3u)] = 0u;
+                d.sync[12 + ((step + 2u) & 3u)] = 0u;
             }
             if (cta == 0)
                 for (int w = (int)threadIdx.x; w < kDenseRowWords; w += (int)blockDim.x) d.live[((step + 2u) & 3u) * kDenseRowWords + w] = 0u;
             ++step;
-            if (!emitted && (!any || level == kDenseHist)) {
+            if (kCore && !emitted && !any) {                     // all levels have a plane: the expansion reads them
+                if (cta == 0 && threadIdx.x == 0) d.core->levels[grp] = level;
+                break;
+            }
+            // The next level needs a plane, or a row of the pool for every vertex.
+            const bool no_room = level >= n_direct && (!kCore || level == kCoreMaxLevels || pool_used > (uint32_t)(kCorePoolPlanes - 1) * (uint32_t)n);
+            if (!emitted && (!any || no_room)) {
+                last_kept = level;
+                if (kCore && cta == 0 && threadIdx.x == 0) { d.core->levels[grp] = 0; d.core->deep = 1; }
                 emit_rows(col0, level);
                 emitted = true;
                 // levels that follow blend into rows this pass wrote from other SMs
@@ -932,6 +1007,8 @@ struct SpdPlan {
     bool dense;                // single large graph: bit-matrix BFS (persistent cooperative kernel)
     int dense_groups;
     size_t dense_off[10];      // vis, frontier planes, acc, acc_cnt, nonempty flags, row_done, item_start, sync, item_rec, acc_row
+    size_t slots_off;
+    CorePlan core;             // behind them
     int32_t dense_acc_rows;    // accumulator rows per CTA group: a bound on the vertices with more than kDenseChunk out-edges
     int threads;
     int grid;
@@ -983,33 +1060,37 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
     // overtakes the multi-source BFS between 14 000 and 15 000 nodes (16 384 nodes: 0.98 against 1.65 ms), before the BFS
     // state stops fitting shared memory at 17 066.
     if ((!pl.smem_state || b->n_total >= kDenseMinNodes) && b->n_graphs == 1) {
-        int dev = 0, coop = 0, per_sm_dense = 0;
+        int dev = 0, coop = 0, per_sm_dense = 0, per_sm_core = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_dense, spd_dense_kernel, 512, 0) == cudaSuccess && per_sm_dense >= 1) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_dense, spd_dense_kernel<false>, 512, 0) == cudaSuccess && per_sm_dense >= 1 &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_core, spd_dense_kernel<true>, 512, 0) == cudaSuccess && per_sm_core >= 1) {
+            if (per_sm_core < per_sm_dense) per_sm_dense = per_sm_core;
             pl.dense = true;
             pl.threads = 512;
             pl.grid = sms * per_sm_dense;
             const size_t n = (size_t)b->n_total;
             const int n_col_blocks = (int)((n + 15 + kDenseBlockBits - 1) / kDenseBlockBits);
             pl.dense_groups = n_col_blocks < kDenseMaxGroups ? n_col_blocks : kDenseMaxGroups;
-            const size_t G = (size_t)pl.dense_groups;
-            const size_t mat = align_up(G * n * kDenseRowWords * sizeof(uint32_t), 256);
+            pl.core = spd_core_plan(b->n_total, pl.dense_groups, 0);
+            const size_t G = (size_t)pl.core.groups, mat = align_up(G * n * kDenseRowWords * sizeof(uint32_t), 256);
             const size_t split_bound = (size_t)(nnz > 0 ? nnz : 0) / (kDenseChunk + 1) + 1;
             pl.dense_acc_rows = (int32_t)(split_bound < n ? split_bound : n);
             size_t off = pl.scratch_off;
             pl.dense_off[0] = off; off += mat;
-            pl.dense_off[1] = off; off += mat * kDensePlanes;
+            pl.dense_off[1] = off; off += align_up((size_t)pl.dense_groups * n * kDenseRowWords * sizeof(uint32_t), 256) * kDensePlanes;
             pl.dense_off[2] = off; off += align_up(G * (size_t)pl.dense_acc_rows * kDenseRowWords * sizeof(uint32_t), 256);
             pl.dense_off[3] = off; off += align_up(G * n * sizeof(uint32_t), 256);
-            pl.dense_off[4] = off; off += align_up(G * align_up(n, 32) * kDensePlanes, 256);
+            pl.dense_off[4] = off; off += align_up(G * align_up(n, 32) * kCoreMaxLevels, 256);
+            pl.slots_off = off; off += pl.core.enabled ? align_up(G * align_up(n, 32) * kCoreMaxLevels * sizeof(uint32_t), 256) : 0;
             pl.dense_off[5] = off; off += align_up(G * n, 256);
             pl.dense_off[6] = off; off += align_up((n + 1) * sizeof(int32_t), 256);
             pl.dense_off[7] = off; off += kDenseSyncBytes;
             // work items: one per vertex plus one per further chunk of out-edges
             pl.dense_off[8] = off; off += align_up((n + (size_t)(nnz > 0 ? nnz : 0) / kDenseChunk + 1) * sizeof(int4), 256);
             pl.dense_off[9] = off; off += align_up(n * sizeof(int32_t), 256);
-            pl.total_bytes = off;
+            pl.core = spd_core_plan(b->n_total, pl.dense_groups, off);
+            pl.total_bytes = pl.core.total_bytes;
         } else {
             cudaGetLastError();
         }
@@ -1065,20 +1146,22 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
     p.max_dist = max_dist;
     p.src_per_batch = pl.src_per_batch;
 
-    GT_CUDA_TRY(cudaMemsetAsync(ws + 8, 0, 8, s));     // work counter and item count
-    spd_setup_kernel<<<1, 1024, 0, s>>>(p);
-    GT_CUDA_TRY(cudaGetLastError());
-    if (pl.dense) {
+    if (!pl.dense) {
+        GT_CUDA_TRY(cudaMemsetAsync(ws + 8, 0, 8, s));     // work counter and item count
+        spd_setup_kernel<<<1, 1024, 0, s>>>(p);
+        GT_CUDA_TRY(cudaGetLastError());
+    } else {
         DenseParams d{};
         d.vis = (uint32_t*)(ws + pl.dense_off[0]);
         d.fr = (uint32_t*)(ws + pl.dense_off[1]);
         d.acc = (uint32_t*)(ws + pl.dense_off[2]);
         d.acc_cnt = (uint32_t*)(ws + pl.dense_off[3]);
         d.nonempty = ws + pl.dense_off[4];
+        d.slots = (uint32_t*)(ws + pl.slots_off);
         d.row_done = ws + pl.dense_off[5];
         d.item_start = (int32_t*)(ws + pl.dense_off[6]);
         d.sync = (uint32_t*)(ws + pl.dense_off[7]);
-        d.live = d.sync + 64 * kDenseMaxGroups;
+        d.live = d.sync + 64 * kCoreMaxGroups;
         d.item_rec = (int4*)(ws + pl.dense_off[8]);
         d.acc_row = (int32_t*)(ws + pl.dense_off[9]);
         d.acc_rows = pl.dense_acc_rows;
@@ -1103,7 +1186,17 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
         spd_dense_item_rec_kernel<<<(unsigned)((batch->n_total + 255) / 256), 256, 0, s>>>(row_ptr, d.item_start, batch->n_total, d.item_rec);
         GT_CUDA_TRY(cudaGetLastError());
         void* args[] = {(void*)&p, (void*)&d};
-        GT_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)spd_dense_kernel, dim3((unsigned)pl.grid), dim3((unsigned)pl.threads), args, 0, s));
+        const dim3 grid((unsigned)pl.grid), threads((unsigned)pl.threads);
+        CoreParams core{};
+        if (pl.core.enabled) {
+            st = spd_core_launch(pl.core, core, ws, row_ptr, col_idx, batch->n_total, nnz, d.item_rec, d.item_start, pl.dense_groups * kDensePlanes * kDenseRowWords, s);
+            if (st != GT_OK) return st;
+            d.core = core.info;
+            d.column = core.column;
+            GT_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)spd_dense_kernel<true>, grid, threads, args, 0, s));
+            if ((st = spd_core_expand(core, d.fr, d.nonempty, d.slots, d.n_pad, kCoreMaxLevels, max_dist, spd_out, s)) != GT_OK) return st;
+        }
+        GT_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)spd_dense_kernel<false>, grid, threads, args, 0, s));
         return GT_OK;
     }
     {

@@ -1,0 +1,60 @@
+"""gt_spd_build for one large graph, where only a core of its targets is searched for: bit-exact against the BFS oracle."""
+import numpy as np
+import pytest
+
+from paper_2609_34420_b200 import workloads as wl
+
+from test_gpu_spd import check, pytestmark  # noqa: F401  (GPU tests)
+
+
+def edges(csr):
+    return np.repeat(np.arange(len(csr[0]) - 1), np.diff(csr[0])), csr[1]
+
+
+def power_law(n, degree, tail=0, keep=1.0):
+    """A power-law graph, every edge's two directions kept with probability `keep`, and a path of `tail` vertices behind vertex 0."""
+    src, dst = edges(wl.chung_lu_power_law(n - tail, float(degree), 2.1, n))
+    if keep < 1.0:
+        kept = np.random.Generator(np.random.PCG64(n)).random(len(src)) < keep
+        src, dst = src[kept], dst[kept]
+    return with_tail(n, src, dst, tail)
+
+
+def with_tail(n, src, dst, tail):
+    t = np.arange(n - tail, n)
+    back = np.concatenate([[0], t[:-1]])[:tail]
+    return wl.csr_from_edges(n, np.concatenate([src, back, t]), np.concatenate([dst, t, back]), symmetric=False)
+
+
+def tree(n):
+    """A random recursive tree: dozens of levels, and more than half of its vertices are leaves or next to one."""
+    i = np.arange(1, n)
+    return wl.csr_from_edges(n, i, (np.random.Generator(np.random.PCG64(n)).random(n - 1) * i).astype(np.int64))
+
+
+def star(n, inward):
+    i, hub = np.arange(1, n), np.zeros(n - 1, np.int64)
+    return wl.csr_from_edges(n, i, hub, symmetric=False) if inward else wl.csr_from_edges(n, hub, i)
+
+
+GRAPHS = {
+    "a plane for every level": (lambda: power_law(32768, 14), 24),
+    "sources and columns ragged, distances clipped": (lambda: power_law(32775, 8), 4),
+    "clipped just where four bits end": (lambda: power_law(32901, 6), 14),
+    "directed": (lambda: power_law(33003, 8, keep=0.6), 254),
+    # room for eleven levels, of which nine have a plane of their own: five to six levels and the path's
+    "levels that share planes": (lambda: with_tail(32777, *edges(wl.barabasi_albert(32770, 5, 3)), 7), 40),
+    "more levels than four bits hold in one column block only": (lambda: power_law(33000, 8, tail=20), 17),
+    # at every level nearly every row gains something
+    "more rows gain late than there is room for": (lambda: wl.random_geometric(32769, 4.0, 1), 12),
+    "a tree": (lambda: tree(32800), 30),
+    "a core of one": (lambda: star(32770, False), 3),
+    "in-neighbours only": (lambda: star(32772, True), 1),
+    "no edges: no core": (lambda: wl.csr_from_edges(32768, np.zeros(0, np.int64), np.zeros(0, np.int64)), 5),
+}
+
+
+@pytest.mark.parametrize("name", GRAPHS)
+def test_targets_that_follow_from_others(name):
+    make, D = GRAPHS[name]
+    check(wl.Workload("core", wl.pack_graphs([make()]), 1, 32, D))
