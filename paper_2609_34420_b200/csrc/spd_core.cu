@@ -17,6 +17,8 @@ namespace gt {
 namespace {
 
 constexpr int kSegmentGroups = kCoreSegment / 32;
+constexpr int kSegmentWarps = kSegmentGroups / 8;                    // that work on a segment, eight groups each
+constexpr int kStageWords = 4 * kCoreSegment;                        // two segments of either half of a block
 constexpr int kSegmentList = kCoreSegment * kCoreMaxDegree / 2;      // words
 constexpr int kCoreSmem = 222 * 1024;                                // and 5 KB of static arrays
 constexpr int kMaxWords = kCoreMaxNodes / 32;
@@ -108,6 +110,9 @@ __global__ void __launch_bounds__(256) spd_core_bits_kernel(CoreParams p)
 // columns each do not meet in the same banks.
 __device__ __forceinline__ uint32_t word_of_column(uint32_t c) { return (c & ~31u) | ((((c >> 2) ^ (c >> 5)) & 7u) << 2) | (c & 3u); }
 
+// Segments are for the halves of a block in turn, and each has room for two.
+__device__ __forceinline__ uint32_t stage_of(int seg) { return (uint32_t)(seg & 3) * kCoreSegment; }
+
 // A block per segment of targets: columns, the targets left out by their number of in-neighbours in groups of 32, and their lists.
 __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
 {
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
     const int groups = max(1, (n_cols + 8191) / 8192);
     const int block_bits = max(1, ((n_cols + groups - 1) / groups + 127) / 128) * 128;
     // Not worth while (the expansion reads what the search would have written) or no room
-    const bool reduced = !hopeless(p) && n_cols <= (int)(0.7f * (float)n) && groups * block_bits <= n && groups <= p.n_groups && (groups * block_bits + 4 + 2 * kCoreSegment) * 4 <= kCoreSmem;
+    const bool reduced = !hopeless(p) && n_cols <= (int)(0.7f * (float)n) && groups * block_bits <= n && groups <= p.n_groups && (groups * block_bits + 4 + kStageWords) * 4 <= kCoreSmem;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         CoreInfo& o = *p.info;
         o.deep = 0;
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
     __syncthreads();
     auto column = [&](int v) -> uint32_t { return (uint32_t)v - s_before[v >> 5] - (uint32_t)__popc(s_bits[v >> 5] & ((1u << (v & 31)) - 1u)); };
     const int seg = (int)blockIdx.x, t_first = seg * kCoreSegment;
-    const uint32_t stage = (uint32_t)(groups * block_bits) + 4u + (uint32_t)(seg & 1) * kCoreSegment;
+    const uint32_t stage = (uint32_t)(groups * block_bits) + 4u + stage_of(seg);
     const uint32_t none = (uint32_t)(groups * block_bits);           // a word that is "none" for all sources
     constexpr int kPer = kCoreSegment / 1024;
     uint32_t place[kPer];                                            // class << 16 | rank
@@ -186,7 +191,7 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
     if (warp == 0) {                                     // lists in the order in which the expansion's warps go through them
         uint32_t at = 0;
         for (int o = lane; o < kSegmentGroups; o += 32) {
-            const int q = (o >> 3) + 32 * (o & 7);
+            const int q = (o >> 3) + kSegmentWarps * (o & 7);
             const uint32_t pairs = q < n_groups ? (class_at(min(32 * q + 31, n_left - 1)) + 1) / 2 : 0u;
             const int words = 32 * (int)pairs, x = warp_scan(words, lane);
             const uint32_t first_word = at + (uint32_t)(x - words);
@@ -194,7 +199,7 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
             uint32_t head = pairs << (3 * (o & 7)) | (q < n_groups ? 1u << 24 : 0u);       // of the eight groups of a warp: pairs of edges, and how many
 #pragma unroll
             for (int off = 1; off < 8; off <<= 1) head += __shfl_xor_sync(0xffffffffu, head, off);
-            if ((o & 7) == 0) p.groups[seg * 32 + (o >> 3)] = make_uint2((uint32_t)seg * kSegmentList + first_word, head);
+            if ((o & 7) == 0) p.groups[seg * kSegmentWarps + (o >> 3)] = make_uint2((uint32_t)seg * kSegmentList + first_word, head);
             at += (uint32_t)__shfl_sync(0xffffffffu, x, 31);
         }
     }
@@ -299,9 +304,12 @@ __device__ __forceinline__ uint32_t smaller(uint32_t a, uint32_t b, uint32_t gua
 //   output   words of eight neighbouring targets -> eight bytes of every row
 // Of four-bit words without a distance beyond 6 the minimum is one of three-bit fields, whose fourth bit is the guard; else
 // of every other field at a time.
-// What bounds it: the pipe of logic and shifts, 61 % busy (issue slots as much; 2.0 TB/s of DRAM traffic), and the barrier of a segment.
-// 65 536 nodes, degree 12 (28 500 targets searched for, 37 000 with 3.0 in-neighbours on average): 2.4 ms; with four accumulators of 16-bit
-// minima, which have no instruction here, and without the table of the output 3.3 ms.
+// What bounds it: the pipe of logic and shifts, 61 % busy when all warps went through a segment together (issue slots as much; 2.0 TB/s
+// of DRAM traffic): they gathered, then wrote, and waited for each other in between.  So each half of a block takes every other
+// segment and meets only itself: one gathers while the other writes.
+// 65 536 nodes, degree 12 (28 500 targets searched for, 37 000 with 3.0 in-neighbours on average): the whole build 4.96 -> 4.71 ms by the
+// halves, the expansion 2.4 -> 2.15 ms of it; with four accumulators of 16-bit minima, which have no instruction here, and without the
+// table of the output it took 3.3 ms.
 template <int kBits>
 __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p)
 {
@@ -345,18 +353,19 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
         if (any && l < n_direct)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(plane + ((size_t)l * n + s0) * row_words), "r"((uint32_t)(here * row_words) * 4u) : "memory");
     };
-    // A warp's groups of a segment, warp + 32 i: where their lists begin, pairs of edges of each (three bits), and how many; the words of
+    // A warp's groups of a segment, warp + 16 i: where their lists begin, pairs of edges of each (three bits), and how many; the words of
     // a list; a thread's targets.
-    static_assert(kSegmentGroups == 8 * 32 && kCoreSegment == 8 * 1024, "eight groups per warp, eight targets per thread");
-    auto groups_of = [&](int seg) -> uint2 { return seg < n_segments ? __ldg(&p.c.groups[seg * 32 + warp]) : make_uint2(0u, 0u); };
+    static_assert(kSegmentWarps == 16 && kCoreSegment == 8 * 512, "eight groups per warp and eight targets per thread of half a block");
+    const int half = warp / kSegmentWarps, half_warp = warp % kSegmentWarps, half_thread = (int)threadIdx.x & 511;
+    auto groups_of = [&](int seg) -> uint2 { return seg < n_segments ? __ldg(&p.c.groups[seg * kSegmentWarps + half_warp]) : make_uint2(0u, 0u); };
     auto words_at = [&](uint32_t off, int pairs, uint32_t (&u)[kCoreMaxDegree / 2]) {
 #pragma unroll
         for (int j = 0; j < kCoreMaxDegree / 2; ++j)
             if (j < pairs) u[j] = __ldg(p.c.list + off + 32 * j);
     };
     auto locs_of = [&](int seg) -> uint4 {
-        const int q = seg * 1024 + (int)threadIdx.x;
-        return q < n_eights ? __ldg((const uint4*)p.c.loc + q) : make_uint4(0u, 0u, 0u, 0u);
+        const int q = seg * 512 + half_thread;
+        return seg < n_segments && q < n_eights ? __ldg((const uint4*)p.c.loc + q) : make_uint4(0u, 0u, 0u, 0u);
     };
     const uint32_t code_lo = (max_dist + 1u) | 1u << 8 | min(2u, max_dist) << 16 | min(3u, max_dist) << 24;
     const uint32_t code_hi = min(4u, max_dist) | min(5u, max_dist) << 8 | min(6u, max_dist) << 16 | min(7u, max_dist) << 24;
@@ -438,17 +447,17 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
         }
         const bool far = s_far[turn] != 0 || max_dist >= 127u;                   // (the table's first byte has no sign)
         if (threadIdx.x == 0) s_far[turn ^ 1] = 0;
-        uint2 mine = groups_of(0);
-        uint4 loc = locs_of(0);
+        uint2 mine = groups_of(half);
+        uint4 loc = locs_of(half);
         __syncthreads();
         if (s0 + (int)gridDim.x * kSources < n) fetch_rows(s0 + (int)gridDim.x * kSources, turn ^ 1);       // (read behind further barriers)
         uint32_t u[kCoreMaxDegree / 2];
         words_at(mine.x + lane, (int)(mine.y & 7u), u);
         // f(minimum over nothing, the words of a group's in-neighbours in pairs) -> word
         auto gather = [&](int seg, auto least) {
-            uint32_t* to = stage + (seg & 1) * kCoreSegment + 32 * warp + lane;
+            uint32_t* to = stage + stage_of(seg) + 32 * half_warp + lane;
             uint32_t off = mine.x + (uint32_t)lane, head = mine.y;
-            for (int left = (int)(head >> 24); left > 0; --left, to += 1024, head >>= 3) {
+            for (int left = (int)(head >> 24); left > 0; --left, to += 32 * kSegmentWarps, head >>= 3) {
                 uint32_t v[kCoreMaxDegree / 2];
                 const int k = (int)(head & 7u);
                 off += 32u * (uint32_t)k;
@@ -503,7 +512,7 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
             return a + (__vcmpltu4(a, max_dist * 0x01010101u) & 0x01010101u);
         };
         auto output = [&](int seg, uint4 at) {
-            const int q = seg * 1024 + (int)threadIdx.x;
+            const int q = seg * 512 + half_thread;
             if (q >= n_eights) return;
             const uint32_t at4[4] = {at.x, at.y, at.z, at.w};
             uint32_t x[8], past[2] = {0u, 0u};
@@ -579,16 +588,17 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
                 store(a, b, 0, 1);
             }
         };
-        for (int seg = 0; seg < n_segments; ++seg) {
-            const uint2 next = groups_of(seg + 1);                               // ahead of their use
+        // The halves of the block take every other segment, each with its own barrier: one gathers while the other writes.
+        for (int seg = half; seg < n_segments; seg += 2) {
+            const uint2 next = groups_of(seg + 2);                               // ahead of their use
             const uint4 at = loc;
             if constexpr (kBits == 8) gather(seg, least_code);
             else if (far) gather(seg, least_far);
             else gather(seg, least_near);
             mine = next;
             words_at(mine.x + lane, (int)(mine.y & 7u), u);
-            if (seg + 1 < n_segments) loc = locs_of(seg + 1);
-            __syncthreads();
+            loc = locs_of(seg + 2);
+            asm volatile("bar.sync %0, 512;" ::"r"(1 + half) : "memory");
             output(seg, at);
         }
         __syncthreads();                                                         // all words read
@@ -614,7 +624,7 @@ CorePlan spd_core_plan(int32_t n, int groups, size_t off)
     c.col_off = off; off += n_pad * sizeof(int32_t);
     c.loc_off = off; off += n_pad * sizeof(uint16_t);
     const size_t segments = ((size_t)n + kCoreSegment - 1) / kCoreSegment;
-    c.group_off = off; off += align_up(segments * 32 * sizeof(uint2), 256);
+    c.group_off = off; off += align_up(segments * kSegmentWarps * sizeof(uint2), 256);
     c.list_off = off; off += segments * kSegmentList * sizeof(uint32_t);
     c.info_off = off; off += align_up(sizeof(CoreInfo), 256);
     c.total_bytes = off;
@@ -666,7 +676,7 @@ gt_status spd_core_expand(const CoreParams& c, const uint32_t* planes, const uin
     if ((st = grant_smem(spd_core_expand_kernel<4>, granted4, kCoreSmem)) != GT_OK) return st;
     if ((st = grant_smem(spd_core_expand_kernel<8>, granted8, kCoreSmem)) != GT_OK) return st;
     // the targets of the search are at most 0.7 n
-    const size_t most = 4 * ((size_t)(0.7 * c.n) + 128 * kCoreMaxGroups + 32 + 4 + 2 * kCoreSegment);
+    const size_t most = 4 * ((size_t)(0.7 * c.n) + 128 * kCoreMaxGroups + 32 + 4 + kStageWords);
     const size_t smem = most < (size_t)kCoreSmem ? most : (size_t)kCoreSmem;
     const dim3 grid((unsigned)sm_count());
     if ((st = launch_overlapped(spd_core_expand_kernel<4>, grid, 1024, smem, s, p)) != GT_OK) return st;

@@ -6,9 +6,9 @@
 namespace gt {
 
 constexpr int kCoreMaxDegree = 8;          // in-neighbours of a target that is left out, at most
-constexpr int kCoreSegment = 8192;         // targets of one step of the expansion
-// Power-law graphs, all targets searched for -> the core: 32 768 nodes of degree 8 1.72 -> 1.59 ms, 33 000 of degree 6 2.44 -> 1.65, 40 000 of degree 12
-// 3.37 -> 2.34, 65 536 6.60 -> 4.96.  Below, the shorter rows leave the chip idle and the expansion costs more than they save: 24 000 of degree 12
+constexpr int kCoreSegment = 4096;         // targets of one step of half a block of the expansion
+// Power-law graphs, all targets searched for -> the core: 32 768 nodes of degree 8 1.73 -> 1.47 ms, 33 000 of degree 6 2.52 -> 1.60, 40 000 of degree 12
+// 3.30 -> 2.31, 65 536 6.60 -> 4.71.  Below, the shorter rows leave the chip idle and the expansion costs more than they save: 24 000 of degree 12
 // 1.03 -> 1.23, 19 000 of degree 8 0.93 -> 1.18.  A graph without many vertices of few edges pays 15 us (33 000 nodes, degree 25: 2.84 ms as before).
 constexpr int kCoreMinNodes = 32768;
 constexpr int kCoreMaxNodes = 65536;       // vertices are numbered in 16 bits
@@ -50,7 +50,7 @@ struct CoreParams {
     uint32_t* left_out;                    // [n / 32] a bit per vertex
     int32_t* column;                       // [n] column of a target of the search, -1: left out
     uint16_t* loc;                         // [pitch] word of a target in the expansion's shared memory
-    uint2* groups;                         // [segments][32] a warp's groups of 32 targets: their lists, and how long they are
+    uint2* groups;                         // [segments][16] a warp's groups of 32 targets: their lists, and how long they are
     uint32_t* list;                        // [segments][kCoreSegment * kCoreMaxDegree / 2] pairs of words
     CoreInfo* info;
     int32_t n;
