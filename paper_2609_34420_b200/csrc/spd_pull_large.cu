@@ -346,9 +346,11 @@ __global__ void __launch_bounds__(1024, 1) spd_large_pull_kernel(LargeParams p)
                 seen |= c[b];
             }
             const uint32_t reach = cur[v], far = reach & ~seen, none = ~reach;
+            if (far | none) {
 #pragma unroll
-            for (int b = 0; b < 8; ++b) c[b] |= (far & (0u - ((far_code >> b) & 1u))) | (none & (0u - ((none_code >> b) & 1u)));
-            emit_word(c, p.n_planes, out + (int64_t)v * ld, 0, nt, cols);
+                for (int b = 0; b < 8; ++b) c[b] |= (far & (0u - ((far_code >> b) & 1u))) | (none & (0u - ((none_code >> b) & 1u)));
+            }
+            emit_word(c, (c[4] | c[5] | c[6] | c[7]) != 0u ? 8 : 4, out + (int64_t)v * ld, 0, nt, cols);
         }
     }
     __syncthreads();
