@@ -108,13 +108,15 @@ enum FwdBarrier {
     kNumFwdBarriers = kBarODone + 4
 };
 
-template <int D>
+// kPair: half of an SM's shared memory.
+template <int D, bool kPair = false>
 struct FwdSmem {
+    static constexpr int kKStages = kPair ? 1 : gt::kKStages, kVStages = gt::kVStages, kSpdStages = kPair ? 2 : gt::kSpdStages;
     static constexpr int kRowBytes = D * 2;
     static constexpr int kTileBytes = 128 * kRowBytes;
-    static constexpr int kSpdTileBytes = kRowsPerCta * kKvTile;
+    static constexpr int kSpdTileBytes = (kPair ? kRowsPerTile : kRowsPerCta) * kKvTile;
     static constexpr int kQ = 0;
-    static constexpr int kK = kQ + kQTiles * kTileBytes;
+    static constexpr int kK = kQ + (kPair ? 1 : kQTiles) * kTileBytes;
     static constexpr int kV = kK + kKStages * kTileBytes;
     static constexpr int kSpd = kV + kVStages * kTileBytes;
     static constexpr int kBias = kSpd + kSpdStages * kSpdTileBytes;
@@ -165,14 +167,18 @@ __device__ __forceinline__ float norm_max(float a, float b) { return __uint_as_f
 // maximum first, which costs a second pass over the scores.  8 192 nodes, 8 heads of 64: 386 -> 251 us, norms included.
 // kTiles = 1: thread blocks of one 128-row query tile and eight softmax warps, for grids that would leave half
 // of the SMs idle or more (rows_per_block); a cluster of them may share the keys (FwdParams::split).  Two score buffers then: with three, a warp could be two key tiles ahead of another.
-template <int D, bool kPartial, bool kShflBias, bool kPrecise = false, int kTiles = kQTiles>
-__global__ void __launch_bounds__(128 + 256 * kTiles, 1)
+// kPair (with one tile): two thread blocks per SM, of which one computes while the other fills, drains or waits for its MMAs; one score
+// buffer, and half of the shared and of the tensor memory (pairs_of_blocks).
+template <int D, bool kPartial, bool kShflBias, bool kPrecise = false, int kTiles = kQTiles, bool kPair = false>
+__global__ void __launch_bounds__(128 + 256 * kTiles, kPair ? 2 : 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_spd,
                 const FwdParams p)
 {
-    using L = FwdSmem<D>;
-    constexpr int kRows = kRowsPerTile * kTiles, kThreads = 128 + 256 * kTiles, kBuffers = kTiles + 1;
+    using L = FwdSmem<D, kPair>;
+    constexpr int kRows = kRowsPerTile * kTiles, kThreads = 128 + 256 * kTiles, kBuffers = kPair ? 1 : kTiles + 1;
+    constexpr int kKStages = L::kKStages, kVStages = L::kVStages, kSpdStages = L::kSpdStages;
+    constexpr uint32_t kTmemCols = kPair ? 256 : 512, kOCol = kPair ? 128 : 384;
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment by pointer arithmetic on the __shared__ array itself, so that every derived
     // pointer keeps its shared address space (integer round trips would turn the accesses generic)
@@ -184,7 +190,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     int h = blockIdx.x, g = kPartial ? 0 : (int)blockIdx.z;
     int32_t q_block = (int32_t)blockIdx.y + p.q_block0;
     const int chunk = kPartial ? (int)blockIdx.z : 0;
-    constexpr bool kShared = kTiles == 1 && !kPartial;       // blocks of a cluster may share the keys
+    constexpr bool kShared = kTiles == 1 && !kPartial && !kPair;       // blocks of a cluster may share the keys
     const int rank = kShared ? (int)blockIdx.x % p.split : 0;
     if constexpr (kShared) h = (int)blockIdx.x / p.split;
 
@@ -252,7 +258,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         prefetch_tensormap(&tmap_v);
         if (p.spd_tma && !p.maps) prefetch_tensormap(&tmap_spd);
     }
-    if (warp == 1) { tmem_alloc(smem_u32(&misc[0]), 512); tmem_relinquish(); }
+    if (warp == 1) { tmem_alloc(smem_u32(&misc[0]), kTmemCols); tmem_relinquish(); }
     grid_wait();
     // The first tiles are on their way while the block is still setting up: the thread that set up the barriers is the one that loads.
     // (4 096 nodes, 8 heads: 59.4 -> 57.6 us, a packed batch of 64 graphs 1 033 -> 1 007.)
@@ -291,7 +297,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     if (warp < 4) {
         // =========================== producer / MMA / SPD warps ===========================
-        if constexpr (kTiles == 2) setmaxnreg_dec_32();
+        if constexpr (kTiles == 2 || kPair) setmaxnreg_dec_32();
         if (warp == 0) {
             for (int j = 1; j < n_kv; ++j) {
                 mbar_wait(bar(kBarKEmpty + j % kKStages), ((j / kKStages) & 1) ^ 1, abort_flag, p.status, 10);
@@ -352,13 +358,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
                             for (int k = 0; k < kKvTile / 16; ++k) {    // hi and lo term of key chunk k at the start of its own 16 score columns
                                 const uint32_t a = tm + b * 128 + (k / (kCols / 16)) * kCols + (k % (kCols / 16)) * 16;
-                                mma_ts(tm + 384 + t * 64, a, advance_desc(dv, k * 16 * L::kRowBytes), idesc_o, k > 0 ? 1u : acc0);
-                                mma_ts(tm + 384 + t * 64, a + 8, advance_desc(dv, k * 16 * L::kRowBytes), idesc_o, 1u);
+                                mma_ts(tm + kOCol + t * 64, a, advance_desc(dv, k * 16 * L::kRowBytes), idesc_o, k > 0 ? 1u : acc0);
+                                mma_ts(tm + kOCol + t * 64, a + 8, advance_desc(dv, k * 16 * L::kRowBytes), idesc_o, 1u);
                             }
                         } else {
 #pragma unroll
                         for (int k = 0; k < kKvTile / 16; ++k)      // P of key half hf sits at the start of that half's score columns
-                            mma_ts(tm + 384 + t * 64, tm + b * 128 + (k / (kCols / 16)) * kCols + (k % (kCols / 16)) * 8,
+                            mma_ts(tm + kOCol + t * 64, tm + b * 128 + (k / (kCols / 16)) * kCols + (k % (kCols / 16)) * 8,
                                    advance_desc(dv, k * 16 * L::kRowBytes), idesc_o, k > 0 ? 1u : acc0);
                         }
                         mma_commit(bar(kBarODone + 2 * t + (j & 1)));
@@ -402,6 +408,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     } else {
         // =================================== softmax warps ===================================
         if constexpr (kTiles == 2) setmaxnreg_inc_112();
+        if constexpr (kPair) setmaxnreg_inc_104();       // 128 x 32 + 256 x 104 = 384 x 80 registers, which the block was launched with
         const int sw = warp - 4;
         const int t = sw / (4 * kHalves);
         const int hf = (sw >> 2) & (kHalves - 1);
@@ -409,7 +416,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         constexpr int kOC = D / kHalves;                 // output columns per thread
         constexpr int kOP = kOC < 32 ? kOC : 32;         // ... per TMEM access
-        const uint32_t tO = tmem + 384 + t * 64 + hf * kOC + lane_off;
+        const uint32_t tO = tmem + kOCol + t * 64 + hf * kOC + lane_off;
         const uint32_t pair_bar = kNbPair + t * 4 + (warp & 3);
         float* xchg = (float*)(smem + L::kXchg) + t * 512;
         float m = 0.f, l = 0.f;
@@ -728,7 +735,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) __nanosleep(200000);    // let copies that may still be in flight land
-    if (warp == 1) tmem_dealloc(tmem, 512);
+    if (warp == 1) tmem_dealloc(tmem, kTmemCols);
     if (kShared && sharers > 1) {
         // Every block merges its part of the rows' channels from all blocks' shares.
         cluster_sync();
@@ -930,6 +937,7 @@ constexpr int32_t kNormsMinNodes = 513;
 
 // Tensor maps of a packed batch, a thread per graph, behind its work list (unless `list` is null), a warp per graph.
 constexpr int kBatchThreads = 128;
+template <int kRows>
 __global__ void __launch_bounds__(kBatchThreads) fwd_batch_kernel(const __grid_constant__ CUtensorMap model, uint8_t* maps, int4* list, int32_t entries,
                                                                   const uint8_t* spd, const int64_t* spd_offsets, const int32_t* cu_seqlens, int32_t n_graphs)
 {
@@ -938,7 +946,7 @@ __global__ void __launch_bounds__(kBatchThreads) fwd_batch_kernel(const __grid_c
     int32_t w = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (list != nullptr) {
         if (w < n_graphs) {
-            write_work_list<kRowsPerCta>(list, entries, cu_seqlens, n_graphs, w);
+            write_work_list<kRows>(list, entries, cu_seqlens, n_graphs, w);
             return;
         }
         w -= n_graphs;
@@ -957,6 +965,23 @@ inline int32_t rows_per_block(const gt_batch* b, int32_t n_heads)
     return (int64_t)((b->max_seqlen + kRowsPerTile - 1) / kRowsPerTile) * b->n_graphs * n_heads <= sm_count() ? kRowsPerTile : kRowsPerCta;
 }
 
+// Two blocks of one tile per SM, for packed batches of small graphs.  A block of ten key tiles spends a quarter of its time filling and draining,
+// and padding of 256 rows is more than half of a graph of a hundred; a tile itself takes a fifth longer, with one score buffer.
+// Graphs and nodes each, heads of d: 64 of 16-300, 4 of 32: 25.7 -> 21.2 us; 200 of 64-1 000, 4 of 32: 217 -> 209; 20 of 1 000-1 100, 8 of 64:
+// 129 -> 120; but 64 of 512-2 048, 16 of 64: 1 035 -> 1 076, and where every block has an SM of its own: 8 of 500-600, 2 of 64: 14.9 -> 16.1.
+constexpr int32_t kPairMaxNodes = 1152;
+constexpr int kPairRegisters = 80;           // per thread at launch: what setmaxnreg shares out
+inline bool small_graphs(const gt_batch* b) { return b->n_graphs > 1 && b->max_seqlen <= kPairMaxNodes; }
+inline size_t fwd_workspace(const gt_batch* b, int32_t n_heads, int32_t list_rows)
+{
+    return kHeaderBytes + maps_bytes(b->n_graphs) + list_bytes(b, list_rows) + norms_bytes(b, n_heads);
+}
+// A workspace without room for a list by 128 rows is used as for large graphs.
+inline bool pairs_of_blocks(const gt_batch* b, int32_t n_heads, size_t workspace_bytes)
+{
+    return small_graphs(b) && rows_per_block(b, n_heads) == kRowsPerCta && workspace_bytes >= fwd_workspace(b, n_heads, kRowsPerTile);
+}
+
 // Blocks that share a query tile's keys (cluster_split): a key tile takes 1.2 us, the cluster and the merge 2 to 3 us.  1 000 nodes, heads
 // of 64: 8 heads 13.9 -> 12.6 us, 4 heads 13.7 -> 10.8; 2 048 nodes, 4 heads 22.3 -> 17.1; 512 nodes, 8 heads 10.5 -> 10.7; 8 graphs of
 // 500 nodes, 2 heads 11.6 -> 12.2: from six key tiles on.
@@ -964,10 +989,10 @@ constexpr int32_t kMinSplitTiles = 6;
 
 template <int D, bool kPartial>
 gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tspd,
-                     FwdParams p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0)
+                     FwdParams p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0, bool pair = false)
 {
     const bool shfl = p.n_buckets <= 32;
-    const int32_t rows = kPartial ? kRowsPerCta : rows_per_block(batch, p.n_heads);
+    const int32_t rows = kPartial ? kRowsPerCta : pair ? kRowsPerTile : rows_per_block(batch, p.n_heads);
     auto kern = shfl ? attn_fwd_kernel<D, kPartial, true> : attn_fwd_kernel<D, kPartial, false>;
     if constexpr (!kPartial) {
         if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true> : attn_fwd_kernel<D, false, false, true>;
@@ -975,25 +1000,30 @@ gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
             kern = shfl ? attn_fwd_kernel<D, false, true, false, 1> : attn_fwd_kernel<D, false, false, false, 1>;
             if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1> : attn_fwd_kernel<D, false, false, true, 1>;
         }
+        if (pair) {
+            kern = shfl ? attn_fwd_kernel<D, false, true, false, 1, true> : attn_fwd_kernel<D, false, false, false, 1, true>;
+            if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1, true> : attn_fwd_kernel<D, false, false, true, 1, true>;
+        }
     }
-    static std::atomic<uint64_t> granted[8] = {};
+    const size_t smem = pair ? FwdSmem<D, true>::kDynamic : FwdSmem<D>::kDynamic;
+    static std::atomic<uint64_t> granted[12] = {};
     static ClusterFit max_clusters[4];
     const int form = (shfl ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0);
-    const gt_status st = grant_smem(kern, granted[form + (rows == kRowsPerTile ? 4 : 0)], FwdSmem<D>::kDynamic);
+    const gt_status st = grant_smem(kern, granted[form + (pair ? 8 : rows == kRowsPerTile ? 4 : 0)], smem, pair ? kPairRegisters : 0);
     if (st != GT_OK) return st;
     const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + rows - 1) / rows;
-    dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, kRowsPerCta) * p.n_heads))
+    dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, rows) * p.n_heads))
                        : dim3((unsigned)p.n_heads, (unsigned)row_blocks, (unsigned)grid_z);
     p.split = 1;
     const int32_t tiles = (batch->max_seqlen + kKvTile - 1) / kKvTile;
-    if (rows == kRowsPerTile && tiles >= kMinSplitTiles)
-        p.split = cluster_split(kern, 128 + 2 * rows, FwdSmem<D>::kDynamic, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, tiles, 3.0f, 2.0f);
+    if (!pair && rows == kRowsPerTile && tiles >= kMinSplitTiles)
+        p.split = cluster_split(kern, 128 + 2 * rows, smem, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, tiles, 3.0f, 2.0f);
     grid.x *= (unsigned)p.split;
     // As in the backward: with several waves of blocks the next kernel's blocks take SMs that the last wave frees one by one, and a
     // backward behind this forward starts ragged (forward and backward, 8 heads of 64: 14 000 nodes 2 452 -> 2 329 us, 16 384 nodes
     // 3 400 -> 3 228, 24 000 nodes 7 349 -> 7 176; the forward alone the same).
-    p.early_release = (int64_t)grid.x * grid.y * grid.z <= sm_count();
-    return launch_overlapped_cluster(kern, grid, 128 + 2 * rows, FwdSmem<D>::kDynamic, p.split, s, tq, tk, tv, tspd, p);
+    p.early_release = (int64_t)grid.x * grid.y * grid.z <= (pair ? 2 : 1) * sm_count();
+    return launch_overlapped_cluster(kern, grid, 128 + 2 * rows, smem, p.split, s, tq, tk, tv, tspd, p);
 }
 
 gt_status check_fwd_args(const void* q, const void* k, const void* v, const uint8_t* spd, const int64_t* spd_offsets,
@@ -1015,7 +1045,7 @@ extern "C" size_t gt_biased_attn_fwd_workspace(const gt_batch* batch, int32_t n_
 {
     (void)head_dim;
     if (gt::validate_batch(batch) != GT_OK || n_heads < 1) return gt::kHeaderBytes;
-    return gt::kHeaderBytes + gt::maps_bytes(batch->n_graphs) + gt::list_bytes(batch, gt::kRowsPerCta) + gt::norms_bytes(batch, n_heads);
+    return gt::fwd_workspace(batch, n_heads, gt::small_graphs(batch) ? gt::kRowsPerTile : gt::kRowsPerCta);
 }
 
 extern "C" gt_status gt_biased_attn_fwd(const void* q, const void* k, const void* v,
@@ -1046,13 +1076,15 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     if ((st = encode_thd_map(&tv, v, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
     CUtensorMap tspd = tq;                       // placeholder when the cp.async loader is used
     FwdParams p{};
-    const int32_t rows = rows_per_block(batch, n_heads);
+    const bool pair = pairs_of_blocks(batch, n_heads, workspace_bytes);
+    const int32_t list_rows = pair ? kRowsPerTile : kRowsPerCta;
+    const int32_t rows = pair ? kRowsPerTile : rows_per_block(batch, n_heads);
     p.spd_tma = batch->n_graphs == 1 ? 1 : 0;
-    const bool room = workspace_bytes >= gt_biased_attn_fwd_workspace(batch, n_heads, head_dim);
+    const bool room = workspace_bytes >= fwd_workspace(batch, n_heads, list_rows);
     if (batch->n_graphs > 1 && room) {
         p.maps = maps_at((uint8_t*)workspace + kHeaderBytes);
         // The list costs 1 us before the first block; that has to come back from the empty blocks that it saves.
-        if (rows == kRowsPerCta && list_saves(batch, kRowsPerCta, n_heads, kListMinSaved))
+        if ((pair || rows == kRowsPerCta) && list_saves(batch, rows, n_heads, kListMinSaved))
             p.list = (const int4*)((uint8_t*)workspace + kHeaderBytes + maps_bytes(batch->n_graphs));
         p.spd_tma = 1;
     }
@@ -1071,7 +1103,7 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     p.c1 = kLog2e / sqrtf((float)head_dim);
     cudaStream_t s = (cudaStream_t)stream;
     if (out_f32 != nullptr && room && batch->max_seqlen >= kNormsMinNodes) {
-        float* norms = (float*)((uint8_t*)workspace + kHeaderBytes + maps_bytes(batch->n_graphs) + list_bytes(batch, kRowsPerCta));
+        float* norms = (float*)((uint8_t*)workspace + kHeaderBytes + maps_bytes(batch->n_graphs) + list_bytes(batch, list_rows));
         const dim3 grid((unsigned)((batch->n_total + kNormRows - 1) / kNormRows), (unsigned)n_heads);
         st = head_dim == 64 ? launch_overlapped(key_norms_kernel<64>, grid, 256, 0, s, (const uint4*)k, norms, batch->n_total, n_heads)
                             : launch_overlapped(key_norms_kernel<32>, grid, 256, 0, s, (const uint4*)k, norms, batch->n_total, n_heads);
@@ -1081,12 +1113,12 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     }
     if (p.maps) {
         const int32_t warps = (batch->n_graphs + 31) / 32 + (p.list ? batch->n_graphs : 0);
-        st = launch_overlapped(fwd_batch_kernel, dim3((unsigned)((warps * 32 + kBatchThreads - 1) / kBatchThreads)), kBatchThreads, 0, s, tspd,
-                               (uint8_t*)p.maps, (int4*)p.list, (int32_t)list_entries(batch, kRowsPerCta), spd, p.spd_offsets, p.cu_seqlens, batch->n_graphs);
+        st = launch_overlapped(pair ? fwd_batch_kernel<kRowsPerTile> : fwd_batch_kernel<kRowsPerCta>, dim3((unsigned)((warps * 32 + kBatchThreads - 1) / kBatchThreads)), kBatchThreads, 0, s, tspd,
+                               (uint8_t*)p.maps, (int4*)p.list, (int32_t)list_entries(batch, list_rows), spd, p.spd_offsets, p.cu_seqlens, batch->n_graphs);
         if (st != GT_OK) return st;
     }
-    return head_dim == 64 ? launch_fwd<64, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s)
-                          : launch_fwd<32, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s);
+    return head_dim == 64 ? launch_fwd<64, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s, 0, pair)
+                          : launch_fwd<32, false>(tq, tk, tv, tspd, p, batch, batch->n_graphs, s, 0, pair);
 }
 
 extern "C" size_t gt_biased_attn_fwd_chunked_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim,

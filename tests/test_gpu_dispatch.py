@@ -30,6 +30,22 @@ def test_packed_batches_with_and_without_a_work_list(n_graphs, largest, d):
     assert torch.equal(out, out2) and torch.equal(lse, lse2)
 
 
+# up to 1 152 nodes two blocks of one query tile share an SM, if the workspace has room for their list; else blocks of two tiles
+@pytest.mark.parametrize("largest,d,D", [(1152, 64, 6), (1153, 64, 6), (1152, 32, 40), (1100, 64, 40)])
+def test_packed_batches_of_small_graphs(largest, d, D):
+    w = wl.small_workload([largest, 1, 128, 129, 255, 256, 257] + sizes(12, largest), 4, d, D, seed=largest + D, avg_degree=1.8)
+    case, out, lse = check_forward(w)
+    _, _, out32 = case.forward_ex()
+    assert rel_l2(to_f64(out32), oracle_forward(case)[0]) <= 1e-4        # as for the precise forward below
+    need = gt.gt_biased_attn_fwd_workspace(case.batch, case.w.n_heads, d)
+    for size in (need - 1, 256):
+        ws = torch.zeros(size, dtype=torch.uint8, device=case.q.device)
+        out2, lse2 = torch.full_like(out, float("nan")), torch.full_like(lse, float("nan"))
+        gt.gt_biased_attn_fwd(case.q, case.k, case.v, case.spd, case.bias, case.batch, D, out2, lse2, ws)
+        gt.gt_check(ws)
+        assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
 @pytest.mark.parametrize("n_graphs,largest,d", [(2, 129, 32), (64, 700, 64), (65, 700, 32)])
 def test_packed_backward_work_list(n_graphs, largest, d):
     check_backward(wl.small_workload(sizes(n_graphs, largest), 2, d, 6, seed=n_graphs, avg_degree=1.8))
