@@ -389,7 +389,7 @@ constexpr int kDenseBatch = 4;                           // work items a warp ta
 constexpr int kDenseMaxGroups = 4;                       // CTA groups working on different column blocks at once (one more where only a core is searched for)
 constexpr int kDensePlanes = 7;                          // levels whose frontier matrices are kept, with blocks of 8192 (more with narrower ones): the output
                                                          // pass reads them, later levels blend into written rows
-constexpr size_t kDenseSyncBytes = (size_t)(256 + 4 * kDenseRowWords * 4) * kCoreMaxGroups;        // sync words, then live targets
+constexpr size_t dense_sync_bytes(int groups) { return (size_t)(256 + 4 * kDenseRowWords * 4) * groups; }        // sync words, then live targets
 constexpr int kDenseFlagWords = 8192;                    // row flags of a level kept as a bitmap in shared memory (graphs up to 262 144 vertices)
 constexpr uint32_t kGridWaitIterations = 1u << 24;
 
@@ -400,7 +400,7 @@ struct DenseParams {
     int32_t* acc_row;       // [n_max] accumulator row of a split vertex (vertices with more than kDenseChunk out-edges)
     int32_t acc_rows;       // accumulator rows per CTA group
     uint32_t* acc_cnt;      // [n_max] finished chunks of a split vertex
-    uint8_t* nonempty;      // [kCoreMaxLevels][n_pad] the row of that plane is valid and has a bit set (rows without the flag are never read)
+    uint8_t* nonempty;      // [kCoreMaxLevels, or kDensePlanes without a core][n_pad] the row of that plane is valid and has a bit set (rows without the flag are never read)
     uint32_t* slots;        // [kCoreMaxLevels][n_pad] where the row is, of a level without a plane of its own (core only)
     uint8_t* row_done;      // [n_max] every valid target of the block is visited
     int32_t* item_start;    // [n_max + 1] prefix sum of chunks per vertex (of the current graph)
@@ -588,6 +588,7 @@ __device__ __forceinline__ int dense_word(int lane, int q, int j) { return q * 1
 template <bool kCore>
 __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DenseParams d)
 {
+    constexpr int kFlagLevels = kCore ? kCoreMaxLevels : kDensePlanes;
     if ((d.core != nullptr && d.core->reduced != 0) != kCore) return;
     // CTA group g (CTAs g, g + G, ...) works on column blocks g, g + G, ... with its own bit matrices, flags
     // and barrier: while one group waits for its slowest warp at a level barrier, the CTAs of the other groups
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     {
         const size_t m = (size_t)grp * d.n_max;
         d.vis += m * row_words; d.fr += m * n_planes * row_words; d.acc += (size_t)grp * d.acc_rows * row_words;
-        d.acc_cnt += m; d.nonempty += (size_t)grp * d.n_pad * kCoreMaxLevels; d.row_done += m;
+        d.acc_cnt += m; d.nonempty += (size_t)grp * d.n_pad * kFlagLevels; d.row_done += m;
         d.slots += (size_t)grp * d.n_pad * kCoreMaxLevels;
         d.sync += grp * 64;
         d.live += grp * 4 * kDenseRowWords;
@@ -755,7 +756,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 }
                 if (inside(q)) *(uint4*)&d.vis[(size_t)s * row_words + dense_word(lane, q, 0)] = make_uint4(bit[0], bit[1], bit[2], bit[3]);
             }
-            if (lane < kCoreMaxLevels) d.nonempty[(size_t)lane * d.n_pad + s] = 0;
+            if (lane < kFlagLevels) d.nonempty[(size_t)lane * d.n_pad + s] = 0;
             if (lane == 0) d.row_done[s] = 0;
         }
         if (!dense_grid_sync(d.sync, epoch, p.header, n_ctas, d.barrier_extra, d.barrier_limit)) return;
@@ -1017,8 +1018,8 @@ struct SpdPlan {
     size_t batch_start_off, scratch_off, scratch_words_per_cta, comp_off, sym_off, total_bytes;
 };
 
-// `in_place`: the caller has no workspace to speak of (gt_spd_build_static).
-SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_place = false)
+// `in_place`: the caller has no workspace to speak of (gt_spd_build_static).  `core`: with room for the choice of a core, where that pays.
+SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_place = false, bool core = true)
 {
     SpdPlan pl{};
     if (nnz < 0) nnz = 0;
@@ -1072,7 +1073,7 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
             const size_t n = (size_t)b->n_total;
             const int n_col_blocks = (int)((n + 15 + kDenseBlockBits - 1) / kDenseBlockBits);
             pl.dense_groups = n_col_blocks < kDenseMaxGroups ? n_col_blocks : kDenseMaxGroups;
-            pl.core = spd_core_plan(b->n_total, pl.dense_groups, 0);
+            pl.core = spd_core_plan(b->n_total, pl.dense_groups, 0, core);
             const size_t G = (size_t)pl.core.groups, mat = align_up(G * n * kDenseRowWords * sizeof(uint32_t), 256);
             const size_t split_bound = (size_t)(nnz > 0 ? nnz : 0) / (kDenseChunk + 1) + 1;
             pl.dense_acc_rows = (int32_t)(split_bound < n ? split_bound : n);
@@ -1081,15 +1082,15 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
             pl.dense_off[1] = off; off += align_up((size_t)pl.dense_groups * n * kDenseRowWords * sizeof(uint32_t), 256) * kDensePlanes;
             pl.dense_off[2] = off; off += align_up(G * (size_t)pl.dense_acc_rows * kDenseRowWords * sizeof(uint32_t), 256);
             pl.dense_off[3] = off; off += align_up(G * n * sizeof(uint32_t), 256);
-            pl.dense_off[4] = off; off += align_up(G * align_up(n, 32) * kCoreMaxLevels, 256);
+            pl.dense_off[4] = off; off += align_up(G * align_up(n, 32) * (pl.core.enabled ? kCoreMaxLevels : kDensePlanes), 256);
             pl.slots_off = off; off += pl.core.enabled ? align_up(G * align_up(n, 32) * kCoreMaxLevels * sizeof(uint32_t), 256) : 0;
             pl.dense_off[5] = off; off += align_up(G * n, 256);
             pl.dense_off[6] = off; off += align_up((n + 1) * sizeof(int32_t), 256);
-            pl.dense_off[7] = off; off += kDenseSyncBytes;
+            pl.dense_off[7] = off; off += dense_sync_bytes(pl.core.enabled ? kCoreMaxGroups : kDenseMaxGroups);
             // work items: one per vertex plus one per further chunk of out-edges
             pl.dense_off[8] = off; off += align_up((n + (size_t)(nnz > 0 ? nnz : 0) / kDenseChunk + 1) * sizeof(int4), 256);
             pl.dense_off[9] = off; off += align_up(n * sizeof(int32_t), 256);
-            pl.core = spd_core_plan(b->n_total, pl.dense_groups, off);
+            pl.core = spd_core_plan(b->n_total, pl.dense_groups, off, core);
             pl.total_bytes = pl.core.total_bytes;
         } else {
             cudaGetLastError();
@@ -1119,8 +1120,9 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
     if (max_dist < 1 || max_dist > 254) return GT_ERR_INVALID_ARG;
     if (batch->n_graphs > 1 && spd_offsets == nullptr) return GT_ERR_INVALID_ARG;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
-    SpdPlan pl = make_plan(batch, nnz, max_dist, in_place);
-    if (workspace_bytes < pl.total_bytes && !in_place) pl = make_plan(batch, nnz, max_dist, true);      // what does with less, more slowly
+    SpdPlan pl = make_plan(batch, nnz, max_dist, in_place, !in_place);
+    if (workspace_bytes < pl.total_bytes && !in_place) pl = make_plan(batch, nnz, max_dist, false, false);      // what does with less, more slowly
+    if (workspace_bytes < pl.total_bytes && !in_place) pl = make_plan(batch, nnz, max_dist, true, false);
     if (workspace == nullptr || workspace_bytes < pl.total_bytes || misaligned16(workspace)) return GT_ERR_WORKSPACE;
 
     cudaStream_t s = (cudaStream_t)stream;
@@ -1161,7 +1163,8 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
         d.row_done = ws + pl.dense_off[5];
         d.item_start = (int32_t*)(ws + pl.dense_off[6]);
         d.sync = (uint32_t*)(ws + pl.dense_off[7]);
-        d.live = d.sync + 64 * kCoreMaxGroups;
+        const int sync_groups = pl.core.enabled ? kCoreMaxGroups : kDenseMaxGroups;
+        d.live = d.sync + 64 * sync_groups;
         d.item_rec = (int4*)(ws + pl.dense_off[8]);
         d.acc_row = (int32_t*)(ws + pl.dense_off[9]);
         d.acc_rows = pl.dense_acc_rows;
@@ -1173,7 +1176,7 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
         g_barrier_overcount = 0;
         // accumulator rows, their counters and the barrier words start at zero
         GT_CUDA_TRY(cudaMemsetAsync(ws + pl.dense_off[2], 0, pl.dense_off[4] - pl.dense_off[2], s));
-        GT_CUDA_TRY(cudaMemsetAsync(ws + pl.dense_off[7], 0, kDenseSyncBytes, s));
+        GT_CUDA_TRY(cudaMemsetAsync(ws + pl.dense_off[7], 0, dense_sync_bytes(sync_groups), s));
         {
             // the block totals borrow the start of the item records, which are written afterwards
             const unsigned scan_blocks = (unsigned)((batch->n_total + kScanBlock - 1) / kScanBlock);
@@ -1285,7 +1288,7 @@ extern "C" gt_status gt_spd_build_static(const int32_t* row_ptr, const int32_t* 
     if (st != GT_OK) return st;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
     if (max_dist < 1 || max_dist > 254) return GT_ERR_INVALID_ARG;
-    const size_t need = make_plan(batch, nnz, max_dist, true).total_bytes;
+    const size_t need = make_plan(batch, nnz, max_dist, true, false).total_bytes;
     if (need > kStaticScratchBytes) {
         if (getenv("GT_DEBUG"))
             fprintf(stderr, "[gt_attn] gt_spd_build_static: this batch needs %zu bytes of scratch, the built-in "

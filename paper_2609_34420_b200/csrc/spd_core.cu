@@ -607,10 +607,10 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
 
 }  // namespace
 
-CorePlan spd_core_plan(int32_t n, int groups, size_t off)
+CorePlan spd_core_plan(int32_t n, int groups, size_t off, bool wanted)
 {
     CorePlan c{};
-    c.enabled = n >= kCoreMinNodes && n <= kCoreMaxNodes;
+    c.enabled = wanted && n >= kCoreMinNodes && n <= kCoreMaxNodes;
     c.groups = c.enabled && n > 8192 * groups * 10 / 7 ? groups + 1 : groups;
     if (c.groups > kCoreMaxGroups) c.groups = kCoreMaxGroups;
     c.clear_off = off;

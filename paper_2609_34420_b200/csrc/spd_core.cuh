@@ -36,7 +36,7 @@ struct CorePlan {
     size_t slot_off, bits_off, col_off, loc_off, group_off, list_off, info_off, total_bytes;
 };
 
-CorePlan spd_core_plan(int32_t n, int groups, size_t off);
+CorePlan spd_core_plan(int32_t n, int groups, size_t off, bool wanted);
 
 struct CoreParams {
     const int32_t* row_ptr;

@@ -1,9 +1,12 @@
 """gt_spd_build for one large graph, where only a core of its targets is searched for: bit-exact against the BFS oracle."""
 import numpy as np
 import pytest
+import torch
 
+from paper_2609_34420_b200 import binding as gt
 from paper_2609_34420_b200 import workloads as wl
 
+from gpu_util import device_batch, device_csr
 from test_gpu_spd import check, pytestmark  # noqa: F401  (GPU tests)
 
 
@@ -58,3 +61,14 @@ GRAPHS = {
 def test_targets_that_follow_from_others(name):
     make, D = GRAPHS[name]
     check(wl.Workload("core", wl.pack_graphs([make()]), 1, 32, D))
+
+
+def test_workspace_without_room_for_the_core():
+    w = wl.Workload("core", wl.pack_graphs([power_law(32777, 8)]), 1, 32, 9)
+    exp = check(w)
+    batch, (rp, ci) = device_batch(w.batch, "cuda"), device_csr(w.batch, "cuda")
+    ws = torch.zeros(gt.gt_spd_build_workspace(batch, len(w.batch.col_idx), w.max_dist) - 1, dtype=torch.uint8, device="cuda")
+    out = torch.full((w.batch.spd_bytes,), 0xEE, dtype=torch.uint8, device="cuda")
+    gt.gt_spd_build(rp, ci, batch, w.max_dist, out, ws)
+    gt.gt_check(ws)
+    np.testing.assert_array_equal(out.cpu().numpy(), exp)
