@@ -335,8 +335,8 @@ gt_status gt_biased_attn_bwd_step_finish(const float* dq_acc, const float* dk_ac
  * w = round_up(ceil(N / n_kv_chunks), 128) rows (the last may be short or empty); each chunk
  * yields a partial (out_c, lse_c) using spd[i][j] at the GLOBAL column j; partials are then
  * merged:  lse = log sum_c exp(lse_c),  out = sum_c exp(lse_c - lse) out_c.
- * Consecutive chunks are merged on the chip, by carrying the running softmax state from one to the next, unless
- * lse_chunks is given or partials through the workspace fill the GPU better.
+ * Unless lse_chunks is given, the same thread blocks may take several consecutive chunks, with the running softmax state on the
+ * chip and their partials added up in fp32; that fills the GPU better or worse than blocks for every chunk, by its size.
  * Results equal gt_biased_attn_fwd up to rounding.  Single graph only (n_graphs == 1).
  * lse_chunks: optional fp32 [n_kv_chunks, H, N] receiving lse_c (-inf for empty chunks), or NULL.
  * ------------------------------------------------------------------------------------- */

@@ -35,6 +35,8 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "attn_common.cuh"
 #include "sm100_primitives.cuh"
 
@@ -74,7 +76,9 @@ struct FwdParams {
     int32_t n_total;
     int32_t n_heads;
     int32_t n_buckets;
-    int32_t kv_chunk_rows;     // chunked: keys per chunk (multiple of 128)
+    int32_t kv_chunk_rows;     // chunked: keys of a share (multiple of 128): a chunk, or several behind one another
+    float* chunk_sums;         //   sums over a share's chunks, [thread blocks][D / 8][softmax threads] of four channels of a row (nullptr: one chunk)
+    int32_t chunk_tiles;       //   key tiles per chunk
     int32_t use_ranges;        // step entry point: key ranges given explicitly, one per grid z
     int32_t range_begin[2];
     int32_t range_end[2];
@@ -123,7 +127,8 @@ struct FwdSmem {
     static constexpr int kXchg = kBias + 256 * 4;             // [2 tiles][max | sum][2 halves][128 rows] float
     static constexpr int kBars = kXchg + 2 * 512 * 4;
     static constexpr int kMisc = kBars + kNumFwdBarriers * 8;
-    static constexpr int kTotal = kMisc + 16;
+    static constexpr int kSums = kMisc + 16;                  // kFold: [softmax threads] {reference, l} of the chunks before
+    static constexpr int kTotal = kSums + (kPair ? 0 : 512 * 8);
     static constexpr int kDynamic = kTotal + 1024;   // slack for the 1024-byte alignment
 };
 
@@ -169,7 +174,10 @@ __device__ __forceinline__ float norm_max(float a, float b) { return __uint_as_f
 // of the SMs idle or more (rows_per_block); a cluster of them may share the keys (FwdParams::split).  Two score buffers then: with three, a warp could be two key tiles ahead of another.
 // kPair (with one tile): two thread blocks per SM, of which one computes while the other fills, drains or waits for its MMAs; one score
 // buffer, and half of the shared and of the tensor memory (pairs_of_blocks).
-template <int D, bool kPartial, bool kShflBias, bool kPrecise = false, int kTiles = kQTiles, bool kPair = false>
+// kFold: the chunked forward with all chunks behind one another.  Every chunk of keys is a chain of MMAs of its own, as if its share went
+// through memory, and is added to the chunks before with rounding: one chain over all of them would be less exact, because the tensor
+// core cuts off what its accumulator cannot hold, an error that grows with the chain.
+template <int D, bool kPartial, bool kShflBias, bool kPrecise = false, int kTiles = kQTiles, bool kPair = false, bool kFold = false>
 __global__ void __launch_bounds__(128 + 256 * kTiles, kPair ? 2 : 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                 const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_spd,
@@ -190,7 +198,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     int h = blockIdx.x, g = kPartial ? 0 : (int)blockIdx.z;
     int32_t q_block = (int32_t)blockIdx.y + p.q_block0;
     const int chunk = kPartial ? (int)blockIdx.z : 0;
-    constexpr bool kShared = kTiles == 1 && !kPartial && !kPair;       // blocks of a cluster may share the keys
+    constexpr bool kShared = kTiles == 1 && !kPartial && !kPair && !kFold;       // blocks of a cluster may share the keys
     const int rank = kShared ? (int)blockIdx.x % p.split : 0;
     if constexpr (kShared) h = (int)blockIdx.x / p.split;
 
@@ -343,11 +351,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             constexpr uint32_t idesc_o = make_idesc_bf16(128, D, false, true);
             const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
             const uint64_t desc_v0 = make_smem_desc(smem_u32(smem + L::kV), L::kRowBytes, 0);
+            [[maybe_unused]] int begin = 0;             // key tile that begins the next chunk
             for (int j = 0; j < n_kv; ++j) {
                 const int vs = j % kVStages;
                 mbar_wait(bar(kBarVFull + vs), (j / kVStages) & 1, abort_flag, p.status, 25);
                 const uint64_t dv = advance_desc(desc_v0, vs * L::kTileBytes);
-                const uint32_t acc0 = j > 0 ? 1u : 0u;
+                uint32_t acc0 = j > 0 ? 1u : 0u;
+                if constexpr (kFold) {
+                    acc0 = j != begin ? 1u : 0u;
+                    if (j == begin) begin += p.chunk_tiles;
+                }
 #pragma unroll
                 for (int t = 0; t < kTiles; ++t) {
                     const int b = (kTiles * j + t) % kBuffers;
@@ -421,6 +434,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         float* xchg = (float*)(smem + L::kXchg) + t * 512;
         float m = 0.f, l = 0.f;
         bool shifted = false;                   // the reference of this warp's rows may differ from 0
+        // kFold: O and l are of the chunk at work; what the chunks before add up to is in memory and, {reference, l}, in `sums`
+        [[maybe_unused]] int next_chunk = p.chunk_tiles;
+        [[maybe_unused]] float2* sums = (float2*)(smem + L::kSums) + (kFold ? tid - 128 : 0);
+        [[maybe_unused]] auto o_sum = [&](int i) -> float4* {       // of four channels of this thread's row
+            return (float4*)p.chunk_sums + ((size_t)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (kOC / 4) + i) * (256 * kTiles) + (tid - 128);
+        };
 
         // lane b of every softmax warp keeps table entry b (scaled by log2 e); entries past the
         // table repeat the last one.  With at most 32 buckets a score's bias is fetched by a
@@ -618,6 +637,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarSpdEmpty + (j % kSpdStages)));
+            if constexpr (kFold) {
+                if (j == next_chunk) {
+                    if (j > p.chunk_tiles) l += sums->y * ex2_approx(sums->x - m);
+                    sums->y = l;
+                    l = 0.f;
+                }
+            }
             l += tile_sum;
 
             // P over the first half of this thread's own score columns
@@ -626,6 +652,34 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 for (int c = 0; c < kCols / 64; ++c) tmem_st32(tS + c * 32, pk[c]);
             }
             tmem_wait_st();
+            if constexpr (kFold) {
+                if (j == next_chunk) {          // the chunk before joins the sum; PV(j) then overwrites it
+                    mbar_wait(bar(kBarODone + 2 * t + ((j - 1) & 1)), ((j - 1) >> 1) & 1, abort_flag, p.status, 44);
+                    tc_fence_after();
+                    uint32_t o[kOC];
+                    tmem_ld<kOC>(tO, o);
+                    tmem_wait_ld();
+                    if (j == p.chunk_tiles) {
+#pragma unroll
+                        for (int i = 0; i < kOC / 4; ++i) *(uint4*)o_sum(i) = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                    } else {
+                        const float m_sum = sums->x;
+                        if (__any_sync(0xffffffffu, m != m_sum)) {
+                            const float w = ex2_approx(m_sum - m);
+#pragma unroll 1
+                            for (int i = 0; i < kOC / 4; ++i) {
+                                float4 a = __ldcg(o_sum(i));
+                                a.x *= w; a.y *= w; a.z *= w; a.w *= w;
+                                *o_sum(i) = a;
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < kOC / 4; ++i) red_add_f32x4(o_sum(i), o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                    }
+                    sums->x = m;
+                    next_chunk += p.chunk_tiles;
+                }
+            }
             tc_fence_before();
             // Warps of a tile can be one step apart (nothing in the speculative pass waits for the
             // previous PV MMA), so odd and even key tiles use different barriers, here and for the
@@ -639,12 +693,18 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // ---- epilogue: O / l, LSE ----
         mbar_wait(bar(kBarODone + 2 * t + ((n_kv - 1) & 1)), ((n_kv - 1) >> 1) & 1, abort_flag, p.status, 43);
         tc_fence_after();
+        [[maybe_unused]] float w_sum = 0.f;
+        [[maybe_unused]] const bool summed = kFold && n_kv > p.chunk_tiles;
+        if (summed) {
+            w_sum = ex2_approx(sums->x - m);
+            l += sums->y * w_sum;
+        }
         xchg[256 + hf * 128 + r] = l;
         named_barrier_sync(pair_bar, 64);
         l += xchg[256 + (hf ^ 1) * 128 + r];
         const int32_t q = q0 + t * kRowsPerTile + r;
         const float inv_l = 1.0f / l;
-        const float lse_nat = (m + log2f(l)) * kLn2;
+        const float lse_nat = kFold ? m * kLn2 + logf(l) : (m + log2f(l)) * kLn2;       // (the merge of shares took a natural logarithm, too)
         if (kShared && sharers > 1) {
             // This block's share of O, not normalised, and its m and l, to its own shared memory (over K and V: every MMA is done).
 #pragma unroll
@@ -657,7 +717,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 for (int i = 0; i < kOP / 4; ++i) part[i * 128] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
             }
             if (hf == 0) *(float2*)(smem + L::kXchg + 512 * 4 + r * 8) = make_float2(m, l);
-        } else if (kPartial && p.state_o != nullptr) {
+        } else if (kPartial && !kFold && p.state_o != nullptr) {
             // Merge into the carried state: lse' = log(e^lse0 + e^lse), o' = e^(lse0-lse') o0 + e^(lse-lse') o.
             const bool mine = q >= p.state_q_begin && q < p.state_q_end;
             float* lse_ptr = p.state_lse + (size_t)h * p.n_total + q;
@@ -696,12 +756,22 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             uint32_t o[kOP];
             tmem_ld<kOP>(tO + c * kOP, o);
             tmem_wait_ld();
+            if (summed) {
+#pragma unroll
+                for (int i = 0; i < kOP / 4; ++i) {
+                    const float4 a = __ldcg(o_sum(c * (kOP / 4) + i));
+                    o[4 * i] = __float_as_uint(__uint_as_float(o[4 * i]) + w_sum * a.x);
+                    o[4 * i + 1] = __float_as_uint(__uint_as_float(o[4 * i + 1]) + w_sum * a.y);
+                    o[4 * i + 2] = __float_as_uint(__uint_as_float(o[4 * i + 2]) + w_sum * a.z);
+                    o[4 * i + 3] = __float_as_uint(__uint_as_float(o[4 * i + 3]) + w_sum * a.w);
+                }
+            }
             if (q < n_g) {
                 if (kPartial) {
                     float4* dst = (float4*)(p.part_o + (((size_t)chunk * p.n_total + q) * p.n_heads + h) * D + hf * kOC + c * kOP);
 #pragma unroll
                     for (int i = 0; i < kOP / 4; ++i)
-                        dst[i] = make_float4(__uint_as_float(o[4 * i]) * inv_l, __uint_as_float(o[4 * i + 1]) * inv_l,
+                        *(kFold ? o_sum(c * (kOP / 4) + i) : &dst[i]) = make_float4(__uint_as_float(o[4 * i]) * inv_l, __uint_as_float(o[4 * i + 1]) * inv_l,
                                              __uint_as_float(o[4 * i + 2]) * inv_l, __uint_as_float(o[4 * i + 3]) * inv_l);
                 } else {
                     uint4* dst = (uint4*)(p.out + ((size_t)(node0 + q) * p.n_heads + h) * D + hf * kOC + c * kOP);
@@ -812,6 +882,46 @@ __global__ void chunk_merge_kernel(const float* __restrict__ part_o, const float
     if (v == 0) lse[(size_t)h * n_total + row] = mx + logf(den);
 }
 
+// The same for shares in the layout of FwdParams::chunk_sums, in thread blocks of 256 rows: block (rows and head, 16 channels).
+template <int D>
+__global__ void __launch_bounds__(kRowsPerCta) share_merge_kernel(const float4* __restrict__ sums, const float* __restrict__ part_lse, __nv_bfloat16* __restrict__ out,
+                                                                  float* __restrict__ lse, int32_t n_total, int32_t n_heads, int32_t n_shares)
+{
+    grid_wait();
+    grid_release();
+    constexpr int kOC = D / kHalves;
+    const int h = (int)(blockIdx.x % (unsigned)n_heads), row = (int)threadIdx.x, c = (int)blockIdx.y * 16;
+    const int32_t q = (int32_t)(blockIdx.x / (unsigned)n_heads) * kRowsPerCta + row;
+    if (q >= n_total) return;
+    auto lse_of = [&](int k) -> float { return part_lse[((size_t)k * n_heads + h) * n_total + q]; };
+    float mx = -INFINITY;
+    for (int k = 0; k < n_shares; ++k) mx = fmaxf(mx, lse_of(k));
+    float den = 0.f;
+    float4 acc[4] = {};
+    for (int k = 0; k < n_shares; ++k) {
+        const float lc = lse_of(k);
+        if (lc == -INFINITY) continue;
+        const float w = exp2f((lc - mx) * kLog2e);
+        den += w;
+        const float4* src = sums + (((size_t)k * gridDim.x + blockIdx.x) * (kOC / 4) + (c % kOC) / 4) * 512 + (row / 128) * 256 + (c / kOC) * 128 + row % 128;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 o = src[i * 512];
+            acc[i].x += w * o.x; acc[i].y += w * o.y; acc[i].z += w * o.z; acc[i].w += w * o.w;
+        }
+    }
+    const float inv = 1.0f / den;
+    uint4 pk[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        pk[i] = make_uint4(pack_bf16x2(acc[2 * i].x * inv, acc[2 * i].y * inv), pack_bf16x2(acc[2 * i].z * inv, acc[2 * i].w * inv),
+                           pack_bf16x2(acc[2 * i + 1].x * inv, acc[2 * i + 1].y * inv), pack_bf16x2(acc[2 * i + 1].z * inv, acc[2 * i + 1].w * inv));
+    uint4* to = (uint4*)(out + ((size_t)q * n_heads + h) * D + c);
+    to[0] = pk[0];
+    to[1] = pk[1];
+    if (c == 0) lse[(size_t)h * n_total + q] = mx + logf(den);
+}
+
 // One ring step's merge: the carried state (normalised accumulator o_acc, lse_acc) of the query rows
 // [q_begin, q_end) absorbs up to two partial results (the step's regular key range and its super-node
 // range):  lse' = log sum exp(lse_i),  o' = sum exp(lse_i - lse') o_i.  Rows with nothing to attend to yet
@@ -869,30 +979,6 @@ int32_t chunk_rows(int32_t n, int32_t n_chunks)
 {
     int32_t w = (n + n_chunks - 1) / n_chunks;
     return (w + kKvTile - 1) / kKvTile * kKvTile;
-}
-
-// Parts that a chunked forward takes its chunks in.  A thread block walks through the consecutive chunks of a part with the softmax
-// state on the chip, as from one ring step to the next; parts go through memory as partial results and are merged.  One part unless
-// more of them fill the grid's last wave better.  A 256 x 128 tile takes 1.55 us, a block's fill and drain 7, the merge 3 and its bytes
-// (written and read, 5 TB/s).  Every chunk a part of its own, as it was -> now, 8 heads of 64: 4 096 nodes, 8 chunks 113.6 -> 59.8 us; 30 000 nodes,
-// 8 chunks 3 104 -> 2 612; 4 heads: 10 000 nodes, 2 chunks 221 us as it was, and 264 in one part.
-int32_t chunk_parts(int32_t n, int32_t n_heads, int32_t head_dim, int32_t n_chunks)
-{
-    const int64_t blocks = (int64_t)((n + kRowsPerCta - 1) / kRowsPerCta) * n_heads;
-    const int32_t tiles = chunk_rows(n, n_chunks) / kKvTile;
-    int32_t best = 1;
-    double least = 0.0;
-    for (int32_t parts = 1; parts <= n_chunks && parts <= 64; ++parts) {
-        const int32_t per = (n_chunks + parts - 1) / parts;
-        if ((n_chunks + per - 1) / per != parts) continue;                 // (the same as fewer parts)
-        double us = (double)((blocks * parts + sm_count() - 1) / sm_count()) * (1.55 * per * tiles + 7.0);
-        if (parts > 1) us += 3.0 + 8e-6 / 5.0 * parts * (double)n * n_heads * head_dim;
-        if (parts == 1 || us < 0.95 * least) {
-            best = parts;
-            least = us;
-        }
-    }
-    return best;
 }
 
 constexpr size_t kListMinSaved = 128;     // thread blocks
@@ -965,6 +1051,34 @@ inline int32_t rows_per_block(const gt_batch* b, int32_t n_heads)
     return (int64_t)((b->max_seqlen + kRowsPerTile - 1) / kRowsPerTile) * b->n_graphs * n_heads <= sm_count() ? kRowsPerTile : kRowsPerCta;
 }
 
+// Chunks of a chunked forward that the same thread blocks take one behind the other.  Blocks of several fill and drain less often and leave
+// fewer shares to merge; more blocks fill the grid's last wave better.  `room`: floats in the workspace for the shares.  A 256 x 128 tile
+// takes 1.50 to 1.61 us (heads of 32 and of 64), a 128 x 128 tile 1.0 where all blocks are of one, a block's fill and drain 7, an addition
+// to the sums 0.9 to 2.5, the merge 3 and its bytes (5 TB/s).  us with every chunk in blocks of its own -> by this rule, 8 chunks: 8 heads of
+// 64: 4 096 nodes 109 -> 65 (one share), 10 000 nodes 460 -> 370 (two), 65 536 nodes 13 700 -> 13 300 (one); 4 heads: 6 000 nodes 109 -> 77
+// (three), 4 096 nodes, 5 chunks 62 -> 45 (one-tile blocks); 5 000 nodes, 5 chunks stay with 68 (98 in one share).
+int32_t chunks_in_turn(const gt_batch* b, int32_t n_heads, int32_t head_dim, int32_t n_chunks, int32_t chunk_tiles, size_t room)
+{
+    const int64_t n = b->n_total, sms = sm_count(), blocks = (n + kRowsPerCta - 1) / kRowsPerCta * n_heads, tiles = (n + kKvTile - 1) / kKvTile;
+    const bool one_tile = rows_per_block(b, n_heads) == kRowsPerTile;
+    int32_t best = n_chunks;
+    double least = one_tile ? 1.0 * tiles + 0.8 * (n_chunks - 1) + 7.0 : 1e30;
+    for (int32_t shares = 1; shares <= n_chunks && shares <= 64; ++shares) {
+        const int32_t per = (n_chunks + shares - 1) / shares;
+        if ((n_chunks + per - 1) / per != shares) continue;                // (the same as fewer shares)
+        if (shares == 1 && one_tile) continue;
+        if (shares > 1 && per > 1 && (size_t)shares * blocks * kRowsPerCta * head_dim > room) continue;
+        const int64_t longest = std::min<int64_t>(tiles, (int64_t)per * chunk_tiles);
+        double us = (double)((blocks * shares + sms - 1) / sms) * (1.55 * longest + 1.5 * (per - 1) + 7.0);
+        if (shares > 1) us += 3.0 + 8e-6 / 5.0 * shares * (double)n * n_heads * head_dim;
+        if (us < 0.97 * least) {
+            best = per;
+            least = us;
+        }
+    }
+    return best;
+}
+
 // Two blocks of one tile per SM, for packed batches of small graphs.  A block of ten key tiles spends a quarter of its time filling and draining,
 // and padding of 256 rows is more than half of a graph of a hundred; a tile itself takes a fifth longer, with one score buffer.
 // Graphs and nodes each, heads of d: 64 of 16-300, 4 of 32: 25.7 -> 21.2 us; 200 of 64-1 000, 4 of 32: 217 -> 209; 20 of 1 000-1 100, 8 of 64:
@@ -991,32 +1105,34 @@ template <int D, bool kPartial>
 gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tspd,
                      FwdParams p, const gt_batch* batch, int grid_z, cudaStream_t s, int grid_y = 0, bool pair = false)
 {
-    const bool shfl = p.n_buckets <= 32;
+    const bool shfl = p.n_buckets <= 32, in_turn = p.chunk_sums != nullptr;
     const int32_t rows = kPartial ? kRowsPerCta : pair ? kRowsPerTile : rows_per_block(batch, p.n_heads);
     auto kern = shfl ? attn_fwd_kernel<D, kPartial, true> : attn_fwd_kernel<D, kPartial, false>;
+    if (in_turn) kern = shfl ? attn_fwd_kernel<D, kPartial, true, false, kQTiles, false, true> : attn_fwd_kernel<D, kPartial, false, false, kQTiles, false, true>;
     if constexpr (!kPartial) {
         if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true> : attn_fwd_kernel<D, false, false, true>;
         if (rows == kRowsPerTile) {
             kern = shfl ? attn_fwd_kernel<D, false, true, false, 1> : attn_fwd_kernel<D, false, false, false, 1>;
             if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1> : attn_fwd_kernel<D, false, false, true, 1>;
         }
+        if (in_turn && rows == kRowsPerTile) kern = shfl ? attn_fwd_kernel<D, false, true, false, 1, false, true> : attn_fwd_kernel<D, false, false, false, 1, false, true>;
         if (pair) {
             kern = shfl ? attn_fwd_kernel<D, false, true, false, 1, true> : attn_fwd_kernel<D, false, false, false, 1, true>;
             if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1, true> : attn_fwd_kernel<D, false, false, true, 1, true>;
         }
     }
     const size_t smem = pair ? FwdSmem<D, true>::kDynamic : FwdSmem<D>::kDynamic;
-    static std::atomic<uint64_t> granted[12] = {};
+    static std::atomic<uint64_t> granted[16] = {};
     static ClusterFit max_clusters[4];
     const int form = (shfl ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0);
-    const gt_status st = grant_smem(kern, granted[form + (pair ? 8 : rows == kRowsPerTile ? 4 : 0)], smem, pair ? kPairRegisters : 0);
+    const gt_status st = grant_smem(kern, granted[form + (in_turn ? (rows == kRowsPerTile ? 14 : 12) : pair ? 8 : rows == kRowsPerTile ? 4 : 0)], smem, pair ? kPairRegisters : 0);
     if (st != GT_OK) return st;
     const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + rows - 1) / rows;
     dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, rows) * p.n_heads))
                        : dim3((unsigned)p.n_heads, (unsigned)row_blocks, (unsigned)grid_z);
     p.split = 1;
     const int32_t tiles = (batch->max_seqlen + kKvTile - 1) / kKvTile;
-    if (!pair && rows == kRowsPerTile && tiles >= kMinSplitTiles)
+    if (!pair && !in_turn && rows == kRowsPerTile && tiles >= kMinSplitTiles)
         p.split = cluster_split(kern, 128 + 2 * rows, smem, max_clusters[form], (int64_t)grid.x * grid.y * grid.z, tiles, 3.0f, 2.0f);
     grid.x *= (unsigned)p.split;
     // As in the backward: with several waves of blocks the next kernel's blocks take SMs that the last wave frees one by one, and a
@@ -1144,42 +1260,59 @@ extern "C" gt_status gt_biased_attn_fwd_chunked(const void* q, const void* k, co
     const size_t need = gt_biased_attn_fwd_chunked_workspace(batch, n_heads, head_dim, n_kv_chunks);
     if (workspace == nullptr || workspace_bytes < need || misaligned16(workspace)) return GT_ERR_WORKSPACE;
     if (sm_count() <= 0) return GT_ERR_NO_DEVICE;
-    const int32_t parts = lse_chunks != nullptr ? n_kv_chunks                         // each chunk's own lse is wanted
-                          : rows_per_block(batch, n_heads) == kRowsPerTile ? 1 : chunk_parts(batch->n_total, n_heads, head_dim, n_kv_chunks);
-    if (parts == 1 && lse_chunks == nullptr)
+    const int32_t width = chunk_rows(batch->n_total, n_kv_chunks), n_filled = (batch->n_total + width - 1) / width;      // (chunks behind those are empty)
+    const size_t rows = (size_t)batch->n_total * n_heads, room = (size_t)n_kv_chunks * rows * head_dim;
+    const int32_t per = lse_chunks != nullptr ? 1 : chunks_in_turn(batch, n_heads, head_dim, n_filled, width / kKvTile, room);      // (each chunk's own lse is wanted)
+    const int32_t shares = lse_chunks != nullptr ? n_kv_chunks : (n_filled + per - 1) / per;
+    const bool whole = shares == 1 && lse_chunks == nullptr;                           // nothing to merge
+    if (n_filled == 1 && lse_chunks == nullptr)
         return gt_biased_attn_fwd_ex(q, k, v, spd, nullptr, bias, batch, n_heads, head_dim, max_dist, out, lse, nullptr, workspace, workspace_bytes, stream);
     CUtensorMap tq, tk, tv;
     if ((st = encode_thd_map(&tq, q, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
     if ((st = encode_thd_map(&tk, k, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
     if ((st = encode_thd_map(&tv, v, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
-    const size_t rows = (size_t)batch->n_total * n_heads;
     uint8_t* ws = (uint8_t*)workspace;
     CUtensorMap tspd;
-    if ((st = encode_spd_map(&tspd, spd, batch->n_total, 256)) != GT_OK) return st;
+    if ((st = encode_spd_map(&tspd, spd, batch->n_total, whole ? rows_per_block(batch, n_heads) : kRowsPerCta)) != GT_OK) return st;
     FwdParams p{};
     p.spd_tma = 1;
     p.spd = spd;
     p.bias = bias;
     p.part_lse = (float*)(ws + kHeaderBytes);
     p.part_o = (float*)(ws + kHeaderBytes + align_up((size_t)n_kv_chunks * rows * sizeof(float), 256));
+    if (per > 1) {                               // (one share: there is room for two, which is more than whole blocks of rows take)
+        p.chunk_sums = p.part_o;
+        p.chunk_tiles = width / kKvTile;
+    }
+    if (whole) {
+        p.out = (__nv_bfloat16*)out;
+        p.lse = lse;
+    }
     p.status = (uint32_t*)workspace;
     p.n_total = batch->n_total;
     p.n_heads = n_heads;
     p.n_buckets = max_dist + 2;
-    p.kv_chunk_rows = chunk_rows(batch->n_total, n_kv_chunks) * ((n_kv_chunks + parts - 1) / parts);
+    p.kv_chunk_rows = width * per;
     p.c1 = kLog2e / sqrtf((float)head_dim);
     cudaStream_t s = (cudaStream_t)stream;
-    st = head_dim == 64 ? launch_fwd<64, true>(tq, tk, tv, tspd, p, batch, parts, s)
-                        : launch_fwd<32, true>(tq, tk, tv, tspd, p, batch, parts, s);
+    if (whole)
+        return head_dim == 64 ? launch_fwd<64, false>(tq, tk, tv, tspd, p, batch, 1, s) : launch_fwd<32, false>(tq, tk, tv, tspd, p, batch, 1, s);
+    st = head_dim == 64 ? launch_fwd<64, true>(tq, tk, tv, tspd, p, batch, shares, s)
+                        : launch_fwd<32, true>(tq, tk, tv, tspd, p, batch, shares, s);
     if (st != GT_OK) return st;
+    if (per > 1) {
+        const dim3 merge((unsigned)((batch->n_total + kRowsPerCta - 1) / kRowsPerCta * n_heads), (unsigned)head_dim / 16);
+        return head_dim == 64 ? launch_overlapped(share_merge_kernel<64>, merge, kRowsPerCta, 0, s, (const float4*)p.chunk_sums, p.part_lse, (__nv_bfloat16*)out, lse, batch->n_total, n_heads, shares)
+                              : launch_overlapped(share_merge_kernel<32>, merge, kRowsPerCta, 0, s, (const float4*)p.chunk_sums, p.part_lse, (__nv_bfloat16*)out, lse, batch->n_total, n_heads, shares);
+    }
     const size_t n_thr = rows * (head_dim / 4);
     const unsigned blocks = (unsigned)((n_thr + 255) / 256);
     if (head_dim == 64)
         st = launch_overlapped(chunk_merge_kernel<64>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
-                                                      batch->n_total, n_heads, parts);
+                                                      batch->n_total, n_heads, shares);
     else
         st = launch_overlapped(chunk_merge_kernel<32>, dim3(blocks), 256, 0, s, p.part_o, p.part_lse, (__nv_bfloat16*)out, lse, lse_chunks,
-                                                      batch->n_total, n_heads, parts);
+                                                      batch->n_total, n_heads, shares);
     return st;
 }
 
