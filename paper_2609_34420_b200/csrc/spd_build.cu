@@ -401,12 +401,11 @@ struct DenseParams {
     int32_t acc_rows;       // accumulator rows per CTA group
     uint32_t* acc_cnt;      // [n_max] finished chunks of a split vertex
     uint8_t* nonempty;      // [kCoreMaxLevels, or kDensePlanes without a core][n_pad] the row of that plane is valid and has a bit set (rows without the flag are never read)
-    uint32_t* slots;        // [kCoreMaxLevels][n_pad] where the row is, of a level without a plane of its own (core only)
     uint8_t* row_done;      // [n_max] every valid target of the block is visited
     int32_t* item_start;    // [n_max + 1] prefix sum of chunks per vertex (of the current graph)
     int4* item_rec;         // [n_items] {vertex, first edge, one past the last edge, chunks of the vertex} of a work item
     uint32_t* live;         // [4][kDenseRowWords] targets that some vertex gained, by level mod 4
-    uint32_t* sync;         // [0] barrier counter, [1] abort, [2..5] "some frontier bit", [8..11] work counter and [12..15] rows taken of the pool, by level mod 4
+    uint32_t* sync;         // [0] barrier counter, [1] abort, [2..5] "some frontier bit" and [8..11] work counter, by level mod 4
     int32_t n_max;
     int32_t n_pad;          // n_max rounded up to 32: pitch of the flag arrays
     int32_t n_groups;       // CTA groups that work on different column blocks at the same time (own state each)
@@ -583,6 +582,15 @@ __device__ __forceinline__ void dense_blend_word(uint8_t* row, int32_t t0, uint3
 // vector q of all lanes together is a contiguous 512-byte piece of the row
 __device__ __forceinline__ int dense_word(int lane, int q, int j) { return q * 128 + lane * 4 + j; }
 
+// The frontier rows of a level: vector q of row s.
+struct FrontierRows {
+    uint32_t* base;
+    size_t pitch;                        // words
+    uint32_t vec0, vec1;                 // where the vectors begin
+    __device__ __forceinline__ uint32_t* at(int s, int lane, int q) const { return base + (size_t)s * pitch + (q ? vec1 : vec0) + (uint32_t)lane * 4; }
+};
+static_assert(kDenseVecs == 2, "two vectors per row");
+
 // kCore: only the targets that *d.core names are searched for, with rows of what length they need (1 % to 10 % on top where all are).
 // Of the two launched kernels the one that it does not say so returns.
 template <bool kCore>
@@ -595,9 +603,8 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     // on the same SMs keep the memory system busy.
     const int block_bits = kCore ? d.core->block_bits : kDenseBlockBits;
     const int row_words = kCore ? block_bits / 32 : kDenseRowWords;
-    // Levels that have a plane each; only few rows gain anything at later ones, and in a search for a core those take rows of a
-    // pool in turn, until it might overflow (pool_rows: room for one level's rows in full at its beginning).
-    const int n_planes = kCore ? d.core->n_planes : kDensePlanes, n_direct = kCore ? d.core->n_direct : kDensePlanes;
+    // Levels that have a plane each.  Of a core, what later ones gain waits in the rows of the matrix, which the expansion writes.
+    const int n_planes = kCore ? d.core->n_planes : kDensePlanes;
     if (kCore) d.n_groups = d.core->n_groups;
     const int grp = (int)blockIdx.x % d.n_groups;
     const int cta = (int)blockIdx.x / d.n_groups;                                   // index within the group
@@ -606,7 +613,6 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
         const size_t m = (size_t)grp * d.n_max;
         d.vis += m * row_words; d.fr += m * n_planes * row_words; d.acc += (size_t)grp * d.acc_rows * row_words;
         d.acc_cnt += m; d.nonempty += (size_t)grp * d.n_pad * kFlagLevels; d.row_done += m;
-        d.slots += (size_t)grp * d.n_pad * kCoreMaxLevels;
         d.sync += grp * 64;
         d.live += grp * 4 * kDenseRowWords;
     }
@@ -629,13 +635,12 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     // one item at a time where a warp has few (a batch is one chain of loads after the other)
     const int batch_items = kCore ? min(kDenseBatch, max(1, n_items / (4 * n_gw))) : kDenseBatch;
     uint32_t epoch = 0;
-    uint32_t pool_used = 0;                    // rows of the pool that the levels so far hold
     uint32_t step = 0;                         // levels over all column blocks: index of the rotating "any" flags
 
     // finalise vertex s for this level: new bits (left in acc), visited, next frontier row, flags.  While the
     // levels still have a plane each (blend == false) no output byte is written here: the output pass reads the
     // planes once.  Later levels blend their bytes into the rows that pass has written.
-    auto finalise = [&](int s, uint32_t (&acc)[kDenseVecs][4], int32_t col0, uint32_t* vis_row, uint32_t* next, uint32_t* next_slot,
+    auto finalise = [&](int s, uint32_t (&acc)[kDenseVecs][4], int32_t col0, uint32_t* vis_row, const FrontierRows& next,
                         uint8_t* next_nonempty, uint32_t code, uint32_t flag_idx, bool blend) {
         bool any_new = false, full = true;
 #pragma unroll
@@ -668,15 +673,9 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
         const bool row_new = __any_sync(0xffffffffu, any_new);
         const bool row_full = __all_sync(0xffffffffu, full);
         if (row_new) {                 // the whole row, zeros included: a flagged row is read in full
-            uint32_t at = (uint32_t)s;
-            if (kCore && next_slot != nullptr) {
-                if (lane == 0) { at = pool_used + atomicAdd(&d.sync[12 + flag_idx], 1u); next_slot[s] = at; }
-                at = __shfl_sync(0xffffffffu, at, 0);
-            }
-            uint32_t* next_row = next + (size_t)at * row_words;
 #pragma unroll
             for (int q = 0; q < kDenseVecs; ++q)
-                if (inside(q)) *(uint4*)&next_row[dense_word(lane, q, 0)] = make_uint4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+                if (inside(q)) *(uint4*)next.at(s, lane, q) = make_uint4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
         }
         if (lane == 0) {
             next_nonempty[s] = row_new ? 1 : 0;
@@ -688,6 +687,10 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
     // Output pass of a column block: every byte of the block's columns is written once, from the frontier planes
     // of levels 1..n_levels (a pair is in at most one of them): its level, clamped; 0 on the diagonal; the
     // unreachable code where no plane has the pair (later levels, if any, overwrite that); 255 in the padding.
+    auto rows_of = [&](int l, int32_t col0) -> FrontierRows {                    // of level l
+        if (kCore && l > n_planes) return {(uint32_t*)(p.spd + col0), (size_t)ld / 4, core_late_word(l - 1 - n_planes, 0, row_words), core_late_word(l - 1 - n_planes, 128, row_words)};
+        return {d.fr + (size_t)(l - 1) * d.n_max * row_words, (size_t)row_words, 0, 128};
+    };
     auto emit_rows = [&](int32_t col0, int n_levels) {
         static_assert(kDensePlanes <= 15 && kCoreMaxLevels <= 15, "four bit slices hold the level codes");
         for (int s = gw; s < n; s += n_gw) {
@@ -697,7 +700,8 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
             const int32_t own = column(s);
 #pragma unroll
             for (int q = 0; q < kDenseVecs; ++q) {
-                if (!inside(q)) continue;
+                const bool in = inside(q);
+                if (!kCore && !in) continue;
                 uint32_t cb[4][4], found[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) { found[j] = 0u; cb[0][j] = cb[1][j] = cb[2][j] = cb[3][j] = 0u; }
@@ -706,13 +710,9 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                     m &= m - 1;
                     int l1 = 0;
                     if (m) { l1 = __ffs(m) - 1; m &= m - 1; }
-                    auto row_of = [&](int l) -> const uint32_t* {
-                        const size_t at = !kCore || l <= n_direct ? (size_t)(l - 1) * d.n_max + s : (size_t)n_direct * d.n_max + __ldcg(&d.slots[(size_t)(l - 1) * d.n_pad + s]);
-                        return d.fr + at * row_words + dense_word(lane, q, 0);
-                    };
-                    const uint4 x = __ldcg((const uint4*)row_of(l0));
-                    uint4 y = make_uint4(0u, 0u, 0u, 0u);
-                    if (l1) y = __ldcg((const uint4*)row_of(l1));
+                    uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
+                    if (in) x = __ldcg((const uint4*)rows_of(l0, col0).at(s, lane, q));
+                    if (in && l1) y = __ldcg((const uint4*)rows_of(l1, col0).at(s, lane, q));
                     const uint32_t c0 = (uint32_t)min(l0, p.max_dist), c1 = (uint32_t)min(l1, p.max_dist);
                     const uint32_t xw[4] = {x.x, x.y, x.z, x.w}, yw[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
@@ -724,6 +724,12 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
 #pragma unroll
                     for (int j = 0; j < 4; ++j) found[j] |= xw[j] | yw[j];
                 }
+                if (kCore && n_levels > n_planes) {      // the output goes where these levels are: the last one, which is still wanted, to plane 1
+                    if (in && ((valid >> n_levels) & 1u))
+                        *(uint4*)rows_of(2, col0).at(s, lane, q) = __ldcg((const uint4*)rows_of(n_levels, col0).at(s, lane, q));
+                    __syncwarp();                        // the whole vector is read
+                }
+                if (!in) continue;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int32_t t0 = col0 + dense_word(lane, q, j) * 32;
@@ -766,17 +772,13 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
         for (int level = 1;; ++level) {
             const uint32_t code = (uint32_t)min(level, p.max_dist);
             const uint32_t flag_idx = step & 3u;
-            // Level l <= n_direct writes plane l - 1, further ones up to the output pass write rows of the pool; the levels behind it take
-            // planes 0 and 1 in turn, which are free then.  Level 1 reads the edges only.
-            const bool late = kCore && !emitted && level > n_direct, from_pool = kCore && level - 1 > n_direct && (!emitted || level - 1 == last_kept);
+            // Level l writes plane l - 1 or, beyond the planes, the matrix; the levels behind the output pass take planes 0 and 1 in
+            // turn, which are free then.  Level 1 reads the edges only.
             const int turn = (level - last_kept) & 1;
-            const int pl_cur = emitted && level - 1 > last_kept ? turn : (from_pool ? n_direct : max(level - 2, 0));
-            const int pl_next = emitted ? turn ^ 1 : min(level - 1, n_direct);
-            const int fl_cur = emitted && level - 1 > last_kept ? turn : max(level - 2, 0), fl_next = emitted ? turn ^ 1 : level - 1;
-            const uint32_t* fcur = d.fr + (size_t)pl_cur * d.n_max * row_words;
-            const uint32_t* slot_cur = from_pool ? d.slots + (size_t)(level - 2) * d.n_pad : nullptr;
-            uint32_t* fnext = d.fr + (size_t)pl_next * d.n_max * row_words;
-            uint32_t* slot_next = late ? d.slots + (size_t)(level - 1) * d.n_pad : nullptr;
+            const bool resumed = emitted && level - 1 == last_kept;              // reads the last level before that pass
+            const FrontierRows cur = rows_of(emitted ? (!resumed ? turn + 1 : kCore && last_kept > n_planes ? 2 : last_kept) : max(level - 1, 1), col0);
+            const FrontierRows next = rows_of(emitted ? (turn ^ 1) + 1 : level, col0);
+            const int fl_cur = emitted && !resumed ? turn : max(level - 2, 0), fl_next = emitted ? turn ^ 1 : level - 1;
             const uint8_t* ne_cur = d.nonempty + (size_t)fl_cur * d.n_pad;
             uint8_t* ne_next = d.nonempty + (size_t)fl_next * d.n_pad;
             // Targets that some vertex gained at the level before: no other target can be gained at this one (a path to it of this
@@ -856,7 +858,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 {
                     uint32_t m = __shfl_sync(0xffffffffu, m_mine, k_item);
                     const int32_t e0 = __shfl_sync(0xffffffffu, rec_mine.y, k_item);
-                    int32_t u = (m >> lane) & 1u ? ci[e0 + lane] : -1;
+                    const int32_t u = (m >> lane) & 1u ? ci[e0 + lane] : -1;
                     if (m) {
                         // bits this vertex still misses and may gain: once the neighbours read so far cover them all, the rest
                         // of the edge list cannot add anything (at the dense levels a few rows are enough)
@@ -896,7 +898,6 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                             __syncwarp();
                             m = 0u;
                         }
-                        if (kCore && slot_cur != nullptr && u >= 0) u = (int32_t)__ldcg(&slot_cur[u]);
                         while (m) {                                   // two frontier rows (2 x 1 KB) in flight
                             const int b0 = __ffs(m) - 1;
                             m &= m - 1;
@@ -904,17 +905,15 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                             int u1 = -1;
                             if (m) { const int b1 = __ffs(m) - 1; m &= m - 1; u1 = __shfl_sync(0xffffffffu, u, b1); }
                             uint4 x[kDenseVecs], y[kDenseVecs];
-                            const uint32_t* r0 = fcur + (size_t)u0 * row_words;
 #pragma unroll
                             for (int q = 0; q < kDenseVecs; ++q) {
                                 x[q] = y[q] = make_uint4(0u, 0u, 0u, 0u);
-                                if (inside(q)) x[q] = __ldcg((const uint4*)&r0[dense_word(lane, q, 0)]);
+                                if (inside(q)) x[q] = __ldcg((const uint4*)cur.at(u0, lane, q));
                             }
                             if (u1 >= 0) {
-                                const uint32_t* r1 = fcur + (size_t)u1 * row_words;
 #pragma unroll
                                 for (int q = 0; q < kDenseVecs; ++q)
-                                    if (inside(q)) y[q] = __ldcg((const uint4*)&r1[dense_word(lane, q, 0)]);
+                                    if (inside(q)) y[q] = __ldcg((const uint4*)cur.at(u1, lane, q));
                             }
 #pragma unroll
                             for (int q = 0; q < kDenseVecs; ++q) {
@@ -931,7 +930,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                     }
                 }
                 if (n_chunks == 1) {
-                    finalise(s, acc, col0, vis_row, fnext, slot_next, ne_next, code, flag_idx, emitted);
+                    finalise(s, acc, col0, vis_row, next, ne_next, code, flag_idx, emitted);
                 } else {
                     uint32_t* acc_row = d.acc + (size_t)d.acc_row[s] * row_words;
 #pragma unroll
@@ -954,7 +953,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                             if (a4.x | a4.y | a4.z | a4.w) *(uint4*)&acc_row[dense_word(lane, q, 0)] = make_uint4(0u, 0u, 0u, 0u);
                         }
                         if (lane == 0) d.acc_cnt[s] = 0u;
-                        finalise(s, acc, col0, vis_row, fnext, slot_next, ne_next, code, flag_idx, emitted);
+                        finalise(s, acc, col0, vis_row, next, ne_next, code, flag_idx, emitted);
                     }
                 }
               }
@@ -964,11 +963,9 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 if (s_gained[w]) atomicOr(&d.live[(step & 3u) * kDenseRowWords + w], s_gained[w]);
             if (!dense_grid_sync(d.sync, epoch, p.header, n_ctas, d.barrier_extra, d.barrier_limit)) return;
             const uint32_t any = *(volatile uint32_t*)&d.sync[2 + flag_idx];
-            if (late) pool_used += *(volatile uint32_t*)&d.sync[12 + flag_idx];
             if (cta == 0 && threadIdx.x == 0) {                 // next written two levels from now
                 d.sync[2 + ((step + 2u) & 3u)] = 0u;
                 d.sync[8 + ((step + 2u) & 3u)] = 0u;
-                d.sync[12 + ((step + 2u) & 3u)] = 0u;
             }
             if (cta == 0)
                 for (int w = (int)threadIdx.x; w < kDenseRowWords; w += (int)blockDim.x) d.live[((step + 2u) & 3u) * kDenseRowWords + w] = 0u;
@@ -977,9 +974,7 @@ __global__ void __launch_bounds__(512, 2) spd_dense_kernel(SpdParams p, DensePar
                 if (cta == 0 && threadIdx.x == 0) d.core->levels[grp] = level;
                 break;
             }
-            // The next level needs a plane, or a row of the pool for every vertex.
-            const bool no_room = level >= n_direct && (!kCore || level == kCoreMaxLevels || pool_used > (uint32_t)(kCorePoolPlanes - 1) * (uint32_t)n);
-            if (!emitted && (!any || no_room)) {
+            if (!emitted && (!any || level == (kCore ? kCoreMaxLevels : kDensePlanes))) {
                 last_kept = level;
                 if (kCore && cta == 0 && threadIdx.x == 0) { d.core->levels[grp] = 0; d.core->deep = 1; }
                 emit_rows(col0, level);
@@ -1008,7 +1003,6 @@ struct SpdPlan {
     bool dense;                // single large graph: bit-matrix BFS (persistent cooperative kernel)
     int dense_groups;
     size_t dense_off[10];      // vis, frontier planes, acc, acc_cnt, nonempty flags, row_done, item_start, sync, item_rec, acc_row
-    size_t slots_off;
     CorePlan core;             // behind them
     int32_t dense_acc_rows;    // accumulator rows per CTA group: a bound on the vertices with more than kDenseChunk out-edges
     int threads;
@@ -1083,7 +1077,6 @@ SpdPlan make_plan(const gt_batch* b, int64_t nnz, int32_t max_dist, bool in_plac
             pl.dense_off[2] = off; off += align_up(G * (size_t)pl.dense_acc_rows * kDenseRowWords * sizeof(uint32_t), 256);
             pl.dense_off[3] = off; off += align_up(G * n * sizeof(uint32_t), 256);
             pl.dense_off[4] = off; off += align_up(G * align_up(n, 32) * (pl.core.enabled ? kCoreMaxLevels : kDensePlanes), 256);
-            pl.slots_off = off; off += pl.core.enabled ? align_up(G * align_up(n, 32) * kCoreMaxLevels * sizeof(uint32_t), 256) : 0;
             pl.dense_off[5] = off; off += align_up(G * n, 256);
             pl.dense_off[6] = off; off += align_up((n + 1) * sizeof(int32_t), 256);
             pl.dense_off[7] = off; off += dense_sync_bytes(pl.core.enabled ? kCoreMaxGroups : kDenseMaxGroups);
@@ -1159,7 +1152,6 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
         d.acc = (uint32_t*)(ws + pl.dense_off[2]);
         d.acc_cnt = (uint32_t*)(ws + pl.dense_off[3]);
         d.nonempty = ws + pl.dense_off[4];
-        d.slots = (uint32_t*)(ws + pl.slots_off);
         d.row_done = ws + pl.dense_off[5];
         d.item_start = (int32_t*)(ws + pl.dense_off[6]);
         d.sync = (uint32_t*)(ws + pl.dense_off[7]);
@@ -1197,7 +1189,7 @@ gt_status spd_build(const int32_t* row_ptr, const int32_t* col_idx, int64_t nnz,
             d.core = core.info;
             d.column = core.column;
             GT_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)spd_dense_kernel<true>, grid, threads, args, 0, s));
-            if ((st = spd_core_expand(core, d.fr, d.nonempty, d.slots, d.n_pad, kCoreMaxLevels, max_dist, spd_out, s)) != GT_OK) return st;
+            if ((st = spd_core_expand(core, d.fr, d.nonempty, d.n_pad, kCoreMaxLevels, max_dist, spd_out, s)) != GT_OK) return st;
         }
         GT_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)spd_dense_kernel<false>, grid, threads, args, 0, s));
         return GT_OK;

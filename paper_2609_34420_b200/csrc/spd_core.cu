@@ -141,8 +141,10 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
     const int n_cols = n - (int)s_warp[31];
     const int groups = max(1, (n_cols + 8191) / 8192);
     const int block_bits = max(1, ((n_cols + groups - 1) / groups + 127) / 128) * 128;
+    const int n_planes = min(kCoreMaxLevels, p.plane_words / (groups * (block_bits / 32)));
     // Not worth while (the expansion reads what the search would have written) or no room
-    const bool reduced = !hopeless(p) && n_cols <= (int)(0.7f * (float)n) && groups * block_bits <= n && groups <= p.n_groups && (groups * block_bits + 4 + kStageWords) * 4 <= kCoreSmem;
+    const bool reduced = !hopeless(p) && n_cols <= (int)(0.7f * (float)n) && groups * block_bits <= n && groups <= p.n_groups && (groups * block_bits + 4 + kStageWords) * 4 <= kCoreSmem &&
+                         n_planes + kCoreLateLevels >= kCoreMaxLevels;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         CoreInfo& o = *p.info;
         o.deep = 0;
@@ -152,8 +154,7 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
         o.block_bits = block_bits;
         o.row_words = block_bits / 32;
         o.n_groups = groups;
-        o.n_planes = min(kCoreMaxLevels + kCorePoolPlanes, p.plane_words / (groups * (block_bits / 32)));
-        o.n_direct = o.n_planes - kCorePoolPlanes;
+        o.n_planes = n_planes;
     }
     if (!reduced) return;
     __syncthreads();
@@ -241,9 +242,8 @@ __global__ void __launch_bounds__(1024) spd_core_lists_kernel(CoreParams p)
 
 struct ExpandParams {
     CoreParams c;
-    const uint32_t* planes;                // [groups][levels][n][row_words]
+    const uint32_t* planes;                // [groups][levels][n][row_words]; further levels are in the rows of spd
     const uint8_t* nonempty;               // [groups][flag_planes][n_pad]
-    const uint32_t* slots;                 // [groups][flag_planes][n_pad] of the levels without a plane of their own
     uint8_t* spd;
     int32_t n_pad;
     int32_t flag_planes;
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
     if (!info.reduced || (info.deep != 0) != (kBits == 8)) return;
     const int n = p.c.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t ld = (int64_t)((n + 15) & ~15);
-    const int row_words = info.row_words, n_words = info.n_groups * row_words, n_planes = info.n_planes, n_direct = info.n_direct;
+    const int row_words = info.row_words, n_words = info.n_groups * row_words, n_planes = info.n_planes;
     const int n_segments = (n + kCoreSegment - 1) / kCoreSegment, n_eights = (int)(ld / 8);
     const uint32_t max_dist = (uint32_t)p.max_dist;
     uint32_t* const stage = s_word + 32 * n_words + 4;
@@ -345,12 +345,12 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
 #pragma unroll
         for (int r = 0; r < kSources; ++r) {
             const bool there = r < here && set[r] != 0;
-            const size_t row = l < n_direct ? (size_t)l * n + s0 + r : (size_t)n_direct * n + (there ? p.slots[at + r] : 0u);
-            s_row[block][l][r] = there ? plane + row * row_words : nullptr;
+            const uint32_t* row = l < n_planes ? plane + ((size_t)l * n + s0 + r) * row_words : (const uint32_t*)(p.spd + (s0 + r) * ld + block * row_words * 32);
+            s_row[block][l][r] = there ? row : nullptr;
             any = any || there;
         }
         if (any && l >= 6) s_far[turn] = 1;
-        if (any && l < n_direct)
+        if (any && l < n_planes)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(plane + ((size_t)l * n + s0) * row_words), "r"((uint32_t)(here * row_words) * 4u) : "memory");
     };
     // A warp's groups of a segment, warp + 16 i: where their lists begin, pairs of edges of each (three bits), and how many; the words of
@@ -383,11 +383,12 @@ __global__ void __launch_bounds__(1024, 1) spd_core_expand_kernel(ExpandParams p
 #pragma unroll
                 for (int l = 0; l < kCoreMaxLevels; ++l) {
                     if (l >= levels) break;
+                    const uint32_t at = l < n_planes ? (uint32_t)word : core_late_word(l - n_planes, word, row_words);
                     uint32_t x[kSources];
 #pragma unroll
                     for (int r = 0; r < kSources; ++r) {
                         const uint32_t* row = s_row[block][l][r];
-                        x[r] = row != nullptr ? __ldcs(row + word) : 0u;
+                        x[r] = row != nullptr ? __ldcs(row + at) : 0u;
                     }
 #pragma unroll
                     for (int b = 0; b < 4; ++b)
@@ -667,10 +668,10 @@ gt_status spd_core_launch(const CorePlan& c, CoreParams& p, uint8_t* ws, const i
     return launch_overlapped(spd_core_lists_kernel, dim3((unsigned)segments), 1024, 0, s, p);
 }
 
-gt_status spd_core_expand(const CoreParams& c, const uint32_t* planes, const uint8_t* nonempty, const uint32_t* slots, int32_t n_pad, int flag_planes,
+gt_status spd_core_expand(const CoreParams& c, const uint32_t* planes, const uint8_t* nonempty, int32_t n_pad, int flag_planes,
                           int32_t max_dist, uint8_t* spd, cudaStream_t s)
 {
-    ExpandParams p{c, planes, nonempty, slots, spd, n_pad, flag_planes, max_dist, 0xffffffffu};
+    ExpandParams p{c, planes, nonempty, spd, n_pad, flag_planes, max_dist, 0xffffffffu};
     static std::atomic<uint64_t> granted4{0}, granted8{0};
     gt_status st;
     if ((st = grant_smem(spd_core_expand_kernel<4>, granted4, kCoreSmem)) != GT_OK) return st;
