@@ -21,12 +21,12 @@
 //
 // Softmax is single pass and speculative: a key tile is exponentiated against the row's current
 // reference without looking at the tile's own maximum first; the row sum of the tile tells
-// afterwards whether the reference was out of reach (sum above a threshold, or not finite, or the first tile's
-// below its reciprocal), and only then the tile is redone the classical way (maximum, rescale of l and O,
-// exponentials).  References are integers in log2 units, so rescale factors are exact powers of two and the
-// bf16 mantissa of a P entry does not depend on the reference, nor on how the keys are tiled or chunked.  They start
-// at 0 (scores are mostly within some powers of two of 1), where nothing has to be subtracted: 4 096 nodes, 8 heads of 64:
-// 60.2 -> 59.4 us, 64 graphs of 512-2 048 nodes, 16 heads: 1 068 -> 1 033 (with the first tile's maximum taken first before).
+// afterwards whether the reference was out of reach (sum above a threshold, or not finite), and only then the
+// tile is redone the classical way (maximum, rescale of l and O, exponentials).  References are integers in log2
+// units, so rescale factors are exact powers of two (a P entry depends on the reference in the rounding of its exponent's
+// argument only).  They start at 0, as scores are mostly within some powers of two of 1; a few scores of the first tile tell where they
+// are not.  With the first tile's maximum always taken first -> so: 4 096 nodes, 8 heads of 64: 59.5 -> 57.9 us, 64 graphs of 512-2 048
+// nodes, 16 heads: 1 078 -> 1 028; all scores shifted by -40, which the classical first tile costs: 59.3 -> 58.6, 1 061 -> 1 051.
 //
 // TMEM columns: three score buffers [0,128) [128,256) [256,384) used in rotation by the steps
 // (key tile j, query tile t) -> buffer (2j+t) mod 3, so that the S MMA of a step never waits for a
@@ -58,7 +58,8 @@ constexpr int kCols = kKvTile / kHalves;      // score columns per softmax threa
 constexpr int kCW = 16;                       // columns per TMEM load
 constexpr int kChunks = kCols / kCW;
 static_assert(kChunks == 4, "the softmax pass is written for four chunks");
-constexpr float kSumThreshold = 0x1p24f;       // tile row sum above which the reference is raised (the first tile's: lowered below 1 / it)
+constexpr float kSumThreshold = 0x1p24f;       // tile row sum above which the reference is raised
+constexpr float kPeekReach = 24.0f;            // log2 units within which a row's first scores leave the starting reference as it is
 constexpr int kNormRows = 256;                // precise variant: rows per entry of key_norms
 constexpr float kReach = 60.0f;               // precise variant: log2 of the largest P entry that needs no new reference (and of the smallest at first)
 
@@ -433,7 +434,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t pair_bar = kNbPair + t * 4 + (warp & 3);
         float* xchg = (float*)(smem + L::kXchg) + t * 512;
         float m = 0.f, l = 0.f;
-        bool shifted = false;                   // the reference of this warp's rows may differ from 0
+        // Precise variant: the reference of this warp's rows may differ from 0; nothing is subtracted where it cannot (8 192 nodes, 8 heads of 64:
+        // 255 -> 242 us; the other one gains 1 % by a pass of its own for that and loses 2 % to 3 % where references differ).
+        [[maybe_unused]] bool m_moved = false;
         // kFold: O and l are of the chunk at work; what the chunks before add up to is in memory and, {reference, l}, in `sums`
         [[maybe_unused]] int next_chunk = p.chunk_tiles;
         [[maybe_unused]] float2* sums = (float2*)(smem + L::kSums) + (kFold ? tid - 128 : 0);
@@ -520,6 +523,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             float tile_sum = 0.f;
             bool loaded = true;                    // chunk 0 is already on its way
             bool exact = false;                    // take the tile maximum first
+            // Is the starting reference in reach of the first tile?  Four of the thread's first 16 scores tell: none of them far above 0 and one not far
+            // below, so that the row's sum is not, either.  Otherwise the tile takes the classical way at once.
+            if (!kPrecise && j == 0) {
+                tmem_wait_ld();
+                const uint32_t word[4] = {wa[0].x, wa[0].y, wa[0].z, wa[0].w};
+                float top = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float b = kShflBias ? __shfl_sync(0xffffffffu, tbl, word[i]) : s_bias[word[i] & 0xffu];
+                    if (4 * i < valid) top = fmaxf(top, fmaf(__uint_as_float(sa[4 * i]), p.c1, b));
+                }
+                exact = named_barrier_or(pair_bar, 64, valid > 0 && !(fabsf(top) <= kPeekReach));       // (a half without valid columns has no say)
+            }
             // The precise variant's P overwrites the scores chunk by chunk, so a tile cannot be redone: it goes the speculative way
             // only where the row's reference leaves no score out of reach (both column halves decide alike).
             if constexpr (kPrecise) exact = __any_sync(0xffffffffu, !(limit <= m + kReach) || (j == 0 && !(low >= -kReach)));
@@ -574,7 +590,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         }
                     }
                     m = m_new;
-                    shifted = true;
+                    m_moved = true;
                 }
 
                 // ---- P = 2^(s c1 + bias - m), row sum ----
@@ -620,7 +636,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tmem_wait_ld(); exp_chunk(3, sb, wb, rag, ref);
                 };
                 if (ragged) exp_pass(BoolTag<true>{}, BoolTag<true>{});
-                else if (shifted) exp_pass(BoolTag<false>{}, BoolTag<true>{});
+                else if (!kPrecise || m_moved) exp_pass(BoolTag<false>{}, BoolTag<true>{});
                 else exp_pass(BoolTag<false>{}, BoolTag<false>{});
                 loaded = false;
                 {
@@ -629,9 +645,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tile_sum = lo + hi;
                 }
                 if (kPrecise || exact) break;
-                // Reference too low (the first: too high) for some row of this warp (pair of warps)?  Also catches inf / NaN.  A half without
-                // valid columns has nothing to say.
-                const bool need = !(tile_sum <= kSumThreshold) || (j == 0 && valid > 0 && !(tile_sum >= 1.0f / kSumThreshold));
+                // reference too low for some row of this warp (pair of warps)?  Also catches inf / NaN.
+                const bool need = !(tile_sum <= kSumThreshold);
                 if (!named_barrier_or(pair_bar, 64, need)) break;
                 exact = true;
             }

@@ -174,6 +174,28 @@ def test_scores_far_from_the_first_reference(n, shift, masked):
     check_forward(w)
 
 
+# The same in the other forms of the kernel, with the fp32 output (whose tiles cannot be done twice) and with the chunks' own lse.
+FORMS = {"one query tile": ([700], 2), "two query tiles": ([1100], 20), "two blocks per SM": (sizes(40, 500), 4)}
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("shift,masked", [(60.0, False), (-60.0, False), (-90.0, False), (0.0, True), (-90.0, True)])
+def test_scores_far_from_the_first_reference_in_every_form(form, shift, masked):
+    sizes_, heads = FORMS[form]
+    w = wl.small_workload(sizes_, heads, 64, 6, seed=heads, avg_degree=1.2)
+    w.tensors().bias[:] += shift
+    if masked:
+        w.tensors().bias[:, 7] = -1e30
+    case, out, lse = check_forward(w)
+    _, lse32, out32 = case.forward_ex()
+    ro, rl = oracle_forward(case)
+    assert rel_l2(to_f64(out32), ro) <= 1e-4 and np.abs(to_f64(lse32) - rl).max() <= LSE_MAX_ABS
+    if len(sizes_) == 1:
+        for own in (True, False):
+            oc, lc, _ = case.forward_chunked(5, want_chunk_lse=own)
+            assert np.abs(to_f64(lc) - rl).max() <= LSE_MAX_ABS and rel_l2(to_f64(oc), to_f64(out)) <= 1e-3
+
+
 # Without the chunks' own lse, on 148 SMs: each chunk in blocks of its own, all behind one another in blocks of one query tile and of
 # two, and two or three behind one another (the last share as long, shorter, a single chunk).  Every chunk is a sum of its own in all
 # of them and is added in fp32: beside the results with the chunks' own lse only values next to a tie of bf16 differ (relative
