@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import attention as oattn
 from paper_2609_34420_b200 import binding as gt
 from paper_2609_34420_b200 import workloads as wl
 
@@ -186,10 +187,16 @@ def test_scores_far_from_the_first_reference_in_every_form(form, shift, masked):
     w.tensors().bias[:] += shift
     if masked:
         w.tensors().bias[:, 7] = -1e30
-    case, out, lse = check_forward(w)
+    case = DeviceCase(w)
+    out, lse = case.forward()
     _, lse32, out32 = case.forward_ex()
     ro, rl = oracle_forward(case)
-    assert rel_l2(to_f64(out32), ro) <= 1e-4 and np.abs(to_f64(lse32) - rl).max() <= LSE_MAX_ABS
+    # bf16 rounds each P and the result by up to 2^-8 of it (a masked row may be left with two nodes whose values nearly cancel)
+    q, k, v, _, b = case.host_f64()
+    weight, _ = oattn.forward_batch(q, k, np.abs(v), case.spd_host, w.batch.spd_offsets, w.batch.cu_seqlens, b)
+    assert (np.abs(to_f64(out) - ro) <= 2.0 ** -8 * (weight + np.abs(ro)) + 1e-4).all()
+    assert rel_l2(to_f64(out32), ro) <= 1e-4
+    assert max(np.abs(to_f64(x) - rl).max() for x in (lse, lse32)) <= LSE_MAX_ABS
     if len(sizes_) == 1:
         for own in (True, False):
             oc, lc, _ = case.forward_chunked(5, want_chunk_lse=own)
