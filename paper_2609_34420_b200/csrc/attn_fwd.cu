@@ -1099,16 +1099,40 @@ int32_t chunks_in_turn(const gt_batch* b, int32_t n_heads, int32_t head_dim, int
 // Graphs and nodes each, heads of d: 64 of 16-300, 4 of 32: 25.7 -> 21.2 us; 200 of 64-1 000, 4 of 32: 217 -> 209; 20 of 1 000-1 100, 8 of 64:
 // 129 -> 120; but 64 of 512-2 048, 16 of 64: 1 035 -> 1 076, and where every block has an SM of its own: 8 of 500-600, 2 of 64: 14.9 -> 16.1.
 constexpr int32_t kPairMaxNodes = 1152;
-constexpr int kPairRegisters = 80;           // per thread at launch: what setmaxnreg shares out
+constexpr int kPairRegisters = 80;           // per thread at launch: what setmaxnreg shares out, which would wait forever for more than there are
+template <int D>
+auto pair_kernel(bool shfl, bool precise)
+{
+    if (precise) return shfl ? attn_fwd_kernel<D, false, true, true, 1, true> : attn_fwd_kernel<D, false, false, true, 1, true>;
+    return shfl ? attn_fwd_kernel<D, false, true, false, 1, true> : attn_fwd_kernel<D, false, false, false, 1, true>;
+}
+template <int D>
+bool pair_registers(bool shfl, bool precise)
+{
+    static std::atomic<int> registers[4] = {};               // as compiled (allocated in eights); 0: not asked yet
+    std::atomic<int>& known = registers[(shfl ? 1 : 0) + (precise ? 2 : 0)];
+    int n = known.load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaFuncAttributes a;
+        if (cudaFuncGetAttributes(&a, pair_kernel<D>(shfl, precise)) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        n = (a.numRegs + 7) / 8 * 8;
+        known.store(n, std::memory_order_relaxed);
+    }
+    return n >= kPairRegisters;
+}
 inline bool small_graphs(const gt_batch* b) { return b->n_graphs > 1 && b->max_seqlen <= kPairMaxNodes; }
 inline size_t fwd_workspace(const gt_batch* b, int32_t n_heads, int32_t list_rows)
 {
     return kHeaderBytes + maps_bytes(b->n_graphs) + list_bytes(b, list_rows) + norms_bytes(b, n_heads);
 }
-// A workspace without room for a list by 128 rows is used as for large graphs.
-inline bool pairs_of_blocks(const gt_batch* b, int32_t n_heads, size_t workspace_bytes)
+// A workspace without room for a list by 128 rows is used as for large graphs, and so is everything if the kernel came out with too few registers.
+inline bool pairs_of_blocks(const gt_batch* b, int32_t n_heads, int32_t head_dim, int32_t n_buckets, bool precise, size_t workspace_bytes)
 {
-    return small_graphs(b) && rows_per_block(b, n_heads) == kRowsPerCta && workspace_bytes >= fwd_workspace(b, n_heads, kRowsPerTile);
+    return small_graphs(b) && rows_per_block(b, n_heads) == kRowsPerCta && workspace_bytes >= fwd_workspace(b, n_heads, kRowsPerTile) &&
+           (head_dim == 64 ? pair_registers<64>(n_buckets <= 32, precise) : pair_registers<32>(n_buckets <= 32, precise));
 }
 
 // Blocks that share a query tile's keys (cluster_split): a key tile takes 1.2 us, the cluster and the merge 2 to 3 us.  1 000 nodes, heads
@@ -1131,16 +1155,13 @@ gt_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
             if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1> : attn_fwd_kernel<D, false, false, true, 1>;
         }
         if (in_turn && rows == kRowsPerTile) kern = shfl ? attn_fwd_kernel<D, false, true, false, 1, false, true> : attn_fwd_kernel<D, false, false, false, 1, false, true>;
-        if (pair) {
-            kern = shfl ? attn_fwd_kernel<D, false, true, false, 1, true> : attn_fwd_kernel<D, false, false, false, 1, true>;
-            if (p.out_f32 != nullptr) kern = shfl ? attn_fwd_kernel<D, false, true, true, 1, true> : attn_fwd_kernel<D, false, false, true, 1, true>;
-        }
+        if (pair) kern = pair_kernel<D>(shfl, p.out_f32 != nullptr);
     }
     const size_t smem = pair ? FwdSmem<D, true>::kDynamic : FwdSmem<D>::kDynamic;
     static std::atomic<uint64_t> granted[16] = {};
     static ClusterFit max_clusters[4];
     const int form = (shfl ? 1 : 0) + (!kPartial && p.out_f32 ? 2 : 0);
-    const gt_status st = grant_smem(kern, granted[form + (in_turn ? (rows == kRowsPerTile ? 14 : 12) : pair ? 8 : rows == kRowsPerTile ? 4 : 0)], smem, pair ? kPairRegisters : 0);
+    const gt_status st = grant_smem(kern, granted[form + (in_turn ? (rows == kRowsPerTile ? 14 : 12) : pair ? 8 : rows == kRowsPerTile ? 4 : 0)], smem);
     if (st != GT_OK) return st;
     const int32_t row_blocks = grid_y > 0 ? grid_y : (batch->max_seqlen + rows - 1) / rows;
     dim3 grid = p.list ? dim3((unsigned)(list_entries(batch, rows) * p.n_heads))
@@ -1207,7 +1228,7 @@ extern "C" gt_status gt_biased_attn_fwd_ex(const void* q, const void* k, const v
     if ((st = encode_thd_map(&tv, v, batch->n_total, n_heads, head_dim)) != GT_OK) return st;
     CUtensorMap tspd = tq;                       // placeholder when the cp.async loader is used
     FwdParams p{};
-    const bool pair = pairs_of_blocks(batch, n_heads, workspace_bytes);
+    const bool pair = pairs_of_blocks(batch, n_heads, head_dim, max_dist + 2, out_f32 != nullptr, workspace_bytes);
     const int32_t list_rows = pair ? kRowsPerTile : kRowsPerCta;
     const int32_t rows = pair ? kRowsPerTile : rows_per_block(batch, n_heads);
     p.spd_tma = batch->n_graphs == 1 ? 1 : 0;

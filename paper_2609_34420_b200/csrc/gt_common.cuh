@@ -79,18 +79,12 @@ inline gt_status launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigne
 
 // Lets a kernel use up to `bytes` of dynamic shared memory, once per device: `granted` is that kernel's own (a bit per device),
 // `bytes` always the same, so it does not matter how many threads ask at once.
-// A kernel whose warps share out registers between them (setmaxnreg) would wait forever with fewer than it counts on: refused here.
 template <class Kernel>
-inline gt_status grant_smem(Kernel kernel, std::atomic<uint64_t>& granted, size_t bytes, int least_registers = 0)
+inline gt_status grant_smem(Kernel kernel, std::atomic<uint64_t>& granted, size_t bytes)
 {
     int dev = 0;
     GT_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 64 && ((granted.load(std::memory_order_relaxed) >> dev) & 1u)) return GT_OK;
-    if (least_registers > 0) {
-        cudaFuncAttributes a;
-        GT_CUDA_TRY(cudaFuncGetAttributes(&a, kernel));
-        if (a.numRegs < least_registers) return GT_ERR_UNSUPPORTED;
-    }
     GT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     if (dev < 64) granted.fetch_or(1ull << dev, std::memory_order_relaxed);
     return GT_OK;
