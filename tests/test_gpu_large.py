@@ -63,16 +63,22 @@ def run_large(name: str, n_slab: int, full_spd_oracle: bool):
     out, out_c = torch.empty_like(q), torch.empty_like(q)
     lse, lse_c = torch.empty(H, n, device=dev), torch.empty(H, n, device=dev)
     gt.gt_check(gt.gt_biased_attn_fwd(q, k, v, spd, bias, bt, D, out, lse))
-    gt.gt_check(gt.gt_biased_attn_fwd_chunked(q, k, v, spd, bias, bt, D, out_c, lse_c, max(w.n_kv_chunks, 2)))
-    assert rel_l2(to_f64(out_c), to_f64(out)) <= CHUNK_REL_L2
-    assert (lse_c - lse).abs().max().item() <= LSE_MAX_ABS
+    C = max(w.n_kv_chunks, 2)
+    lse_chunks = torch.empty(C, H, n, device=dev)
+    for own in (lse_chunks, None):             # each chunk in blocks of its own, then as the call likes best
+        gt.gt_check(gt.gt_biased_attn_fwd_chunked(q, k, v, spd, bias, bt, D, out_c, lse_c, C, own))
+        assert rel_l2(to_f64(out_c), to_f64(out)) <= CHUNK_REL_L2
+        assert (lse_c - lse).abs().max().item() <= LSE_MAX_ABS
+    assert (torch.logsumexp(lse_chunks, 0) - lse).abs().max().item() <= LSE_MAX_ABS
+    del lse_chunks
 
     f = wl.bf16_bits_to_f64
     qf, kf, vf, dof, bf = f(t.q), f(t.k), f(t.v), f(t.dout), t.bias.astype(np.float64)
     ro, rl = oattn.forward_single(qf, kf, vf, spd_rows, bf, rows=rows, compact_spd=True)
     rows_t = torch.from_numpy(rows).to(dev)
-    assert np.abs(to_f64(out[rows_t]) - ro).max() <= O_MAX_ABS
-    assert np.abs(to_f64(lse[:, rows_t]) - rl).max() <= LSE_MAX_ABS
+    for o, l in ((out, lse), (out_c, lse_c)):
+        assert np.abs(to_f64(o[rows_t]) - ro).max() <= O_MAX_ABS
+        assert np.abs(to_f64(l[:, rows_t]) - rl).max() <= LSE_MAX_ABS
 
     # ---- backward with dO restricted to the slab ----
     do_masked = torch.zeros_like(do)
@@ -94,7 +100,6 @@ def run_large(name: str, n_slab: int, full_spd_oracle: bool):
         assert (dq[mask].float().abs().max().item() == 0.0)
 
     # ---- chunked backward (same dO): equals the unchunked backward, chunk shares add up ----
-    C = max(w.n_kv_chunks, 2)
     dq_c, dk_c, dv_c = (torch.empty_like(q) for _ in range(3))
     dbias_c = torch.empty_like(bias)
     db_chunks = torch.empty((C,) + tuple(bias.shape), device=dev)
