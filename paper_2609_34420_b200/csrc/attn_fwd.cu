@@ -434,14 +434,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint32_t pair_bar = kNbPair + t * 4 + (warp & 3);
         float* xchg = (float*)(smem + L::kXchg) + t * 512;
         float m = 0.f, l = 0.f;
-        // Precise variant: the reference of this warp's rows may differ from 0; nothing is subtracted where it cannot (8 192 nodes, 8 heads of 64:
-        // 255 -> 242 us; the other one gains 1 % by a pass of its own for that and loses 2 % to 3 % where references differ).
-        [[maybe_unused]] bool m_moved = false;
+        // A form of the pass without the subtraction, for warps whose references are all 0.  8 192 nodes, 8 heads of 64, fp32 output: 255 -> 242 us; heads
+        // of 32: 16 384 nodes, 4 heads 424 -> 409, 64 graphs of 512-2 048 nodes, 16 heads 955 -> 938.  Heads of 64 gain 1 % at 0 (217.2 -> 215.3) and
+        // lose 2 % where references differ (223 -> 228), two blocks per SM lose either way (195 -> 198, 209 -> 217).
+        constexpr bool kOwnFormAtZero = kPrecise || (D == 32 && !kPair);
+        [[maybe_unused]] bool m_moved = false;             // some reference of this warp may not be 0
         // kFold: O and l are of the chunk at work; what the chunks before add up to is in memory and, {reference, l}, in `sums`
         [[maybe_unused]] int next_chunk = p.chunk_tiles;
         [[maybe_unused]] float2* sums = (float2*)(smem + L::kSums) + (kFold ? tid - 128 : 0);
-        [[maybe_unused]] auto o_sum = [&](int i) -> float4* {       // of four channels of this thread's row
-            return (float4*)p.chunk_sums + ((size_t)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (kOC / 4) + i) * (256 * kTiles) + (tid - 128);
+        constexpr int kSumStep = 256 * kTiles;
+        [[maybe_unused]] auto o_sum = [&]() -> float4* {            // of this thread's row, four channels every kSumStep
+            uint32_t x, y, z, at;               // (by asm: nothing of the address is to be kept in registers through the loop, which costs 2 %)
+            asm volatile("mov.u32 %0, %%ctaid.x; mov.u32 %1, %%ctaid.y; mov.u32 %2, %%ctaid.z; mov.u32 %3, %%tid.x;" : "=r"(x), "=r"(y), "=r"(z), "=r"(at));
+            return (float4*)p.chunk_sums + ((size_t)((z * gridDim.y + y) * gridDim.x + x) * (kOC / 4)) * kSumStep + (at - 128);
         };
 
         // lane b of every softmax warp keeps table entry b (scaled by log2 e); entries past the
@@ -636,7 +641,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     tmem_wait_ld(); exp_chunk(3, sb, wb, rag, ref);
                 };
                 if (ragged) exp_pass(BoolTag<true>{}, BoolTag<true>{});
-                else if (!kPrecise || m_moved) exp_pass(BoolTag<false>{}, BoolTag<true>{});
+                else if (!kOwnFormAtZero || m_moved) exp_pass(BoolTag<false>{}, BoolTag<true>{});
                 else exp_pass(BoolTag<false>{}, BoolTag<false>{});
                 loaded = false;
                 {
@@ -652,14 +657,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarSpdEmpty + (j % kSpdStages)));
-            if constexpr (kFold) {
-                if (j == next_chunk) {
-                    if (j > p.chunk_tiles) l += sums->y * ex2_approx(sums->x - m);
-                    sums->y = l;
-                    l = 0.f;
-                }
-            }
-            l += tile_sum;
+            if constexpr (!kFold) l += tile_sum;
 
             // P over the first half of this thread's own score columns
             if constexpr (!kPrecise) {
@@ -671,29 +669,33 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (j == next_chunk) {          // the chunk before joins the sum; PV(j) then overwrites it
                     mbar_wait(bar(kBarODone + 2 * t + ((j - 1) & 1)), ((j - 1) >> 1) & 1, abort_flag, p.status, 44);
                     tc_fence_after();
+                    float4* const sum = o_sum();
                     uint32_t o[kOC];
                     tmem_ld<kOC>(tO, o);
                     tmem_wait_ld();
                     if (j == p.chunk_tiles) {
 #pragma unroll
-                        for (int i = 0; i < kOC / 4; ++i) *(uint4*)o_sum(i) = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                        for (int i = 0; i < kOC / 4; ++i) *(uint4*)&sum[i * kSumStep] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                     } else {
                         const float m_sum = sums->x;
                         if (__any_sync(0xffffffffu, m != m_sum)) {
                             const float w = ex2_approx(m_sum - m);
 #pragma unroll 1
                             for (int i = 0; i < kOC / 4; ++i) {
-                                float4 a = __ldcg(o_sum(i));
+                                float4 a = __ldcg(&sum[i * kSumStep]);
                                 a.x *= w; a.y *= w; a.z *= w; a.w *= w;
-                                *o_sum(i) = a;
+                                sum[i * kSumStep] = a;
                             }
                         }
 #pragma unroll
-                        for (int i = 0; i < kOC / 4; ++i) red_add_f32x4(o_sum(i), o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                        for (int i = 0; i < kOC / 4; ++i) red_add_f32x4(&sum[i * kSumStep], o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                     }
-                    sums->x = m;
+                    if (j > p.chunk_tiles) l += sums->y * ex2_approx(sums->x - m);
+                    *sums = make_float2(m, l);
+                    l = 0.f;
                     next_chunk += p.chunk_tiles;
                 }
+                l += tile_sum;
             }
             tc_fence_before();
             // Warps of a tile can be one step apart (nothing in the speculative pass waits for the
@@ -774,7 +776,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             if (summed) {
 #pragma unroll
                 for (int i = 0; i < kOP / 4; ++i) {
-                    const float4 a = __ldcg(o_sum(c * (kOP / 4) + i));
+                    const float4 a = __ldcg(&o_sum()[(c * (kOP / 4) + i) * kSumStep]);
                     o[4 * i] = __float_as_uint(__uint_as_float(o[4 * i]) + w_sum * a.x);
                     o[4 * i + 1] = __float_as_uint(__uint_as_float(o[4 * i + 1]) + w_sum * a.y);
                     o[4 * i + 2] = __float_as_uint(__uint_as_float(o[4 * i + 2]) + w_sum * a.z);
@@ -786,7 +788,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     float4* dst = (float4*)(p.part_o + (((size_t)chunk * p.n_total + q) * p.n_heads + h) * D + hf * kOC + c * kOP);
 #pragma unroll
                     for (int i = 0; i < kOP / 4; ++i)
-                        *(kFold ? o_sum(c * (kOP / 4) + i) : &dst[i]) = make_float4(__uint_as_float(o[4 * i]) * inv_l, __uint_as_float(o[4 * i + 1]) * inv_l,
+                        *(kFold ? &o_sum()[(c * (kOP / 4) + i) * kSumStep] : &dst[i]) = make_float4(__uint_as_float(o[4 * i]) * inv_l, __uint_as_float(o[4 * i + 1]) * inv_l,
                                              __uint_as_float(o[4 * i + 2]) * inv_l, __uint_as_float(o[4 * i + 3]) * inv_l);
                 } else {
                     uint4* dst = (uint4*)(p.out + ((size_t)(node0 + q) * p.n_heads + h) * D + hf * kOC + c * kOP);
@@ -1070,8 +1072,8 @@ inline int32_t rows_per_block(const gt_batch* b, int32_t n_heads)
 // fewer shares to merge; more blocks fill the grid's last wave better.  `room`: floats in the workspace for the shares.  A 256 x 128 tile
 // takes 1.50 to 1.61 us (heads of 32 and of 64), a 128 x 128 tile 1.0 where all blocks are of one, a block's fill and drain 7, an addition
 // to the sums 0.9 to 2.5, the merge 3 and its bytes (5 TB/s).  us with every chunk in blocks of its own -> by this rule, 8 chunks: 8 heads of
-// 64: 4 096 nodes 109 -> 65 (one share), 10 000 nodes 460 -> 370 (two), 65 536 nodes 13 700 -> 13 300 (one); 4 heads: 6 000 nodes 109 -> 77
-// (three), 4 096 nodes, 5 chunks 62 -> 45 (one-tile blocks); 5 000 nodes, 5 chunks stay with 68 (98 in one share).
+// 64: 4 096 nodes 110 -> 66 (one share), 10 000 nodes 466 -> 380 (two), 65 536 nodes 14 060 -> 13 660 (one); 4 heads: 6 000 nodes 111 -> 78
+// (three), 4 096 nodes 62 -> 42 (one-tile blocks); 5 000 nodes, 5 chunks stay with 69 (98 in one share).
 int32_t chunks_in_turn(const gt_batch* b, int32_t n_heads, int32_t head_dim, int32_t n_chunks, int32_t chunk_tiles, size_t room)
 {
     const int64_t n = b->n_total, sms = sm_count(), blocks = (n + kRowsPerCta - 1) / kRowsPerCta * n_heads, tiles = (n + kKvTile - 1) / kKvTile;
