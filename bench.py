@@ -48,7 +48,7 @@ BWD_KERNEL_DRAM_BYTES_PER_N2 = 1037.7e6 / (16384.0 ** 2)
 # The same for the forward kernel (16 384 nodes) and for the bit-matrix SPD build (32 768 nodes, search and expansion
 # together; its traffic also grows with the number of BFS levels, so the scaled figure is an estimate).
 FWD_KERNEL_DRAM_BYTES_PER_N2 = 438.1e6 / (16384.0 ** 2)
-SPD_DENSE_DRAM_BYTES_PER_N2 = 2.300e9 / (32768.0 ** 2)
+SPD_DENSE_DRAM_BYTES_PER_N2 = 2.262e9 / (32768.0 ** 2)
 
 
 def load_peaks():

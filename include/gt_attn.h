@@ -100,10 +100,13 @@ gt_status gt_check(void* workspace, void* stream);
  * 4 bytes per node, bit of max_dist + 1 and thread block in flight (up to two per SM; 24 MB at 8 192 nodes; below 14 500 nodes a
  * call that is handed 4 n_total + 1 024 bytes does without, more slowly); a larger single graph, or one of 14 500 nodes or
  * more with over 32 edges per node, what the bit matrices of its traversal need: about 8 KB per node
- * for each of min(4, ceil(n/8192)) groups of thread blocks (eight bit matrices of 1 KB rows per group: visited, and one
- * frontier per level up to 6; later levels reuse two of them) plus 1 KB per 33 edges per group (rows for vertices with more
- * than 32 out-edges) and 16 bytes per 32 edges -- 2.2 GB at 65 536 nodes with 786 000 edges -- and a device that supports
- * cooperative launches; other batches with a larger graph: 4(G+1) + 4 n_total + 4 G bytes (per-graph offsets, and the
+ * for each of min(4, ceil(n/8192)) groups of thread blocks (bit matrices of 1 KB rows: visited, and the frontiers of seven
+ * levels, two of which later levels use again) plus 1 KB per 33 edges per group (rows for vertices with more
+ * than 32 out-edges) and 16 bytes per 32 edges, and a device that supports cooperative launches.  From 32 768 to 65 536 nodes,
+ * where the build may search for part of the targets only, 13 bytes per node and group and 45 per node more, and beyond 46 811 nodes
+ * everything but the frontiers for a fifth group: 2.34 GB at 65 536 nodes with 786 000 edges; a call that is handed what the search
+ * for all targets takes (2.25 GB) searches for all, more slowly.  Until the build is done spd_out may hold parts of its state.
+ * Other batches with a larger graph: 4(G+1) + 4 n_total + 4 G bytes (per-graph offsets, and the
  * connected-component label of every node: the search of an undirected graph without a vertex of more than 64 out-edges
  * stops at level max_dist), and beyond 17 066 nodes 12 bytes per node of the largest graph for each of up to
  * 2 x (number of SMs) thread blocks.
@@ -181,8 +184,8 @@ void gt_test_hook_barrier_overcount(int32_t extra);
  * accumulation and softmax, bf16 `out` [T,H,d], fp32 `lse` [H,T].
  * bias: fp32 [n_heads, max_dist+2].
  * Workspace: 256 bytes, 4 bytes per head and 256 rows (norms of the keys, for the fp32 output), and for a packed batch 128 bytes per
- * graph (descriptors of the SPD blocks) and 16 bytes per graph and per 256 rows (a list of the work); a call that is handed the
- * 256 bytes alone does without all of it, more slowly.
+ * graph (descriptors of the SPD blocks) and 16 bytes per graph and per 256 rows (a list of the work; per 128 rows where no graph has more
+ * than 1 152 nodes).  A call that is handed room for the list by 256 rows, or the 256 bytes alone, does without the rest, more slowly.
  * ------------------------------------------------------------------------------------- */
 size_t gt_biased_attn_fwd_workspace(const gt_batch* batch, int32_t n_heads, int32_t head_dim);
 gt_status gt_biased_attn_fwd(const void* q, const void* k, const void* v,
@@ -337,6 +340,7 @@ gt_status gt_biased_attn_bwd_step_finish(const float* dq_acc, const float* dk_ac
  * merged:  lse = log sum_c exp(lse_c),  out = sum_c exp(lse_c - lse) out_c.
  * Unless lse_chunks is given, the same thread blocks may take several consecutive chunks, with the running softmax state on the
  * chip and their partials added up in fp32; that fills the GPU better or worse than blocks for every chunk, by its size.
+ * Workspace in every case: 256 bytes and, per row, head and chunk, head_dim + 1 floats.
  * Results equal gt_biased_attn_fwd up to rounding.  Single graph only (n_graphs == 1).
  * lse_chunks: optional fp32 [n_kv_chunks, H, N] receiving lse_c (-inf for empty chunks), or NULL.
  * ------------------------------------------------------------------------------------- */

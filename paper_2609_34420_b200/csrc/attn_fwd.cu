@@ -25,8 +25,8 @@
 // tile is redone the classical way (maximum, rescale of l and O, exponentials).  References are integers in log2
 // units, so rescale factors are exact powers of two (a P entry depends on the reference in the rounding of its exponent's
 // argument only).  They start at 0, as scores are mostly within some powers of two of 1; a few scores of the first tile tell where they
-// are not.  With the first tile's maximum always taken first -> so: 4 096 nodes, 8 heads of 64: 59.5 -> 57.9 us, 64 graphs of 512-2 048
-// nodes, 16 heads: 1 078 -> 1 028; all scores shifted by -40, which the classical first tile costs: 59.3 -> 58.6, 1 061 -> 1 051.
+// are not.  With the first tile's maximum always taken first, and the first loads behind the set-up -> now: 4 096 nodes, 8 heads of 64:
+// 59.4 -> 58.6 us, 64 graphs of 512-2 048 nodes, 16 heads: 1 052 -> 1 019; all scores shifted by -40: 60.7 -> 60.8, 1 088 -> 1 085.
 //
 // TMEM columns: three score buffers [0,128) [128,256) [256,384) used in rotation by the steps
 // (key tile j, query tile t) -> buffer (2j+t) mod 3, so that the S MMA of a step never waits for a
@@ -270,7 +270,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     if (warp == 1) { tmem_alloc(smem_u32(&misc[0]), kTmemCols); tmem_relinquish(); }
     grid_wait();
     // The first tiles are on their way while the block is still setting up: the thread that set up the barriers is the one that loads.
-    // (4 096 nodes, 8 heads: 59.4 -> 57.6 us, a packed batch of 64 graphs 1 033 -> 1 007.)
     const void* spd_map = !kPartial && p.maps ? (const void*)(p.maps + (size_t)g * kMapBytes) : &tmap_spd;
     auto load_k = [&](int j) {
         const int s = j % kKStages;

@@ -20,7 +20,7 @@
 // shifts, which has half the rate, in the edge lists' making and in the output.  One graph of 4 096 nodes, clocks of a block:
 // order and lists 19k, state 4k, five passes 39k, output 13k of 79k.  The lists' offsets by all warps, groups of vertices in turns that
 // go back and forth (they come by falling degree), lanes of finished vertices left out, and no work on planes and codes that a graph
-// does not have: 41.5 -> 37.7 us, a packed batch of 64 graphs of 512 to 2 048 nodes 277 -> 263 us.
+// does not have: 41.1 -> 38.4 us, a packed batch of 64 graphs of 512 to 2 048 nodes 291 -> 278 us.
 #include "spd_pull.cuh"
 
 namespace gt {
