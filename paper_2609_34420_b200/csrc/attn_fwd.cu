@@ -6,8 +6,8 @@
 // back to tensor memory as the A operand of the P V MMA.
 //
 // One CTA = one head x 256 query rows (two 128-row tiles, so the tensor pipe works on one tile
-// while the other is in its softmax) x all key tiles of the graph (or of one key chunk for the
-// chunked entry point).
+// while the other is in its softmax) x all key tiles of the graph (or of one key chunk, or several behind one
+// another, for the chunked entry point).
 //
 //   warp 0      TMA producer: Q once; K and V through separate 2-stage rings; on a single graph
 //               also the 256x128-byte SPD tile (3-stage ring, 128-byte swizzle)
